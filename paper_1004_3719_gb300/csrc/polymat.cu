@@ -6,16 +6,32 @@
 // arrays: A[k][i][j] is the coefficient of x^k in entry (i, j).
 //
 // F_p itself has roots of unity of order at most 16 when p = 65521, so the
-// transforms run over three primes with large power-of-two roots instead: the
-// exact integer coefficients of C are below s * (min(da, db) + 1) * (p-1)^2
-// < P0 P1 P2, so C is computed modulo each of
-// them by number-theoretic transforms (length L, the power of two >= da+db+1;
-// one CTA per polynomial, in shared memory), a pointwise s x s matrix product
-// at each of the L points, and the inverse transforms, then brought back to
-// Z/pZ by Garner's mixed-radix reconstruction.  Forward transforms are
-// decimation in frequency (natural order in, bit-reversed out) and the inverse
-// ones decimation in time (bit-reversed in, natural out), so no permutation
-// pass is needed; the pointwise products do not care about the order.
+// transforms run over primes with large power-of-two roots instead: the
+// exact integer coefficients of C are below s * (min(da, db) + 1) * (p-1)^2,
+// so C is computed modulo as many primes as that bound needs (one, two or
+// three: two for p = 65521 at every length, three for p near 2^31), by
+// number-theoretic transforms of length L (a power of two >= da+db+1), a
+// pointwise matrix product at each of the L points, and the inverse
+// transforms, then brought back to Z/pZ by Garner's mixed-radix
+// reconstruction.
+//
+// Layout.  Every array stays point-major, [prime][point][entry]: the entries
+// of one matrix are contiguous, like the coefficients that come in and go
+// out.  A transform works on all entries at once, one (entry, column) item
+// per lane, so that every global access of a warp is 32 consecutive words
+// whatever the matrix size; nothing is transposed.  L = L1 L2: a first
+// kernel transforms along k1 (k = k1 L2 + k2, stride L2) and multiplies by
+// the cross twiddles w^(j1 k2), a second along k2; the inverse runs the same
+// two axes backwards, so the frequencies are never reordered.  L <= 256
+// takes one kernel each way.  One tile is up to 256 points x 32 items: two
+// register transforms of up to 16 points per thread with one exchange
+// through shared memory between them.
+//
+// What bounds it: at s = 16, degree 6250 (L = 16384, two primes) the planes
+// of A, B and C are 33.5 MB each, and each is written and read twice; the
+// butterflies (about 7 instructions each on values kept in [0, 2P)) are the
+// rest.  Measured with the former one-polynomial-per-CTA radix-2 kernels over
+// three primes: 1170 us per product; with these: 148 us.
 #include <algorithm>
 #include <cstring>
 
@@ -26,212 +42,517 @@ namespace ff {
 namespace {
 
 constexpr int kPmPrimes = 3;
-constexpr u32 kPmP[kPmPrimes] = {998244353u, 167772161u, 469762049u};  // c 2^k + 1, k = 23, 25, 26
+constexpr u32 kPmP0 = 998244353u, kPmP1 = 469762049u, kPmP2 = 167772161u;  // c 2^k + 1, k = 23, 26, 25
+constexpr u32 kPmP[kPmPrimes] = {kPmP0, kPmP1, kPmP2};
 constexpr u32 kPmGen = 3;                                            // a primitive root of each
-constexpr int kPmMaxLog = 15;                                        // L <= 2^15: 128 KB of shared memory
-constexpr int kNttThreads = 512;
+constexpr int kPmMaxLog = 15;
+constexpr int kPmMinLog = 4;
+constexpr int kPmLanes = 32;                                         // items per tile
 
-struct PmConsts {
-    Mod P[kPmPrimes];
-    u32 root[kPmPrimes], iroot[kPmPrimes], linv[kPmPrimes], linv_q[kPmPrimes];
-    int reduce_input;    // p > the smallest prime: inputs need a reduction mod P_q
-    Mod mp;              // the output modulus p
-    u32 inv01, inv02, inv12;  // P0^-1 mod P1, P0^-1 mod P2, P1^-1 mod P2
-    u32 p0_mod_p, p0p1_mod_p;
+// ---------------------------------------------------------------------------
+// Roots of unity, computed by the compiler.
+struct alignas(8) PmW {
+    u32 w, q;  // a constant and floor(w 2^32 / P), its Shoup quotient
 };
 
-__device__ __forceinline__ u32 mulm(u32 a, u32 b, const Mod &M) { return red64((u64)a * b, M); }
-
-// a * w mod P for a fixed w with wq = floor(w 2^32 / P), P < 2^31 (Shoup): the
-// quotient estimate umulhi(a, wq) is the true quotient or one less, so the
-// 32-bit remainder lies in [0, 2P).
-__device__ __forceinline__ u32 mul_shoup(u32 a, u32 w, u32 wq, u32 P)
-{
-    const u32 r = a * w - __umulhi(a, wq) * P;
-    return r >= P ? r - P : r;
-}
-
-__device__ u32 powm(u32 a, u32 e, const Mod &M)
-{
-    u32 r = 1u % M.m;
-    while (e) {
-        if (e & 1u) r = mulm(r, a, M);
-        a = mulm(a, a, M);
-        e >>= 1;
-    }
-    return r;
-}
-
-// tw[q][0][i] = (root_q^i, its Shoup quotient), tw[q][1][i] the same for root_q^-i, i < L/2
-__global__ void k_pm_twiddles(uint2 *tw, int L, const __grid_constant__ PmConsts c)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int h = L / 2;
-    if (t >= (long long)kPmPrimes * 2 * h) return;
-    const int i = (int)(t % h), dir = (int)(t / h % 2), q = (int)(t / (2 * h));
-    const u32 w = powm(dir ? c.iroot[q] : c.root[q], (u32)i, c.P[q]);
-    tw[t] = make_uint2(w, (u32)(((u64)w << 32) / c.P[q].m));
-}
-
-// dst[q][e][k] = src[k][e] mod P_q for k <= d, 0 up to L = 2^lg (all indices
-// below 2^31: 3 * 32^2 * 2^15 entries at most)
-__global__ void k_pm_load(const u32 *__restrict__ src, long long d, int s2, int lg, u32 *__restrict__ dst,
-                          const __grid_constant__ PmConsts c)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= kPmPrimes * s2 << lg) return;
-    const int k = t & ((1 << lg) - 1), qe = t >> lg;
-    const int e = qe % s2, q = qe / s2;
-    const u32 v = k <= d ? src[(long long)k * s2 + e] : 0u;
-    dst[t] = c.reduce_input ? v % c.P[q].m : v;
-}
-
-// One polynomial of length L per CTA, transformed in shared memory.
-template <bool INV>
-__global__ void __launch_bounds__(kNttThreads) k_ntt(u32 *__restrict__ data, int L, int s2, const uint2 *__restrict__ tw,
-                                                     const __grid_constant__ PmConsts c)
-{
-    extern __shared__ u32 a[];
-    const int q = blockIdx.x / s2;
-    const u32 P = c.P[q].m;
-    const uint2 *w = tw + ((size_t)q * 2 + (INV ? 1 : 0)) * (L / 2);
-    u32 *g = data + (size_t)blockIdx.x * L;
-    for (int i = threadIdx.x; i < L; i += kNttThreads) a[i] = g[i];
-    __syncthreads();
-    const int h = L / 2;
-    if (!INV) {
-        for (int lgl = __ffs(h) - 1; lgl >= 0; --lgl) {  // decimation in frequency, len = 2^lgl
-            const int len = 1 << lgl, step = h >> lgl;
-            for (int b0 = threadIdx.x; b0 < h; b0 += 8 * kNttThreads) {
-                uint2 wv[8];  // this thread's twiddles, all requested before any is used
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int b = b0 + u * kNttThreads;
-                    wv[u] = b < h ? __ldg(w + (b & (len - 1)) * step) : make_uint2(0u, 0u);
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int b = b0 + u * kNttThreads;
-                    if (b >= h) break;
-                    const int j = b & (len - 1), i0 = ((b >> lgl) << (lgl + 1)) + j, i1 = i0 + len;
-                    const u32 x0 = a[i0], x1 = a[i1];
-                    a[i0] = x0 + x1 >= P ? x0 + x1 - P : x0 + x1;
-                    a[i1] = mul_shoup(x0 >= x1 ? x0 - x1 : x0 + P - x1, wv[u].x, wv[u].y, P);
-                }
-            }
-            __syncthreads();
-        }
-        for (int i = threadIdx.x; i < L; i += kNttThreads) g[i] = a[i];
-    } else {
-        for (int lgl = 0; (1 << lgl) <= h; ++lgl) {  // decimation in time, len = 2^lgl
-            const int len = 1 << lgl, step = h >> lgl;
-            for (int b0 = threadIdx.x; b0 < h; b0 += 8 * kNttThreads) {
-                uint2 wv[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int b = b0 + u * kNttThreads;
-                    wv[u] = b < h ? __ldg(w + (b & (len - 1)) * step) : make_uint2(0u, 0u);
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int b = b0 + u * kNttThreads;
-                    if (b >= h) break;
-                    const int j = b & (len - 1), i0 = ((b >> lgl) << (lgl + 1)) + j, i1 = i0 + len;
-                    const u32 x0 = a[i0], x1 = mul_shoup(a[i1], wv[u].x, wv[u].y, P);
-                    a[i0] = x0 + x1 >= P ? x0 + x1 - P : x0 + x1;
-                    a[i1] = x0 >= x1 ? x0 - x1 : x0 + P - x1;
-                }
-            }
-            __syncthreads();
-        }
-        for (int i = threadIdx.x; i < L; i += kNttThreads) g[i] = mul_shoup(a[i], c.linv[q], c.linv_q[q], P);
-    }
-}
-
-// Ch[q][i s + j][t] = sum_k Ah[q][i s + k][t] Bh[q][k s + j][t] mod P_q.  A CTA
-// takes TP consecutive points of one prime: the s x s matrices of A and B at
-// those points are read once into shared memory, [entry][point], and every
-// output is formed there.
-constexpr int kPwThreads = 256;
-
-__global__ void __launch_bounds__(kPwThreads) k_pm_pointwise(const u32 *__restrict__ Ah, const u32 *__restrict__ Bh,
-                                                            u32 *__restrict__ Ch, int s, int L, int lgtp,
-                                                            const __grid_constant__ PmConsts c)
-{
-    const int TP = 1 << lgtp;
-    extern __shared__ u32 pw[];
-    const int s2 = s * s;
-    u32 *As = pw, *Bs = pw + (size_t)s2 * TP;
-    const int nblk = (L + TP - 1) / TP;
-    const int q = blockIdx.x / nblk, t0 = (blockIdx.x % nblk) * TP;
-    const int tp = min(TP, L - t0);
-    const Mod &M = c.P[q];
-    const u32 *ag = Ah + (size_t)q * s2 * L + t0, *bg = Bh + (size_t)q * s2 * L + t0;
-    for (int idx = threadIdx.x; idx < s2 * TP; idx += kPwThreads) {
-        const int e = idx >> lgtp, tt = idx & (TP - 1);
-        As[idx] = tt < tp ? ag[(size_t)e * L + tt] : 0u;
-        Bs[idx] = tt < tp ? bg[(size_t)e * L + tt] : 0u;
-    }
-    __syncthreads();
-    u32 *cg = Ch + (size_t)q * s2 * L + t0;
-    for (int o = threadIdx.x; o < s2 * TP; o += kPwThreads) {
-        const int e = o >> lgtp, tt = o & (TP - 1);
-        if (tt >= tp) continue;
-        const int i = e / s, j = e % s;
-        const u32 *ar = As + (size_t)i * s * TP + tt, *bc = Bs + (size_t)j * TP + tt;
-        u64 acc = 0;
-        u32 r = 0;
-        for (int k = 0; k < s; ++k) {
-            acc += (u64)ar[(size_t)k * TP] * bc[(size_t)k * s * TP];  // each below 2^60
-            if ((k & 7) == 7) {
-                r = red64((u64)r + red64(acc, M), M);
-                acc = 0;
-            }
-        }
-        cg[(size_t)e * L + tt] = red64((u64)r + red64(acc, M), M);
-    }
-}
-
-// C[k][e] = the integer with residues Ch[0..2][e][k], mod p (Garner)
-__global__ void k_pm_crt(const u32 *__restrict__ Ch, u32 *__restrict__ C, long long dc, int s2, int L,
-                         const __grid_constant__ PmConsts c)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int)(dc + 1) * s2) return;
-    const int e = t % s2, k = t / s2;
-    const size_t plane = (size_t)s2 * L;
-    const u32 r0 = Ch[(size_t)e * L + k], r1 = Ch[plane + (size_t)e * L + k], r2 = Ch[2 * plane + (size_t)e * L + k];
-    const Mod &M1 = c.P[1], &M2 = c.P[2];
-    const u32 x1 = r0;                                           // < P0
-    const u32 x1m1 = x1 % M1.m, x1m2 = x1 % M2.m;
-    const u32 x2 = mulm(r1 >= x1m1 ? r1 - x1m1 : r1 + M1.m - x1m1, c.inv01, M1);  // < P1
-    u32 t3 = mulm(r2 >= x1m2 ? r2 - x1m2 : r2 + M2.m - x1m2, c.inv02, M2);
-    const u32 x2m2 = x2 % M2.m;
-    t3 = t3 >= x2m2 ? t3 - x2m2 : t3 + M2.m - x2m2;
-    const u32 x3 = mulm(t3, c.inv12, M2);                        // < P2
-    // value = x1 + P0 x2 + P0 P1 x3, reduced mod p term by term
-    const Mod &mp = c.mp;
-    u64 v = (u64)(x1 % mp.m) + red64((u64)c.p0_mod_p * x2, mp) + red64((u64)c.p0p1_mod_p * x3, mp);
-    C[(size_t)k * s2 + e] = red64(v, mp);
-}
-
-u32 powmod_host(u64 a, u64 e, u64 m)
+constexpr u32 pm_pow(u64 a, u64 e, u64 m)
 {
     u64 r = 1 % m;
     a %= m;
     while (e) {
-        if (e & 1) r = (unsigned __int128)r * a % m;
-        a = (unsigned __int128)a * a % m;
+        if (e & 1) r = r * a % m;   // m < 2^30
+        a = a * a % m;
         e >>= 1;
     }
     return (u32)r;
 }
 
-int pm_log2(long long da, long long db)
+constexpr u32 pm_inv32(u32 m)  // m^-1 mod 2^32, m odd (Newton)
 {
-    int lg = 0;
-    while ((1LL << lg) < da + db + 1) ++lg;
-    return std::max(lg, 1);
+    u32 y = m;
+    for (int i = 0; i < 4; ++i) y *= 2u - m * y;
+    return y;
+}
+
+constexpr u32 pm_root(int q, int lg) { return pm_pow(kPmGen, (kPmP[q] - 1) >> lg, kPmP[q]); }
+
+constexpr PmW pm_w(u64 w, u64 P) { return PmW{(u32)w, (u32)((w << 32) / P)}; }
+
+struct PmConstTab {
+    PmW w16[2][kPmPrimes][8];     // powers of the 16th root and of its inverse
+    PmW w256[kPmPrimes][256];     // powers of the 256th root
+};
+
+constexpr PmConstTab pm_make_const()
+{
+    PmConstTab t{};
+    for (int q = 0; q < kPmPrimes; ++q) {
+        const u64 P = kPmP[q];
+        for (int dir = 0; dir < 2; ++dir) {
+            const u64 r = dir ? pm_pow(pm_root(q, 4), P - 2, P) : pm_root(q, 4);
+            u64 w = 1;
+            for (int i = 0; i < 8; ++i) {
+                t.w16[dir][q][i] = pm_w(w, P);
+                w = w * r % P;
+            }
+        }
+        u64 w = 1;
+        const u64 r = pm_root(q, 8);
+        for (int i = 0; i < 256; ++i) {
+            t.w256[q][i] = pm_w(w, P);
+            w = w * r % P;
+        }
+    }
+    return t;
+}
+
+// Powers of the 2^15-th root w in Montgomery form: w^(256 h) at hi[h], w^l at
+// lo[l]; w^i is the Montgomery product of two entries.
+struct PmCrossTab {
+    u32 hi[kPmPrimes][128], lo[kPmPrimes][256];
+};
+
+constexpr PmCrossTab pm_make_cross()
+{
+    PmCrossTab t{};
+    for (int q = 0; q < kPmPrimes; ++q) {
+        const u64 P = kPmP[q], R = ((u64)1 << 32) % P;
+        u64 w = R, r = pm_root(q, 7);
+        for (int i = 0; i < 128; ++i) {
+            t.hi[q][i] = (u32)w;
+            w = w * r % P;
+        }
+        w = R;
+        r = pm_root(q, 15);
+        for (int i = 0; i < 256; ++i) {
+            t.lo[q][i] = (u32)w;
+            w = w * r % P;
+        }
+    }
+    return t;
+}
+
+__constant__ const PmConstTab c_pm = pm_make_const();
+__device__ const PmCrossTab d_pm_cross = pm_make_cross();
+
+// ---------------------------------------------------------------------------
+// Arithmetic mod P < 2^30 on lazy values in [0, 2P).
+__device__ __forceinline__ u32 pm_csub(u32 x, u32 m) { return min(x, x - m); }  // x < 2m: x mod m up to m
+
+// a w mod P in [0, 2P) for any 32-bit a and a fixed w < P (Shoup): the
+// quotient estimate umulhi(a, q) is the true quotient or one less.
+__device__ __forceinline__ u32 pm_shoup(u32 a, u32 w, u32 q, u32 P) { return a * w - __umulhi(a, q) * P; }
+
+// hi 2^32 + lo, times 2^-32, mod P (Montgomery, 1985): in [0, P + hi] without
+// overflow when hi + P < 2^32.
+__device__ __forceinline__ u32 pm_redc(u32 lo, u32 hi, u32 P, u32 pinv) { return hi + P - __umulhi(lo * pinv, P); }
+
+// a b 2^-32 mod P in [0, 2P), for a < 2^32 and b < P
+__device__ __forceinline__ u32 pm_mont(u32 a, u32 b, u32 P, u32 pinv)
+{
+    const u64 t = (u64)a * b;
+    return pm_redc((u32)t, (u32)(t >> 32), P, pinv);
+}
+
+struct PmPrime {
+    u32 P, pinv, mu;  // mu = floor(2^32 / P)
+};
+
+__device__ __forceinline__ PmPrime pm_prime(int q)
+{
+    PmPrime r;
+    r.P = q == 0 ? kPmP0 : q == 1 ? kPmP1 : kPmP2;
+    constexpr u32 i0 = pm_inv32(kPmP0), i1 = pm_inv32(kPmP1), i2 = pm_inv32(kPmP2);
+    constexpr u32 m0 = (u32)(((u64)1 << 32) / kPmP0), m1 = (u32)(((u64)1 << 32) / kPmP1),
+                  m2 = (u32)(((u64)1 << 32) / kPmP2);
+    r.pinv = q == 0 ? i0 : q == 1 ? i1 : i2;
+    r.mu = q == 0 ? m0 : q == 1 ? m1 : m2;
+    return r;
+}
+
+// v < 2^bits with its bits reversed, bits <= 4
+__host__ __device__ constexpr int pm_bitrev(int v, int bits)
+{
+    return ((v & 1) << 3 | (v & 2) << 1 | (v & 4) >> 1 | (v & 8) >> 3) >> (4 - bits);
+}
+
+// Stages ST, ST - 1, ..., 0 of a decimation in frequency over 2^LOG points in
+// registers: X_j ends at register bitrev(j).  Values in and out in [0, 2P).
+template <int LOG, int ST, bool INV>
+__device__ __forceinline__ void pm_stages(u32 (&x)[1 << LOG], int q, u32 P)
+{
+    constexpr int len = 1 << ST;
+    const u32 P2 = 2u * P;
+#pragma unroll
+    for (int h = 0; h < (1 << LOG) / 2; ++h) {
+        const int i = h & (len - 1), k = ((h >> ST) << (ST + 1)) + i;
+        const u32 u = x[k], v = x[k + len], d = u - v + P2;
+        x[k] = pm_csub(u + v, P2);
+        if (i == 0) {
+            x[k + len] = pm_csub(d, P2);
+        } else {
+            const PmW w = c_pm.w16[INV ? 1 : 0][q][i * (8 >> ST)];
+            x[k + len] = pm_shoup(d, w.w, w.q, P);
+        }
+    }
+    if constexpr (ST > 0) pm_stages<LOG, ST - 1, INV>(x, q, P);
+}
+
+template <int LOG, bool INV>
+__device__ __forceinline__ void pm_dft(u32 (&x)[1 << LOG], int q, u32 P)
+{
+    pm_stages<LOG, LOG - 1, INV>(x, q, P);
+}
+
+// The tile transform of 2^(LA+LB) points for one lane's item: x holds points
+// n = na 2^LB + g (g the thread's group) on entry; on return y(r, jb) is
+// frequency j = ja + 2^LA jb of ja = g + r 2^LB, at register
+// r 2^LB + bitrev(jb).  `sm` is the tile's exchange buffer.
+template <int LA, int LB, bool INV>
+__device__ __forceinline__ void pm_tile(u32 (&x)[1 << LA], u32 *sm, int g, int lane, int q, u32 P)
+{
+    constexpr int NA = 1 << LA, NB = 1 << LB;
+    static_assert(LA >= LB, "a group's step B takes NA / NB frequencies ja");
+    pm_dft<LA, INV>(x, q, P);
+#pragma unroll
+    for (int ja = 0; ja < NA; ++ja) {
+        u32 v = x[pm_bitrev(ja, LA)];
+        if (ja) {
+            const int e = (ja * g) << (8 - LA - LB);  // exponent of the 256th root
+            const PmW w = c_pm.w256[q][INV ? (256 - e) & 255 : e];
+            v = pm_shoup(v, w.w, w.q, P);
+        }
+        sm[(ja * NB + g) * kPmLanes + lane] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < NA / NB; ++r) {
+        u32 y[NB];
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb) y[nb] = sm[((g + r * NB) * NB + nb) * kPmLanes + lane];
+        pm_dft<LB, INV>(y, q, P);
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb) x[r * NB + nb] = y[nb];
+    }
+}
+
+// One operand of a transform launch: `ne` entries per point.
+struct PmOp {
+    const u32 *src;      // coefficients (first forward pass), else unused
+    long long nsrc;      // words of src
+    u32 *plane;          // [prime][L][ne]
+    int ne;
+    unsigned tiles;      // CTAs of this operand
+};
+
+enum PmMode { PM_F1, PM_F2, PM_F, PM_I1 };
+
+// One pass over one axis of L = L1 L2 for one or two operands (blockIdx.x)
+// and one prime (blockIdx.y).  PM_F1: along k1, coefficients in, times the
+// cross twiddles; PM_F2: along k2, values out below P; PM_F: the only pass
+// (L2 = 1), coefficients in, values out below P; PM_I1: inverse along j2,
+// times the inverse cross twiddles.
+template <int LA, int LB, int MODE>
+__global__ void __launch_bounds__(kPmLanes << LB) k_pm_pass(const PmOp A, const PmOp B, int lg, int lg2)
+{
+    constexpr int NA = 1 << LA, NB = 1 << LB, LN = LA + LB;
+    constexpr bool INV = MODE == PM_I1, FIRST = MODE == PM_F1 || MODE == PM_F;
+    __shared__ u32 sm[(1 << LN) * kPmLanes];
+    const bool isB = blockIdx.x >= A.tiles;
+    const PmOp &O = isB ? B : A;
+    const unsigned tile = isB ? blockIdx.x - A.tiles : blockIdx.x;
+    const int q = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const PmPrime pr = pm_prime(q);
+    const u32 P = pr.P;
+    const int ne = O.ne;
+    // items: (k2, entry) along k1, (j1, entry) along k2
+    const u32 other = 1u << (lg - LN);   // points of the other axis
+    const u32 w = tile * kPmLanes + lane;
+    const bool ok = w < other * (u32)ne;
+    const u32 kk = w / (u32)ne;
+    const u32 stride = FIRST ? ((u32)ne << lg2) : (u32)ne;
+    const u32 base = FIRST ? w : kk * ((u32)ne << lg2) + (w - kk * (u32)ne);
+    u32 *pl = O.plane + (size_t)q * ((size_t)ne << lg);
+    u32 x[NA];
+#pragma unroll
+    for (int na = 0; na < NA; ++na) {
+        const u32 n = (u32)(na * NB + g), idx = base + n * stride;
+        x[na] = 0u;
+        if (FIRST) {
+            if (ok && (long long)idx < O.nsrc) {
+                const u32 v = __ldg(O.src + idx);
+                x[na] = v - __umulhi(v, pr.mu) * P;  // below 2P (Barrett, 1986)
+            }
+        } else if (ok) {
+            x[na] = pl[idx];
+        }
+    }
+    pm_tile<LA, LB, INV>(x, sm, g, lane, q, P);
+    if (!ok) return;
+    // cross twiddle of frequency j: the 2^15-th root to the power +-j kk 2^(15-lg),
+    // Montgomery form; from one jb to the next it takes a fixed factor
+    auto cross = [&](u32 e) {
+        e = (INV ? (1u << kPmMaxLog) - e : e) & ((1u << kPmMaxLog) - 1u);
+        return pm_csub(pm_mont(__ldg(&d_pm_cross.hi[q][e >> 8]), __ldg(&d_pm_cross.lo[q][e & 255u]), P, pr.pinv), P);
+    };
+    const u32 ke = kk << (kPmMaxLog - lg);
+    const u32 step = (MODE == PM_F1 || MODE == PM_I1) ? cross(NA * ke) : 0u;
+#pragma unroll
+    for (int r = 0; r < NA / NB; ++r) {
+        const u32 j0 = (u32)(g + r * NB);
+        u32 t = (MODE == PM_F1 || MODE == PM_I1) ? cross(j0 * ke) : 0u;
+#pragma unroll
+        for (int jb = 0; jb < NB; ++jb) {
+            u32 v = x[r * NB + pm_bitrev(jb, LB)];
+            if (MODE == PM_F1 || MODE == PM_I1) {
+                v = pm_mont(v, t, P, pr.pinv);
+                if (jb + 1 < NB) t = pm_csub(pm_mont(t, step, P, pr.pinv), P);
+            } else {
+                v = pm_csub(v, P);
+            }
+            pl[base + (j0 + NA * jb) * stride] = v;
+        }
+    }
+}
+
+struct PmOut {
+    Mod mp;                    // the output modulus p
+    u32 linv[kPmPrimes], linv_q[kPmPrimes];  // 2^32 / L mod P and its Shoup quotient
+    u32 inv01, inv01q, inv02, inv02q, inv12, inv12q;  // P0^-1 mod P1, mod P2, P1^-1 mod P2, with quotients
+    u32 p0_mod_p, p0p1_mod_p;
+};
+
+// x mod P for x < 2^30 and P < 2^30 with mu = floor(2^32 / P)
+__device__ __forceinline__ u32 pm_mod(u32 x, u32 P, u32 mu) { return pm_csub(x - __umulhi(x, mu) * P, P); }
+
+// The integer with residues r[0..NPR-1] (each below its prime), mod p (Garner)
+template <int NPR>
+__device__ __forceinline__ u32 pm_crt(const u32 (&r)[NPR], const PmOut &c)
+{
+    if constexpr (NPR == 1) return red64(r[0], c.mp);
+    if constexpr (NPR >= 2) {
+        constexpr u32 P0 = kPmP0, P1 = kPmP1, P2 = kPmP2;
+        constexpr u32 mu1 = (u32)(((u64)1 << 32) / P1), mu2 = (u32)(((u64)1 << 32) / P2);
+        const u32 d1 = r[1] + P1 - pm_mod(r[0], P1, mu1);
+        const u32 x2 = pm_csub(pm_shoup(d1, c.inv01, c.inv01q, P1), P1);
+        if constexpr (NPR == 2) return red64((u64)r[0] + (u64)P0 * x2, c.mp);   // below P0 P1 < 2^59
+        if constexpr (NPR == 3) {
+            const u32 d2 = r[2] + P2 - pm_mod(r[0], P2, mu2);
+            const u32 t2 = pm_csub(pm_shoup(d2, c.inv02, c.inv02q, P2), P2);
+            const u32 d3 = t2 + P2 - pm_mod(x2, P2, mu2);
+            const u32 x3 = pm_csub(pm_shoup(d3, c.inv12, c.inv12q, P2), P2);
+            // r0 + P0 x2 + P0 P1 x3, term by term
+            const u64 v = (u64)red64(r[0], c.mp) + red64((u64)c.p0_mod_p * x2, c.mp) + red64((u64)c.p0p1_mod_p * x3, c.mp);
+            return red64(v, c.mp);
+        }
+    }
+}
+
+// The last inverse pass, along j1, for every prime in turn, then the
+// reconstruction: coefficients klo..khi of C are written from C on.
+template <int LA, int LB, int NPR>
+__global__ void __launch_bounds__(kPmLanes << LB) k_pm_out(const u32 *__restrict__ Ch, u32 *__restrict__ C, int ne, int lg,
+                                                          int lg2, long long klo, long long khi, const __grid_constant__ PmOut c)
+{
+    constexpr int NA = 1 << LA, NB = 1 << LB, LN = LA + LB;
+    __shared__ u32 sm[(1 << LN) * kPmLanes];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const u32 w = blockIdx.x * kPmLanes + lane;
+    const bool ok = w < ((u32)ne << (lg - LN));
+    const u32 stride = (u32)ne << lg2;
+    u32 res[NPR][NA];
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) {
+        const u32 *pl = Ch + (size_t)q * ((size_t)ne << lg);
+#pragma unroll
+        for (int na = 0; na < NA; ++na) res[q][na] = ok ? pl[w + (u32)(na * NB + g) * stride] : 0u;
+        if (q) __syncthreads();  // the previous prime's exchange has been read
+        pm_tile<LA, LB, true>(res[q], sm, g, lane, q, pm_prime(q).P);
+    }
+    if (!ok) return;
+    const long long lo = klo * ne, hi = (khi + 1) * ne;
+#pragma unroll
+    for (int r = 0; r < NA / NB; ++r)
+#pragma unroll
+        for (int jb = 0; jb < NB; ++jb) {
+            const long long idx = w + (long long)(g + r * NB + NA * jb) * stride;
+            if (idx < lo || idx >= hi) continue;
+            u32 v[NPR];
+#pragma unroll
+            for (int q = 0; q < NPR; ++q)
+                v[q] = pm_csub(pm_shoup(res[q][r * NB + pm_bitrev(jb, LB)], c.linv[q], c.linv_q[q], pm_prime(q).P), pm_prime(q).P);
+            C[idx - lo] = pm_crt<NPR>(v, c);
+        }
+}
+
+// ---------------------------------------------------------------------------
+// Ch[q][t] = Ah[q][t] Bh[q][t] 2^-32 mod P_q, an (sr x si) by (si x sc) product
+// at every point.  A CTA takes TP consecutive points of one prime, both
+// matrices of each in shared memory (rows padded to four words); a thread
+// forms 4 x 4 outputs of one point (rows ti + nti r, columns 4 tj ..), reading
+// four words of four rows of A and of B at a time: 64 multiply-adds per eight
+// 16-byte loads.  Terms are below P^2 < 2^59.8, so 16 of them fit in 64 bits;
+// longer rows fold multiples of 2 P 2^32 away every eight terms.
+constexpr int kPwThreads = 256;
+
+struct PmPw {
+    int sr, si, sc;
+    int si4, sc4;        // si, sc rounded up to 4
+    int nti, ntj;        // threads per point: rows (sr / 4), columns (sc / 4), rounded up
+    int tp;              // points per CTA
+    int ast, bst;        // words of shared memory per point of A and of B
+    int L;
+    u32 m_a, m_si, m_b, m_sc;  // ceil(2^32 / d) for d = sr si, si, si sc, sc: exact quotients below 2^16
+};
+
+__device__ __forceinline__ u32 pm_div(u32 x, u32 magic) { return __umulhi(x, magic); }
+
+__global__ void __launch_bounds__(kPwThreads) k_pm_pointwise(const u32 *__restrict__ Ah, const u32 *__restrict__ Bh,
+                                                            u32 *__restrict__ Ch, const __grid_constant__ PmPw a)
+{
+    extern __shared__ __align__(16) u32 pw[];
+    u32 *As = pw, *Bs = pw + (size_t)a.tp * a.ast;
+    const int q = blockIdx.y, t0 = blockIdx.x * a.tp, np = min(a.tp, a.L - t0);
+    const PmPrime pr = pm_prime(q);
+    const u32 ea = (u32)(a.sr * a.si), eb = (u32)(a.si * a.sc), ec = (u32)(a.sr * a.sc);
+    const u32 *ag = Ah + ((size_t)q * a.L + t0) * ea, *bg = Bh + ((size_t)q * a.L + t0) * eb;
+    // rows and columns past the matrices are never used but read: zero them
+    if (a.si != a.si4 || a.sc != a.sc4 || a.sr != 4 * a.nti) {
+        for (int i = threadIdx.x; i < a.tp * (a.ast + a.bst); i += kPwThreads) pw[i] = 0u;
+        __syncthreads();
+        for (u32 i = threadIdx.x; i < (u32)np * ea; i += kPwThreads) {
+            const u32 t = ea == 1u ? i : pm_div(i, a.m_a), e = i - t * ea;
+            const u32 r = a.si == 1 ? e : pm_div(e, a.m_si), k = e - r * (u32)a.si;
+            As[t * a.ast + r * a.si4 + k] = ag[i];
+        }
+        for (u32 i = threadIdx.x; i < (u32)np * eb; i += kPwThreads) {
+            const u32 t = eb == 1u ? i : pm_div(i, a.m_b), e = i - t * eb;
+            const u32 r = a.sc == 1 ? e : pm_div(e, a.m_sc), k = e - r * (u32)a.sc;
+            Bs[t * a.bst + r * a.sc4 + k] = bg[i];
+        }
+    } else {
+        // multiples of four: whole 16-byte blocks (the planes are 16-byte aligned)
+        for (u32 i = threadIdx.x; i < (u32)np * ea / 4; i += kPwThreads) {
+            const u32 t = pm_div(4 * i, a.m_a);
+            *reinterpret_cast<uint4 *>(As + t * a.ast + (4 * i - t * ea)) = reinterpret_cast<const uint4 *>(ag)[i];
+        }
+        for (u32 i = threadIdx.x; i < (u32)np * eb / 4; i += kPwThreads) {
+            const u32 t = pm_div(4 * i, a.m_b);
+            *reinterpret_cast<uint4 *>(Bs + t * a.bst + (4 * i - t * eb)) = reinterpret_cast<const uint4 *>(bg)[i];
+        }
+    }
+    __syncthreads();
+    const int per = a.nti * a.ntj, t = threadIdx.x / per, u = threadIdx.x - t * per;
+    if (t >= np) return;
+    const int ti = u / a.ntj, tj = u - ti * a.ntj;
+    const u32 *ap = As + t * a.ast + ti * a.si4, *bp = Bs + t * a.bst + 4 * tj;
+    u64 acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0;
+    const u32 P2 = 2u * pr.P;
+    for (int k = 0; k < a.si4; k += 4) {
+        uint4 av[4], bv[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) av[r] = *reinterpret_cast<const uint4 *>(ap + r * a.nti * a.si4 + k);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) bv[r] = *reinterpret_cast<const uint4 *>(bp + (k + r) * a.sc4);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const u32 ar[4] = {av[r].x, av[r].y, av[r].z, av[r].w};
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                acc[r][0] += (u64)ar[h] * bv[h].x;
+                acc[r][1] += (u64)ar[h] * bv[h].y;
+                acc[r][2] += (u64)ar[h] * bv[h].z;
+                acc[r][3] += (u64)ar[h] * bv[h].w;
+            }
+        }
+        if (a.si > 16 && (k & 4)) {
+            // eight more terms add below 8 P^2 < 2^62.8 to at most 2 P 2^32 < 2^62.9
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const u32 h = (u32)(acc[r][c] >> 32);
+                    acc[r][c] = (u64)min(h, h - P2) << 32 | (u32)acc[r][c];
+                }
+        }
+    }
+    u32 *cg = Ch + ((size_t)q * a.L + t0 + t) * ec;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = ti + r * a.nti;
+        if (i >= a.sr) break;
+        u32 o[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            // the high word is below 3.8 P (16 terms) or 4P: one or two steps of 2P
+            u32 h = (u32)(acc[r][c] >> 32);
+            h = min(h, h - P2);
+            const u32 v = pm_redc((u32)acc[r][c], h, pr.P, pr.pinv);   // below 3P
+            o[c] = pm_csub(v, P2);
+        }
+        if (a.sc == a.sc4) {
+            *reinterpret_cast<uint4 *>(cg + (size_t)i * a.sc + 4 * tj) = make_uint4(o[0], o[1], o[2], o[3]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (4 * tj + c < a.sc) cg[(size_t)i * a.sc + 4 * tj + c] = o[c];
+        }
+    }
+}
+
+int pm_log2(long long points)
+{
+    int lg = kPmMinLog;
+    while ((1LL << lg) < points) ++lg;
+    return lg;
+}
+
+// Launches of one axis of 2^ln points (4 <= ln <= 8).
+template <int MODE>
+ffspmv_status pm_pass(int ln, const PmOp &A, const PmOp &B, int lg, int lg2, int npr, cudaStream_t st)
+{
+    const dim3 grid(A.tiles + B.tiles, (unsigned)npr);
+    switch (ln) {
+    case 4: k_pm_pass<2, 2, MODE><<<grid, kPmLanes << 2, 0, st>>>(A, B, lg, lg2); break;
+    case 5: k_pm_pass<3, 2, MODE><<<grid, kPmLanes << 2, 0, st>>>(A, B, lg, lg2); break;
+    case 6: k_pm_pass<3, 3, MODE><<<grid, kPmLanes << 3, 0, st>>>(A, B, lg, lg2); break;
+    case 7: k_pm_pass<4, 3, MODE><<<grid, kPmLanes << 3, 0, st>>>(A, B, lg, lg2); break;
+    default: k_pm_pass<4, 4, MODE><<<grid, kPmLanes << 4, 0, st>>>(A, B, lg, lg2); break;
+    }
+    FF_CUDA(cudaGetLastError());
+    return FFSPMV_OK;
+}
+
+template <int NPR>
+ffspmv_status pm_out(int ln, const u32 *Ch, u32 *C, int ne, int lg, int lg2, long long klo, long long khi, const PmOut &c,
+                     cudaStream_t st)
+{
+    const unsigned tiles = (unsigned)((((long long)ne << (lg - ln)) + kPmLanes - 1) / kPmLanes);
+    switch (ln) {
+    case 4: k_pm_out<2, 2, NPR><<<tiles, kPmLanes << 2, 0, st>>>(Ch, C, ne, lg, lg2, klo, khi, c); break;
+    case 5: k_pm_out<3, 2, NPR><<<tiles, kPmLanes << 2, 0, st>>>(Ch, C, ne, lg, lg2, klo, khi, c); break;
+    case 6: k_pm_out<3, 3, NPR><<<tiles, kPmLanes << 3, 0, st>>>(Ch, C, ne, lg, lg2, klo, khi, c); break;
+    case 7: k_pm_out<4, 3, NPR><<<tiles, kPmLanes << 3, 0, st>>>(Ch, C, ne, lg, lg2, klo, khi, c); break;
+    default: k_pm_out<4, 4, NPR><<<tiles, kPmLanes << 4, 0, st>>>(Ch, C, ne, lg, lg2, klo, khi, c); break;
+    }
+    FF_CUDA(cudaGetLastError());
+    return FFSPMV_OK;
+}
+
+// Primes whose product exceeds every exact coefficient; 0 when three do not.
+int pm_primes(u32 p, int si, long long terms)
+{
+    const long double bound = (long double)si * (long double)terms * (long double)(p - 1) * (long double)(p - 1);
+    long double prod = 1;
+    for (int q = 0; q < kPmPrimes; ++q) {
+        prod *= kPmP[q];
+        if (bound < prod) return q + 1;
+    }
+    return 0;
 }
 
 }  // namespace
@@ -242,9 +563,8 @@ using namespace ff;
 extern "C" ffspmv_status polymat_mul_workspace(int32_t s, int64_t da, int64_t db, int64_t *bytes)
 {
     if (!bytes || s < 1 || s > 32 || da < 0 || db < 0) return FFSPMV_ERR_ARG;
-    const int lg = pm_log2(da, db);
-    if (lg > kPmMaxLog) return FFSPMV_ERR_UNSUPPORTED;
-    const long long L = 1LL << lg;
+    if (da + db + 1 > (1LL << kPmMaxLog)) return FFSPMV_ERR_UNSUPPORTED;
+    const long long L = 1LL << pm_log2(da + db + 1);
     *bytes = 3LL * kPmPrimes * s * s * L * 4 + (long long)kPmPrimes * L * 8 + 256;
     return FFSPMV_OK;
 }
@@ -259,57 +579,68 @@ extern "C" ffspmv_status polymat_mul(uint32_t p, int32_t s, int64_t da, int64_t 
     ffspmv_status r = polymat_mul_workspace(s, da, db, &need);
     if (r != FFSPMV_OK) return r;
     if (work_bytes < need || ((uintptr_t)d_work & 15)) return FFSPMV_ERR_ARG;
-    // the exact coefficients must stay below P0 P1 P2
-    const long double bound = (long double)s * (long double)(std::min(da, db) + 1) * (long double)(p - 1) *
-                              (long double)(p - 1);
-    const long double prod = (long double)kPmP[0] * kPmP[1] * kPmP[2];
-    if (bound >= prod) return FFSPMV_ERR_UNSUPPORTED;
-    const int lg = pm_log2(da, db);
-    const int L = 1 << lg, s2 = s * s;
-    PmConsts c;
+    // the exact coefficients must stay below the product of the primes
+    const int npr = pm_primes(p, s, std::min(da, db) + 1);
+    if (!npr) return FFSPMV_ERR_UNSUPPORTED;
+    cudaStream_t st = (cudaStream_t)stream;
+    const int lg = pm_log2(da + db + 1);
+    // L <= 256 in one pass, else two axes of at most 256 points
+    const int lg2 = lg <= 8 ? 0 : lg / 2, lg1 = lg - lg2;
+    const long long L = 1LL << lg;
+    const int ne = s * s;
+    u32 *Ah = (u32 *)d_work, *Bh = Ah + (size_t)npr * L * ne, *Ch = Bh + (size_t)npr * L * ne;
+    auto tiles = [&](int ln) { return (unsigned)((((long long)ne << (lg - ln)) + kPmLanes - 1) / kPmLanes); };
+    PmOp A = {d_A, (da + 1) * ne, Ah, ne, tiles(lg1)}, B = {d_B, (db + 1) * ne, Bh, ne, tiles(lg1)};
+    if (lg2 == 0) {
+        if ((r = pm_pass<PM_F>(lg1, A, B, lg, lg2, npr, st)) != FFSPMV_OK) return r;
+    } else {
+        if ((r = pm_pass<PM_F1>(lg1, A, B, lg, lg2, npr, st)) != FFSPMV_OK) return r;
+        A.tiles = B.tiles = tiles(lg2);
+        if ((r = pm_pass<PM_F2>(lg2, A, B, lg, lg2, npr, st)) != FFSPMV_OK) return r;
+    }
+    PmPw w;
+    memset(&w, 0, sizeof(w));
+    w.sr = w.si = w.sc = s;
+    w.si4 = (w.si + 3) / 4 * 4;
+    w.sc4 = (w.sc + 3) / 4 * 4;
+    w.nti = (w.sr + 3) / 4;
+    w.ntj = w.sc4 / 4;
+    w.tp = kPwThreads / (w.nti * w.ntj);
+    w.ast = 4 * w.nti * w.si4 + 4;   // 4 words of padding: neighbouring points start in other banks
+    w.bst = w.si4 * w.sc4 + 4;
+    w.L = (int)L;
+    auto magic = [](int d) { return (u32)((((u64)1 << 32) + d - 1) / d); };
+    w.m_a = magic(w.sr * w.si);
+    w.m_si = magic(w.si);
+    w.m_b = magic(w.si * w.sc);
+    w.m_sc = magic(w.sc);
+    const size_t pw_smem = (size_t)w.tp * (w.ast + w.bst) * 4;
+    FF_CUDA(cudaFuncSetAttribute(k_pm_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw_smem));
+    k_pm_pointwise<<<dim3((unsigned)((L + w.tp - 1) / w.tp), (unsigned)npr), kPwThreads, pw_smem, st>>>(Ah, Bh, Ch, w);
+    FF_CUDA(cudaGetLastError());
+    PmOut c;
     memset(&c, 0, sizeof(c));
-    for (int q = 0; q < kPmPrimes; ++q) {
+    c.mp = make_mod(p, 1, 0);
+    for (int q = 0; q < npr; ++q) {
         const u64 P = kPmP[q];
-        c.P[q] = make_mod((u32)P, 1, 0);
-        c.root[q] = powmod_host(kPmGen, (P - 1) >> lg, P);
-        // order exactly L: root^(L/2) = -1
-        if (powmod_host(c.root[q], (u64)L / 2, P) != P - 1) return FFSPMV_ERR_UNSUPPORTED;
-        c.iroot[q] = powmod_host(c.root[q], P - 2, P);
-        c.linv[q] = powmod_host((u64)L, P - 2, P);
+        // the pointwise products carry 2^-32, the inverse transform a factor L
+        c.linv[q] = (u32)((u64)pm_pow((u64)L, P - 2, P) * (((u64)1 << 32) % P) % P);
         c.linv_q[q] = (u32)(((u64)c.linv[q] << 32) / P);
     }
-    c.reduce_input = p > std::min({kPmP[0], kPmP[1], kPmP[2]}) ? 1 : 0;
-    c.mp = make_mod(p, 1, 0);
-    c.inv01 = powmod_host(kPmP[0] % kPmP[1], kPmP[1] - 2, kPmP[1]);
-    c.inv02 = powmod_host(kPmP[0] % kPmP[2], kPmP[2] - 2, kPmP[2]);
-    c.inv12 = powmod_host(kPmP[1] % kPmP[2], kPmP[2] - 2, kPmP[2]);
+    auto inv = [](u64 a, u64 P, u32 &v, u32 &vq) {
+        v = pm_pow(a, P - 2, P);
+        vq = (u32)(((u64)v << 32) / P);
+    };
+    inv(kPmP[0], kPmP[1], c.inv01, c.inv01q);
+    inv(kPmP[0], kPmP[2], c.inv02, c.inv02q);
+    inv(kPmP[1], kPmP[2], c.inv12, c.inv12q);
     c.p0_mod_p = (u32)(kPmP[0] % p);
     c.p0p1_mod_p = (u32)((unsigned __int128)kPmP[0] * kPmP[1] % p);
-
-    cudaStream_t st = (cudaStream_t)stream;
-    const size_t plane = (size_t)kPmPrimes * s2 * L;
-    u32 *Ah = (u32 *)d_work, *Bh = Ah + plane, *Ch = Bh + plane;
-    uint2 *tw = reinterpret_cast<uint2 *>(Ch + plane);  // 8-byte aligned: plane is a multiple of 2
-    const int T = 256;
-    auto blocks = [&](long long n) { return (unsigned)((n + T - 1) / T); };
-    k_pm_twiddles<<<blocks((long long)kPmPrimes * L), T, 0, st>>>(tw, L, c);
-    k_pm_load<<<blocks(plane), T, 0, st>>>(d_A, da, s2, lg, Ah, c);
-    k_pm_load<<<blocks(plane), T, 0, st>>>(d_B, db, s2, lg, Bh, c);
-    FF_CUDA(cudaGetLastError());
-    const size_t smem = (size_t)L * 4;
-    FF_CUDA(cudaFuncSetAttribute(k_ntt<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    FF_CUDA(cudaFuncSetAttribute(k_ntt<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_ntt<false><<<(unsigned)(kPmPrimes * s2), kNttThreads, smem, st>>>(Ah, L, s2, tw, c);
-    k_ntt<false><<<(unsigned)(kPmPrimes * s2), kNttThreads, smem, st>>>(Bh, L, s2, tw, c);
-    // points per CTA: both s x s tiles in at most 64 KB of shared memory
-    int lgtp = 5;  // 32 points per CTA, fewer when s^2 is large
-    while (lgtp > 0 && ((size_t)s2 << lgtp) > 8192) --lgtp;
-    const int TP = 1 << lgtp;
-    const size_t pw_smem = (size_t)2 * s2 * TP * 4;
-    FF_CUDA(cudaFuncSetAttribute(k_pm_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw_smem));
-    k_pm_pointwise<<<(unsigned)(kPmPrimes * ((L + TP - 1) / TP)), kPwThreads, pw_smem, st>>>(Ah, Bh, Ch, s, L, lgtp, c);
-    k_ntt<true><<<(unsigned)(kPmPrimes * s2), kNttThreads, smem, st>>>(Ch, L, s2, tw, c);
-    k_pm_crt<<<blocks((da + db + 1) * s2), T, 0, st>>>(Ch, d_C, da + db, s2, L, c);
-    FF_CUDA(cudaGetLastError());
-    return FFSPMV_OK;
+    if (lg2) {
+        const PmOp Cc = {nullptr, 0, Ch, ne, tiles(lg2)}, none = {nullptr, 0, nullptr, 1, 0};
+        if ((r = pm_pass<PM_I1>(lg2, Cc, none, lg, lg2, npr, st)) != FFSPMV_OK) return r;
+    }
+    return npr == 1   ? pm_out<1>(lg1, Ch, d_C, ne, lg, lg2, 0, da + db, c, st)
+           : npr == 2 ? pm_out<2>(lg1, Ch, d_C, ne, lg, lg2, 0, da + db, c, st)
+                      : pm_out<3>(lg1, Ch, d_C, ne, lg, lg2, 0, da + db, c, st);
 }
