@@ -131,13 +131,19 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
  * beta y and its block form).  d_x: ncols x nvec (ldx), d_y: nrows x nvec
  * (ldy); 1 <= nvec; alpha, beta < m (reduced if not).  beta = 0 never reads
  * d_y ("apply": y <- A x).  d_x and d_y must not overlap.  On a handle whose
- * plan is the x-panel layout, a block runs in passes of 4 vectors (m <=
+ * format the library chose (FFSPMV_FMT_AUTO) most blocks run on a layout of
+ * their own, up to 32 vectors per pass, with the rows of X packed next to
+ * each other: the first such block builds it (synchronous, host work plus
+ * one allocation per handle and direction); while the stream is captured
+ * before that, or when it cannot be built, the block runs as follows.  On a
+ * handle whose plan is the x-panel layout, a block runs in passes of 4 vectors (m <=
  * 2^16) or 2, then 1: each pass reads the matrix once for all its vectors
  * (Sec. 2.5.1) on an x-panel layout built for that width; the first block
  * that needs a width builds its layout and times one pass of it against the
  * same vectors one at a time (synchronous, host work plus one allocation
  * per handle, direction and width), and keeps it only if it is faster.  Calls on one handle must not
- * overlap on the GPU (the x-panel plans stage x in buffers of the handle).
+ * overlap on the GPU (x-panel plans and blocks stage x in buffers of the
+ * handle).
  */
 ffspmv_status spmv_apply(ffspmv_t h, const uint32_t *d_x, int64_t ldx,
                          uint32_t *d_y, int64_t ldy, int32_t nvec,
@@ -253,8 +259,8 @@ ffspmv_status spmv_describe_plan(ffspmv_t h, char *buf, size_t len);
 
 /* Number of kernel launches that one spmv_apply (transpose = 0) or
  * spmv_apply_transpose (transpose = 1) call with nvec vectors enqueues
- * (nothing is enqueued; on an x-panel handle this builds the layouts for
- * the pass widths the block needs, as spmv_apply does). */
+ * (nothing is enqueued; this builds the layouts that the block needs, as
+ * spmv_apply does; blocks are taken as contiguous and 16-byte aligned). */
 ffspmv_status spmv_count_launches(ffspmv_t h, int32_t transpose, int32_t nvec,
                                   int64_t *launches);
 

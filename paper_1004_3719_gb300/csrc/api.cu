@@ -4,6 +4,7 @@
 #include <vector>
 
 #include "ff_internal.cuh"
+#include "ff_block.h"
 #include "ff_plan.h"
 #include "ff_select.h"
 #include "../../include/ffspmv_select.h"
@@ -57,6 +58,7 @@ void destroy_handle(ffspmv_handle *h)
     free_sequence_state(h);
     batch_forget(h);
     free_gf2(h);
+    free_block(h);
     delete h;
 }
 
@@ -404,6 +406,28 @@ static ffspmv_status next_pass(ffspmv_t h, bool transpose, const Plan *P, int le
     return FFSPMV_OK;
 }
 
+// The layout that a block of nvec vectors runs on when it is not the plan's
+// own: the block layout, for handles whose format the library chose.
+//   x-panel plan: from 4 vectors on (m <= 256), 3 (m <= 2^16) or 2.  One pass
+//     of the panels for 2 vectors still wins at m <= 2^16 (1M power-law
+//     matrix: 65 us against 92; 3 vectors at m = 251: 85 against 94, at
+//     m = 65521: 106 against 93; 2 vectors at m = 2^31 - 1: 128 against 92).
+//   binned plan: unless the work is small and the plan takes fewer launches
+//     (20 000 x 20 000, 10 per row, m = 65521: 4 vectors in 10 us against 12,
+//     16 in 15.8 against 12; 90 001 x 120 011 power-law, 23 per row: 2
+//     vectors in 62 us against 17, 16 in 515 against 20).
+static const BlockPlan *block_path(ffspmv_t h, bool transpose, int nvec, cudaStream_t st)
+{
+    if (h->opt.priority_format != FFSPMV_FMT_AUTO || nvec < 2 || (h->opt.test_hooks & 12)) return nullptr;
+    const Plan &P = transpose ? h->AT : h->A;
+    if (P.panel.on) {
+        if (nvec < (h->m <= 256u ? 4 : h->m <= 65536u ? 3 : 2)) return nullptr;
+    } else if (P.nnz * nvec < (1LL << 21) && count_plan_launches(P, nvec) < 2LL * std::max(1, (nvec + 31) / 32)) {
+        return nullptr;
+    }
+    return ensure_block(h, transpose, st);
+}
+
 static ffspmv_status apply_common(ffspmv_t h, bool transpose, const uint32_t *d_x,
                                   int64_t ldx, uint32_t *d_y, int64_t ldy,
                                   int32_t nvec, uint32_t alpha, uint32_t beta,
@@ -428,6 +452,8 @@ static ffspmv_status apply_common(ffspmv_t h, bool transpose, const uint32_t *d_
     PanelCtl ctl;
     ctl.status = h->d_status + 2;
     ctl.skip_stage = (h->opt.test_hooks & 2) ? 1 : -1;
+    if (const BlockPlan *B = block_path(h, transpose, nvec, st))
+        return run_block(*B, d_x, ldx, d_y, ldy, nvec, h->m, alpha % h->m, beta % h->m, st);
     if (!P->panel.on || nvec == 1)
         return run_plan(*P, d_x, ldx, d_y, ldy, nvec, h->m, alpha % h->m, beta % h->m, st, &ctl);
     // x-panel blocks: passes of 4 or 2 vectors read the matrix once for all
@@ -521,7 +547,10 @@ ffspmv_status spmv_count_launches(ffspmv_t h, int32_t transpose, int32_t nvec, i
         n += 2LL * ((nvec + chunk - 1) / chunk);
     } else {
         const Plan &P = transpose ? h->AT : h->A;
-        if (!P.panel.on || nvec == 1) {
+        const BlockPlan *B = block_path(h, transpose != 0, nvec, nullptr);
+        if (B) {
+            n += block_launches(*B, nvec);
+        } else if (!P.panel.on || nvec == 1) {
             n += count_plan_launches(P, nvec);
         } else {
             for (int c0 = 0; c0 < nvec;) {

@@ -1,0 +1,664 @@
+// Y <- alpha A X + beta Y for blocks of vectors (Sec. 2.5.1): one pass over
+// the matrix for up to 32 vectors.
+//
+// A gather of x costs one 32-byte L2 sector however little of it is used, and
+// the gathers are what bounds a row-wise product (about 250 G sectors/s
+// measured on this chip).  With the residues of one row of X packed next to
+// each other (u16 for m <= 2^16: 16 vectors are 32 bytes), one sector serves
+// all the vectors, so a pass takes about the time of one vector's gathers.
+// The x-panel layout, which is faster for one vector, has no such gain: its
+// panels and row groups shrink as x and the row sums widen.  Measured on the
+// 1M x 1M power-law matrix (15.8M entries, m = 65521), 16 vectors: 643 us
+// in passes of the x-panel layout, 130 us here (14 us of it the packing); 16
+// vectors at m = 2^31 - 1: 1093 -> 192 us; 90 001 x 120 011 with power-law rows
+// (binned plan): 515 -> 20 us.
+//
+// Layout.  Rows are ordered by length class and their entries stored in that
+// order, so that the lanes of a warp do the same number of steps; T lanes
+// hold the 16-byte pieces of a row of X (T = 1, 2, 4, 8), G groups of T lanes
+// share a matrix row (G grows with the class).  Rows above kBlockLong entries
+// are cut into chunks of that many, one warp each; the chunks add reduced
+// sums into 64-bit words and the last one to arrive writes the row.
+#include <algorithm>
+#include <cstring>
+#include <exception>
+#include <thread>
+#include <type_traits>
+
+#include "ff_internal.cuh"
+#include "ff_plan.h"
+#include "ff_block.h"
+
+namespace ff {
+namespace {
+
+constexpr int kBlockThreads = 256;
+constexpr long long kBlockLong = 512;   // entries of a chunk; longer rows are split over warps
+constexpr int kBlockVecs = 32;          // vectors per pass
+constexpr int kBlockClasses = 7;        // by quads of entries: 0, 1, 2, 3-4, 5-8, 9-16, 17-128
+
+int block_class(long long len)
+{
+    const long long quads = (len + 3) / 4;
+    int c = 0;
+    if (quads > 0)
+        for (c = 1; c < kBlockClasses - 1 && (1LL << (c - 1)) < quads; ++c) {}
+    return c;
+}
+
+// groups of lanes that share a row of the class, one quad each per step
+int block_groups(int c)
+{
+    const int g[kBlockClasses] = {1, 1, 1, 2, 4, 8, 32};
+    return g[c];
+}
+
+}  // namespace
+
+struct BlockPlan {
+    bool ok = false;
+    void *arena = nullptr;
+    long long n = 0, ncols = 0;
+    bool small = true;                 // m <= 2^16: u16 values and staged x
+    long long nlong = 0, nchunk = 0;   // rows split over warps, and their chunks
+    long long cls_row[kBlockClasses + 1] = {};  // rows of class c: [cls_row[c], cls_row[c + 1]) of row / ptr
+    const u32 *ptr = nullptr;          // [n - nlong + 1] offsets in quads, rows in class order
+    const u32 *row = nullptr;          // [n - nlong] their matrix rows
+    const uint4 *chunk = nullptr;      // (long row index, first quad, end, chunks of the row)
+    const u32 *lrow = nullptr;         // [nlong] matrix rows
+    const u32 *col = nullptr;
+    const void *val = nullptr;
+    uint4 *xs = nullptr;               // staged rows of X
+    u32 quad1 = 0;                     // the one-quad class: row r at quad quad1 + r (mod 2^32)
+    u64 *carry = nullptr;              // [nlong][kBlockVecs], zero between calls
+    u32 *count = nullptr;              // [nlong] chunks arrived, zero between calls
+};
+
+void free_block(ffspmv_handle *h)
+{
+    for (BlockPlan *&b : h->block) {
+        if (b) {
+            if (b->arena) cudaFree(b->arena);
+            delete b;
+        }
+        b = nullptr;
+    }
+}
+
+namespace {
+
+// Rows of X packed to `pitch` 16-byte words each: u16 or u32 residues, zero
+// past nvec.  One thread per word.
+template <bool SMALL>
+__global__ void __launch_bounds__(kBlockThreads) k_block_stage(const u32 *__restrict__ x, long long ldx, long long n,
+                                                              int nvec, int pitch, int vec4, uint4 *__restrict__ xs)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int C = SMALL ? 8 : 4;
+    const long long t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
+    if (t >= n * pitch) return;
+    const long long i = t / pitch;
+    const int c0 = (int)(t - i * pitch) * C;
+    const u32 *p = x + i * ldx + c0;
+    u32 v[C];
+    if (vec4 && c0 + C <= nvec) {
+#pragma unroll
+        for (int u = 0; u < C / 4; ++u) {
+            const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p) + u);
+            v[4 * u] = w.x; v[4 * u + 1] = w.y; v[4 * u + 2] = w.z; v[4 * u + 3] = w.w;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < C; ++u) v[u] = c0 + u < nvec ? __ldg(p + u) : 0u;
+    }
+    uint4 o;
+    if constexpr (SMALL) {
+        o.x = (v[0] & 0xffffu) | v[1] << 16;
+        o.y = (v[2] & 0xffffu) | v[3] << 16;
+        o.z = (v[4] & 0xffffu) | v[5] << 16;
+        o.w = (v[6] & 0xffffu) | v[7] << 16;
+    } else {
+        o = make_uint4(v[0], v[1], v[2], v[3]);
+    }
+    xs[t] = o;
+}
+
+struct BlockArgs {
+    const u32 *ptr, *row, *col, *lrow;
+    const uint4 *chunk;
+    const void *val;
+    const uint4 *xs;    // rows of X, pitch words of 16 bytes each
+    u64 *carry;
+    u32 *count;
+    u32 *y;
+    long long ldy;
+    int pitch, pieces, nvec, vec4, lgt;  // pieces of 16 bytes per row of X; lgt: log2 of the lanes that hold them
+    int nchunk_warps;             // warps 0 .. nchunk - 1 take the chunks
+    u32 warp0[kBlockClasses + 1]; // first warp of each class, heaviest class first
+    u32 row0[kBlockClasses + 1];  // its rows
+    int lgg[kBlockClasses];       // log2 of groups per row
+    u32 quad1;                    // rows r of the one-quad class: quad quad1 + r
+    int fold;                     // m <= 2^31
+    Mod M;
+};
+
+// Sums of one lane: 8 components of u16 residues (64-bit sums of terms below
+// 2^32, at most 2^32 of them) or 4 of u32 residues (96-bit sums).
+template <bool SMALL>
+struct BlockAcc;
+
+template <>
+struct BlockAcc<true> {
+    static constexpr int C = 8;
+    typedef u64 Sum;
+    u64 a[8];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a[i] = 0;
+    }
+    __device__ __forceinline__ void quad(const uint2 &vv, const uint4 (&x)[4], int)
+    {
+        const u32 v[4] = {vv.x & 0xffffu, vv.x >> 16, vv.y & 0xffffu, vv.y >> 16};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const u32 w[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[2 * i] += (u64)v[u] * (w[i] & 0xffffu);
+                a[2 * i + 1] += (u64)v[u] * (w[i] >> 16);
+            }
+        }
+    }
+    static __device__ __forceinline__ u64 sel(bool b, u64 x, u64 y) { return b ? x : y; }
+    static __device__ __forceinline__ u64 add_from(u64 keep, u64 send, int off)
+    {
+        return keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+    static __device__ __forceinline__ u32 get(u64 s, const Mod &M) { return red64(s, M); }
+};
+
+template <>
+struct BlockAcc<false> {
+    static constexpr int C = 4;
+    typedef AccWide Sum;
+    AccWide a[4];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i].zero();
+    }
+    __device__ __forceinline__ void quad(const uint4 &vv, const uint4 (&x)[4], int fold)
+    {
+        const u32 v[4] = {vv.x, vv.y, vv.z, vv.w};
+        u32 w[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            w[u][0] = x[u].x;
+            w[u][1] = x[u].y;
+            w[u][2] = x[u].z;
+            w[u][3] = x[u].w;
+        }
+        if (fold) {
+            // m <= 2^31: four products, each below 2^62, in one 64-bit word
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const u64 t = (u64)v[0] * w[0][i] + (u64)v[1] * w[1][i] + (u64)v[2] * w[2][i] + (u64)v[3] * w[3][i];
+                asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
+                    : "+r"(a[i].w0), "+r"(a[i].w1), "+r"(a[i].w2)
+                    : "r"((u32)t), "r"((u32)(t >> 32)));
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i].mad(v[u], w[u][i]);
+        }
+    }
+    static __device__ __forceinline__ AccWide sel(bool b, const AccWide &x, const AccWide &y)
+    {
+        AccWide r;
+        r.w0 = b ? x.w0 : y.w0;
+        r.w1 = b ? x.w1 : y.w1;
+        r.w2 = b ? x.w2 : y.w2;
+        return r;
+    }
+    static __device__ __forceinline__ AccWide add_from(AccWide keep, const AccWide &send, int off)
+    {
+        const u32 o0 = __shfl_xor_sync(0xffffffffu, send.w0, off), o1 = __shfl_xor_sync(0xffffffffu, send.w1, off),
+                  o2 = __shfl_xor_sync(0xffffffffu, send.w2, off);
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+            : "+r"(keep.w0), "+r"(keep.w1), "+r"(keep.w2)
+            : "r"(o0), "r"(o1), "r"(o2));
+        return keep;
+    }
+    static __device__ __forceinline__ u32 get(const AccWide &s, const Mod &M) { return (u32)s.partial(M); }
+};
+
+// acc += quads k, k + step, ... below end; xb: this lane's piece of the rows
+// of X.  Rows are padded to whole quads (value 0, column 0).
+template <bool SMALL>
+__device__ __forceinline__ void block_entries(BlockAcc<SMALL> &acc, const BlockArgs &a, u32 k, u32 end, u32 step,
+                                              const char *xb, bool on)
+{
+    typedef typename std::conditional<SMALL, uint2, uint4>::type V;
+    const u32 pb = (u32)a.pitch * 16u;
+    if (k >= end) return;
+    uint4 j = __ldcs(reinterpret_cast<const uint4 *>(a.col) + k);
+    V v = __ldcs(reinterpret_cast<const V *>(a.val) + k);
+    for (;;) {
+        uint4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (on) {
+            x[0] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.x * pb));
+            x[1] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.y * pb));
+            x[2] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.z * pb));
+            x[3] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.w * pb));
+        }
+        // the next quad is on its way from memory while the gathers are
+        const V vc = v;
+        k += step;
+        if (k < end) {
+            j = __ldcs(reinterpret_cast<const uint4 *>(a.col) + k);
+            v = __ldcs(reinterpret_cast<const V *>(a.val) + k);
+        }
+        acc.quad(vc, x, a.fold);
+        if (k >= end) break;
+    }
+}
+
+// R consecutive components from column col0 of a row
+template <int R>
+__device__ __forceinline__ void block_write(const u32 (&r)[R], const BlockArgs &a, u32 row, int col0)
+{
+    u32 *yp = a.y + (long long)row * a.ldy + col0;
+    if (R >= 4 && a.vec4 && col0 + R <= a.nvec) {
+#pragma unroll
+        for (int i = 0; i + 4 <= R; i += 4) {
+            u32 o[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) o[k] = combine(r[i + k], yp + i + k, false, a.M);
+            __stcs(reinterpret_cast<uint4 *>(yp + i), make_uint4(o[0], o[1], o[2], o[3]));
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+            if (col0 + i < a.nvec) yp[i] = combine(r[i], yp + i, false, a.M);
+    }
+}
+
+// The sums of the 2^lgg groups of a row (lanes a multiple of T apart), each
+// component in one group only: every step sends one half of the components
+// to the partner and keeps the other.  R components, from `col0` on, are left
+// in s when the steps S .. end; `emit(s, col0)` takes them from the lanes
+// that hold final sums.
+template <bool SMALL, int R, class Emit>
+__device__ __forceinline__ void block_reduce(typename BlockAcc<SMALL>::Sum (&s)[R], int lgt, int lgg, int step, int lane,
+                                             int col0, Emit emit)
+{
+    typedef BlockAcc<SMALL> A;
+    if (step == lgg) {
+        u32 o[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) o[i] = A::get(s[i], *emit.M);
+        emit(o, col0);
+        return;
+    }
+    const int off = 1 << (lgt + step);
+    if constexpr (R > 1) {
+        const bool up = (lane & off) != 0;
+        typename A::Sum t[R / 2];
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i)
+            t[i] = A::add_from(A::sel(up, s[i + R / 2], s[i]), A::sel(up, s[i], s[i + R / 2]), off);
+        block_reduce<SMALL, R / 2>(t, lgt, lgg, step + 1, lane, col0 + (up ? R / 2 : 0), emit);
+    } else {
+        // one component left: the lanes of the remaining steps all get the sum
+        for (; step < lgg; ++step) s[0] = A::add_from(s[0], s[0], 1 << (lgt + step));
+        // ... and the one whose bits of those steps are 0 writes it
+        constexpr int full = SMALL ? 3 : 2;
+        const bool mine = (lane & (((1 << lgg) - (1 << full)) << lgt)) == 0;
+        u32 o[1] = {A::get(s[0], *emit.M)};
+        if (mine) emit(o, col0);
+    }
+}
+
+struct BlockEmitRow {
+    const BlockArgs *a;
+    const Mod *M;
+    u32 row;
+    bool ok;
+    template <int R>
+    __device__ __forceinline__ void operator()(const u32 (&o)[R], int col0) const
+    {
+        if (ok) block_write<R>(o, *a, row, col0);
+    }
+};
+
+struct BlockEmitCarry {
+    const BlockArgs *a;
+    const Mod *M;
+    u64 *cw;
+    template <int R>
+    __device__ __forceinline__ void operator()(const u32 (&o)[R], int col0) const
+    {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+            if (col0 + i < a->nvec) atomicAdd(cw + col0 + i, (u64)o[i]);
+    }
+};
+
+// One warp per chunk of a long row, or per 32 / (T G) rows of a class.
+template <bool SMALL>
+__global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constant__ BlockArgs a)
+{
+    constexpr int C = BlockAcc<SMALL>::C;
+    const u32 w = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, T = 1 << a.lgt, c = lane & (T - 1);
+    const char *xb = reinterpret_cast<const char *>(a.xs + c);
+    const bool on = c < a.pieces;
+    BlockAcc<SMALL> acc;
+    acc.zero();
+    // the rows of X come from the staging launch before this one
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (w < (u32)a.nchunk_warps) {
+        const uint4 ch = __ldg(a.chunk + w);
+        block_entries<SMALL>(acc, a, ch.y + (u32)(lane >> a.lgt), ch.z, 32u >> a.lgt, xb, on);
+        u64 *cw = a.carry + (size_t)ch.x * kBlockVecs;
+        const BlockEmitCarry emit = {&a, &a.M, cw};
+        block_reduce<SMALL, C>(acc.a, a.lgt, 5 - a.lgt, 0, lane, c * C, emit);
+        // the chunk that arrives last writes the row and clears its words
+        u32 last = 0;
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(a.count + ch.x, 1u) == ch.w - 1u ? 1u : 0u;
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (!last) return;
+        __threadfence();
+        const u32 row = __ldg(a.lrow + ch.x);
+        if (lane < a.nvec) {
+            u32 *yp = a.y + (long long)row * a.ldy + lane;
+            *yp = combine(red64(__ldcg(cw + lane), a.M), yp, false, a.M);
+            cw[lane] = 0;
+        }
+        if (lane == 0) a.count[ch.x] = 0;
+        return;
+    }
+    // the class of this warp (warp0 grows; the last entry ends the list)
+    int b = 0;
+#pragma unroll
+    for (int i = 1; i < kBlockClasses; ++i)
+        if (w >= a.warp0[i]) b = i;
+    if (w >= a.warp0[kBlockClasses]) return;
+    const int lgg = a.lgg[b], lgr = a.lgt + lgg;   // log2 of groups and of lanes per row
+    const u32 r = a.row0[b] + ((w - a.warp0[b]) << (5 - lgr)) + (u32)(lane >> lgr);
+    BlockEmitRow emit = {&a, &a.M, 0u, r < a.row0[b + 1] && on};
+    if (r < a.row0[b + 1]) {
+        // rows of one quad lie one after another: no offset to wait for
+        const bool one = b == kBlockClasses - 2;
+        const u32 s = one ? a.quad1 + r : __ldg(a.ptr + r), e = one ? s + 1u : __ldg(a.ptr + r + 1);
+        emit.row = __ldg(a.row + r);
+        block_entries<SMALL>(acc, a, s + (u32)((lane >> a.lgt) & ((1 << lgg) - 1)), e, 1u << lgg, xb, on);
+    }
+    block_reduce<SMALL, C>(acc.a, a.lgt, lgg, 0, lane, c * C, emit);
+}
+
+// ---------------------------------------------------------------------------
+ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long long *ptr, const int *col,
+                          const u32 *val, u32 m)
+{
+    const long long nnz = ptr[n];
+    // offsets in quads are 32-bit
+    if (nnz / 4 + n >= (1LL << 32) - 1 || n >= (1LL << 32) - 64) return FFSPMV_ERR_UNSUPPORTED;
+    auto quads = [&](long long i) { return (u32)((ptr[i + 1] - ptr[i] + 3) / 4); };
+    B.n = n;
+    B.ncols = ncols;
+    B.small = m <= 65536u;
+    // rows in class order, heaviest first, and where their entries go
+    std::vector<u32> lrow, row, rptr;
+    std::vector<uint4> chunk;
+    long long cnt[kBlockClasses] = {};
+    u32 at = 0;
+    for (long long i = 0; i < n; ++i) {
+        const long long L = ptr[i + 1] - ptr[i];
+        if (L <= kBlockLong) {
+            ++cnt[block_class(L)];
+            continue;
+        }
+        const u32 parts = (u32)((L + kBlockLong - 1) / kBlockLong);
+        for (u32 c = 0; c < parts; ++c)
+            chunk.push_back(make_uint4((u32)lrow.size(), at + c * (u32)(kBlockLong / 4),
+                                       at + std::min(quads(i), (c + 1) * (u32)(kBlockLong / 4)), parts));
+        lrow.push_back((u32)i);
+        at += quads(i);
+    }
+    B.nlong = (long long)lrow.size();
+    B.nchunk = (long long)chunk.size();
+    const long long ns = n - B.nlong;
+    for (int c = 0; c < kBlockClasses; ++c) B.cls_row[c + 1] = B.cls_row[c] + cnt[kBlockClasses - 1 - c];
+    row.resize((size_t)ns);
+    rptr.resize((size_t)ns + 1);
+    long long pos[kBlockClasses];
+    for (int c = 0; c < kBlockClasses; ++c) pos[c] = B.cls_row[kBlockClasses - 1 - c];
+    for (long long i = 0; i < n; ++i) {
+        const long long L = ptr[i + 1] - ptr[i];
+        if (L <= kBlockLong) row[(size_t)pos[block_class(L)]++] = (u32)i;
+    }
+    for (long long r = 0; r < ns; ++r) {
+        rptr[(size_t)r] = at;
+        at += quads(row[(size_t)r]);
+    }
+    rptr[(size_t)ns] = at;
+    // heaviest first: class 1 (one quad) is the last but one
+    const size_t r1 = (size_t)B.cls_row[kBlockClasses - 2];
+    B.quad1 = rptr[r1] - (u32)r1;
+    const int vb = B.small ? 2 : 4;
+    const size_t slots = (size_t)at * 4;
+    std::vector<u32> pcol(std::max<size_t>(slots, 4), 0u);
+    std::vector<unsigned char> pval(std::max<size_t>(slots, 4) * vb, 0);
+    auto copy_row = [&](long long i, u32 quad) {
+        size_t to = (size_t)quad * 4;
+        for (long long k = ptr[i]; k < ptr[i + 1]; ++k, ++to) {
+            pcol[to] = (u32)col[k];
+            const u32 v = val[k] % m;
+            if (B.small) reinterpret_cast<unsigned short *>(pval.data())[to] = (unsigned short)v;
+            else reinterpret_cast<u32 *>(pval.data())[to] = v;
+        }
+    };
+    const int nt = (int)std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
+    auto work = [&](int t) {
+        for (long long r = ns * t / nt; r < ns * (t + 1) / nt; ++r) copy_row(row[(size_t)r], rptr[(size_t)r]);
+        u32 to = 0;
+        for (long long r = 0; r < B.nlong; ++r) {
+            if (r % nt == t) copy_row(lrow[(size_t)r], to);
+            to += quads(lrow[(size_t)r]);
+        }
+    };
+    if (nnz < 200000 || nt == 1) {
+        for (int t = 0; t < nt; ++t) work(t);
+    } else {
+        std::vector<std::thread> th;
+        th.reserve((size_t)nt);
+        for (int t = 0; t < nt; ++t) {
+            try {
+                th.emplace_back(work, t);
+            } catch (const std::exception &) {
+                work(t);  // no thread to be had: this share runs here
+            }
+        }
+        for (auto &t : th) t.join();
+    }
+    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+    size_t o = 0;
+    auto put = [&](size_t bytes) {
+        const size_t here = o;
+        o += al(std::max<size_t>(bytes, 16));
+        return here;
+    };
+    const size_t o_ptr = put(rptr.size() * 4), o_row = put(row.size() * 4), o_chunk = put(chunk.size() * 16),
+                 o_lrow = put(lrow.size() * 4), o_col = put(pcol.size() * 4), o_val = put(pval.size()),
+                 o_carry = put((size_t)B.nlong * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
+                 o_xs = put((size_t)ncols * kBlockVecs * vb);
+    if (cudaMalloc(&B.arena, o) != cudaSuccess) {
+        cudaGetLastError();
+        B.arena = nullptr;
+        return FFSPMV_ERR_OOM;
+    }
+    char *base = (char *)B.arena;
+    auto up = [&](size_t off, const void *src, size_t bytes) {
+        return !bytes || cudaMemcpy(base + off, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+    };
+    const bool ok = up(o_ptr, rptr.data(), rptr.size() * 4) && up(o_row, row.data(), row.size() * 4) &&
+                    up(o_chunk, chunk.data(), chunk.size() * 16) && up(o_lrow, lrow.data(), lrow.size() * 4) &&
+                    up(o_col, pcol.data(), slots * 4) && up(o_val, pval.data(), slots * vb) &&
+                    cudaMemset(base + o_carry, 0, o_xs - o_carry) == cudaSuccess;
+    if (!ok) {
+        cudaFree(B.arena);
+        B.arena = nullptr;
+        cudaGetLastError();
+        return FFSPMV_ERR_CUDA;
+    }
+    B.ptr = (const u32 *)(base + o_ptr);
+    B.row = (const u32 *)(base + o_row);
+    B.chunk = (const uint4 *)(base + o_chunk);
+    B.lrow = (const u32 *)(base + o_lrow);
+    B.col = (const u32 *)(base + o_col);
+    B.val = base + o_val;
+    B.carry = (u64 *)(base + o_carry);
+    B.count = (u32 *)(base + o_count);
+    B.xs = (uint4 *)(base + o_xs);
+    return FFSPMV_OK;
+}
+
+}  // namespace
+
+const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st)
+{
+    BlockPlan *&b = h->block[transpose ? 1 : 0];
+    if (b) return b->ok ? b : nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;  // nothing can be allocated or copied now
+    }
+    BlockPlan *nb = new (std::nothrow) BlockPlan();
+    if (!nb) return nullptr;
+    ffspmv_status r;
+    try {
+        if (!transpose) {
+            r = build_block(*nb, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(), h->h_val.data(), h->m);
+        } else {
+            std::vector<long long> tptr;
+            std::vector<int> tcol;
+            std::vector<u32> tval;
+            transpose_csr(h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(), h->h_val.data(), tptr, tcol, tval);
+            r = build_block(*nb, h->A.ncols, h->A.nrows, tptr.data(), tcol.data(), tval.data(), h->m);
+        }
+    } catch (const std::exception &) {
+        r = FFSPMV_ERR_OOM;
+    }
+    nb->ok = r == FFSPMV_OK;  // a layout that could not be made is not tried again
+    b = nb;
+    return nb->ok ? nb : nullptr;
+}
+
+// Launches of one block of nvec vectors: a staging pass and the product per
+// kBlockVecs vectors; x is read in place where its rows already are whole
+// aligned 16-byte pieces of u32.
+static bool block_in_place(const BlockPlan &B, const u32 *x, long long ldx, int nv)
+{
+    return !B.small && nv % 4 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15u) == 0 && ldx / 4 < (1LL << 30);
+}
+
+long long block_launches(const BlockPlan &B, int nvec)
+{
+    long long n = 0;
+    for (int v0 = 0; v0 < nvec; v0 += kBlockVecs)
+        n += block_in_place(B, nullptr, nvec, std::min(kBlockVecs, nvec - v0)) ? 1 : 2;
+    return n;
+}
+
+ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec, u32 m,
+                        u32 alpha, u32 beta, cudaStream_t st)
+{
+    const int C = B.small ? 8 : 4;
+    for (int v0 = 0; v0 < nvec; v0 += kBlockVecs) {
+        const int nv = std::min(kBlockVecs, nvec - v0);
+        const u32 *xv = x + v0;
+        u32 *yv = y + v0;
+        BlockArgs a;
+        memset(&a, 0, sizeof(a));
+        a.ptr = B.ptr;
+        a.row = B.row;
+        a.col = B.col;
+        a.lrow = B.lrow;
+        a.chunk = B.chunk;
+        a.val = B.val;
+        a.carry = B.carry;
+        a.count = B.count;
+        a.quad1 = B.quad1;
+        a.y = yv;
+        a.ldy = ldy;
+        a.nvec = nv;
+        a.vec4 = (ldy % 4 == 0 && ((uintptr_t)yv & 15u) == 0) ? 1 : 0;
+        a.M = make_mod(m, alpha, beta);
+        a.fold = m <= (1u << 31) ? 1 : 0;
+        const int pieces = (nv + C - 1) / C;
+        while ((1 << a.lgt) < pieces) ++a.lgt;
+        a.pieces = pieces;
+        const bool in_place = block_in_place(B, xv, ldx, nv);
+        if (in_place) {
+            a.xs = reinterpret_cast<const uint4 *>(xv);
+            a.pitch = (int)(ldx / 4);
+        } else {
+            a.xs = B.xs;
+            a.pitch = pieces;
+            const long long words = B.ncols * pieces;
+            const int vec4 = (ldx % 4 == 0 && ((uintptr_t)xv & 15u) == 0) ? 1 : 0;
+            if (words > 0) {
+                const unsigned blocks = (unsigned)((words + kBlockThreads - 1) / kBlockThreads);
+                if (B.small)
+                    k_block_stage<true><<<blocks, kBlockThreads, 0, st>>>(xv, ldx, B.ncols, nv, pieces, vec4, B.xs);
+                else
+                    k_block_stage<false><<<blocks, kBlockThreads, 0, st>>>(xv, ldx, B.ncols, nv, pieces, vec4, B.xs);
+                FF_CUDA(cudaGetLastError());
+            }
+        }
+        // groups per row: by class, doubled while the launch has fewer than
+        // 16 warps per SM (short matrices: more lanes per row, shorter chains)
+        long long warps = 0;
+        for (int boost = 0; boost < 6; ++boost) {
+            warps = B.nchunk;
+            for (int c = 0; c < kBlockClasses; ++c) {
+                const int g = block_groups(kBlockClasses - 1 - c) << boost;
+                int lg = 0;
+                while ((2 << lg) <= std::min(g, 32 >> a.lgt)) ++lg;
+                a.lgg[c] = lg;
+                a.row0[c] = (u32)B.cls_row[c];
+                a.warp0[c] = (u32)warps;
+                const int rpw = 32 >> (a.lgt + lg);
+                warps += (B.cls_row[c + 1] - B.cls_row[c] + rpw - 1) / rpw;
+            }
+            if (warps >= 16 * 152) break;
+        }
+        a.row0[kBlockClasses] = (u32)B.cls_row[kBlockClasses];
+        a.warp0[kBlockClasses] = (u32)warps;
+        a.nchunk_warps = (int)B.nchunk;
+        if (warps == 0) continue;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((warps * 32 + kBlockThreads - 1) / kBlockThreads));
+        cfg.blockDim = dim3(kBlockThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = in_place ? 0 : 1;
+        if (B.small) FF_CUDA(cudaLaunchKernelEx(&cfg, k_block<true>, a));
+        else FF_CUDA(cudaLaunchKernelEx(&cfg, k_block<false>, a));
+    }
+    return FFSPMV_OK;
+}
+
+}  // namespace ff

@@ -285,6 +285,7 @@ struct Plan {
 
 namespace ff {
 struct Gf2Pattern;
+struct BlockPlan;
 }
 
 struct ffspmv_handle {
@@ -315,6 +316,8 @@ struct ffspmv_handle {
     // x-panel plans of A and A^T for 2 and 4 vectors per pass, built on the
     // first block that uses them when the plan is the x-panel layout
     ff::Plan *multi[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    // block layouts of A and A^T (block.cu), built on the first block that uses them
+    ff::BlockPlan *block[2] = {nullptr, nullptr};
 };
 
 namespace ff {
