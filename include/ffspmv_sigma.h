@@ -39,11 +39,12 @@ extern "C" {
 /*
  * Device workspace (bytes, written to *bytes) that sigma_basis needs for
  * these sizes.  1 <= n <= m <= 32, d >= 1; base = 0 picks the default leaf
- * order (the largest power of two <= 32 whose M-Basis leaf fits in one CTA's
- * shared memory), else 1 <= base <= 32.  FFSPMV_ERR_UNSUPPORTED when the
- * leaf does not fit in shared memory, or the largest product of the
- * recursion (ceil(d/2) + d coefficients) exceeds the 2^15-point transforms
- * of polymat_mul.
+ * order (32), else 1 <= base <= 32.  The basis and its degrees do not depend
+ * on base (M-Basis is the limit of the recursion), which the library may cut
+ * into smaller leaves; the degree bound of sigma_basis is taken at orders up
+ * to base.  FFSPMV_ERR_UNSUPPORTED when d > base and the largest product of
+ * the recursion (ceil(d/2) + d coefficients) exceeds the 2^15-point
+ * transforms of polymat_mul.
  */
 ffspmv_status sigma_basis_workspace(int32_t m, int32_t n, int64_t d, int32_t base, int64_t *bytes);
 
@@ -57,8 +58,9 @@ ffspmv_status sigma_basis_workspace(int32_t m, int32_t n, int64_t d, int32_t bas
  * sigma_basis_workspace (PM-Basis hands orders <= base to M-Basis).  d_work:
  * at least sigma_basis_workspace bytes of device memory, 16-byte aligned,
  * owned by the caller and not used by another call at the same time.
- * Synchronous: the recursion reads each leaf's degrees back to size the next
- * products, so the call returns after the stream has finished the work.
+ * Synchronous: the recursion reads the larger halves' degrees back to size
+ * the next products, so the call returns after the stream has finished the
+ * work.
  */
 ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
                           const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,

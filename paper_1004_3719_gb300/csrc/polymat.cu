@@ -36,6 +36,7 @@
 #include <cstring>
 
 #include "ff_internal.cuh"
+#include "ff_polymat.h"
 #include "ffspmv_polymat.h"
 
 namespace ff {
@@ -555,52 +556,199 @@ int pm_primes(u32 p, int si, long long terms)
     return 0;
 }
 
-}  // namespace
-}  // namespace ff
-
-using namespace ff;
-
-extern "C" ffspmv_status polymat_mul_workspace(int32_t s, int64_t da, int64_t db, int64_t *bytes)
+// Smallest transform whose cyclic wrap leaves the coefficients klo..khi
+// alone: coefficient k of the product lands on k mod L, so L > khi and
+// da + db - L < klo.
+int pm_length_log(long long da, long long db, long long klo, long long khi)
 {
-    if (!bytes || s < 1 || s > 32 || da < 0 || db < 0) return FFSPMV_ERR_ARG;
-    if (da + db + 1 > (1LL << kPmMaxLog)) return FFSPMV_ERR_UNSUPPORTED;
-    const long long L = 1LL << pm_log2(da + db + 1);
-    *bytes = 3LL * kPmPrimes * s * s * L * 4 + (long long)kPmPrimes * L * 8 + 256;
+    return pm_log2(std::max(khi + 1, da + db - klo + 1));
+}
+
+// ---------------------------------------------------------------------------
+// Products by the definition.  A CTA forms up to 16 x 16 or 8 x 32 entries of
+// one coefficient of C (2 x 4 per lane); its eight warps take every eighth
+// pair (A_a, B_(k-a)) into shared memory of their own, and their reduced sums
+// meet at the end.  One launch, where the transforms need three to five: what
+// short operands (the lower levels of the sigma-basis recursion) pay for.
+// FOLD: more terms than 64 bits hold.
+constexpr int kPdWarps = 8;
+constexpr int kPdTile = 32 * 36 + 32 * 8;   // words of a warp's tiles: rows of A (padded by 4 words), then B
+static_assert(16 * 36 + 32 * 16 <= kPdTile && 8 * 36 + 32 * 32 <= kPdTile, "16 rows by 16 columns, 8 rows by 32");
+
+struct PmDirect {
+    const u32 *A, *B;
+    u32 *C;
+    int sr, si, sc, da, db, klo;
+    int si4, ast, ntj, lgn;   // si rounded up to 4, row stride of the A tile, column threads and their log2
+    const int *ea, *eb;
+    Mod M;
+    PmNode node;
+};
+
+template <bool FOLD>
+__global__ void __launch_bounds__(kPdWarps * 32) k_pm_direct(const __grid_constant__ PmDirect a)
+{
+    __shared__ __align__(16) u32 tile[kPdWarps][kPdTile];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k = a.klo + blockIdx.x;
+    const int da = a.ea ? min(a.da, __ldg(a.ea)) : a.da, db = a.eb ? min(a.db, __ldg(a.eb)) : a.db;
+    const int nti = 32 >> a.lgn, rows = min(2 * nti, 32), i0 = blockIdx.y * rows;
+    const int ti = lane >> a.lgn, tj = lane & (a.ntj - 1);
+    const int cols4 = 4 * a.ntj, nr = min(rows, a.sr - i0);
+    u32 *As = tile[warp], *Bs = As + rows * a.ast;
+    if (nr < rows || a.si != a.si4 || a.sc != cols4) {
+        // padding rows and columns are never loaded and read as zero
+        for (int i = lane; i < kPdTile; i += 32) As[i] = 0u;
+    }
+    u64 acc[2][4];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0;
+    const bool vec = (a.si & 3) == 0 && (a.sc & 3) == 0;   // rows of 16-byte blocks (device arrays are 16-byte aligned)
+    const u32 *ap = As + min(ti, rows - 1) * a.ast, *ap1 = As + min(ti + nti, rows - 1) * a.ast, *bp = Bs + 4 * tj;
+    for (int x = max(0, k - db) + warp; x <= min(da, k); x += kPdWarps) {
+        const u32 *ag = a.A + ((size_t)x * a.sr + i0) * a.si, *bg = a.B + (size_t)(k - x) * a.si * a.sc;
+        __syncwarp();
+        if (vec) {
+            const int qa = a.si >> 2, qb = a.sc >> 2;
+            for (int e = lane; e < nr * qa; e += 32) {
+                const int r = e / qa, c = e - r * qa;
+                *reinterpret_cast<uint4 *>(As + r * a.ast + 4 * c) = __ldg(reinterpret_cast<const uint4 *>(ag) + e);
+            }
+            for (int e = lane; e < a.si * qb; e += 32) {
+                const int r = e / qb, c = e - r * qb;
+                *reinterpret_cast<uint4 *>(Bs + r * cols4 + 4 * c) = __ldg(reinterpret_cast<const uint4 *>(bg) + e);
+            }
+        } else {
+            for (int e = lane; e < nr * a.si; e += 32) {
+                const int r = e / a.si, c = e - r * a.si;
+                As[r * a.ast + c] = __ldg(ag + e);
+            }
+            for (int e = lane; e < a.si * a.sc; e += 32) {
+                const int r = e / a.sc, c = e - r * a.sc;
+                Bs[r * cols4 + c] = __ldg(bg + e);
+            }
+        }
+        __syncwarp();
+        for (int kk = 0; kk < a.si4; kk += 4) {
+            const uint4 av[2] = {*reinterpret_cast<const uint4 *>(ap + kk), *reinterpret_cast<const uint4 *>(ap1 + kk)};
+            uint4 bv[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) bv[r] = *reinterpret_cast<const uint4 *>(bp + (kk + r) * cols4);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const u32 ar[4] = {av[r].x, av[r].y, av[r].z, av[r].w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    acc[r][0] += (u64)ar[u] * bv[u].x;
+                    acc[r][1] += (u64)ar[u] * bv[u].y;
+                    acc[r][2] += (u64)ar[u] * bv[u].z;
+                    acc[r][3] += (u64)ar[u] * bv[u].w;
+                    if (FOLD && (u & 1)) {
+                        // two products below p^2 < 2^62 on top of less than p 2^32
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const u32 hi = (u32)(acc[r][c] >> 32);
+                            acc[r][c] = (u64)min(hi, hi - a.M.m) << 32 | (u32)acc[r][c];
+                        }
+                    }
+                }
+            }
+        }
+    }
+    // the warps' sums, each below p: entry (ti + nti r, 4 tj + c) at [r][c][lane]
+    __syncthreads();
+    u32 *red = tile[0];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) red[(warp * 8 + r * 4 + c) * 32 + lane] = red64(acc[r][c], a.M);
+    __syncthreads();
+    u32 *cg = a.C + (size_t)blockIdx.x * a.sr * a.sc;
+    {
+        const int l = lane, rc = warp;   // 256 threads: one entry each
+        const int i = (l >> a.lgn) + (rc >> 2) * nti, j = 4 * (l & (a.ntj - 1)) + (rc & 3);
+        u64 s = 0;
+#pragma unroll
+        for (int w = 0; w < kPdWarps; ++w) s += red[(w * 8 + rc) * 32 + l];
+        if (i < nr && j < a.sc) cg[(size_t)(i0 + i) * a.sc + j] = red64(s, a.M);
+    }
+    if (a.node.out && blockIdx.x == 0 && blockIdx.y == 0 && warp == 0) pm_node(a.node, lane);
+}
+
+}  // namespace
+
+size_t pm_product_bytes(int sr, int si, int sc, long long da, long long db, long long klo, long long khi, int npr)
+{
+    const int lg = pm_length_log(da, db, klo, khi);
+    if (lg > kPmMaxLog) return 0;
+    return ((size_t)npr * ((size_t)sr * si + (size_t)si * sc + (size_t)sr * sc) << lg) * 4;
+}
+
+ffspmv_status pm_direct(u32 p, int sr, int si, int sc, int da, int db, const u32 *A, const u32 *B, u32 *C, int klo,
+                        int khi, const int *ea, const int *eb, const PmNode *node, cudaStream_t st)
+{
+    PmDirect a;
+    memset(&a, 0, sizeof(a));
+    a.A = A;
+    a.B = B;
+    a.C = C;
+    a.sr = sr;
+    a.si = si;
+    a.sc = sc;
+    a.da = da;
+    a.db = db;
+    a.klo = klo;
+    a.si4 = (si + 3) / 4 * 4;
+    a.ast = a.si4 + 4;
+    while ((4 << a.lgn) < sc) ++a.lgn;
+    a.ntj = 1 << a.lgn;
+    a.ea = ea;
+    a.eb = eb;
+    a.M = make_mod(p, 1, 0);
+    if (node) a.node = *node;
+    const int rows = std::min(2 * (32 >> a.lgn), 32);
+    const dim3 grid((unsigned)(khi - klo + 1), (unsigned)((sr + rows - 1) / rows));
+    // terms of one warp's sum
+    const unsigned __int128 terms = (unsigned __int128)si * ((std::min(da, db) + kPdWarps) / kPdWarps + 1);
+    const bool fold = terms * (p - 1) * (p - 1) >= ((unsigned __int128)1 << 64);
+    if (fold) k_pm_direct<true><<<grid, kPdWarps * 32, 0, st>>>(a);
+    else k_pm_direct<false><<<grid, kPdWarps * 32, 0, st>>>(a);
+    FF_CUDA(cudaGetLastError());
     return FFSPMV_OK;
 }
 
-extern "C" ffspmv_status polymat_mul(uint32_t p, int32_t s, int64_t da, int64_t db, const uint32_t *d_A,
-                                     const uint32_t *d_B, uint32_t *d_C, void *d_work, int64_t work_bytes,
-                                     ffspmv_stream_t stream)
+ffspmv_status pm_product(u32 p, int sr, int si, int sc, long long da, long long db, const u32 *A_, const u32 *B_, u32 *C_,
+                         long long klo, long long khi, void *work, size_t work_bytes, cudaStream_t st)
 {
-    if (p < 2 || p > (1u << 31) || s < 1 || s > 32 || da < 0 || db < 0 || !d_A || !d_B || !d_C || !d_work)
-        return FFSPMV_ERR_ARG;
-    int64_t need = 0;
-    ffspmv_status r = polymat_mul_workspace(s, da, db, &need);
-    if (r != FFSPMV_OK) return r;
-    if (work_bytes < need || ((uintptr_t)d_work & 15)) return FFSPMV_ERR_ARG;
     // the exact coefficients must stay below the product of the primes
-    const int npr = pm_primes(p, s, std::min(da, db) + 1);
-    if (!npr) return FFSPMV_ERR_UNSUPPORTED;
-    cudaStream_t st = (cudaStream_t)stream;
-    const int lg = pm_log2(da + db + 1);
+    const int npr = pm_primes(p, si, std::min(da, db) + 1);
+    const size_t need = pm_product_bytes(sr, si, sc, da, db, klo, khi, npr);
+    if (!npr || !need) return FFSPMV_ERR_UNSUPPORTED;
+    if (work_bytes < need) return FFSPMV_ERR_ARG;
+    ffspmv_status r;
+    const int lg = pm_length_log(da, db, klo, khi);
     // L <= 256 in one pass, else two axes of at most 256 points
     const int lg2 = lg <= 8 ? 0 : lg / 2, lg1 = lg - lg2;
     const long long L = 1LL << lg;
-    const int ne = s * s;
-    u32 *Ah = (u32 *)d_work, *Bh = Ah + (size_t)npr * L * ne, *Ch = Bh + (size_t)npr * L * ne;
-    auto tiles = [&](int ln) { return (unsigned)((((long long)ne << (lg - ln)) + kPmLanes - 1) / kPmLanes); };
-    PmOp A = {d_A, (da + 1) * ne, Ah, ne, tiles(lg1)}, B = {d_B, (db + 1) * ne, Bh, ne, tiles(lg1)};
+    const int ea = sr * si, eb = si * sc, ec = sr * sc;
+    u32 *Ah = (u32 *)work, *Bh = Ah + (size_t)npr * L * ea, *Ch = Bh + (size_t)npr * L * eb;
+    auto tiles = [&](int ne, int ln) { return (unsigned)((((long long)ne << (lg - ln)) + kPmLanes - 1) / kPmLanes); };
+    PmOp A = {A_, (da + 1) * ea, Ah, ea, tiles(ea, lg1)}, B = {B_, (db + 1) * eb, Bh, eb, tiles(eb, lg1)};
     if (lg2 == 0) {
         if ((r = pm_pass<PM_F>(lg1, A, B, lg, lg2, npr, st)) != FFSPMV_OK) return r;
     } else {
         if ((r = pm_pass<PM_F1>(lg1, A, B, lg, lg2, npr, st)) != FFSPMV_OK) return r;
-        A.tiles = B.tiles = tiles(lg2);
+        A.tiles = tiles(ea, lg2);
+        B.tiles = tiles(eb, lg2);
         if ((r = pm_pass<PM_F2>(lg2, A, B, lg, lg2, npr, st)) != FFSPMV_OK) return r;
     }
     PmPw w;
     memset(&w, 0, sizeof(w));
-    w.sr = w.si = w.sc = s;
+    w.sr = sr;
+    w.si = si;
+    w.sc = sc;
     w.si4 = (w.si + 3) / 4 * 4;
     w.sc4 = (w.sc + 3) / 4 * 4;
     w.nti = (w.sr + 3) / 4;
@@ -608,14 +756,16 @@ extern "C" ffspmv_status polymat_mul(uint32_t p, int32_t s, int64_t da, int64_t 
     w.tp = kPwThreads / (w.nti * w.ntj);
     w.ast = 4 * w.nti * w.si4 + 4;   // 4 words of padding: neighbouring points start in other banks
     w.bst = w.si4 * w.sc4 + 4;
+    // both matrices of every point in at most 96 KB (two CTAs per SM)
+    w.tp = std::max(1, std::min(w.tp, (int)(96 * 1024 / 4) / (w.ast + w.bst)));
     w.L = (int)L;
     auto magic = [](int d) { return (u32)((((u64)1 << 32) + d - 1) / d); };
-    w.m_a = magic(w.sr * w.si);
+    w.m_a = magic(ea);
     w.m_si = magic(w.si);
-    w.m_b = magic(w.si * w.sc);
+    w.m_b = magic(eb);
     w.m_sc = magic(w.sc);
     const size_t pw_smem = (size_t)w.tp * (w.ast + w.bst) * 4;
-    FF_CUDA(cudaFuncSetAttribute(k_pm_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw_smem));
+    FF_CUDA(cudaFuncSetAttribute(k_pm_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
     k_pm_pointwise<<<dim3((unsigned)((L + w.tp - 1) / w.tp), (unsigned)npr), kPwThreads, pw_smem, st>>>(Ah, Bh, Ch, w);
     FF_CUDA(cudaGetLastError());
     PmOut c;
@@ -637,10 +787,36 @@ extern "C" ffspmv_status polymat_mul(uint32_t p, int32_t s, int64_t da, int64_t 
     c.p0_mod_p = (u32)(kPmP[0] % p);
     c.p0p1_mod_p = (u32)((unsigned __int128)kPmP[0] * kPmP[1] % p);
     if (lg2) {
-        const PmOp Cc = {nullptr, 0, Ch, ne, tiles(lg2)}, none = {nullptr, 0, nullptr, 1, 0};
+        const PmOp Cc = {nullptr, 0, Ch, ec, tiles(ec, lg2)}, none = {nullptr, 0, nullptr, 1, 0};
         if ((r = pm_pass<PM_I1>(lg2, Cc, none, lg, lg2, npr, st)) != FFSPMV_OK) return r;
     }
-    return npr == 1   ? pm_out<1>(lg1, Ch, d_C, ne, lg, lg2, 0, da + db, c, st)
-           : npr == 2 ? pm_out<2>(lg1, Ch, d_C, ne, lg, lg2, 0, da + db, c, st)
-                      : pm_out<3>(lg1, Ch, d_C, ne, lg, lg2, 0, da + db, c, st);
+    return npr == 1   ? pm_out<1>(lg1, Ch, C_, ec, lg, lg2, klo, khi, c, st)
+           : npr == 2 ? pm_out<2>(lg1, Ch, C_, ec, lg, lg2, klo, khi, c, st)
+                      : pm_out<3>(lg1, Ch, C_, ec, lg, lg2, klo, khi, c, st);
+}
+
+}  // namespace ff
+
+using namespace ff;
+
+extern "C" ffspmv_status polymat_mul_workspace(int32_t s, int64_t da, int64_t db, int64_t *bytes)
+{
+    if (!bytes || s < 1 || s > 32 || da < 0 || db < 0) return FFSPMV_ERR_ARG;
+    if (da + db + 1 > (1LL << kPmMaxLog)) return FFSPMV_ERR_UNSUPPORTED;
+    const long long L = 1LL << pm_log2(da + db + 1);
+    *bytes = 3LL * kPmPrimes * s * s * L * 4 + (long long)kPmPrimes * L * 8 + 256;
+    return FFSPMV_OK;
+}
+
+extern "C" ffspmv_status polymat_mul(uint32_t p, int32_t s, int64_t da, int64_t db, const uint32_t *d_A,
+                                     const uint32_t *d_B, uint32_t *d_C, void *d_work, int64_t work_bytes,
+                                     ffspmv_stream_t stream)
+{
+    if (p < 2 || p > (1u << 31) || s < 1 || s > 32 || da < 0 || db < 0 || !d_A || !d_B || !d_C || !d_work)
+        return FFSPMV_ERR_ARG;
+    int64_t need = 0;
+    const ffspmv_status r = polymat_mul_workspace(s, da, db, &need);
+    if (r != FFSPMV_OK) return r;
+    if (work_bytes < need || ((uintptr_t)d_work & 15)) return FFSPMV_ERR_ARG;
+    return pm_product(p, s, s, s, da, db, d_A, d_B, d_C, 0, da + db, d_work, (size_t)work_bytes, (cudaStream_t)stream);
 }
