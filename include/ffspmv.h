@@ -206,11 +206,13 @@ ffspmv_status spmv_block_project_finish(uint32_t p, int32_t s, uint64_t *d_Sacc,
  * (not in the paper).  hs: host array of handles (each with its own
  * modulus); d_x / d_y: host arrays of device pointers, X_j: ncols_j x nvec[j]
  * row-major (ld = nvec[j]), Y_j: nrows_j x nvec[j]; 1 <= nvec[j] <= 32.
- * The work list is rebuilt on the host only when the set of handles or nvec
- * changes; that first call also times a few tile shapes (rows per work item,
- * length from which a row gets a whole CTA) on the device and keeps the
- * fastest, writing the outputs several times with the same values.  Not
- * thread-safe: one host thread at a time.
+ * The first batched (or block) product of a handle builds its block layout
+ * (synchronous, host work plus one allocation per handle); after that a call
+ * with any set of handles only launches: one product kernel per 512 matrices,
+ * and one that packs the X_j which are not made of whole aligned 16-byte
+ * pieces.  A handle may appear several times: its products then run one after
+ * another.  Like the other products, calls that share a handle must not
+ * overlap on the GPU.
  */
 ffspmv_status spmv_batch_apply(int32_t count, const ffspmv_t *hs,
                                const uint32_t *const *d_x,

@@ -56,7 +56,6 @@ void destroy_handle(ffspmv_handle *h)
     if (h->csr_arena) cudaFree(h->csr_arena);
     if (h->d_status) cudaFree(h->d_status);
     free_sequence_state(h);
-    batch_forget(h);
     free_gf2(h);
     free_block(h);
     delete h;

@@ -9,8 +9,8 @@
 // The x-panel layout, which is faster for one vector, has no such gain: its
 // panels and row groups shrink as x and the row sums widen.  Measured on the
 // 1M x 1M power-law matrix (15.8M entries, m = 65521), 16 vectors: 643 us
-// in passes of the x-panel layout, 130 us here (14 us of it the packing); 16
-// vectors at m = 2^31 - 1: 1093 -> 192 us; 90 001 x 120 011 with power-law rows
+// in passes of the x-panel layout, 128 us here (14 us of it the packing); 16
+// vectors at m = 2^31 - 1: 1093 -> 181 us; 90 001 x 120 011 with power-law rows
 // (binned plan): 515 -> 20 us.
 //
 // Layout.  Rows are ordered by length class and their entries stored in that
@@ -46,17 +46,26 @@ int block_class(long long len)
     return c;
 }
 
-// groups of lanes that share a row of the class, one quad each per step
-int block_groups(int c)
-{
-    const int g[kBlockClasses] = {1, 1, 1, 2, 4, 8, 32};
-    return g[c];
-}
-
 }  // namespace
+
+// What a launch over many matrices reads of each (k_block_many).
+struct BlockDev {
+    const u32 *ptr, *row, *col, *lrow;
+    const uint4 *chunk;
+    const void *val;
+    uint4 *xs;
+    u64 *carry;
+    u32 *count;
+    long long ncols;
+    u32 row0[kBlockClasses + 1];  // rows of each class, heaviest class first
+    u32 nchunk, quad1;
+    int small, fold;
+    Mod M;
+};
 
 struct BlockPlan {
     bool ok = false;
+    const BlockDev *dev = nullptr;
     void *arena = nullptr;
     long long n = 0, ncols = 0;
     bool small = true;                 // m <= 2^16: u16 values and staged x
@@ -87,16 +96,12 @@ void free_block(ffspmv_handle *h)
 
 namespace {
 
-// Rows of X packed to `pitch` 16-byte words each: u16 or u32 residues, zero
-// past nvec.  One thread per word.
+// Word t of the rows of X packed to `pitch` 16-byte words each: u16 or u32
+// residues, zero past nvec.
 template <bool SMALL>
-__global__ void __launch_bounds__(kBlockThreads) k_block_stage(const u32 *__restrict__ x, long long ldx, long long n,
-                                                              int nvec, int pitch, int vec4, uint4 *__restrict__ xs)
+__device__ __forceinline__ uint4 block_pack(const u32 *__restrict__ x, long long ldx, long long t, int nvec, int pitch, int vec4)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int C = SMALL ? 8 : 4;
-    const long long t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
-    if (t >= n * pitch) return;
     const long long i = t / pitch;
     const int c0 = (int)(t - i * pitch) * C;
     const u32 *p = x + i * ldx + c0;
@@ -111,19 +116,24 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_stage(const u32 *__rest
 #pragma unroll
         for (int u = 0; u < C; ++u) v[u] = c0 + u < nvec ? __ldg(p + u) : 0u;
     }
-    uint4 o;
-    if constexpr (SMALL) {
-        o.x = (v[0] & 0xffffu) | v[1] << 16;
-        o.y = (v[2] & 0xffffu) | v[3] << 16;
-        o.z = (v[4] & 0xffffu) | v[5] << 16;
-        o.w = (v[6] & 0xffffu) | v[7] << 16;
-    } else {
-        o = make_uint4(v[0], v[1], v[2], v[3]);
-    }
-    xs[t] = o;
+    if constexpr (SMALL)
+        return make_uint4((v[0] & 0xffffu) | v[1] << 16, (v[2] & 0xffffu) | v[3] << 16, (v[4] & 0xffffu) | v[5] << 16,
+                          (v[6] & 0xffffu) | v[7] << 16);
+    else
+        return make_uint4(v[0], v[1], v[2], v[3]);
 }
 
-struct BlockArgs {
+template <bool SMALL>
+__global__ void __launch_bounds__(kBlockThreads) k_block_stage(const u32 *__restrict__ x, long long ldx, long long n,
+                                                              int nvec, int pitch, int vec4, uint4 *__restrict__ xs)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long long t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
+    if (t < n * pitch) xs[t] = block_pack<SMALL>(x, ldx, t, nvec, pitch, vec4);
+}
+
+// One matrix and one block of vectors, as a warp needs them.
+struct BlockMat {
     const u32 *ptr, *row, *col, *lrow;
     const uint4 *chunk;
     const void *val;
@@ -133,13 +143,17 @@ struct BlockArgs {
     u32 *y;
     long long ldy;
     int pitch, pieces, nvec, vec4, lgt;  // pieces of 16 bytes per row of X; lgt: log2 of the lanes that hold them
+    u32 quad1;                    // rows r of the one-quad class: quad quad1 + r
+    int fold;                     // m <= 2^31
+    Mod M;
+};
+
+struct BlockArgs {
+    BlockMat m;
     int nchunk_warps;             // warps 0 .. nchunk - 1 take the chunks
     u32 warp0[kBlockClasses + 1]; // first warp of each class, heaviest class first
     u32 row0[kBlockClasses + 1];  // its rows
     int lgg[kBlockClasses];       // log2 of groups per row
-    u32 quad1;                    // rows r of the one-quad class: quad quad1 + r
-    int fold;                     // m <= 2^31
-    Mod M;
 };
 
 // Sums of one lane: 8 components of u16 residues (64-bit sums of terms below
@@ -201,6 +215,9 @@ struct BlockAcc<false> {
         }
         if (fold) {
             // m <= 2^31: four products, each below 2^62, in one 64-bit word
+            // (a run-time test on purpose: it keeps the four gathers and the
+            // next quad's loads ahead of the sums; as a template the sums
+            // moved in between, 236 us against 191 at 16 vectors)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const u64 t = (u64)v[0] * w[0][i] + (u64)v[1] * w[1][i] + (u64)v[2] * w[2][i] + (u64)v[3] * w[3][i];
@@ -238,7 +255,7 @@ struct BlockAcc<false> {
 // acc += quads k, k + step, ... below end; xb: this lane's piece of the rows
 // of X.  Rows are padded to whole quads (value 0, column 0).
 template <bool SMALL>
-__device__ __forceinline__ void block_entries(BlockAcc<SMALL> &acc, const BlockArgs &a, u32 k, u32 end, u32 step,
+__device__ __forceinline__ void block_entries(BlockAcc<SMALL> &acc, const BlockMat &a, u32 k, u32 end, u32 step,
                                               const char *xb, bool on)
 {
     typedef typename std::conditional<SMALL, uint2, uint4>::type V;
@@ -270,7 +287,7 @@ __device__ __forceinline__ void block_entries(BlockAcc<SMALL> &acc, const BlockA
 
 // R consecutive components from column col0 of a row
 template <int R>
-__device__ __forceinline__ void block_write(const u32 (&r)[R], const BlockArgs &a, u32 row, int col0)
+__device__ __forceinline__ void block_write(const u32 (&r)[R], const BlockMat &a, u32 row, int col0)
 {
     u32 *yp = a.y + (long long)row * a.ldy + col0;
     if (R >= 4 && a.vec4 && col0 + R <= a.nvec) {
@@ -325,7 +342,7 @@ __device__ __forceinline__ void block_reduce(typename BlockAcc<SMALL>::Sum (&s)[
 }
 
 struct BlockEmitRow {
-    const BlockArgs *a;
+    const BlockMat *a;
     const Mod *M;
     u32 row;
     bool ok;
@@ -337,7 +354,7 @@ struct BlockEmitRow {
 };
 
 struct BlockEmitCarry {
-    const BlockArgs *a;
+    const BlockMat *a;
     const Mod *M;
     u64 *cw;
     template <int R>
@@ -349,40 +366,67 @@ struct BlockEmitCarry {
     }
 };
 
-// One warp per chunk of a long row, or per 32 / (T G) rows of a class.
+// A warp's chunk of a long row.
 template <bool SMALL>
-__global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constant__ BlockArgs a)
+__device__ __forceinline__ void block_chunk(const BlockMat &a, u32 w, int lane)
 {
     constexpr int C = BlockAcc<SMALL>::C;
-    const u32 w = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31, T = 1 << a.lgt, c = lane & (T - 1);
-    const char *xb = reinterpret_cast<const char *>(a.xs + c);
+    const int T = 1 << a.lgt, c = lane & (T - 1);
+    BlockAcc<SMALL> acc;
+    acc.zero();
+    const uint4 ch = __ldg(a.chunk + w);
+    block_entries<SMALL>(acc, a, ch.y + (u32)(lane >> a.lgt), ch.z, 32u >> a.lgt,
+                         reinterpret_cast<const char *>(a.xs + c), c < a.pieces);
+    u64 *cw = a.carry + (size_t)ch.x * kBlockVecs;
+    const BlockEmitCarry emit = {&a, &a.M, cw};
+    block_reduce<SMALL, C>(acc.a, a.lgt, 5 - a.lgt, 0, lane, c * C, emit);
+    // the chunk that arrives last writes the row and clears its words
+    u32 last = 0;
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) last = atomicAdd(a.count + ch.x, 1u) == ch.w - 1u ? 1u : 0u;
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (!last) return;
+    __threadfence();
+    const u32 row = __ldg(a.lrow + ch.x);
+    if (lane < a.nvec) {
+        u32 *yp = a.y + (long long)row * a.ldy + lane;
+        *yp = combine(red64(__ldcg(cw + lane), a.M), yp, false, a.M);
+        cw[lane] = 0;
+    }
+    if (lane == 0) a.count[ch.x] = 0;
+}
+
+// A warp's 32 / (T G) rows of a class: r0 the first, below rend, G = 2^lgg.
+template <bool SMALL>
+__device__ __forceinline__ void block_rows(const BlockMat &a, u32 r0, u32 rend, int lgg, bool one, int lane)
+{
+    constexpr int C = BlockAcc<SMALL>::C;
+    const int T = 1 << a.lgt, c = lane & (T - 1), lgr = a.lgt + lgg;
     const bool on = c < a.pieces;
     BlockAcc<SMALL> acc;
     acc.zero();
+    const u32 r = r0 + (u32)(lane >> lgr);
+    BlockEmitRow emit = {&a, &a.M, 0u, r < rend && on};
+    if (r < rend) {
+        // rows of one quad lie one after another: no offset to wait for
+        const u32 s = one ? a.quad1 + r : __ldg(a.ptr + r), e = one ? s + 1u : __ldg(a.ptr + r + 1);
+        emit.row = __ldg(a.row + r);
+        block_entries<SMALL>(acc, a, s + (u32)((lane >> a.lgt) & ((1 << lgg) - 1)), e, 1u << lgg,
+                             reinterpret_cast<const char *>(a.xs + c), on);
+    }
+    block_reduce<SMALL, C>(acc.a, a.lgt, lgg, 0, lane, c * C, emit);
+}
+
+template <bool SMALL>
+__global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constant__ BlockArgs a)
+{
+    const u32 w = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     // the rows of X come from the staging launch before this one
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (w < (u32)a.nchunk_warps) {
-        const uint4 ch = __ldg(a.chunk + w);
-        block_entries<SMALL>(acc, a, ch.y + (u32)(lane >> a.lgt), ch.z, 32u >> a.lgt, xb, on);
-        u64 *cw = a.carry + (size_t)ch.x * kBlockVecs;
-        const BlockEmitCarry emit = {&a, &a.M, cw};
-        block_reduce<SMALL, C>(acc.a, a.lgt, 5 - a.lgt, 0, lane, c * C, emit);
-        // the chunk that arrives last writes the row and clears its words
-        u32 last = 0;
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) last = atomicAdd(a.count + ch.x, 1u) == ch.w - 1u ? 1u : 0u;
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (!last) return;
-        __threadfence();
-        const u32 row = __ldg(a.lrow + ch.x);
-        if (lane < a.nvec) {
-            u32 *yp = a.y + (long long)row * a.ldy + lane;
-            *yp = combine(red64(__ldcg(cw + lane), a.M), yp, false, a.M);
-            cw[lane] = 0;
-        }
-        if (lane == 0) a.count[ch.x] = 0;
+        block_chunk<SMALL>(a.m, w, lane);
         return;
     }
     // the class of this warp (warp0 grows; the last entry ends the list)
@@ -391,17 +435,114 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constan
     for (int i = 1; i < kBlockClasses; ++i)
         if (w >= a.warp0[i]) b = i;
     if (w >= a.warp0[kBlockClasses]) return;
-    const int lgg = a.lgg[b], lgr = a.lgt + lgg;   // log2 of groups and of lanes per row
-    const u32 r = a.row0[b] + ((w - a.warp0[b]) << (5 - lgr)) + (u32)(lane >> lgr);
-    BlockEmitRow emit = {&a, &a.M, 0u, r < a.row0[b + 1] && on};
-    if (r < a.row0[b + 1]) {
-        // rows of one quad lie one after another: no offset to wait for
-        const bool one = b == kBlockClasses - 2;
-        const u32 s = one ? a.quad1 + r : __ldg(a.ptr + r), e = one ? s + 1u : __ldg(a.ptr + r + 1);
-        emit.row = __ldg(a.row + r);
-        block_entries<SMALL>(acc, a, s + (u32)((lane >> a.lgt) & ((1 << lgg) - 1)), e, 1u << lgg, xb, on);
+    const int lgg = a.lgg[b];
+    block_rows<SMALL>(a.m, a.row0[b] + ((w - a.warp0[b]) << (5 - a.m.lgt - lgg)), a.row0[b + 1], lgg,
+                      b == kBlockClasses - 2, lane);
+}
+
+// log2 of the groups per row of class i (heaviest first), 2^lgt lanes per row
+// of X.  A group's epilogue (sums joined, one reduction per component) costs
+// about as much as three quads, so rows share as few groups as keep the warp's
+// lanes busy: with four or more lanes per row of X fewer still.  300 007 x
+// 200 003, 22 per row, m = 2^31 - 1, 16 vectors: 79 us with 8 / 4 / 2 groups
+// for classes 1 to 3, 59 with 4 / 2 / 1, 53 with 2 / 1 / 1 (3 vectors: 39, 39,
+// 45).
+__host__ __device__ inline int block_lgg(int i, int lgt)
+{
+    const int lg = i == 0 ? 4 : lgt < 2 ? (i == 1 ? 2 : i == 2 ? 1 : 0) : i == 1 ? 1 : 0;
+    return lg < 5 - lgt ? lg : 5 - lgt;
+}
+
+// Many matrices in one launch, each with its modulus, vectors and packed X:
+// what a launch passes for one of them, and the first warp (or, for the
+// staging, the first CTA) of each.
+constexpr int kMany = 512;
+struct BlockMany {
+    const BlockDev *dev[kMany];
+    const u32 *x[kMany];
+    u32 *y[kMany];
+    u32 first[kMany + 1];
+    unsigned char nvec[kMany], place[kMany];  // place: x is read where it lies
+    int count;
+};
+static_assert(sizeof(BlockMany) < 32000, "launch parameters");
+
+__device__ __forceinline__ int block_find(const BlockMany &P, u32 w)
+{
+    int lo = 0, hi = P.count - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (P.first[mid] <= w) lo = mid;
+        else hi = mid - 1;
     }
-    block_reduce<SMALL, C>(acc.a, a.lgt, lgg, 0, lane, c * C, emit);
+    return lo;
+}
+
+__global__ void __launch_bounds__(kBlockThreads) k_block_stage_many(const __grid_constant__ BlockMany P)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int j = block_find(P, blockIdx.x);
+    const BlockDev &D = *P.dev[j];
+    const int nvec = P.nvec[j], C = D.small ? 8 : 4, pieces = (nvec + C - 1) / C;
+    const u32 *x = P.x[j];
+    const int vec4 = nvec % 4 == 0 && ((uintptr_t)x & 15u) == 0;
+    const long long t = (long long)(blockIdx.x - P.first[j]) * kBlockThreads + threadIdx.x;
+    if (t >= D.ncols * pieces) return;
+    D.xs[t] = D.small ? block_pack<true>(x, nvec, t, nvec, pieces, vec4) : block_pack<false>(x, nvec, t, nvec, pieces, vec4);
+}
+
+__global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_constant__ BlockMany P)
+{
+    const u32 w0 = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
+    if (w0 >= P.first[P.count]) return;
+    const int lane = threadIdx.x & 31, j = block_find(P, w0);
+    const BlockDev &D = *P.dev[j];
+    BlockMat a;
+    a.ptr = D.ptr;
+    a.row = D.row;
+    a.col = D.col;
+    a.lrow = D.lrow;
+    a.chunk = D.chunk;
+    a.val = D.val;
+    a.carry = D.carry;
+    a.count = D.count;
+    a.y = P.y[j];
+    a.nvec = P.nvec[j];
+    a.ldy = a.nvec;
+    const int C = D.small ? 8 : 4;
+    a.pieces = (a.nvec + C - 1) / C;
+    a.lgt = a.pieces > 1 ? 32 - __clz(a.pieces - 1) : 0;
+    a.xs = P.place[j] ? reinterpret_cast<const uint4 *>(P.x[j]) : D.xs;
+    a.pitch = a.pieces;
+    a.vec4 = a.nvec % 4 == 0 && ((uintptr_t)a.y & 15u) == 0;
+    a.quad1 = D.quad1;
+    a.fold = D.fold;
+    a.M = D.M;
+    u32 w = w0 - P.first[j];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (w < D.nchunk) {
+        if (D.small) block_chunk<true>(a, w, lane);
+        else block_chunk<false>(a, w, lane);
+        return;
+    }
+    w -= D.nchunk;
+    int b = 0, lgg = 0;
+    u32 r0 = 0, rend = 0;
+    for (; b < kBlockClasses; ++b) {
+        r0 = D.row0[b];
+        rend = D.row0[b + 1];
+        lgg = block_lgg(b, a.lgt);
+        const int sh = 5 - a.lgt - lgg;
+        const u32 nw = (u32)(((u64)(rend - r0) + (1u << sh) - 1u) >> sh);
+        if (w < nw) {
+            r0 += w << sh;
+            break;
+        }
+        w -= nw;
+    }
+    if (b == kBlockClasses) return;
+    if (D.small) block_rows<true>(a, r0, rend, lgg, b == kBlockClasses - 2, lane);
+    else block_rows<false>(a, r0, rend, lgg, b == kBlockClasses - 2, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -499,7 +640,7 @@ ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long
     const size_t o_ptr = put(rptr.size() * 4), o_row = put(row.size() * 4), o_chunk = put(chunk.size() * 16),
                  o_lrow = put(lrow.size() * 4), o_col = put(pcol.size() * 4), o_val = put(pval.size()),
                  o_carry = put((size_t)B.nlong * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
-                 o_xs = put((size_t)ncols * kBlockVecs * vb);
+                 o_dev = put(sizeof(BlockDev)), o_xs = put((size_t)ncols * kBlockVecs * vb);
     if (cudaMalloc(&B.arena, o) != cudaSuccess) {
         cudaGetLastError();
         B.arena = nullptr;
@@ -512,7 +653,7 @@ ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long
     const bool ok = up(o_ptr, rptr.data(), rptr.size() * 4) && up(o_row, row.data(), row.size() * 4) &&
                     up(o_chunk, chunk.data(), chunk.size() * 16) && up(o_lrow, lrow.data(), lrow.size() * 4) &&
                     up(o_col, pcol.data(), slots * 4) && up(o_val, pval.data(), slots * vb) &&
-                    cudaMemset(base + o_carry, 0, o_xs - o_carry) == cudaSuccess;
+                    cudaMemset(base + o_carry, 0, o_dev - o_carry) == cudaSuccess;
     if (!ok) {
         cudaFree(B.arena);
         B.arena = nullptr;
@@ -528,6 +669,31 @@ ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long
     B.carry = (u64 *)(base + o_carry);
     B.count = (u32 *)(base + o_count);
     B.xs = (uint4 *)(base + o_xs);
+    BlockDev D;
+    memset(&D, 0, sizeof(D));
+    D.ptr = B.ptr;
+    D.row = B.row;
+    D.col = B.col;
+    D.lrow = B.lrow;
+    D.chunk = B.chunk;
+    D.val = B.val;
+    D.xs = B.xs;
+    D.carry = B.carry;
+    D.count = B.count;
+    D.ncols = ncols;
+    for (int c = 0; c <= kBlockClasses; ++c) D.row0[c] = (u32)B.cls_row[c];
+    D.nchunk = (u32)B.nchunk;
+    D.quad1 = B.quad1;
+    D.small = B.small ? 1 : 0;
+    D.fold = m <= (1u << 31) ? 1 : 0;
+    D.M = make_mod(m, 1, 0);
+    if (!up(o_dev, &D, sizeof(D))) {
+        cudaFree(B.arena);
+        B.arena = nullptr;
+        cudaGetLastError();
+        return FFSPMV_ERR_CUDA;
+    }
+    B.dev = (const BlockDev *)(base + o_dev);
     return FFSPMV_OK;
 }
 
@@ -568,7 +734,7 @@ const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st)
 // aligned 16-byte pieces of u32.
 static bool block_in_place(const BlockPlan &B, const u32 *x, long long ldx, int nv)
 {
-    return !B.small && nv % 4 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15u) == 0 && ldx / 4 < (1LL << 30);
+    return !B.small && nv % 4 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15u) == 0 && ldx / 4 < (1LL << 28);
 }
 
 long long block_launches(const BlockPlan &B, int nvec)
@@ -589,31 +755,31 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
         u32 *yv = y + v0;
         BlockArgs a;
         memset(&a, 0, sizeof(a));
-        a.ptr = B.ptr;
-        a.row = B.row;
-        a.col = B.col;
-        a.lrow = B.lrow;
-        a.chunk = B.chunk;
-        a.val = B.val;
-        a.carry = B.carry;
-        a.count = B.count;
-        a.quad1 = B.quad1;
-        a.y = yv;
-        a.ldy = ldy;
-        a.nvec = nv;
-        a.vec4 = (ldy % 4 == 0 && ((uintptr_t)yv & 15u) == 0) ? 1 : 0;
-        a.M = make_mod(m, alpha, beta);
-        a.fold = m <= (1u << 31) ? 1 : 0;
+        a.m.ptr = B.ptr;
+        a.m.row = B.row;
+        a.m.col = B.col;
+        a.m.lrow = B.lrow;
+        a.m.chunk = B.chunk;
+        a.m.val = B.val;
+        a.m.carry = B.carry;
+        a.m.count = B.count;
+        a.m.quad1 = B.quad1;
+        a.m.y = yv;
+        a.m.ldy = ldy;
+        a.m.nvec = nv;
+        a.m.vec4 = (ldy % 4 == 0 && ((uintptr_t)yv & 15u) == 0) ? 1 : 0;
+        a.m.M = make_mod(m, alpha, beta);
+        a.m.fold = m <= (1u << 31) ? 1 : 0;
         const int pieces = (nv + C - 1) / C;
-        while ((1 << a.lgt) < pieces) ++a.lgt;
-        a.pieces = pieces;
+        while ((1 << a.m.lgt) < pieces) ++a.m.lgt;
+        a.m.pieces = pieces;
         const bool in_place = block_in_place(B, xv, ldx, nv);
         if (in_place) {
-            a.xs = reinterpret_cast<const uint4 *>(xv);
-            a.pitch = (int)(ldx / 4);
+            a.m.xs = reinterpret_cast<const uint4 *>(xv);
+            a.m.pitch = (int)(ldx / 4);
         } else {
-            a.xs = B.xs;
-            a.pitch = pieces;
+            a.m.xs = B.xs;
+            a.m.pitch = pieces;
             const long long words = B.ncols * pieces;
             const int vec4 = (ldx % 4 == 0 && ((uintptr_t)xv & 15u) == 0) ? 1 : 0;
             if (words > 0) {
@@ -631,13 +797,11 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
         for (int boost = 0; boost < 6; ++boost) {
             warps = B.nchunk;
             for (int c = 0; c < kBlockClasses; ++c) {
-                const int g = block_groups(kBlockClasses - 1 - c) << boost;
-                int lg = 0;
-                while ((2 << lg) <= std::min(g, 32 >> a.lgt)) ++lg;
+                const int lg = std::min(block_lgg(c, a.m.lgt) + boost, 5 - a.m.lgt);
                 a.lgg[c] = lg;
                 a.row0[c] = (u32)B.cls_row[c];
                 a.warp0[c] = (u32)warps;
-                const int rpw = 32 >> (a.lgt + lg);
+                const int rpw = 32 >> (a.m.lgt + lg);
                 warps += (B.cls_row[c + 1] - B.cls_row[c] + rpw - 1) / rpw;
             }
             if (warps >= 16 * 152) break;
@@ -657,6 +821,71 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
         cfg.numAttrs = in_place ? 0 : 1;
         if (B.small) FF_CUDA(cudaLaunchKernelEx(&cfg, k_block<true>, a));
         else FF_CUDA(cudaLaunchKernelEx(&cfg, k_block<false>, a));
+    }
+    return FFSPMV_OK;
+}
+
+// Y_j = A_j X_j for `count` (at most kMany) different plans, contiguous blocks
+// of nvec[j] <= kBlockVecs vectors.
+static ffspmv_status block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
+                                cudaStream_t st)
+{
+    BlockMany P, S;   // the products, and the staging of the X that are not read in place
+    memset(&P, 0, sizeof(P));
+    memset(&S, 0, sizeof(S));
+    long long warps = 0, stage = 0;
+    for (int j = 0; j < count; ++j) {
+        const BlockPlan &b = *B[j];
+        const int C = b.small ? 8 : 4, pieces = (nvec[j] + C - 1) / C;
+        int lgt = 0;
+        while ((1 << lgt) < pieces) ++lgt;
+        P.dev[j] = b.dev;
+        P.x[j] = x[j];
+        P.y[j] = y[j];
+        P.nvec[j] = (unsigned char)nvec[j];
+        P.place[j] = block_in_place(b, x[j], nvec[j], nvec[j]) ? 1 : 0;
+        P.first[j] = (u32)warps;
+        warps += b.nchunk;
+        for (int c = 0; c < kBlockClasses; ++c) {
+            const int rpw = 1 << (5 - lgt - block_lgg(c, lgt));
+            warps += (b.cls_row[c + 1] - b.cls_row[c] + rpw - 1) / rpw;
+        }
+        if (!P.place[j] && b.ncols > 0) {
+            S.dev[S.count] = b.dev;
+            S.x[S.count] = x[j];
+            S.nvec[S.count] = (unsigned char)nvec[j];
+            S.first[S.count++] = (u32)stage;
+            stage += (b.ncols * pieces + kBlockThreads - 1) / kBlockThreads;
+        }
+    }
+    if (warps >= (1LL << 32) - 64 || stage >= (1LL << 31)) return FFSPMV_ERR_UNSUPPORTED;
+    P.first[count] = (u32)warps;
+    P.count = count;
+    if (stage > 0) {
+        S.first[S.count] = (u32)stage;
+        k_block_stage_many<<<(unsigned)stage, kBlockThreads, 0, st>>>(S);
+        FF_CUDA(cudaGetLastError());
+    }
+    if (warps == 0) return FFSPMV_OK;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((warps * 32 + kBlockThreads - 1) / kBlockThreads));
+    cfg.blockDim = dim3(kBlockThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = stage > 0 ? 1 : 0;
+    FF_CUDA(cudaLaunchKernelEx(&cfg, k_block_many, P));
+    return FFSPMV_OK;
+}
+
+ffspmv_status run_block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
+                             cudaStream_t st)
+{
+    for (int c0 = 0; c0 < count; c0 += kMany) {
+        const ffspmv_status r = block_many(std::min(kMany, count - c0), B + c0, x + c0, y + c0, nvec + c0, st);
+        if (r != FFSPMV_OK) return r;
     }
     return FFSPMV_OK;
 }

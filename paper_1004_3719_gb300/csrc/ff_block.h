@@ -17,4 +17,9 @@ long long block_launches(const BlockPlan &B, int nvec);  // of a contiguous, 16-
 ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec, u32 m,
                         u32 alpha, u32 beta, cudaStream_t st);
 
+// Y_j = A_j X_j of different plans, one product launch per 512 of them:
+// contiguous blocks of nvec[j] <= 32 vectors.
+ffspmv_status run_block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
+                             cudaStream_t st);
+
 }  // namespace ff
