@@ -133,9 +133,10 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
  * d_y ("apply": y <- A x).  d_x and d_y must not overlap.  On a handle whose
  * format the library chose (FFSPMV_FMT_AUTO) most blocks run on a layout of
  * their own, up to 32 vectors per pass, with the rows of X packed next to
- * each other: the first such block builds it (synchronous, host work plus
- * one allocation per handle and direction); while the stream is captured
- * before that, or when it cannot be built, the block runs as follows.  On a
+ * each other: the first such block (the second, unless the plan is the x-panel
+ * layout) builds it on the device (synchronous, one allocation per handle and
+ * direction); before that, while the stream is captured before that, and when
+ * it cannot be built, the block runs as follows.  On a
  * handle whose plan is the x-panel layout, a block runs in passes of 4 vectors (m <=
  * 2^16) or 2, then 1: each pass reads the matrix once for all its vectors
  * (Sec. 2.5.1) on an x-panel layout built for that width; the first block
@@ -207,7 +208,7 @@ ffspmv_status spmv_block_project_finish(uint32_t p, int32_t s, uint64_t *d_Sacc,
  * modulus); d_x / d_y: host arrays of device pointers, X_j: ncols_j x nvec[j]
  * row-major (ld = nvec[j]), Y_j: nrows_j x nvec[j]; 1 <= nvec[j] <= 32.
  * The first batched (or block) product of a handle builds its block layout
- * (synchronous, host work plus one allocation per handle); after that a call
+ * (synchronous, one allocation per handle); after that a call
  * with any set of handles only launches: one product kernel per 512 matrices,
  * and one that packs the X_j which are not made of whole aligned 16-byte
  * pieces.  A handle may appear several times: its products then run one after

@@ -414,8 +414,11 @@ static ffspmv_status next_pass(ffspmv_t h, bool transpose, const Plan *P, int le
 //   binned plan: unless the work is small and the plan takes fewer launches
 //     (20 000 x 20 000, 10 per row, m = 65521: 4 vectors in 10 us against 12,
 //     16 in 15.8 against 12; 90 001 x 120 011 power-law, 23 per row: 2
-//     vectors in 62 us against 17, 16 in 515 against 20).
-static const BlockPlan *block_path(ffspmv_t h, bool transpose, int nvec, cudaStream_t st)
+//     vectors in 62 us against 17, 16 in 515 against 20).  The first such
+//     block still takes the plan: building the layout costs 0.1 to 2 ms,
+//     which a single product would not earn back (a panel plan's first block
+//     would build panel layouts instead, which takes longer).
+static const BlockPlan *block_path(ffspmv_t h, bool transpose, int nvec, cudaStream_t st, bool counting = false)
 {
     if (h->opt.priority_format != FFSPMV_FMT_AUTO || nvec < 2 || (h->opt.test_hooks & 12)) return nullptr;
     const Plan &P = transpose ? h->AT : h->A;
@@ -423,6 +426,9 @@ static const BlockPlan *block_path(ffspmv_t h, bool transpose, int nvec, cudaStr
         if (nvec < (h->m <= 256u ? 4 : h->m <= 65536u ? 3 : 2)) return nullptr;
     } else if (P.nnz * nvec < (1LL << 21) && count_plan_launches(P, nvec) < 2LL * std::max(1, (nvec + 31) / 32)) {
         return nullptr;
+    } else if (!counting && !h->block_seen[transpose ? 1 : 0]) {
+        h->block_seen[transpose ? 1 : 0] = true;
+        if (!h->block[transpose ? 1 : 0]) return nullptr;
     }
     return ensure_block(h, transpose, st);
 }
@@ -546,7 +552,7 @@ ffspmv_status spmv_count_launches(ffspmv_t h, int32_t transpose, int32_t nvec, i
         n += 2LL * ((nvec + chunk - 1) / chunk);
     } else {
         const Plan &P = transpose ? h->AT : h->A;
-        const BlockPlan *B = block_path(h, transpose != 0, nvec, nullptr);
+        const BlockPlan *B = block_path(h, transpose != 0, nvec, nullptr, true);
         if (B) {
             n += block_launches(*B, nvec);
         } else if (!P.panel.on || nvec == 1) {

@@ -21,12 +21,10 @@
 // sums into 64-bit words and the last one to arrive writes the row.
 #include <algorithm>
 #include <cstring>
-#include <exception>
-#include <thread>
+#include <new>
 #include <type_traits>
 
 #include "ff_internal.cuh"
-#include "ff_plan.h"
 #include "ff_block.h"
 
 namespace ff {
@@ -37,13 +35,9 @@ constexpr long long kBlockLong = 512;   // entries of a chunk; longer rows are s
 constexpr int kBlockVecs = 32;          // vectors per pass
 constexpr int kBlockClasses = 7;        // by quads of entries: 0, 1, 2, 3-4, 5-8, 9-16, 17-128
 
-int block_class(long long len)
+__device__ __forceinline__ int block_class(u32 quads)
 {
-    const long long quads = (len + 3) / 4;
-    int c = 0;
-    if (quads > 0)
-        for (c = 1; c < kBlockClasses - 1 && (1LL << (c - 1)) < quads; ++c) {}
-    return c;
+    return quads <= 2u ? (int)quads : min(kBlockClasses - 1, 33 - __clz(quads - 1u));
 }
 
 }  // namespace
@@ -546,90 +540,105 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_co
 }
 
 // ---------------------------------------------------------------------------
-ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long long *ptr, const int *col,
-                          const u32 *val, u32 m)
+// The layout is made on the device from the CSR arrays: the lengths of the
+// output rows (of A: row offsets; of A^T: a histogram of the columns), the
+// rows and quads of each class, each row's place (a warp's rows of a class
+// take consecutive places, so rows stay nearly in order), then the entries.
+// The order of the entries of a row is free: sums mod m are exact.
+struct BlockBuild {
+    const long long *ptr;   // CSR of A
+    const u32 *col, *val;
+    long long nr, n;        // rows of A, output rows
+    u32 *len, *start;       // [n]: entries, first quad
+    u64 *cursor;            // [kBlockClasses + 2]: (rows << 32) + quads of each class and of the long rows; chunks
+    u32 *orow, *optr, *lrow, *ocol;
+    uint4 *chunk;
+    void *oval;
+    int small;
+};
+
+__global__ void __launch_bounds__(kBlockThreads) k_block_lengths(const BlockBuild b, int transpose)
 {
-    const long long nnz = ptr[n];
-    // offsets in quads are 32-bit
-    if (nnz / 4 + n >= (1LL << 32) - 1 || n >= (1LL << 32) - 64) return FFSPMV_ERR_UNSUPPORTED;
-    auto quads = [&](long long i) { return (u32)((ptr[i + 1] - ptr[i] + 3) / 4); };
-    B.n = n;
-    B.ncols = ncols;
-    B.small = m <= 65536u;
-    // rows in class order, heaviest first, and where their entries go
-    std::vector<u32> lrow, row, rptr;
-    std::vector<uint4> chunk;
-    long long cnt[kBlockClasses] = {};
-    u32 at = 0;
-    for (long long i = 0; i < n; ++i) {
-        const long long L = ptr[i + 1] - ptr[i];
-        if (L <= kBlockLong) {
-            ++cnt[block_class(L)];
-            continue;
-        }
-        const u32 parts = (u32)((L + kBlockLong - 1) / kBlockLong);
-        for (u32 c = 0; c < parts; ++c)
-            chunk.push_back(make_uint4((u32)lrow.size(), at + c * (u32)(kBlockLong / 4),
-                                       at + std::min(quads(i), (c + 1) * (u32)(kBlockLong / 4)), parts));
-        lrow.push_back((u32)i);
-        at += quads(i);
-    }
-    B.nlong = (long long)lrow.size();
-    B.nchunk = (long long)chunk.size();
-    const long long ns = n - B.nlong;
-    for (int c = 0; c < kBlockClasses; ++c) B.cls_row[c + 1] = B.cls_row[c] + cnt[kBlockClasses - 1 - c];
-    row.resize((size_t)ns);
-    rptr.resize((size_t)ns + 1);
-    long long pos[kBlockClasses];
-    for (int c = 0; c < kBlockClasses; ++c) pos[c] = B.cls_row[kBlockClasses - 1 - c];
-    for (long long i = 0; i < n; ++i) {
-        const long long L = ptr[i + 1] - ptr[i];
-        if (L <= kBlockLong) row[(size_t)pos[block_class(L)]++] = (u32)i;
-    }
-    for (long long r = 0; r < ns; ++r) {
-        rptr[(size_t)r] = at;
-        at += quads(row[(size_t)r]);
-    }
-    rptr[(size_t)ns] = at;
-    // heaviest first: class 1 (one quad) is the last but one
-    const size_t r1 = (size_t)B.cls_row[kBlockClasses - 2];
-    B.quad1 = rptr[r1] - (u32)r1;
-    const int vb = B.small ? 2 : 4;
-    const size_t slots = (size_t)at * 4;
-    std::vector<u32> pcol(std::max<size_t>(slots, 4), 0u);
-    std::vector<unsigned char> pval(std::max<size_t>(slots, 4) * vb, 0);
-    auto copy_row = [&](long long i, u32 quad) {
-        size_t to = (size_t)quad * 4;
-        for (long long k = ptr[i]; k < ptr[i + 1]; ++k, ++to) {
-            pcol[to] = (u32)col[k];
-            const u32 v = val[k] % m;
-            if (B.small) reinterpret_cast<unsigned short *>(pval.data())[to] = (unsigned short)v;
-            else reinterpret_cast<u32 *>(pval.data())[to] = v;
-        }
-    };
-    const int nt = (int)std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
-    auto work = [&](int t) {
-        for (long long r = ns * t / nt; r < ns * (t + 1) / nt; ++r) copy_row(row[(size_t)r], rptr[(size_t)r]);
-        u32 to = 0;
-        for (long long r = 0; r < B.nlong; ++r) {
-            if (r % nt == t) copy_row(lrow[(size_t)r], to);
-            to += quads(lrow[(size_t)r]);
-        }
-    };
-    if (nnz < 200000 || nt == 1) {
-        for (int t = 0; t < nt; ++t) work(t);
+    const long long nth = (long long)gridDim.x * kBlockThreads, t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
+    if (!transpose) {
+        for (long long i = t; i < b.nr; i += nth) b.len[i] = (u32)(b.ptr[i + 1] - b.ptr[i]);
     } else {
-        std::vector<std::thread> th;
-        th.reserve((size_t)nt);
-        for (int t = 0; t < nt; ++t) {
-            try {
-                th.emplace_back(work, t);
-            } catch (const std::exception &) {
-                work(t);  // no thread to be had: this share runs here
+        const long long nnz = b.ptr[b.nr];
+        for (long long k = t; k < nnz; k += nth) atomicAdd(b.len + b.col[k], 1u);
+    }
+}
+
+// place = 0: the totals of every class into the cursors; place = 1: every row
+// to its place, the cursors holding the first places.
+__global__ void __launch_bounds__(kBlockThreads) k_block_place(const BlockBuild b, int place)
+{
+    const int lane = threadIdx.x & 31;
+    const long long nw = (b.n + 31) / 32, step = (long long)gridDim.x * (kBlockThreads / 32);
+    for (long long w = (long long)blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5); w < nw; w += step) {
+        const long long i = w * 32 + lane;
+        const u32 len = i < b.n ? b.len[i] : 0u, quads = (u32)(((u64)len + 3u) / 4u);
+        const int c = i >= b.n ? -1 : len > (u32)kBlockLong ? kBlockClasses : block_class(quads);
+        const u32 parts = c == kBlockClasses ? (u32)(((u64)len + kBlockLong - 1) / kBlockLong) : 0u;
+        for (int k = 0; k <= kBlockClasses; ++k) {
+            const u32 same = __ballot_sync(0xffffffffu, c == k);
+            if (!same) continue;
+            // this lane's offset among the warp's rows of the class
+            u64 mine = c == k ? ((u64)1 << 32) + quads : 0, sum = mine;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const u64 o = __shfl_up_sync(0xffffffffu, sum, d);
+                if (lane >= d) sum += o;
+            }
+            const u64 all = __shfl_sync(0xffffffffu, sum, 31);
+            u64 base = 0;
+            if (lane == 0) base = atomicAdd(b.cursor + k, all);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (c != k) continue;
+            if (!place) {
+                if (parts) atomicAdd(b.cursor + kBlockClasses + 1, (u64)parts);
+                continue;
+            }
+            const u64 at = base + sum - mine;
+            const u32 slot = (u32)(at >> 32), q = (u32)at;
+            b.start[i] = q;
+            if (k == kBlockClasses) {
+                b.lrow[slot] = (u32)i;
+                const u64 c0 = atomicAdd(b.cursor + kBlockClasses + 1, (u64)parts);
+                for (u32 p = 0; p < parts; ++p)
+                    b.chunk[c0 + p] = make_uint4(slot, q + p * (u32)(kBlockLong / 4),
+                                                 q + min(quads, (p + 1) * (u32)(kBlockLong / 4)), parts);
+            } else {
+                b.orow[slot] = (u32)i;
+                b.optr[slot] = q;
             }
         }
-        for (auto &t : th) t.join();
     }
+}
+
+__global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild b, int transpose)
+{
+    const int lane = threadIdx.x & 31;
+    const long long step = (long long)gridDim.x * (kBlockThreads / 32);
+    for (long long i = (long long)blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5); i < b.nr; i += step) {
+        const long long s = b.ptr[i], e = b.ptr[i + 1];
+        for (long long k = s + lane; k < e; k += 32) {
+            const u32 j = b.col[k], v = b.val[k];
+            const size_t to = transpose ? (size_t)b.start[j] * 4 + (atomicSub(b.len + j, 1u) - 1u)
+                                        : (size_t)b.start[i] * 4 + (size_t)(k - s);
+            b.ocol[to] = transpose ? (u32)i : j;
+            if (b.small) reinterpret_cast<unsigned short *>(b.oval)[to] = (unsigned short)v;
+            else reinterpret_cast<u32 *>(b.oval)[to] = v;
+        }
+    }
+}
+
+// The block layout of A (nr x nc, values below m), or of A^T.
+ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long nc, const long long *ptr, const int *col,
+                          const u32 *val, u32 m, cudaStream_t st, void *&tmp)
+{
+    const long long nnz = ptr[nr], n = transpose ? nc : nr, ncols = transpose ? nr : nc;
+    // offsets in quads and lengths are 32-bit
+    if (nnz >= (1LL << 32) - 1 || nnz / 4 + n >= (1LL << 32) - 1 || n >= (1LL << 32) - 64) return FFSPMV_ERR_UNSUPPORTED;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     size_t o = 0;
     auto put = [&](size_t bytes) {
@@ -637,8 +646,63 @@ ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long
         o += al(std::max<size_t>(bytes, 16));
         return here;
     };
-    const size_t o_ptr = put(rptr.size() * 4), o_row = put(row.size() * 4), o_chunk = put(chunk.size() * 16),
-                 o_lrow = put(lrow.size() * 4), o_col = put(pcol.size() * 4), o_val = put(pval.size()),
+    constexpr int kCur = kBlockClasses + 2;
+    const size_t t_ptr = put((size_t)(nr + 1) * 8), t_col = put((size_t)nnz * 4), t_val = put((size_t)nnz * 4),
+                 t_len = put((size_t)n * 4), t_start = put((size_t)n * 4), t_cur = put(kCur * 8);
+    if (cudaMalloc(&tmp, o) != cudaSuccess) {
+        cudaGetLastError();
+        tmp = nullptr;
+        return FFSPMV_ERR_OOM;
+    }
+    char *t = (char *)tmp;
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const unsigned grid = (unsigned)(8 * std::max(nsm, 1));
+    BlockBuild b;
+    memset(&b, 0, sizeof(b));
+    b.ptr = (const long long *)(t + t_ptr);
+    b.col = (const u32 *)(t + t_col);
+    b.val = (const u32 *)(t + t_val);
+    b.nr = nr;
+    b.n = n;
+    b.len = (u32 *)(t + t_len);
+    b.start = (u32 *)(t + t_start);
+    b.cursor = (u64 *)(t + t_cur);
+    b.small = m <= 65536u ? 1 : 0;
+    u64 cur[kCur] = {};
+    FF_CUDA(cudaMemcpyAsync(t + t_ptr, ptr, (size_t)(nr + 1) * 8, cudaMemcpyHostToDevice, st));
+    if (nnz) {
+        FF_CUDA(cudaMemcpyAsync(t + t_col, col, (size_t)nnz * 4, cudaMemcpyHostToDevice, st));
+        FF_CUDA(cudaMemcpyAsync(t + t_val, val, (size_t)nnz * 4, cudaMemcpyHostToDevice, st));
+    }
+    FF_CUDA(cudaMemsetAsync(t + t_len, 0, o - t_len, st));
+    k_block_lengths<<<grid, kBlockThreads, 0, st>>>(b, transpose ? 1 : 0);
+    k_block_place<<<grid, kBlockThreads, 0, st>>>(b, 0);
+    FF_CUDA(cudaGetLastError());
+    FF_CUDA(cudaMemcpyAsync(cur, b.cursor, sizeof(cur), cudaMemcpyDeviceToHost, st));
+    FF_CUDA(cudaStreamSynchronize(st));
+    // the long rows' quads come first, then the classes, heaviest first
+    B.n = n;
+    B.ncols = ncols;
+    B.small = b.small != 0;
+    B.nlong = (long long)(cur[kBlockClasses] >> 32);
+    B.nchunk = (long long)cur[kBlockClasses + 1];
+    u64 quads = cur[kBlockClasses] & 0xffffffffull, rows = 0;
+    cur[kBlockClasses] = cur[kBlockClasses + 1] = 0;
+    for (int i = 0; i < kBlockClasses; ++i) {
+        const int c = kBlockClasses - 1 - i;
+        const u64 here = cur[c];
+        cur[c] = (rows << 32) + quads;
+        if (c == 1) B.quad1 = (u32)quads - (u32)rows;
+        rows += here >> 32;
+        quads += here & 0xffffffffull;
+        B.cls_row[i + 1] = (long long)rows;
+    }
+    const int vb = B.small ? 2 : 4;
+    o = 0;
+    const size_t o_ptr = put((size_t)(rows + 1) * 4), o_row = put((size_t)rows * 4), o_chunk = put((size_t)B.nchunk * 16),
+                 o_lrow = put((size_t)B.nlong * 4), o_col = put((size_t)quads * 16), o_val = put((size_t)quads * 4 * vb),
                  o_carry = put((size_t)B.nlong * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
                  o_dev = put(sizeof(BlockDev)), o_xs = put((size_t)ncols * kBlockVecs * vb);
     if (cudaMalloc(&B.arena, o) != cudaSuccess) {
@@ -647,53 +711,40 @@ ffspmv_status build_block(BlockPlan &B, long long n, long long ncols, const long
         return FFSPMV_ERR_OOM;
     }
     char *base = (char *)B.arena;
-    auto up = [&](size_t off, const void *src, size_t bytes) {
-        return !bytes || cudaMemcpy(base + off, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
-    };
-    const bool ok = up(o_ptr, rptr.data(), rptr.size() * 4) && up(o_row, row.data(), row.size() * 4) &&
-                    up(o_chunk, chunk.data(), chunk.size() * 16) && up(o_lrow, lrow.data(), lrow.size() * 4) &&
-                    up(o_col, pcol.data(), slots * 4) && up(o_val, pval.data(), slots * vb) &&
-                    cudaMemset(base + o_carry, 0, o_dev - o_carry) == cudaSuccess;
-    if (!ok) {
-        cudaFree(B.arena);
-        B.arena = nullptr;
-        cudaGetLastError();
-        return FFSPMV_ERR_CUDA;
-    }
-    B.ptr = (const u32 *)(base + o_ptr);
-    B.row = (const u32 *)(base + o_row);
-    B.chunk = (const uint4 *)(base + o_chunk);
-    B.lrow = (const u32 *)(base + o_lrow);
-    B.col = (const u32 *)(base + o_col);
-    B.val = base + o_val;
-    B.carry = (u64 *)(base + o_carry);
-    B.count = (u32 *)(base + o_count);
-    B.xs = (uint4 *)(base + o_xs);
     BlockDev D;
     memset(&D, 0, sizeof(D));
-    D.ptr = B.ptr;
-    D.row = B.row;
-    D.col = B.col;
-    D.lrow = B.lrow;
-    D.chunk = B.chunk;
-    D.val = B.val;
-    D.xs = B.xs;
-    D.carry = B.carry;
-    D.count = B.count;
+    D.ptr = B.ptr = (const u32 *)(base + o_ptr);
+    D.row = B.row = (const u32 *)(base + o_row);
+    D.chunk = B.chunk = (const uint4 *)(base + o_chunk);
+    D.lrow = B.lrow = (const u32 *)(base + o_lrow);
+    D.col = B.col = (const u32 *)(base + o_col);
+    D.val = B.val = base + o_val;
+    D.carry = B.carry = (u64 *)(base + o_carry);
+    D.count = B.count = (u32 *)(base + o_count);
+    D.xs = B.xs = (uint4 *)(base + o_xs);
     D.ncols = ncols;
     for (int c = 0; c <= kBlockClasses; ++c) D.row0[c] = (u32)B.cls_row[c];
     D.nchunk = (u32)B.nchunk;
     D.quad1 = B.quad1;
-    D.small = B.small ? 1 : 0;
+    D.small = b.small;
     D.fold = m <= (1u << 31) ? 1 : 0;
     D.M = make_mod(m, 1, 0);
-    if (!up(o_dev, &D, sizeof(D))) {
-        cudaFree(B.arena);
-        B.arena = nullptr;
-        cudaGetLastError();
-        return FFSPMV_ERR_CUDA;
-    }
     B.dev = (const BlockDev *)(base + o_dev);
+    b.optr = (u32 *)(base + o_ptr);
+    b.orow = (u32 *)(base + o_row);
+    b.chunk = (uint4 *)(base + o_chunk);
+    b.lrow = (u32 *)(base + o_lrow);
+    b.ocol = (u32 *)(base + o_col);
+    b.oval = base + o_val;
+    const u32 end = (u32)quads;
+    FF_CUDA(cudaMemcpyAsync(b.cursor, cur, sizeof(cur), cudaMemcpyHostToDevice, st));
+    FF_CUDA(cudaMemcpyAsync(b.optr + rows, &end, 4, cudaMemcpyHostToDevice, st));
+    FF_CUDA(cudaMemcpyAsync(base + o_dev, &D, sizeof(D), cudaMemcpyHostToDevice, st));
+    FF_CUDA(cudaMemsetAsync(base + o_col, 0, o_dev - o_col, st));   // padding entries, sums and counts of long rows
+    k_block_place<<<grid, kBlockThreads, 0, st>>>(b, 1);
+    k_block_fill<<<grid, kBlockThreads, 0, st>>>(b, transpose ? 1 : 0);
+    FF_CUDA(cudaGetLastError());
+    FF_CUDA(cudaStreamSynchronize(st));
     return FFSPMV_OK;
 }
 
@@ -710,19 +761,13 @@ const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st)
     }
     BlockPlan *nb = new (std::nothrow) BlockPlan();
     if (!nb) return nullptr;
-    ffspmv_status r;
-    try {
-        if (!transpose) {
-            r = build_block(*nb, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(), h->h_val.data(), h->m);
-        } else {
-            std::vector<long long> tptr;
-            std::vector<int> tcol;
-            std::vector<u32> tval;
-            transpose_csr(h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(), h->h_val.data(), tptr, tcol, tval);
-            r = build_block(*nb, h->A.ncols, h->A.nrows, tptr.data(), tcol.data(), tval.data(), h->m);
-        }
-    } catch (const std::exception &) {
-        r = FFSPMV_ERR_OOM;
+    void *tmp = nullptr;
+    const ffspmv_status r = build_block(*nb, transpose, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(),
+                                        h->h_val.data(), h->m, st, tmp);
+    if (tmp) cudaFree(tmp);
+    if (r != FFSPMV_OK && nb->arena) {
+        cudaFree(nb->arena);
+        nb->arena = nullptr;
     }
     nb->ok = r == FFSPMV_OK;  // a layout that could not be made is not tried again
     b = nb;

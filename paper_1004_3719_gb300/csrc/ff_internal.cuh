@@ -316,8 +316,10 @@ struct ffspmv_handle {
     // x-panel plans of A and A^T for 2 and 4 vectors per pass, built on the
     // first block that uses them when the plan is the x-panel layout
     ff::Plan *multi[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-    // block layouts of A and A^T (block.cu), built on the first block that uses them
+    // block layouts of A and A^T (block.cu), built on the first block that uses
+    // them (binned plans: the second)
     ff::BlockPlan *block[2] = {nullptr, nullptr};
+    bool block_seen[2] = {false, false};
 };
 
 namespace ff {

@@ -42,6 +42,7 @@ def test_row_lengths_and_widths(lib, m):
 def test_largest_sums(lib, m):
     A = edge_matrix(m, largest=True)
     M = lib.Matrix.from_csr(A, transpose_mode=lib.TRANSPOSE.NONE)
+    assert M.launches(False, 32) <= 2    # builds the layout
     for nvec in (3, 16, 32):
         X = np.full((A.ncols, nvec), m - 1, dtype=np.uint32)
         assert np.array_equal(to_host(M.apply(to_dev(X))), oracle.csr_spmv(A, X))
@@ -52,6 +53,7 @@ def test_strided_and_unaligned_blocks(lib, m):
     import torch
     A = edge_matrix(m)
     M = lib.Matrix.from_csr(A, transpose_mode=lib.TRANSPOSE.NONE)
+    assert M.launches(False, 32) <= 2    # builds the layout
     for nvec, ldx, ldy, ox, oy in ((8, 8, 8, 1, 0), (8, 8, 8, 0, 1), (8, 12, 16, 0, 0), (7, 9, 11, 3, 2), (16, 20, 17, 0, 0)):
         x = rand_block(nvec, A.ncols, ldx, m)
         y0 = rand_block(nvec + 1, A.nrows, ldy, m)
