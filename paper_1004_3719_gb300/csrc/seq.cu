@@ -1,21 +1,40 @@
 // The block Wiedemann matrix sequence S_i = X^T A^i Y (mod p), Sec. 3 step 1,
 // kept on the device as Sec. 2.5.2 asks.
 //
-// Persistent path (p <= 2^16, s <= 16, A square and splittable into a few
-// dense diagonals plus a narrow ELL_R part): one cooperative kernel runs every
-// step.  CTA c owns a contiguous slice of rows; per step it forms its rows of
-// V_{i+1} = A V_i (DIA + ELL_R, Sec. 2.4.4), stores them, and projects them on
-// the matching rows of X with tensor-core MMAs on 8-bit limbs; a bounded grid
-// barrier then publishes V_{i+1} and the per-CTA partial projections, which
-// the CTAs sum into S_{i+1}.  The kernel is captured in a CUDA graph.
+// Persistent path (p <= 2^16, s <= 16, A square, at most 16 entries per row
+// once a few dense diagonals are merged): one cooperative kernel runs every
+// step.  CTA c owns a contiguous slice of rows, its warps 16-row groups: two
+// lanes per row gather the 16-residue rows of V_i that the row's entries name
+// (32 bytes each, from L2), form the row of V_{i+1}, store it, and the warp
+// projects its 16 rows on the matching rows of X with tensor-core MMAs on
+// 8-bit limbs, without meeting the other warps.  A bounded grid barrier then
+// publishes V_{i+1}; each CTA sums and writes its partial projection after it
+// has arrived there, and a warp of its own adds the CTAs' partials of a step up
+// during the step after next.  The kernel is captured in a CUDA graph.
 //
 // Per-launch path (everything else): for every step one projection launch and
 // the plan's SpMM launches.
 //
+// Arithmetic.  Two entries' residues of one component in a 32-bit word and the
+// two values as four bytes: two dp2a instructions (16 x 8 bits, two products
+// each) do two multiply-adds, the low and the high bytes of the values in
+// sums of their own (at most 16 products below 2^24 each), at half the
+// multiplier's time of 64-bit multiply-adds; the two sums are joined and
+// reduced in 32 bits.
+//
 // Exactness of the projection on tensor cores: a residue v < 2^16 splits as
-// v = 256*h + l with h, l < 256, both exact in fp16; one m16n8k16 MMA sums 16
-// products below 2^16 each, so its fp32 result (< 2^20) is an exact integer,
-// converted to u64 at once and weighted by 1, 256 or 65536.
+// v = 256*h + l with h, l < 256, both exact in fp16; a 16-row group adds
+// below 2^20 to an fp32 accumulator of limb products (twice that where the
+// two cross terms share one), which stays an exact integer below 2^23 over
+// kSeqTiles groups and is then folded into integers mod p.
+//
+// Measured, 100 000 x 100 000, 9.5 entries per row, s = 16, p = 65521: 15.1 us
+// per step with 64-bit multiply-adds, row passes that met at CTA barriers and
+// projections published before the barrier; 7.55 us with warps of their own
+// and dp2a, 7.1 us with the projection after the arrival.  Of a step's 13.9
+// thousand clocks the gathers take about 10: 0.95 million 32-byte rows from
+// L2, one line each, near the rate at which this chip serves random sectors
+// (about 250 G/s).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -28,33 +47,32 @@ namespace ff {
 
 namespace {
 
-constexpr int kSeqThreads = 512;
+constexpr int kSeqWorkers = 15;                   // warps that multiply (19: 94.7 ms for 12 502 steps, 23: 91.2, 15: 89.0)
+constexpr int kSeqWarps = kSeqWorkers + 1;        // ... and the one that sums the CTAs' partial projections
+constexpr int kSeqThreads = 32 * kSeqWarps;
 constexpr int kS = 16;                            // block width of the persistent kernel
-constexpr int kCPT = 8;                           // components per thread
-constexpr int kTPR = kS / kCPT;                   // threads per row
-constexpr int kRowsPerPass = kSeqThreads / kTPR;  // 256
-constexpr int kMaxEnt = 16;                       // DIA + ELL_R entries per row
-constexpr int kBatch = 10;                        // entries gathered together per thread
-constexpr int kVsStride = 20;                     // halves per staged row (no bank conflicts)
-constexpr size_t kXfSmemMax = 160 * 1024;         // shared memory for resident X fragments
+constexpr int kMaxEnt = 16;                       // entries per row
+constexpr int kSeqBatch = 5;                      // entry pairs gathered together per lane
+constexpr int kSeqTiles = 3;                      // groups that a warp forms before it projects them
+constexpr int kSeqBufs = 3;                       // partial projections in flight
+constexpr int kVsStride = 24;                     // halves per staged row (no bank conflicts for ldmatrix)
 constexpr unsigned kDefaultSpins = 1u << 22;      // x <= 64 ns sleeps: well under a second
 
 struct SeqArgs {
     long long n;
-    int ndiag, width, s;
+    int s;
+    int npair;                 // entry pairs per row
     long long ld;
     long long nsteps;
-    const int *doff;
-    const unsigned short *dval;
-    const u32 *col;
-    const unsigned short *val;
-    const u32 *rownb;
+    const u32 *col;            // [2 npair][ld]: columns (value 0: the row itself)
+    const u32 *val;            // [npair][ld]: bytes (v0 low, v1 low, v0 high, v1 high)
+    const unsigned char *gnp;  // [n / 16]: pairs in use in a 16-row group
     const uint4 *XF;           // X limbs in MMA A-fragment order: [n/16][limb][lane]
     unsigned short *V0, *V1;   // n x 16
-    u32 *partial;              // [2][nblocks][256]
+    u32 *partial;              // [kSeqBufs][nblocks][256]
     u32 *S;
     u32 *Vnext;
-    unsigned *bar;             // [0] arrivals, [1] generation
+    unsigned *bar;             // [0] arrivals
     int *status;               // [0] timeout flag
     unsigned spin_limit;
     int test_skip;
@@ -63,16 +81,6 @@ struct SeqArgs {
     int mrows;                 // rows of one CTA's resident matrix slice (capacity)
     int mat_off;               // byte offset of that slice in dynamic shared memory
     Mod M;
-};
-
-// A CTA's rows of the DIA + ELL_R layout, resident in shared memory for the
-// whole launch (the matrix is the same at every step): entry-major like the
-// global arrays, row index relative to the CTA's first row.
-struct MatSlice {
-    const unsigned short *dval;  // [ndiag][mrows]
-    const u32 *col;              // [width][mrows]
-    const unsigned short *val;   // [width][mrows]
-    const u32 *rownb;            // [mrows], or null when all rows have `width` entries
 };
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
@@ -89,23 +97,26 @@ __device__ __forceinline__ int ld_volatile_int(const int *p)
     return v;
 }
 
-// Grid barrier with a bounded wait.  The arrival counter (zeroed before the
-// launch) only grows: barrier number `epoch` is passed once it reaches
-// epoch * gridDim.x.  One thread per CTA adds its arrival with release order
-// (after the CTA's __syncthreads, so it publishes the whole CTA's writes) and
-// polls with acquire loads.  Returns false (and sets status[0]) when the wait
-// ran out or another CTA already gave up.
-__device__ bool grid_barrier(const SeqArgs &a, bool skip, unsigned &epoch)
+// Grid barrier with a bounded wait, in two halves.  The arrival counter
+// (zeroed before the launch) only grows: barrier number `epoch` is passed once
+// it reaches epoch * gridDim.x.  One thread per CTA adds its arrival with
+// release order (after the CTA's __syncthreads, so it publishes the whole
+// CTA's writes) and polls with acquire loads.  The wait returns false (and
+// sets status[0]) when it ran out or another CTA already gave up.
+__device__ __forceinline__ void grid_arrive(const SeqArgs &a, bool skip)
+{
+    __syncthreads();
+    if (threadIdx.x == 0 && !skip) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
+}
+
+__device__ bool grid_wait(const SeqArgs &a, bool skip, unsigned epoch)
 {
     __shared__ int s_ok;
-    __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        ++epoch;
+        unsigned it = 0;
         if (!skip) {
             const unsigned target = epoch * gridDim.x;
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
-            unsigned it = 0;
             while ((int)(ld_acquire(a.bar) - target) < 0) {
                 if (++it > a.spin_limit || ((it & 255u) == 0 && ld_volatile_int(a.status) != 0)) {
                     atomicExch(a.status, 1);
@@ -115,8 +126,7 @@ __device__ bool grid_barrier(const SeqArgs &a, bool skip, unsigned &epoch)
                 if (it > 64) __nanosleep(32);
             }
         } else {
-            // test hook: never arrive; wait (bounded) for the others to give up
-            unsigned it = 0;
+            // test hook: never arrived; wait (bounded) for the others to give up
             while (ld_volatile_int(a.status) == 0 && ++it <= a.spin_limit) __nanosleep(64);
             atomicExch(a.status, 1);
             ok = 0;
@@ -146,185 +156,188 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint4 &A, u32 b0, 
 {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 "
-        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(A.x), "r"(A.y), "r"(A.z), "r"(A.w), "r"(b0), "r"(b1),
-          "f"(0.f), "f"(0.f), "f"(0.f), "f"(0.f));
+        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(A.x), "r"(A.y), "r"(A.z), "r"(A.w), "r"(b0), "r"(b1));
 }
 
 struct __align__(16) SeqSmem {
-    union {
-        unsigned short vs[2][kRowsPerPass][kVsStride];  // staged V rows, double buffered
-        u32 red[kSeqThreads / 32][kS * kS];             // per-warp partial projections
-    };
-    int doff[kMaxEnt];
+    u32 red[kSeqWorkers][kS * kS];                       // per-warp partial projections
+    unsigned short vs[kSeqWorkers][kSeqTiles][16 * kVsStride];  // per-warp staged rows of V
+};
+constexpr size_t kXfSmemMax = 225 * 1024 - sizeof(SeqSmem);  // shared memory for resident X fragments and matrix rows
+
+// t mod m up to m (in [0, 2m)), mu = floor(2^32 / m) (Barrett, 1986)
+__device__ __forceinline__ u32 seq_mod2(u32 t, u32 m, u32 mu) { return t - __umulhi(t, mu) * m; }
+// lo + 256 hi mod m for lo, hi < 2^29
+__device__ __forceinline__ u32 seq_join(u32 lo, u32 hi, u32 m, u32 mu)
+{
+    const u32 t = seq_mod2(seq_mod2(hi, m, mu) * 256u + lo, m, mu);   // hi mod m < 2^17, the sum below 2^30
+    return min(t, t - m);
+}
+
+// One warp's fp32 sums of limb products: rows 8h + g of X^T against columns
+// 8 nt + 2t, 2t + 1: [weight 1, 256, 65536][nt][e].
+struct SeqSums {
+    float d[3][2][4];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int w = 0; w < 3; ++w)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) d[w][nt][e] = 0.0f;
+    }
 };
 
-// V_out rows [r0, r1) = A * V_in (when `compute`), and, when `project`, the
-// partial X^T V_out over those rows accumulated in pacc.  Two threads share a
-// row (8 components each); warp w then runs k-step w of every 256-row pass
-// with both X limbs against both V limbs (8 MMAs).  Indices are 32-bit: the
-// layout guarantees 16 n < 2^31.
-__device__ void spmm_and_project(const SeqArgs &a, SeqSmem &sm, const uint4 *xfs, const MatSlice &ms,
-                                 const unsigned short *Vin, unsigned short *Vout, int r0, int r1,
-                                 bool compute, bool project, u32 (&pacc)[2][2][4])
+// The sums, mod p, into (first) or onto this warp's words of sm.red.
+__device__ __forceinline__ void seq_flush(const SeqArgs &a, u32 *red, SeqSums &P, bool first, u32 mu)
 {
-    const int R = a.mrows;
-    const int rip = threadIdx.x / kTPR;
-    const int c0 = (threadIdx.x % kTPR) * kCPT;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    const int nd = a.ndiag, n = (int)a.n, ld = (int)a.ld;
-    int pass = 0;
-    for (int base = r0; base < r1; base += kRowsPerPass, ++pass) {
-        const int row = base + rip;
-        uint4 outq = make_uint4(0u, 0u, 0u, 0u);
-        if (row < r1) {
-            if (compute) {
-                const int lr = row - r0;
-                const int ntot =
-                    nd + (a.rownb ? (a.mat_smem ? (int)ms.rownb[lr] : (int)__ldg(a.rownb + row)) : a.width);
-                u64 acc[kCPT];
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
-                for (int k = 0; k < kCPT; ++k) acc[k] = 0;
-#pragma unroll
-                for (int e0 = 0; e0 < kMaxEnt; e0 += kBatch) {
-                    if (e0 >= ntot) break;
-                    uint4 q[kBatch];
-                    u32 v[kBatch];
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        const int e = e0 + u;
-                        q[u] = make_uint4(0u, 0u, 0u, 0u);
-                        v[u] = 0;
-                        if (e < nd) {
-                            const int j = row + sm.doff[e];
-                            if ((unsigned)j < (unsigned)n) {
-                                v[u] = a.mat_smem ? ms.dval[e * R + lr] : __ldg(a.dval + e * ld + row);
-                                q[u] = __ldcg(reinterpret_cast<const uint4 *>(Vin + j * kS + c0));
-                            }
-                        } else if (e < ntot) {
-                            int j;
-                            if (a.mat_smem) {
-                                const int li = (e - nd) * R + lr;
-                                j = (int)ms.col[li];
-                                v[u] = ms.val[li];
-                            } else {
-                                const int idx = (e - nd) * ld + row;
-                                j = (int)__ldg(a.col + idx);
-                                v[u] = __ldg(a.val + idx);
-                            }
-                            q[u] = __ldcg(reinterpret_cast<const uint4 *>(Vin + j * kS + c0));
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        const u32 qq[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            acc[2 * k] += (u64)v[u] * (qq[k] & 0xffffu);
-                            acc[2 * k + 1] += (u64)v[u] * (qq[k] >> 16);
-                        }
-                    }
-                }
-                outq.x = red64(acc[0], a.M) | (red64(acc[1], a.M) << 16);
-                outq.y = red64(acc[2], a.M) | (red64(acc[3], a.M) << 16);
-                outq.z = red64(acc[4], a.M) | (red64(acc[5], a.M) << 16);
-                outq.w = red64(acc[6], a.M) | (red64(acc[7], a.M) << 16);
-                *reinterpret_cast<uint4 *>(Vout + row * kS + c0) = outq;
-            } else {
-                outq = __ldcg(reinterpret_cast<const uint4 *>(Vin + row * kS + c0));
-            }
-        }
-        if (!project) continue;
-        unsigned short(*vs)[kVsStride] = sm.vs[pass & 1];
-        *reinterpret_cast<uint2 *>(&vs[rip][c0]) = make_uint2(outq.x, outq.y);
-        *reinterpret_cast<uint2 *>(&vs[rip][c0 + 4]) = make_uint2(outq.z, outq.w);
-        __syncthreads();
-        // each pass adds below 2^29 per element: reduce every 4 passes
-        if ((pass & 3) == 3) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) pacc[i][j][e] = red64(pacc[i][j][e], a.M);
-        }
-        const int q16 = (base >> 4) + w;
-        if (q16 * 16 < r1) {
-            uint4 A0, A1;
-            if (a.xf_smem) {
-                const uint4 *f = xfs + ((size_t)(q16 - (r0 >> 4)) * 2) * 32 + lane;
-                A0 = f[0];
-                A1 = f[32];
-            } else {
-                A0 = __ldg(a.XF + ((size_t)q16 * 2 + 0) * 32 + lane);
-                A1 = __ldg(a.XF + ((size_t)q16 * 2 + 1) * 32 + lane);
-            }
-            const int k0 = w * 16;
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                const int nn = nt * 8 + g;
-                const u32 p0 = vs[k0 + 2 * t][nn] | ((u32)vs[k0 + 2 * t + 1][nn] << 16);
-                const u32 p1 = vs[k0 + 2 * t + 8][nn] | ((u32)vs[k0 + 2 * t + 9][nn] << 16);
-#pragma unroll
-                for (int vl = 0; vl < 2; ++vl) {
-                    const u32 b0 = bytes_to_half2(vl ? (p0 >> 8) & 0x00ff00ffu : p0 & 0x00ff00ffu);
-                    const u32 b1 = bytes_to_half2(vl ? (p1 >> 8) & 0x00ff00ffu : p1 & 0x00ff00ffu);
-                    float d0[4], d1[4];
-                    mma16816(d0, A0, b0, b1);
-                    mma16816(d1, A1, b0, b1);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        pacc[vl][nt][e] += f32_to_u32(d0[e]) + (f32_to_u32(d1[e]) << 8);
-                }
-            }
-        }
-    }
-}
-
-// Add the warps' fragments into sm.acc, then write this CTA's partial
-// projection (reduced) and clear the accumulators.
-__device__ void publish_partial(const SeqArgs &a, SeqSmem &sm, int buf, u32 (&pacc)[2][2][4])
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    __syncthreads();  // the last pass's MMAs have read the staged rows
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-        const int b = nt * 8 + 2 * t;
-        u32 c[4];
+    for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            c[e] = red64((u64)pacc[0][nt][e] + ((u64)pacc[1][nt][e] << 8), a.M);  // V limb weights 1, 256
-            pacc[0][nt][e] = pacc[1][nt][e] = 0;
+            const u32 cross = f32_to_u32(P.d[1][nt][e]), hi = f32_to_u32(P.d[2][nt][e]), lo = f32_to_u32(P.d[0][nt][e]);
+            const u32 v = seq_join(lo, seq_join(cross, hi, a.M.m, mu), a.M.m, mu);
+            u32 *r = red + (g + (e >> 1) * 8) * kS + nt * 8 + 2 * t + (e & 1);
+            *r = first ? v : *r + v;
         }
-        sm.red[w][g * kS + b] = c[0];
-        sm.red[w][g * kS + b + 1] = c[1];
-        sm.red[w][(g + 8) * kS + b] = c[2];
-        sm.red[w][(g + 8) * kS + b + 1] = c[3];
-    }
-    __syncthreads();
-    u32 *dst = a.partial + ((size_t)buf * gridDim.x + blockIdx.x) * (kS * kS);
-    for (int o = threadIdx.x; o < kS * kS; o += blockDim.x) {
-        u64 tot = 0;
-#pragma unroll
-        for (int i = 0; i < kSeqThreads / 32; ++i) tot += sm.red[i][o];
-        dst[o] = red64(tot, a.M);
-    }
-    __syncthreads();  // sm.red aliases the staging rows of the next step
 }
 
-// S_step[o] = sum over CTAs of their partials (mod p); one warp per output,
-// output o on warp o / gridDim.x of CTA o % gridDim.x, so that every CTA has
-// at most two.
-__device__ void reduce_step(const SeqArgs &a, int buf, long long step)
+// X^T times the staged rows of a worker warp's groups base, base +
+// kSeqWorkers, ... (at most kSeqTiles of them) into (first) or onto its words
+// of sm.red.
+__device__ __forceinline__ void seq_project(const SeqArgs &a, SeqSmem &sm, const uint4 *xf, int base, int ngroups, bool first,
+                                            u32 mu)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __syncwarp();   // the rows are staged
+    SeqSums P;
+    P.zero();
+    for (int k = 0; k < kSeqTiles; ++k) {
+        const int grp = base + k * kSeqWorkers;
+        if (grp >= ngroups) break;
+        // B fragments of both column tiles: rows 0-7 and 8-15 of each
+        u32 b[4];
+        const u32 at = (u32)__cvta_generic_to_shared(
+            sm.vs[w][k] + ((lane & 7) + ((lane >> 3) & 1) * 8) * kVsStride + (lane >> 4) * 8);
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                     : "r"(at)
+                     : "memory");
+        const uint4 *f = xf + (size_t)grp * 64 + lane;
+        const uint4 A0 = f[0], A1 = f[32];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            const u32 b0 = b[2 * nt], b1 = b[2 * nt + 1];
+            const u32 l0 = bytes_to_half2(b0 & 0x00ff00ffu), l1 = bytes_to_half2(b1 & 0x00ff00ffu);
+            const u32 h0 = bytes_to_half2((b0 >> 8) & 0x00ff00ffu), h1 = bytes_to_half2((b1 >> 8) & 0x00ff00ffu);
+            mma16816(P.d[0][nt], A0, l0, l1);
+            mma16816(P.d[1][nt], A0, h0, h1);
+            mma16816(P.d[1][nt], A1, l0, l1);
+            mma16816(P.d[2][nt], A1, h0, h1);
+        }
+    }
+    seq_flush(a, sm.red[w], P, first, mu);
+    __syncwarp();   // the fragments have been read
+}
+
+// A worker warp's 16-row groups of rows [r0, r1): V_out = A V_in (when
+// COMPUTE; else V_in itself), staged for the projection kSeqTiles groups at a
+// time.  All but the last of these batches are projected here (their sums need
+// the registers that the gathers take); the first group of the last one is
+// returned for seq_project, which then runs after the CTA has arrived at the
+// grid barrier.  `col`, `val`, `gnp` start at row r0 with `ld` rows per entry.
+template <bool COMPUTE>
+__device__ __forceinline__ int seq_rows(const SeqArgs &a, SeqSmem &sm, const uint4 *xf, const u32 *col, const u32 *val,
+                                         const unsigned char *gnp, size_t ld, const unsigned short *Vin,
+                                         unsigned short *Vout, int r0, int r1, bool project, u32 mu)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c0 = (lane & 1) * 8;
+    const int ngroups = (r1 - r0 + 15) >> 4;
+    for (int base = w;; base += kSeqTiles * kSeqWorkers) {
+        for (int k = 0; k < kSeqTiles; ++k) {
+            const int grp = base + k * kSeqWorkers;
+            if (grp >= ngroups) break;
+            const int lr = grp * 16 + (lane >> 1), row = r0 + lr;
+            uint4 out = make_uint4(0u, 0u, 0u, 0u);
+            if (COMPUTE) {
+                u32 lo[8], hi[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) lo[i] = hi[i] = 0u;
+                const int np = gnp[grp];   // warp-uniform
+                const bool live = row < r1;
+                const u32 *cp = col + lr, *vp = val + lr;
+                const unsigned short *vin = Vin + c0;
+                for (int p0 = 0; p0 < np; p0 += kSeqBatch) {
+                    uint4 q[kSeqBatch][2];
+                    u32 v[kSeqBatch];
+#pragma unroll
+                    for (int u = 0; u < kSeqBatch; ++u) {
+                        q[u][0] = q[u][1] = make_uint4(0u, 0u, 0u, 0u);
+                        v[u] = 0u;
+                        if (p0 + u < np && live) {
+                            const u32 j0 = cp[(size_t)(2 * (p0 + u)) * ld], j1 = cp[(size_t)(2 * (p0 + u) + 1) * ld];
+                            v[u] = vp[(size_t)(p0 + u) * ld];
+                            q[u][0] = __ldcg(reinterpret_cast<const uint4 *>(vin + (size_t)j0 * kS));
+                            q[u][1] = __ldcg(reinterpret_cast<const uint4 *>(vin + (size_t)j1 * kS));
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kSeqBatch; ++u) {
+                        const u32 x0[4] = {q[u][0].x, q[u][0].y, q[u][0].z, q[u][0].w};
+                        const u32 x1[4] = {q[u][1].x, q[u][1].y, q[u][1].z, q[u][1].w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const u32 e0 = __byte_perm(x0[i], x1[i], 0x5410), e1 = __byte_perm(x0[i], x1[i], 0x7632);
+                            lo[2 * i] = __dp2a_lo(e0, v[u], lo[2 * i]);
+                            hi[2 * i] = __dp2a_hi(e0, v[u], hi[2 * i]);
+                            lo[2 * i + 1] = __dp2a_lo(e1, v[u], lo[2 * i + 1]);
+                            hi[2 * i + 1] = __dp2a_hi(e1, v[u], hi[2 * i + 1]);
+                        }
+                    }
+                }
+                u32 r[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) r[i] = seq_join(lo[i], hi[i], a.M.m, mu);
+                out = make_uint4(r[0] | r[1] << 16, r[2] | r[3] << 16, r[4] | r[5] << 16, r[6] | r[7] << 16);
+                if (live) *reinterpret_cast<uint4 *>(Vout + (size_t)row * kS + c0) = out;
+            } else if (row < r1) {
+                out = __ldcg(reinterpret_cast<const uint4 *>(Vin + (size_t)row * kS + c0));
+            }
+            *reinterpret_cast<uint4 *>(sm.vs[w][k] + (lane >> 1) * kVsStride + c0) = out;
+        }
+        if (base + kSeqTiles * kSeqWorkers >= ngroups) return base;
+        if (project) seq_project(a, sm, xf, base, ngroups, base == w, mu);
+    }
+}
+// both cross products of kSeqTiles groups of 16 rows stay below 2^23 (f32_to_u32)
+static_assert(2 * kSeqTiles * 16 * 255 * 255 < (1 << 23), "exact fp32 sums");
+
+// This CTA's partial projection (reduced) from the workers' words; the caller
+// synchronises before and after.
+__device__ __forceinline__ void publish_partial(const SeqArgs &a, const SeqSmem &sm, int buf)
+{
+    u32 *dst = a.partial + ((size_t)buf * gridDim.x + blockIdx.x) * (kS * kS);
+    if (threadIdx.x < kS * kS) {
+        u64 tot = 0;
+#pragma unroll
+        for (int i = 0; i < kSeqWorkers; ++i) tot += sm.red[i][threadIdx.x];
+        dst[threadIdx.x] = red64(tot, a.M);
+    }
+}
+
+// S_step[o] = sum over CTAs of their partials (mod p), one warp per output:
+// outputs blockIdx.x + gridDim.x (wi + k nw) for warp wi of nw.
+__device__ void reduce_step(const SeqArgs &a, long long step, int wi, int nw)
 {
     const int nb = gridDim.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-    const u32 *src = a.partial + (size_t)buf * nb * (kS * kS);
-    for (int o = blockIdx.x + w * nb; o < kS * kS; o += nb * nw) {
+    const int lane = threadIdx.x & 31;
+    const u32 *src = a.partial + (size_t)(step % kSeqBufs) * nb * (kS * kS);
+    for (int o = blockIdx.x + wi * nb; o < kS * kS; o += nb * nw) {
         u64 s = 0;
         for (int c = lane; c < nb; c += 32) s += __ldcg(src + (size_t)c * (kS * kS) + o);
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -335,84 +348,93 @@ __device__ void reduce_step(const SeqArgs &a, int buf, long long step)
 
 __global__ void __launch_bounds__(kSeqThreads, 1) k_sequence(const __grid_constant__ SeqArgs a)
 {
-    __shared__ SeqSmem sm;
-    extern __shared__ uint4 xfs[];  // X fragments of this CTA's 16-row groups (if they fit)
-    if (threadIdx.x < kMaxEnt) sm.doff[threadIdx.x] = threadIdx.x < a.ndiag ? a.doff[threadIdx.x] : 0;
-    __syncthreads();
+    extern __shared__ __align__(16) unsigned char seq_smem[];
+    SeqSmem &sm = *reinterpret_cast<SeqSmem *>(seq_smem);
+    unsigned char *seq_dyn = seq_smem + sizeof(SeqSmem);
     const long long nb = gridDim.x;
-    // 16-row aligned slices, so that every k-step covers one 16-row group
+    // 16-row aligned slices: every group of 16 rows belongs to one warp
     const int r0 = (int)(((a.n * blockIdx.x / nb) >> 4) << 4);
     const int r1 = blockIdx.x + 1 == nb ? (int)a.n : (int)(((a.n * (blockIdx.x + 1) / nb) >> 4) << 4);
     if (a.nsteps <= 0 && !a.Vnext) return;
+    const int g0 = r0 >> 4, ng = (r1 - r0 + 15) >> 4, nr = r1 - r0;
+    const uint4 *xf = a.XF + (size_t)g0 * 64;
+    const u32 *col = a.col + r0, *val = a.val + r0;
+    const unsigned char *gnp = a.gnp + g0;
+    size_t ld = (size_t)a.ld;
     if (a.xf_smem) {
-        // constant across steps: keep the CTA's X fragments resident
-        const int q0 = r0 >> 4, q1 = (r1 + 15) >> 4;
-        for (int t = threadIdx.x; t < (q1 - q0) * 64; t += blockDim.x) xfs[t] = __ldg(a.XF + (size_t)q0 * 64 + t);
+        // constant across steps: the CTA's X fragments
+        uint4 *d = reinterpret_cast<uint4 *>(seq_dyn);
+        for (int t = threadIdx.x; t < ng * 64; t += kSeqThreads) d[t] = __ldg(xf + t);
+        xf = d;
     }
-    MatSlice ms = {nullptr, nullptr, nullptr, nullptr};
     if (a.mat_smem) {
         // constant across steps too: the CTA's rows of the matrix
-        unsigned char *base = reinterpret_cast<unsigned char *>(xfs) + a.mat_off;
-        const int R = a.mrows, nr = r1 - r0, ld = (int)a.ld;
-        const size_t b_d = ((size_t)a.ndiag * R * 2 + 15) / 16 * 16, b_c = (size_t)a.width * R * 4;
-        const size_t b_v = ((size_t)a.width * R * 2 + 15) / 16 * 16;
-        unsigned short *dv = reinterpret_cast<unsigned short *>(base);
-        u32 *cl = reinterpret_cast<u32 *>(base + b_d);
-        unsigned short *vl = reinterpret_cast<unsigned short *>(base + b_d + b_c);
-        u32 *rb = a.rownb ? reinterpret_cast<u32 *>(base + b_d + b_c + b_v) : nullptr;
-        for (int t = threadIdx.x; t < a.ndiag * nr; t += blockDim.x) {
+        const int R = a.mrows;
+        u32 *dc = reinterpret_cast<u32 *>(seq_dyn + a.mat_off), *dv = dc + (size_t)2 * a.npair * R;
+        unsigned char *dg = reinterpret_cast<unsigned char *>(dv + (size_t)a.npair * R);
+        for (int t = threadIdx.x; t < 2 * a.npair * nr; t += kSeqThreads) {
             const int e = t / nr, r = t - e * nr;
-            dv[e * R + r] = __ldg(a.dval + (size_t)e * ld + r0 + r);
+            dc[e * R + r] = __ldg(col + (size_t)e * ld + r);
         }
-        for (int t = threadIdx.x; t < a.width * nr; t += blockDim.x) {
+        for (int t = threadIdx.x; t < a.npair * nr; t += kSeqThreads) {
             const int e = t / nr, r = t - e * nr;
-            cl[e * R + r] = __ldg(a.col + (size_t)e * ld + r0 + r);
-            vl[e * R + r] = __ldg(a.val + (size_t)e * ld + r0 + r);
+            dv[e * R + r] = __ldg(val + (size_t)e * ld + r);
         }
-        if (rb)
-            for (int r = threadIdx.x; r < nr; r += blockDim.x) rb[r] = __ldg(a.rownb + r0 + r);
-        ms.dval = dv;
-        ms.col = cl;
-        ms.val = vl;
-        ms.rownb = rb;
+        for (int t = threadIdx.x; t < ng; t += kSeqThreads) dg[t] = __ldg(gnp + t);
+        col = dc;
+        val = dv;
+        gnp = dg;
+        ld = (size_t)R;
     }
     __syncthreads();
     const bool skip = a.test_skip && blockIdx.x == 0;
-    unsigned epoch = 0;  // grid barriers passed (thread 0)
-    u32 pacc[2][2][4];
-    for (int i = 0; i < 2; ++i)
-        for (int j = 0; j < 2; ++j)
-            for (int e = 0; e < 4; ++e) pacc[i][j][e] = 0;
-    // The partials of S_j are summed during the next step, after its SpMM and
-    // before its barrier (they sit in buffer j & 1, which is written again only
-    // after that barrier), so no CTA starts a step late.
-    long long pending = -1;  // step whose partials are published but not yet summed
+    const bool worker = threadIdx.x < 32 * kSeqWorkers;
+    const u32 mu = (u32)(a.M.mu >> 32);   // floor(2^32 / m)
+    // few CTAs have many outputs each: then every warp takes some
+    const bool alone = kS * kS <= 3 * nb;
+    const int wi = alone ? 0 : (int)(threadIdx.x >> 5), nw = alone ? 1 : kSeqWarps;
+    unsigned epoch = 0;  // grid barriers passed
     // S_0 = X^T Y
     if (a.nsteps > 0) {
-        spmm_and_project(a, sm, xfs, ms, a.V0, a.V0, r0, r1, false, true, pacc);
-        publish_partial(a, sm, 0, pacc);
-        if (!grid_barrier(a, skip, epoch)) return;
-        pending = 0;
+        if (worker) {
+            const int last = seq_rows<false>(a, sm, xf, col, val, gnp, ld, a.V0, a.V0, r0, r1, true, mu);
+            seq_project(a, sm, xf, last, ng, last < kSeqWorkers, mu);
+        }
+        __syncthreads();
+        publish_partial(a, sm, 0);
+        grid_arrive(a, skip);
+        if (!grid_wait(a, skip, ++epoch)) return;
     }
-    long long done = 0;  // SpMMs done: V_done is current
-    for (long long i = 0; i < a.nsteps; ++i) {
-        const bool need = (i + 1 < a.nsteps) || a.Vnext;
-        if (!need) break;
+    // Step i forms V_{i+1} and S_{i+1}'s partials.  These are written after
+    // this CTA has arrived at the step's barrier, so they are seen after the
+    // next one and summed in step i + 2; a buffer is written again only after
+    // every CTA has arrived at the end of that step (kSeqBufs = 3).
+    const long long steps = a.Vnext ? a.nsteps : a.nsteps - 1;   // products
+    for (long long i = 0; i < steps; ++i) {
         const unsigned short *Vin = (i & 1) ? a.V1 : a.V0;
         unsigned short *Vout = (i & 1) ? a.V0 : a.V1;
         const bool proj = i + 1 < a.nsteps;
-        spmm_and_project(a, sm, xfs, ms, Vin, Vout, r0, r1, true, proj, pacc);
-        if (pending >= 0) reduce_step(a, (int)(pending & 1), pending);
-        pending = -1;
-        if (proj) publish_partial(a, sm, (int)((i + 1) & 1), pacc);
-        if (!grid_barrier(a, false, epoch)) return;
-        done = i + 1;
-        if (proj) pending = i + 1;
+        if (i > 0 && (!worker || !alone)) reduce_step(a, i - 1, wi, nw);
+        int last = 0;
+        if (worker) last = seq_rows<true>(a, sm, xf, col, val, gnp, ld, Vin, Vout, r0, r1, proj, mu);
+        grid_arrive(a, false);   // V_{i+1} is stored: the rest runs while the other CTAs arrive
+        if (proj) {
+            if (worker) seq_project(a, sm, xf, last, ng, last < kSeqWorkers, mu);
+            __syncthreads();
+            publish_partial(a, sm, (int)((i + 1) % kSeqBufs));
+        }
+        if (!grid_wait(a, false, ++epoch)) return;
     }
-    if (pending >= 0) reduce_step(a, (int)(pending & 1), pending);
+    // the last partials have to be seen, then the last two steps are summed
+    if (a.nsteps > 1 && steps > 0) {
+        grid_arrive(a, false);
+        if (!grid_wait(a, false, ++epoch)) return;
+    }
+    for (long long j = steps > 1 ? steps - 1 : 0; j < a.nsteps; ++j)
+        reduce_step(a, j, (int)(threadIdx.x >> 5), kSeqWarps);
     if (a.Vnext) {
-        const unsigned short *Vf = (done & 1) ? a.V1 : a.V0;
-        for (long long t = (long long)r0 * a.s + threadIdx.x; t < (long long)r1 * a.s; t += blockDim.x) {
+        const unsigned short *Vf = (steps & 1) ? a.V1 : a.V0;
+        for (long long t = (long long)r0 * a.s + threadIdx.x; t < (long long)r1 * a.s; t += kSeqThreads) {
             const long long row = t / a.s;
             const int c = (int)(t - row * a.s);
             a.Vnext[t] = __ldcg(Vf + row * kS + c);
@@ -500,17 +522,14 @@ __global__ void k_reduce_copy(long long n, const u32 *__restrict__ src, u32 *__r
 
 // ---------------------------------------------------------------------------
 struct SeqState {
-    // DIA + ELL_R layout
+    // entry pairs, row by row
     bool layout_tried = false, layout_ok = false;
     long long n = 0;
-    int ndiag = 0, width = 0;
+    int npair = 0;
     long long ld = 0;
     void *arena = nullptr;
-    const int *doff = nullptr;
-    const unsigned short *dval = nullptr;
-    const u32 *col = nullptr;
-    const unsigned short *val = nullptr;
-    const u32 *rownb = nullptr;
+    const u32 *col = nullptr, *val = nullptr;
+    const unsigned char *gnp = nullptr;
     // work buffers
     void *work = nullptr;
     size_t work_bytes = 0;
@@ -543,7 +562,8 @@ void free_sequence_state(ffspmv_handle *h)
 
 namespace {
 
-// Split A into its densest diagonals (DIA) and an ELL_R part for the rest.
+// The rows as pairs of entries: the densest diagonals first (their entries
+// merged), then the rest in order.  Refused when a row needs more than kMaxEnt.
 bool build_seq_layout(ffspmv_handle *h, SeqState &q)
 {
     const long long n = h->A.nrows;
@@ -582,44 +602,41 @@ bool build_seq_layout(ffspmv_handle *h, SeqState &q)
     }
     if (width + (long long)diag.size() > kMaxEnt) return false;  // short rows only
     if (n * kS >= (1LL << 31) || width * ld >= (1LL << 31)) return false;  // 32-bit indices
-    std::vector<u32> ecol((size_t)(width * ld), 0), rownb(n);
-    std::vector<unsigned short> eval((size_t)(width * ld), 0);
-    bool uniform = true;
+    const int nd = (int)diag.size(), npair = (int)((nd + width + 1) / 2);
+    std::vector<u32> ecol((size_t)2 * npair * ld), eval((size_t)npair * ld, 0);
+    std::vector<unsigned char> gnp((size_t)(n + 15) / 16, 0);
+    for (size_t e = 0; e < (size_t)2 * npair; ++e)
+        for (long long i = 0; i < ld; ++i) ecol[e * ld + i] = (u32)std::min<long long>(i, n - 1);
     for (long long i = 0; i < n; ++i) {
-        long long j = 0;
-        for (long long k = ptr[i]; k < ptr[i + 1]; ++k) {
-            long long off = col[k] - i;
-            if (std::find(diag.begin(), diag.end(), (int)off) != diag.end()) continue;
-            ecol[(size_t)(j * ld + i)] = (u32)col[k];
-            eval[(size_t)(j * ld + i)] = (unsigned short)val[k];
+        int j = 0;   // entries without a value are left out
+        auto put = [&](long long c, u32 v) {
+            if (!v) return;
+            ecol[(size_t)j * ld + i] = (u32)c;
+            eval[(size_t)(j / 2) * ld + i] |= ((v & 255u) | (v >> 8) << 16) << (j & 1 ? 8 : 0);
             ++j;
-        }
-        rownb[i] = (u32)j;
-        if (j != width) uniform = false;
+        };
+        for (int d = 0; d < nd; ++d) put(i + diag[d], dval[(size_t)d * ld + i]);
+        for (long long k = ptr[i]; k < ptr[i + 1]; ++k)
+            if (std::find(diag.begin(), diag.end(), (int)(col[k] - i)) == diag.end()) put(col[k], val[k]);
+        unsigned char &g = gnp[(size_t)(i >> 4)];
+        g = (unsigned char)std::max<int>(g, (j + 1) / 2);
     }
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    size_t o_doff = 0, o_dval = al(diag.size() * 4 + 4), o_col = o_dval + al(dval.size() * 2 + 2);
-    size_t o_val = o_col + al(ecol.size() * 4 + 4), o_nb = o_val + al(eval.size() * 2 + 2);
-    size_t total = o_nb + al(rownb.size() * 4 + 4);
+    const size_t o_val = al(ecol.size() * 4 + 4), o_gnp = o_val + al(eval.size() * 4 + 4), total = o_gnp + al(gnp.size() + 4);
     if (cudaMalloc(&q.arena, total) != cudaSuccess) {
         q.arena = nullptr;
         return false;
     }
     char *b = (char *)q.arena;
-    cudaMemcpy(b + o_doff, diag.data(), diag.size() * 4, cudaMemcpyHostToDevice);
-    cudaMemcpy(b + o_dval, dval.data(), dval.size() * 2, cudaMemcpyHostToDevice);
-    cudaMemcpy(b + o_col, ecol.data(), ecol.size() * 4, cudaMemcpyHostToDevice);
-    cudaMemcpy(b + o_val, eval.data(), eval.size() * 2, cudaMemcpyHostToDevice);
-    cudaMemcpy(b + o_nb, rownb.data(), rownb.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(b, ecol.data(), ecol.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(b + o_val, eval.data(), eval.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(b + o_gnp, gnp.data(), gnp.size(), cudaMemcpyHostToDevice);
     q.n = n;
-    q.ndiag = (int)diag.size();
-    q.width = (int)width;
+    q.npair = npair;
     q.ld = ld;
-    q.doff = (const int *)(b + o_doff);
-    q.dval = (const unsigned short *)(b + o_dval);
-    q.col = (const u32 *)(b + o_col);
-    q.val = (const unsigned short *)(b + o_val);
-    q.rownb = uniform ? nullptr : (const u32 *)(b + o_nb);
+    q.col = (const u32 *)b;
+    q.val = (const u32 *)(b + o_val);
+    q.gnp = (const unsigned char *)(b + o_gnp);
     return cudaGetLastError() == cudaSuccess;
 }
 
@@ -629,7 +646,7 @@ ffspmv_status ensure_work(SeqState &q, long long n, int nblocks)
     const size_t nq = (size_t)((n + 15) / 16);
     size_t xb = al(nq * 64 * sizeof(uint4));
     size_t vb = al((size_t)n * kS * 2 + 16);
-    size_t pb = al((size_t)2 * nblocks * kS * kS * 4);
+    size_t pb = al((size_t)kSeqBufs * nblocks * kS * kS * 4);
     size_t need = xb + 2 * vb + pb + 256;
     if (need > q.work_bytes) {
         if (q.work) cudaFree(q.work);
@@ -742,8 +759,8 @@ extern "C" ffspmv_status spmv_block_sequence(ffspmv_t h, const uint32_t *d_X, co
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaFuncSetAttribute(k_sequence, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXfSmemMax);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sequence, kSeqThreads, kXfSmemMax);
+        cudaFuncSetAttribute(k_sequence, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(SeqSmem) + kXfSmemMax));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sequence, kSeqThreads, sizeof(SeqSmem) + kXfSmemMax);
         nblocks = nsm * std::min(per_sm, 1);
         if (!coop || per_sm < 1) persistent = false;
         // keep at least one pass of rows per CTA
@@ -757,16 +774,13 @@ extern "C" ffspmv_status spmv_block_sequence(ffspmv_t h, const uint32_t *d_X, co
     SeqArgs a;
     memset(&a, 0, sizeof(a));
     a.n = n;
-    a.ndiag = q->ndiag;
-    a.width = q->width;
+    a.npair = q->npair;
     a.s = s;
     a.ld = q->ld;
     a.nsteps = nsteps;
-    a.doff = q->doff;
-    a.dval = q->dval;
     a.col = q->col;
     a.val = q->val;
-    a.rownb = q->rownb;
+    a.gnp = q->gnp;
     a.XF = q->XF;
     a.V0 = q->V0;
     a.V1 = q->V1;
@@ -782,11 +796,10 @@ extern "C" ffspmv_status spmv_block_sequence(ffspmv_t h, const uint32_t *d_X, co
     a.xf_smem = xf_bytes <= kXfSmemMax ? 1 : 0;
     // the CTA's matrix rows as well, when they fit beside the X fragments
     a.mrows = (int)(((n + nblocks - 1) / nblocks / 16 + 2) * 16);
-    const size_t mat_bytes = ((size_t)q->ndiag * a.mrows * 2 + 15) / 16 * 16 + (size_t)q->width * a.mrows * 4 +
-                             ((size_t)q->width * a.mrows * 2 + 15) / 16 * 16 + (q->rownb ? (size_t)a.mrows * 4 : 0);
+    const size_t mat_bytes = (size_t)3 * q->npair * a.mrows * 4 + (size_t)a.mrows / 16 + 16;
     a.mat_off = a.xf_smem ? (int)xf_bytes : 0;
     a.mat_smem = (size_t)a.mat_off + mat_bytes <= kXfSmemMax ? 1 : 0;
-    const size_t dyn_smem = (size_t)a.mat_off + (a.mat_smem ? mat_bytes : 0);
+    const size_t dyn_smem = sizeof(SeqSmem) + (size_t)a.mat_off + (a.mat_smem ? mat_bytes : 0);
     a.M = make_mod(h->m, 1, 0);
 
     // the graph: prepare X/Y, clear barrier + status, run the persistent kernel
