@@ -246,26 +246,42 @@ struct BlockAcc<false> {
     static __device__ __forceinline__ u32 get(const AccWide &s, const Mod &M) { return (u32)s.partial(M); }
 };
 
+// COH: X is a buffer that earlier kernels of the stream wrote (L2 only), else
+// the read-only path.
+template <bool COH>
+__device__ __forceinline__ uint4 block_gather(const char *p)
+{
+    if constexpr (COH) return __ldcg(reinterpret_cast<const uint4 *>(p));
+    else return __ldg(reinterpret_cast<const uint4 *>(p));
+}
+
 // acc += quads k, k + step, ... below end; xb: this lane's piece of the rows
 // of X.  Rows are padded to whole quads (value 0, column 0).
-template <bool SMALL>
+// X (and the y that earlier products read) belong to the kernel before this one
+// in the stream: it is waited for with the first quad already on its way.
+template <bool SMALL, bool COH>
 __device__ __forceinline__ void block_entries(BlockAcc<SMALL> &acc, const BlockMat &a, u32 k, u32 end, u32 step,
                                               const char *xb, bool on)
 {
     typedef typename std::conditional<SMALL, uint2, uint4>::type V;
     const u32 pb = (u32)a.pitch * 16u;
-    if (k >= end) return;
-    uint4 j = __ldcs(reinterpret_cast<const uint4 *>(a.col) + k);
-    V v = __ldcs(reinterpret_cast<const V *>(a.val) + k);
-    for (;;) {
+    uint4 j = make_uint4(0u, 0u, 0u, 0u);
+    V v = V{};
+    if (k < end) {
+        j = __ldcs(reinterpret_cast<const uint4 *>(a.col) + k);
+        v = __ldcs(reinterpret_cast<const V *>(a.val) + k);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (COH) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next step may load its quads
+    while (k < end) {
         uint4 x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = make_uint4(0u, 0u, 0u, 0u);
         if (on) {
-            x[0] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.x * pb));
-            x[1] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.y * pb));
-            x[2] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.z * pb));
-            x[3] = __ldg(reinterpret_cast<const uint4 *>(xb + (u64)j.w * pb));
+            x[0] = block_gather<COH>(xb + (u64)j.x * pb);
+            x[1] = block_gather<COH>(xb + (u64)j.y * pb);
+            x[2] = block_gather<COH>(xb + (u64)j.z * pb);
+            x[3] = block_gather<COH>(xb + (u64)j.w * pb);
         }
         // the next quad is on its way from memory while the gathers are
         const V vc = v;
@@ -275,7 +291,6 @@ __device__ __forceinline__ void block_entries(BlockAcc<SMALL> &acc, const BlockM
             v = __ldcs(reinterpret_cast<const V *>(a.val) + k);
         }
         acc.quad(vc, x, a.fold);
-        if (k >= end) break;
     }
 }
 
@@ -361,7 +376,7 @@ struct BlockEmitCarry {
 };
 
 // A warp's chunk of a long row.
-template <bool SMALL>
+template <bool SMALL, bool COH = false>
 __device__ __forceinline__ void block_chunk(const BlockMat &a, u32 w, int lane)
 {
     constexpr int C = BlockAcc<SMALL>::C;
@@ -369,7 +384,7 @@ __device__ __forceinline__ void block_chunk(const BlockMat &a, u32 w, int lane)
     BlockAcc<SMALL> acc;
     acc.zero();
     const uint4 ch = __ldg(a.chunk + w);
-    block_entries<SMALL>(acc, a, ch.y + (u32)(lane >> a.lgt), ch.z, 32u >> a.lgt,
+    block_entries<SMALL, COH>(acc, a, ch.y + (u32)(lane >> a.lgt), ch.z, 32u >> a.lgt,
                          reinterpret_cast<const char *>(a.xs + c), c < a.pieces);
     u64 *cw = a.carry + (size_t)ch.x * kBlockVecs;
     const BlockEmitCarry emit = {&a, &a.M, cw};
@@ -392,7 +407,7 @@ __device__ __forceinline__ void block_chunk(const BlockMat &a, u32 w, int lane)
 }
 
 // A warp's 32 / (T G) rows of a class: r0 the first, below rend, G = 2^lgg.
-template <bool SMALL>
+template <bool SMALL, bool COH = false>
 __device__ __forceinline__ void block_rows(const BlockMat &a, u32 r0, u32 rend, int lgg, bool one, int lane)
 {
     constexpr int C = BlockAcc<SMALL>::C;
@@ -402,27 +417,22 @@ __device__ __forceinline__ void block_rows(const BlockMat &a, u32 r0, u32 rend, 
     acc.zero();
     const u32 r = r0 + (u32)(lane >> lgr);
     BlockEmitRow emit = {&a, &a.M, 0u, r < rend && on};
+    u32 s = 0, e = 0;
     if (r < rend) {
         // rows of one quad lie one after another: no offset to wait for
-        const u32 s = one ? a.quad1 + r : __ldg(a.ptr + r), e = one ? s + 1u : __ldg(a.ptr + r + 1);
+        s = one ? a.quad1 + r : __ldg(a.ptr + r);
+        e = one ? s + 1u : __ldg(a.ptr + r + 1);
         emit.row = __ldg(a.row + r);
-        block_entries<SMALL>(acc, a, s + (u32)((lane >> a.lgt) & ((1 << lgg) - 1)), e, 1u << lgg,
-                             reinterpret_cast<const char *>(a.xs + c), on);
     }
+    block_entries<SMALL, COH>(acc, a, s + (u32)((lane >> a.lgt) & ((1 << lgg) - 1)), e, 1u << lgg,
+                              reinterpret_cast<const char *>(a.xs + c), on);
     block_reduce<SMALL, C>(acc.a, a.lgt, lgg, 0, lane, c * C, emit);
 }
 
-template <bool SMALL>
-__global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constant__ BlockArgs a)
+// The rows of warp w >= nchunk_warps.
+template <bool SMALL, bool COH>
+__device__ __forceinline__ void block_class_rows(const BlockArgs &a, u32 w, int lane)
 {
-    const u32 w = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    // the rows of X come from the staging launch before this one
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (w < (u32)a.nchunk_warps) {
-        block_chunk<SMALL>(a.m, w, lane);
-        return;
-    }
     // the class of this warp (warp0 grows; the last entry ends the list)
     int b = 0;
 #pragma unroll
@@ -430,8 +440,94 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constan
         if (w >= a.warp0[i]) b = i;
     if (w >= a.warp0[kBlockClasses]) return;
     const int lgg = a.lgg[b];
-    block_rows<SMALL>(a.m, a.row0[b] + ((w - a.warp0[b]) << (5 - a.m.lgt - lgg)), a.row0[b + 1], lgg,
-                      b == kBlockClasses - 2, lane);
+    block_rows<SMALL, COH>(a.m, a.row0[b] + ((w - a.warp0[b]) << (5 - a.m.lgt - lgg)), a.row0[b + 1], lgg,
+                           b == kBlockClasses - 2, lane);
+}
+
+template <bool SMALL>
+__global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constant__ BlockArgs a)
+{
+    const u32 w = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w < (u32)a.nchunk_warps) {
+        block_chunk<SMALL>(a.m, w, lane);
+        return;
+    }
+    block_class_rows<SMALL, false>(a, w, lane);
+}
+
+// One step of a block sequence at m > 2^16: V_{i+1} = A V_i and S_i = X^T V_i in
+// one launch, both read V_i.  CTAs below `spmm` multiply; each of the next
+// `proj` projects its rows (four outputs of one row of S per thread, the
+// threads in groups that take every ngrp-th row) and writes its reduced sums;
+// one more adds up the sums of the step before and writes S_{i-1}, so that no
+// CTA waits for another.  V: rows of ldv words (a multiple of four, zero past
+// s).  A kernel lets the next one start once the one before it is complete.
+struct BlockStep {
+    BlockArgs b;
+    unsigned spmm, proj;      // CTAs of each kind
+    int s, tiles, ngrp;       // tiles of four outputs, groups of threads
+    long long n, ldv, per;    // rows, words per row of V, rows per projecting CTA
+    const u32 *X, *V;
+    u32 *part, *prev;         // [proj][s s]: this step's sums, the step before's (null: none)
+    u32 *S;                   // S_{i-1}
+};
+
+__global__ void __launch_bounds__(kBlockThreads, 3) k_block_step(const __grid_constant__ BlockStep a)
+{
+    __shared__ u32 red[4 * kBlockThreads];
+    const int tid = threadIdx.x;
+    if (blockIdx.x < a.spmm) {
+        const u32 w = (blockIdx.x * kBlockThreads + tid) >> 5;
+        if (w < (u32)a.b.nchunk_warps) block_chunk<false, true>(a.b.m, w, tid & 31);
+        else if (w < a.b.warp0[kBlockClasses]) block_class_rows<false, true>(a.b, w, tid & 31);
+        return;
+    }
+    const Mod &M = a.b.m.M;
+    const int outs = a.s * a.s;
+    if (blockIdx.x == gridDim.x - 1) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (!a.prev) return;
+        for (int o = tid; o < outs; o += kBlockThreads) {
+            u64 sum = 0;
+#pragma unroll 8
+            for (unsigned c = 0; c < a.proj; ++c) sum += __ldcg(a.prev + (size_t)c * outs + o);
+            a.S[o] = red64(sum, M);
+        }
+        return;
+    }
+    const long long r0 = (long long)(blockIdx.x - a.spmm) * a.per, r1 = min(a.n, r0 + a.per);
+    const int g = tid / a.tiles, t = tid - g * a.tiles, bt = (a.s + 3) / 4;   // tile: row t / bt of S, columns 4 (t mod bt) ..
+    const int ai = t / bt, c0 = 4 * (t - ai * bt);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    AccWide acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i].zero();
+    if (g < a.ngrp) {
+#pragma unroll 4
+        for (long long r = r0 + g; r < r1; r += a.ngrp) {
+            const u32 x = __ldg(a.X + r * a.s + ai);
+            const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(a.V + r * a.ldv + c0));
+            acc[0].mad(x, v.x);
+            acc[1].mad(x, v.y);
+            acc[2].mad(x, v.z);
+            acc[3].mad(x, v.w);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) red[i * kBlockThreads + tid] = g < a.ngrp ? (u32)acc[i].partial(M) : 0u;
+    __syncthreads();
+    if (tid < a.tiles) {
+        u32 *dst = a.part + (size_t)(blockIdx.x - a.spmm) * outs + ai * a.s;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            u64 sum = 0;
+            for (int k = 0; k < a.ngrp; ++k) sum += red[i * kBlockThreads + k * a.tiles + tid];
+            if (c0 + i < a.s) dst[c0 + i] = red64(sum, M);
+        }
+    }
 }
 
 // log2 of the groups per row of class i (heaviest first), 2^lgt lanes per row
@@ -513,7 +609,6 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_co
     a.fold = D.fold;
     a.M = D.M;
     u32 w = w0 - P.first[j];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (w < D.nchunk) {
         if (D.small) block_chunk<true>(a, w, lane);
         else block_chunk<false>(a, w, lane);
@@ -790,6 +885,57 @@ long long block_launches(const BlockPlan &B, int nvec)
     return n;
 }
 
+// What a launch needs of the layout and of one block of nv vectors (X is
+// filled in by the caller).
+static BlockArgs block_args(const BlockPlan &B, u32 *y, long long ldy, int nv, u32 m, u32 alpha, u32 beta)
+{
+    BlockArgs a;
+    memset(&a, 0, sizeof(a));
+    a.m.ptr = B.ptr;
+    a.m.row = B.row;
+    a.m.col = B.col;
+    a.m.lrow = B.lrow;
+    a.m.chunk = B.chunk;
+    a.m.val = B.val;
+    a.m.carry = B.carry;
+    a.m.count = B.count;
+    a.m.quad1 = B.quad1;
+    a.m.y = y;
+    a.m.ldy = ldy;
+    a.m.nvec = nv;
+    a.m.vec4 = (ldy % 4 == 0 && ((uintptr_t)y & 15u) == 0) ? 1 : 0;
+    a.m.M = make_mod(m, alpha, beta);
+    a.m.fold = m <= (1u << 31) ? 1 : 0;
+    const int C = B.small ? 8 : 4;
+    a.m.pieces = (nv + C - 1) / C;
+    while ((1 << a.m.lgt) < a.m.pieces) ++a.m.lgt;
+    return a;
+}
+
+// The warps of a launch, class by class; returns their number.
+static long long block_warps(const BlockPlan &B, BlockArgs &a)
+{
+    // groups per row: by class, doubled while the launch has fewer than
+    // 16 warps per SM (short matrices: more lanes per row, shorter chains)
+    long long warps = 0;
+    for (int boost = 0; boost < 6; ++boost) {
+        warps = B.nchunk;
+        for (int c = 0; c < kBlockClasses; ++c) {
+            const int lg = std::min(block_lgg(c, a.m.lgt) + boost, 5 - a.m.lgt);
+            a.lgg[c] = lg;
+            a.row0[c] = (u32)B.cls_row[c];
+            a.warp0[c] = (u32)warps;
+            const int rpw = 32 >> (a.m.lgt + lg);
+            warps += (B.cls_row[c + 1] - B.cls_row[c] + rpw - 1) / rpw;
+        }
+        if (warps >= 16 * 152) break;
+    }
+    a.row0[kBlockClasses] = (u32)B.cls_row[kBlockClasses];
+    a.warp0[kBlockClasses] = (u32)warps;
+    a.nchunk_warps = (int)B.nchunk;
+    return warps;
+}
+
 ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec, u32 m,
                         u32 alpha, u32 beta, cudaStream_t st)
 {
@@ -798,26 +944,8 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
         const int nv = std::min(kBlockVecs, nvec - v0);
         const u32 *xv = x + v0;
         u32 *yv = y + v0;
-        BlockArgs a;
-        memset(&a, 0, sizeof(a));
-        a.m.ptr = B.ptr;
-        a.m.row = B.row;
-        a.m.col = B.col;
-        a.m.lrow = B.lrow;
-        a.m.chunk = B.chunk;
-        a.m.val = B.val;
-        a.m.carry = B.carry;
-        a.m.count = B.count;
-        a.m.quad1 = B.quad1;
-        a.m.y = yv;
-        a.m.ldy = ldy;
-        a.m.nvec = nv;
-        a.m.vec4 = (ldy % 4 == 0 && ((uintptr_t)yv & 15u) == 0) ? 1 : 0;
-        a.m.M = make_mod(m, alpha, beta);
-        a.m.fold = m <= (1u << 31) ? 1 : 0;
+        BlockArgs a = block_args(B, yv, ldy, nv, m, alpha, beta);
         const int pieces = (nv + C - 1) / C;
-        while ((1 << a.m.lgt) < pieces) ++a.m.lgt;
-        a.m.pieces = pieces;
         const bool in_place = block_in_place(B, xv, ldx, nv);
         if (in_place) {
             a.m.xs = reinterpret_cast<const uint4 *>(xv);
@@ -836,24 +964,7 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
                 FF_CUDA(cudaGetLastError());
             }
         }
-        // groups per row: by class, doubled while the launch has fewer than
-        // 16 warps per SM (short matrices: more lanes per row, shorter chains)
-        long long warps = 0;
-        for (int boost = 0; boost < 6; ++boost) {
-            warps = B.nchunk;
-            for (int c = 0; c < kBlockClasses; ++c) {
-                const int lg = std::min(block_lgg(c, a.m.lgt) + boost, 5 - a.m.lgt);
-                a.lgg[c] = lg;
-                a.row0[c] = (u32)B.cls_row[c];
-                a.warp0[c] = (u32)warps;
-                const int rpw = 32 >> (a.m.lgt + lg);
-                warps += (B.cls_row[c + 1] - B.cls_row[c] + rpw - 1) / rpw;
-            }
-            if (warps >= 16 * 152) break;
-        }
-        a.row0[kBlockClasses] = (u32)B.cls_row[kBlockClasses];
-        a.warp0[kBlockClasses] = (u32)warps;
-        a.nchunk_warps = (int)B.nchunk;
+        const long long warps = block_warps(B, a);
         if (warps == 0) continue;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)((warps * 32 + kBlockThreads - 1) / kBlockThreads));
@@ -931,6 +1042,58 @@ ffspmv_status run_block_many(int count, const BlockPlan *const *B, const u32 *co
     for (int c0 = 0; c0 < count; c0 += kMany) {
         const ffspmv_status r = block_many(std::min(kMany, count - c0), B + c0, x + c0, y + c0, nvec + c0, st);
         if (r != FFSPMV_OK) return r;
+    }
+    return FFSPMV_OK;
+}
+
+// projecting CTAs: four rows per group of threads, two CTAs per SM at most
+static unsigned step_proj(long long n, int s)
+{
+    const int ngrp = kBlockThreads / (s * ((s + 3) / 4));
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return (unsigned)std::max<long long>(1, std::min<long long>((n + 4LL * ngrp - 1) / (4LL * ngrp), 2LL * std::max(nsm, 1)));
+}
+
+size_t block_steps_bytes(long long n, int s) { return (size_t)2 * step_proj(n, s) * s * s * 4; }
+
+ffspmv_status run_block_steps(const BlockPlan &B, long long n, int s, u32 m, const u32 *X, u32 *V0, u32 *V1, u32 *part,
+                              long long nsteps, bool next, u32 *S, cudaStream_t st)
+{
+    const int ldv = (s + 3) / 4 * 4;
+    BlockStep a;
+    memset(&a, 0, sizeof(a));
+    a.s = s;
+    a.tiles = s * (ldv / 4);
+    a.ngrp = kBlockThreads / a.tiles;
+    a.n = n;
+    a.ldv = ldv;
+    a.X = X;
+    a.proj = step_proj(n, s);
+    a.per = (n + a.proj - 1) / a.proj;
+    u32 *parts[2] = {part, part + (size_t)a.proj * s * s};
+    for (long long i = 0; i <= nsteps; ++i) {
+        const u32 *Vi = (i & 1) ? V1 : V0;
+        a.b = block_args(B, (i & 1) ? V0 : V1, ldv, s, m, 1, 0);
+        a.b.m.xs = reinterpret_cast<const uint4 *>(Vi);
+        a.b.m.pitch = ldv / 4;
+        const long long warps = block_warps(B, a.b);
+        a.spmm = i + 1 < nsteps || (next && i < nsteps) ? (unsigned)((warps * 32 + kBlockThreads - 1) / kBlockThreads) : 0u;
+        a.V = Vi;
+        a.part = parts[i & 1];
+        a.prev = i ? parts[(i + 1) & 1] : nullptr;
+        a.S = i ? S + (i - 1) * s * s : nullptr;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(a.spmm + (i < nsteps ? a.proj : 0u) + 1u);
+        cfg.blockDim = dim3(kBlockThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        FF_CUDA(cudaLaunchKernelEx(&cfg, k_block_step, a));
     }
     return FFSPMV_OK;
 }

@@ -22,4 +22,12 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
 ffspmv_status run_block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
                              cudaStream_t st);
 
+// nsteps >= 1 steps of a block sequence at m > 2^16, one launch each and one
+// more: S_i = X^T V_i (at S + i s s) and V_{i+1} = A V_i between V0 and V1 (n
+// rows of s words rounded up to 4, zero past s; V_0 in V0; `next`: V_nsteps is
+// formed too).  part: block_steps_bytes of scratch.
+size_t block_steps_bytes(long long n, int s);
+ffspmv_status run_block_steps(const BlockPlan &B, long long n, int s, u32 m, const u32 *X, u32 *V0, u32 *V1, u32 *part,
+                              long long nsteps, bool next, u32 *S, cudaStream_t st);
+
 }  // namespace ff

@@ -36,7 +36,7 @@ struct GdRows {
     int r[kGdMaxN];  // physical row of each position of the elimination
 };
 
-__device__ __forceinline__ u32 mulmod(u32 a, u32 b, u32 p) { return (u32)((u64)a * b % p); }
+__device__ __forceinline__ u32 mulmod(u32 a, u32 b, const Mod &M) { return red64((u64)a * b, M); }
 
 // W[i][c][k], k < K: coefficient k of U_ic (rev = 0) or of U~_ic (rev = 1),
 // U_ic = entry (sel[i], c) of the basis P ((d+1) x m x m, coefficient-major).
@@ -98,17 +98,17 @@ __global__ void k_gd_val(const u32 *__restrict__ W, int n, int K, int c, int pre
 
 // inv = 1 / u mod x^L, u_k = coefficient v + k of the pivot entry: inv_0 =
 // u_0^(p-2) (Fermat), inv_k = -inv_0 sum_{j=1..k} u_j inv_{k-j}.  One CTA.
-__global__ void k_gd_inv(const u32 *__restrict__ W, int n, int K, int c, int v, int L, GdRows R, u32 p,
+__global__ void k_gd_inv(const u32 *__restrict__ W, int n, int K, int c, int v, int L, GdRows R, const Mod M,
                          u32 *__restrict__ inv)
 {
     __shared__ u64 part[kGdThreads / 32];
     __shared__ u32 inv0;
     const u32 *u = W + ((long long)R.r[c] * n + c) * K + v;
     if (threadIdx.x == 0) {
-        u32 b = u[0], e = p - 2, r = 1;
+        u32 b = u[0], e = M.m - 2u, r = 1;
         while (e) {
-            if (e & 1u) r = mulmod(r, b, p);
-            b = mulmod(b, b, p);
+            if (e & 1u) r = mulmod(r, b, M);
+            b = mulmod(b, b, M);
             e >>= 1;
         }
         inv0 = r;
@@ -117,14 +117,14 @@ __global__ void k_gd_inv(const u32 *__restrict__ W, int n, int K, int c, int v, 
     __syncthreads();
     for (int k = 1; k < L; ++k) {
         u64 s = 0;  // below L 2^31 < 2^47
-        for (int j = 1 + threadIdx.x; j <= k; j += blockDim.x) s += mulmod(u[j], inv[k - j], p);
+        for (int j = 1 + threadIdx.x; j <= k; j += blockDim.x) s += mulmod(u[j], inv[k - j], M);
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
         if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
         __syncthreads();
         if (threadIdx.x == 0) {
             u64 t = 0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w];
-            inv[k] = mulmod(inv0, (p - (u32)(t % p)) % p, p);
+            inv[k] = mulmod(inv0, red64(M.m - red64(t, M), M), M);
         }
         __syncthreads();
     }
@@ -132,7 +132,7 @@ __global__ void k_gd_inv(const u32 *__restrict__ W, int n, int K, int c, int v, 
 
 // f_pos = (entry (pos, c) / x^v) * inv mod x^L for the positions below c
 // (CTA b: position c + 1 + b).
-__global__ void k_gd_factor(const u32 *__restrict__ W, int n, int K, int c, int v, int L, GdRows R, u32 p,
+__global__ void k_gd_factor(const u32 *__restrict__ W, int n, int K, int c, int v, int L, GdRows R, const Mod M,
                             const u32 *__restrict__ inv, u32 *__restrict__ F)
 {
     const int pos = c + 1 + blockIdx.x;
@@ -140,14 +140,14 @@ __global__ void k_gd_factor(const u32 *__restrict__ W, int n, int K, int c, int 
     u32 *f = F + (long long)pos * K;
     for (int k = threadIdx.x; k < L; k += blockDim.x) {
         u64 s = 0;
-        for (int j = 0; j <= k; ++j) s += mulmod(a[j], inv[k - j], p);
-        f[k] = (u32)(s % p);
+        for (int j = 0; j <= k; ++j) s += mulmod(a[j], inv[k - j], M);
+        f[k] = red64(s, M);
     }
 }
 
 // row_pos -= f_pos row_c (columns > c, coefficients < L); CTA (b, j): position
 // c + 1 + b, column c + 1 + j.
-__global__ void k_gd_update(u32 *__restrict__ W, int n, int K, int c, int L, GdRows R, u32 p,
+__global__ void k_gd_update(u32 *__restrict__ W, int n, int K, int c, int L, GdRows R, const Mod M,
                             const u32 *__restrict__ F)
 {
     const int w = n - c - 1;
@@ -157,8 +157,8 @@ __global__ void k_gd_update(u32 *__restrict__ W, int n, int K, int c, int L, GdR
     const u32 *f = F + (long long)pos * K;
     for (int k = threadIdx.x; k < L; k += blockDim.x) {
         u64 s = 0;
-        for (int j = 0; j <= k; ++j) s += mulmod(f[j], q[k - j], p);
-        t[k] = (u32)(((u64)t[k] + p - (u32)(s % p)) % p);
+        for (int j = 0; j <= k; ++j) s += mulmod(f[j], q[k - j], M);
+        t[k] = red64((u64)t[k] + M.m - red64(s, M), M);
     }
 }
 
@@ -196,6 +196,7 @@ bool gd_prime(u64 q)
 
 struct GdRun {
     u32 p = 0;
+    Mod M = {};
     int m = 0, n = 0;
     long long d = 0;
     const u32 *P = nullptr;
@@ -234,11 +235,13 @@ ffspmv_status gd_valuation(GdRun &G, int rev, int K, long long *out, bool *ok)
         sum += v;
         const int L = prec - v;
         if (c + 1 < n) {
-            k_gd_inv<<<1, kGdThreads, 0, G.st>>>(G.W, n, K, c, v, L, R, G.p, G.inv);
+            // a short series takes one warp: its 2 L block barriers were most of
+            // the kernel (48 us at L = 32 with 256 threads)
+            k_gd_inv<<<1, L <= 128 ? 32 : kGdThreads, 0, G.st>>>(G.W, n, K, c, v, L, R, G.M, G.inv);
             FF_CUDA(cudaGetLastError());
-            k_gd_factor<<<n - c - 1, kGdThreads, 0, G.st>>>(G.W, n, K, c, v, L, R, G.p, G.inv, G.F);
+            k_gd_factor<<<n - c - 1, kGdThreads, 0, G.st>>>(G.W, n, K, c, v, L, R, G.M, G.inv, G.F);
             FF_CUDA(cudaGetLastError());
-            k_gd_update<<<(n - c - 1) * (n - c - 1), kGdThreads, 0, G.st>>>(G.W, n, K, c, L, R, G.p, G.F);
+            k_gd_update<<<(n - c - 1) * (n - c - 1), kGdThreads, 0, G.st>>>(G.W, n, K, c, L, R, G.M, G.F);
             FF_CUDA(cudaGetLastError());
         }
         prec = L;
@@ -318,6 +321,7 @@ extern "C" ffspmv_status sigma_generator_degrees(uint32_t p, int32_t m, int32_t 
     std::vector<int> sel(order.begin(), order.begin() + n);
     GdRun G;
     G.p = p;
+    G.M = make_mod(p, 1, 0);
     G.m = m;
     G.n = n;
     G.d = d;
