@@ -447,7 +447,7 @@ __device__ __forceinline__ void block_class_rows(const BlockArgs &a, u32 w, int 
 template <bool SMALL>
 __global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constant__ BlockArgs a)
 {
-    const u32 w = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
+    const u32 w = blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (w < (u32)a.nchunk_warps) {
         block_chunk<SMALL>(a.m, w, lane);
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kBlockThreads, 3) k_block_step(const __grid_co
     __shared__ u32 red[4 * kBlockThreads];
     const int tid = threadIdx.x;
     if (blockIdx.x < a.spmm) {
-        const u32 w = (blockIdx.x * kBlockThreads + tid) >> 5;
+        const u32 w = blockIdx.x * (kBlockThreads / 32) + (tid >> 5);
         if (w < (u32)a.b.nchunk_warps) block_chunk<false, true>(a.b.m, w, tid & 31);
         else if (w < a.b.warp0[kBlockClasses]) block_class_rows<false, true>(a.b, w, tid & 31);
         return;
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_stage_many(const __grid
 
 __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_constant__ BlockMany P)
 {
-    const u32 w0 = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
+    const u32 w0 = blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5);
     if (w0 >= P.first[P.count]) return;
     const int lane = threadIdx.x & 31, j = block_find(P, w0);
     const BlockDev &D = *P.dev[j];
