@@ -299,7 +299,8 @@ class Matrix:
         words = x.shape[1] if x.dim() == 2 else 1
         out_rows = self.ncols if transpose else self.nrows
         if y is None:
-            y = torch.zeros((out_rows, words) if x.dim() == 2 else (out_rows,), dtype=torch.int64, device=dev)
+            make = torch.zeros if accumulate else torch.empty   # without accumulate every word is written
+            y = make((out_rows, words) if x.dim() == 2 else (out_rows,), dtype=torch.int64, device=dev)
         spmv_apply_gf2(self.handle, transpose, x, y, words, accumulate, stream)
         return y
 

@@ -30,11 +30,6 @@
 namespace ff {
 namespace {
 
-constexpr int kBlockThreads = 256;
-constexpr long long kBlockLong = 512;   // entries of a chunk; longer rows are split over warps
-constexpr int kBlockVecs = 32;          // vectors per pass
-constexpr int kBlockClasses = 7;        // by quads of entries: 0, 1, 2, 3-4, 5-8, 9-16, 17-128
-
 __device__ __forceinline__ int block_class(u32 quads)
 {
     return quads <= 2u ? (int)quads : min(kBlockClasses - 1, 33 - __clz(quads - 1u));
@@ -57,33 +52,10 @@ struct BlockDev {
     Mod M;
 };
 
-struct BlockPlan {
-    bool ok = false;
-    const BlockDev *dev = nullptr;
-    void *arena = nullptr;
-    long long n = 0, ncols = 0;
-    bool small = true;                 // m <= 2^16: u16 values and staged x
-    long long nlong = 0, nchunk = 0;   // rows split over warps, and their chunks
-    long long cls_row[kBlockClasses + 1] = {};  // rows of class c: [cls_row[c], cls_row[c + 1]) of row / ptr
-    const u32 *ptr = nullptr;          // [n - nlong + 1] offsets in quads, rows in class order
-    const u32 *row = nullptr;          // [n - nlong] their matrix rows
-    const uint4 *chunk = nullptr;      // (long row index, first quad, end, chunks of the row)
-    const u32 *lrow = nullptr;         // [nlong] matrix rows
-    const u32 *col = nullptr;
-    const void *val = nullptr;
-    uint4 *xs = nullptr;               // staged rows of X
-    u32 quad1 = 0;                     // the one-quad class: row r at quad quad1 + r (mod 2^32)
-    u64 *carry = nullptr;              // [nlong][kBlockVecs], zero between calls
-    u32 *count = nullptr;              // [nlong] chunks arrived, zero between calls
-};
-
 void free_block(ffspmv_handle *h)
 {
     for (BlockPlan *&b : h->block) {
-        if (b) {
-            if (b->arena) cudaFree(b->arena);
-            delete b;
-        }
+        free_block_plan(b);
         b = nullptr;
     }
 }
@@ -530,19 +502,6 @@ __global__ void __launch_bounds__(kBlockThreads, 3) k_block_step(const __grid_co
     }
 }
 
-// log2 of the groups per row of class i (heaviest first), 2^lgt lanes per row
-// of X.  A group's epilogue (sums joined, one reduction per component) costs
-// about as much as three quads, so rows share as few groups as keep the warp's
-// lanes busy: with four or more lanes per row of X fewer still.  300 007 x
-// 200 003, 22 per row, m = 2^31 - 1, 16 vectors: 79 us with 8 / 4 / 2 groups
-// for classes 1 to 3, 59 with 4 / 2 / 1, 53 with 2 / 1 / 1 (3 vectors: 39, 39,
-// 45).
-__host__ __device__ inline int block_lgg(int i, int lgt)
-{
-    const int lg = i == 0 ? 4 : lgt < 2 ? (i == 1 ? 2 : i == 2 ? 1 : 0) : i == 1 ? 1 : 0;
-    return lg < 5 - lgt ? lg : 5 - lgt;
-}
-
 // Many matrices in one launch, each with its modulus, vectors and packed X:
 // what a launch passes for one of them, and the first warp (or, for the
 // staging, the first CTA) of each.
@@ -649,17 +608,26 @@ struct BlockBuild {
     u32 *orow, *optr, *lrow, *ocol;
     uint4 *chunk;
     void *oval;
-    int small;
+    int small, odd;         // odd: the pattern of the odd values only, without values
 };
 
 __global__ void __launch_bounds__(kBlockThreads) k_block_lengths(const BlockBuild b, int transpose)
 {
     const long long nth = (long long)gridDim.x * kBlockThreads, t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
-    if (!transpose) {
+    if (!transpose && !b.odd) {
         for (long long i = t; i < b.nr; i += nth) b.len[i] = (u32)(b.ptr[i + 1] - b.ptr[i]);
+    } else if (!transpose) {
+        for (long long w = t >> 5; w < b.nr; w += nth >> 5) {   // a warp per row
+            const long long e = b.ptr[w + 1];
+            u32 c = 0;
+            for (long long k = b.ptr[w] + (threadIdx.x & 31); k < e; k += 32) c += b.val[k] & 1u;
+            c = __reduce_add_sync(0xffffffffu, c);
+            if ((threadIdx.x & 31) == 0) b.len[w] = c;
+        }
     } else {
         const long long nnz = b.ptr[b.nr];
-        for (long long k = t; k < nnz; k += nth) atomicAdd(b.len + b.col[k], 1u);
+        for (long long k = t; k < nnz; k += nth)
+            if (!b.odd || (b.val[k] & 1u)) atomicAdd(b.len + b.col[k], 1u);
     }
 }
 
@@ -718,9 +686,12 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild b
         const long long s = b.ptr[i], e = b.ptr[i + 1];
         for (long long k = s + lane; k < e; k += 32) {
             const u32 j = b.col[k], v = b.val[k];
-            const size_t to = transpose ? (size_t)b.start[j] * 4 + (atomicSub(b.len + j, 1u) - 1u)
-                                        : (size_t)b.start[i] * 4 + (size_t)(k - s);
+            if (b.odd && !(v & 1u)) continue;
+            const u32 r = transpose ? j : (u32)i;
+            const size_t to = (size_t)b.start[r] * 4 +
+                              (transpose || b.odd ? (size_t)(atomicSub(b.len + r, 1u) - 1u) : (size_t)(k - s));
             b.ocol[to] = transpose ? (u32)i : j;
+            if (b.odd) continue;
             if (b.small) reinterpret_cast<unsigned short *>(b.oval)[to] = (unsigned short)v;
             else reinterpret_cast<u32 *>(b.oval)[to] = v;
         }
@@ -729,11 +700,19 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild b
 
 // The block layout of A (nr x nc, values below m), or of A^T.
 ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long nc, const long long *ptr, const int *col,
-                          const u32 *val, u32 m, cudaStream_t st, void *&tmp)
+                          const u32 *val, u32 m, bool odd, cudaStream_t st, void *&tmp)
 {
     const long long nnz = ptr[nr], n = transpose ? nc : nr, ncols = transpose ? nr : nc;
-    // offsets in quads and lengths are 32-bit
-    if (nnz >= (1LL << 32) - 1 || nnz / 4 + n >= (1LL << 32) - 1 || n >= (1LL << 32) - 64) return FFSPMV_ERR_UNSUPPORTED;
+    // offsets in quads and lengths of rows are 32-bit; with values, 32-bit row numbers are rounded up to a warp's
+    constexpr long long kLim = (1LL << 32) - 1;
+    if (nnz / 4 + std::min(n, nnz) >= kLim || (!odd && (nnz >= kLim || n >= kLim - 63))) return FFSPMV_ERR_UNSUPPORTED;
+    if (nnz >= kLim) {
+        std::vector<long long> len((size_t)n, 0);
+        for (long long i = 0; i < nr; ++i)
+            for (long long k = ptr[i]; k < ptr[i + 1]; ++k) ++len[transpose ? (size_t)col[k] : (size_t)i];
+        for (long long l : len)
+            if (l >= kLim) return FFSPMV_ERR_UNSUPPORTED;
+    }
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     size_t o = 0;
     auto put = [&](size_t bytes) {
@@ -765,6 +744,7 @@ ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long 
     b.start = (u32 *)(t + t_start);
     b.cursor = (u64 *)(t + t_cur);
     b.small = m <= 65536u ? 1 : 0;
+    b.odd = odd ? 1 : 0;
     u64 cur[kCur] = {};
     FF_CUDA(cudaMemcpyAsync(t + t_ptr, ptr, (size_t)(nr + 1) * 8, cudaMemcpyHostToDevice, st));
     if (nnz) {
@@ -794,11 +774,11 @@ ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long 
         quads += here & 0xffffffffull;
         B.cls_row[i + 1] = (long long)rows;
     }
-    const int vb = B.small ? 2 : 4;
+    const int vb = odd ? 0 : B.small ? 2 : 4;
     o = 0;
     const size_t o_ptr = put((size_t)(rows + 1) * 4), o_row = put((size_t)rows * 4), o_chunk = put((size_t)B.nchunk * 16),
                  o_lrow = put((size_t)B.nlong * 4), o_col = put((size_t)quads * 16), o_val = put((size_t)quads * 4 * vb),
-                 o_carry = put((size_t)B.nlong * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
+                 o_carry = put((size_t)(odd ? 0 : B.nlong) * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
                  o_dev = put(sizeof(BlockDev)), o_xs = put((size_t)ncols * kBlockVecs * vb);
     if (cudaMalloc(&B.arena, o) != cudaSuccess) {
         cudaGetLastError();
@@ -835,7 +815,9 @@ ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long 
     FF_CUDA(cudaMemcpyAsync(b.cursor, cur, sizeof(cur), cudaMemcpyHostToDevice, st));
     FF_CUDA(cudaMemcpyAsync(b.optr + rows, &end, 4, cudaMemcpyHostToDevice, st));
     FF_CUDA(cudaMemcpyAsync(base + o_dev, &D, sizeof(D), cudaMemcpyHostToDevice, st));
-    FF_CUDA(cudaMemsetAsync(base + o_col, 0, o_dev - o_col, st));   // padding entries, sums and counts of long rows
+    // padding entries (value 0, or no column), sums and counts of long rows
+    FF_CUDA(cudaMemsetAsync(base + o_col, odd ? 0xff : 0, o_val - o_col, st));
+    FF_CUDA(cudaMemsetAsync(base + o_val, 0, o_dev - o_val, st));
     k_block_place<<<grid, kBlockThreads, 0, st>>>(b, 1);
     k_block_fill<<<grid, kBlockThreads, 0, st>>>(b, transpose ? 1 : 0);
     FF_CUDA(cudaGetLastError());
@@ -845,28 +827,44 @@ ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long 
 
 }  // namespace
 
-const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st)
+static bool capturing(cudaStream_t st)
 {
-    BlockPlan *&b = h->block[transpose ? 1 : 0];
-    if (b) return b->ok ? b : nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return nullptr;  // nothing can be allocated or copied now
-    }
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) return false;
+    cudaGetLastError();
+    return true;
+}
+
+ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, cudaStream_t st, BlockPlan **out)
+{
+    *out = nullptr;
+    if (capturing(st)) return FFSPMV_ERR_CUDA;  // nothing can be allocated or copied now
     BlockPlan *nb = new (std::nothrow) BlockPlan();
-    if (!nb) return nullptr;
+    if (!nb) return FFSPMV_ERR_OOM;
     void *tmp = nullptr;
     const ffspmv_status r = build_block(*nb, transpose, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(),
-                                        h->h_val.data(), h->m, st, tmp);
+                                        h->h_val.data(), h->m, odd, st, tmp);
     if (tmp) cudaFree(tmp);
     if (r != FFSPMV_OK && nb->arena) {
         cudaFree(nb->arena);
         nb->arena = nullptr;
     }
-    nb->ok = r == FFSPMV_OK;  // a layout that could not be made is not tried again
-    b = nb;
-    return nb->ok ? nb : nullptr;
+    nb->ok = r == FFSPMV_OK;
+    *out = nb;
+    return r;
+}
+
+void free_block_plan(BlockPlan *b)
+{
+    if (b && b->arena) cudaFree(b->arena);
+    delete b;
+}
+
+const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st)
+{
+    BlockPlan *&b = h->block[transpose ? 1 : 0];
+    if (!b) make_block(h, transpose, false, st, &b);   // a layout that could not be made is not tried again
+    return b && b->ok ? b : nullptr;
 }
 
 // Launches of one block of nvec vectors: a staging pass and the product per

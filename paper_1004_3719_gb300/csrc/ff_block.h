@@ -5,7 +5,53 @@
 
 namespace ff {
 
-struct BlockPlan;
+constexpr int kBlockThreads = 256;
+constexpr long long kBlockLong = 512;   // entries of a chunk; longer rows are split over warps
+constexpr int kBlockVecs = 32;          // vectors per pass
+constexpr int kBlockClasses = 7;        // by quads of entries: 0, 1, 2, 3-4, 5-8, 9-16, 17-128
+
+// log2 of the groups per row of class i (heaviest first), 2^lgt lanes per row
+// of X.  A group's epilogue (sums joined, one reduction per component) costs
+// about as much as three quads, so rows share as few groups as keep the warp's
+// lanes busy: with four or more lanes per row of X fewer still.  300 007 x
+// 200 003, 22 per row, m = 2^31 - 1, 16 vectors: 79 us with 8 / 4 / 2 groups
+// for classes 1 to 3, 59 with 4 / 2 / 1, 53 with 2 / 1 / 1 (3 vectors: 39, 39,
+// 45).
+__host__ __device__ inline int block_lgg(int i, int lgt)
+{
+    const int lg = i == 0 ? 4 : lgt < 2 ? (i == 1 ? 2 : i == 2 ? 1 : 0) : i == 1 ? 1 : 0;
+    return lg < 5 - lgt ? lg : 5 - lgt;
+}
+
+struct BlockDev;   // what a launch over many matrices reads of each (block.cu)
+
+struct BlockPlan {
+    bool ok = false;
+    const BlockDev *dev = nullptr;
+    void *arena = nullptr;
+    long long n = 0, ncols = 0;
+    bool small = true;                 // m <= 2^16: u16 values and staged x
+    long long nlong = 0, nchunk = 0;   // rows split over warps, and their chunks
+    long long cls_row[kBlockClasses + 1] = {};  // rows of class c: [cls_row[c], cls_row[c + 1]) of row / ptr
+    const u32 *ptr = nullptr;          // [n - nlong + 1] offsets in quads, rows in class order
+    const u32 *row = nullptr;          // [n - nlong] their matrix rows
+    const uint4 *chunk = nullptr;      // (long row index, first quad, end, chunks of the row)
+    const u32 *lrow = nullptr;         // [nlong] matrix rows
+    const u32 *col = nullptr;
+    const void *val = nullptr;
+    uint4 *xs = nullptr;               // staged rows of X
+    u32 quad1 = 0;                     // the one-quad class: row r at quad quad1 + r (mod 2^32)
+    u64 *carry = nullptr;              // [nlong][kBlockVecs], zero between calls
+    u32 *count = nullptr;              // [nlong] chunks arrived, zero between calls
+};
+
+// A block layout of A or A^T, made on the device (synchronous); `odd`: of the
+// pattern of the odd values, padded with columns 2^32 - 1, without values and
+// without sums of long rows.  On
+// an error other than a stream under capture or no host memory *out is a plan
+// with ok = false.
+ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, cudaStream_t st, BlockPlan **out);
+void free_block_plan(BlockPlan *b);
 
 // The block layout of A (or A^T), built on first use from the handle's host
 // copy of the matrix (synchronous, one allocation); null while `st` is being

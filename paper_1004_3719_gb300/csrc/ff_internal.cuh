@@ -284,7 +284,6 @@ struct Plan {
 }  // namespace ff
 
 namespace ff {
-struct Gf2Pattern;
 struct BlockPlan;
 }
 
@@ -312,7 +311,7 @@ struct ffspmv_handle {
     void *seq_state = nullptr;
     int *d_status = nullptr;   // device status word (timeouts)
     // patterns of the odd entries of A and A^T for the GF(2) products
-    ff::Gf2Pattern *gf2[2] = {nullptr, nullptr};
+    ff::BlockPlan *gf2[2] = {nullptr, nullptr};
     // x-panel plans of A and A^T for 2 and 4 vectors per pass, built on the
     // first block that uses them when the plan is the x-panel layout
     ff::Plan *multi[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};

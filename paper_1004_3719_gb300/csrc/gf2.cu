@@ -5,216 +5,164 @@
 // into words is the binary case the paper's closing remarks point to.
 //
 // Only the pattern of the odd entries is kept (built on the first call, for A
-// or A^T).  Rows of at most kGf2Long entries: G lanes per row (G from the mean
-// row length), each lane over every G-th entry, then an exclusive or across
-// the group.  Longer rows are cut into chunks of kGf2Chunk entries, one warp
-// each, whose results meet in y by atomic exclusive or (the row kernel first
-// clears those rows of y, unless accumulating).  A lane gathers W words of
-// each x row it names (the host walks the words four at a time).
+// or A^T), in the block layout (block.cu): rows in length classes, columns in
+// quads, so that a lane loads four columns at once and has four gathers in
+// flight while the next quad is on its way.  A lane gathers one 64-bit word of
+// a row of X, or two where the rows are 16-byte aligned; T lanes take a row's
+// words and G groups of them share a row of A.  The chunks of a row above 512
+// entries meet in Y by atomic exclusive or: a launch before clears those rows
+// (unless accumulating), and only the chunks' last step waits for it.  Nothing
+// of the handle is written, so calls on one handle may overlap.
+//
+// The gathers bound it: one random L2 sector per entry, 63 us for 15.8M at 250 G
+// sectors/s.  1M power-law pattern, 64 / 256 vectors: 91 / 211 us with a lane
+// group per short row, a second launch for the long rows and 8-byte offsets;
+// 66 / 87 us here (16 words: 1359 -> 302).
 #include <algorithm>
-#include <cstring>
 
+#include "ff_block.h"
 #include "ff_internal.cuh"
-#include "ff_plan.h"
-#include "ff_select.h"
 
 namespace ff {
 
-constexpr int kGf2Threads = 256;
-constexpr long long kGf2Long = 32;
-constexpr long long kGf2Chunk = 1024;
-
-struct Gf2Pattern {
-    void *arena = nullptr;
-    const long long *ptr = nullptr;  // [n + 1]
-    const u32 *col = nullptr;        // odd entries only
-    const long long *chunks = nullptr;  // [nlong][3]: row, first entry, end of a long-row chunk
-    long long n = 0, ncols = 0, nnz = 0, nlong = 0;  // nlong: chunks
-    int G = 1;
-};
-
 void free_gf2(ffspmv_handle *h)
 {
-    for (int t = 0; t < 2; ++t) {
-        if (h->gf2[t]) {
-            if (h->gf2[t]->arena) cudaFree(h->gf2[t]->arena);
-            delete h->gf2[t];
-            h->gf2[t] = nullptr;
-        }
+    for (BlockPlan *&g : h->gf2) {
+        free_block_plan(g);
+        g = nullptr;
     }
 }
 
 namespace {
 
-template <int W>
-__global__ void __launch_bounds__(kGf2Threads)
-k_gf2_rows(const long long *__restrict__ ptr, const u32 *__restrict__ col, long long n, int G,
-           const u64 *__restrict__ X, u64 *__restrict__ Y, int w, int w0, int accumulate)
+constexpr int kGf2Lanes = 8;   // lanes per row of X in one pass
+
+struct Gf2Args {
+    const u32 *ptr, *row, *col, *lrow;
+    const uint4 *chunk;
+    const u64 *X;
+    u64 *Y;
+    int w, pieces, lgt, accumulate;   // words per row of X and Y; pieces of this pass; log2 of the lanes that take them
+    u32 nchunk;
+    u32 quad1;
+    u32 warp0[kBlockClasses + 1], row0[kBlockClasses + 1];
+    int lgg[kBlockClasses];
+};
+
+// One piece of a row of X: E 64-bit words.
+template <int E>
+struct Gf2Piece;
+template <>
+struct Gf2Piece<1> {
+    u64 a;
+    __device__ __forceinline__ void zero() { a = 0; }
+    __device__ __forceinline__ void load(const u64 *p) { a = __ldg(p); }
+    __device__ __forceinline__ void add(const Gf2Piece &o) { a ^= o.a; }
+    __device__ __forceinline__ void shfl(int off) { a ^= __shfl_xor_sync(0xffffffffu, a, off); }
+    __device__ __forceinline__ u64 get(int) const { return a; }
+};
+template <>
+struct Gf2Piece<2> {
+    u64 a, b;
+    __device__ __forceinline__ void zero() { a = b = 0; }
+    __device__ __forceinline__ void load(const u64 *p)
+    {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(p));
+        a = v.x;
+        b = v.y;
+    }
+    __device__ __forceinline__ void add(const Gf2Piece &o)
+    {
+        a ^= o.a;
+        b ^= o.b;
+    }
+    __device__ __forceinline__ void shfl(int off)
+    {
+        a ^= __shfl_xor_sync(0xffffffffu, a, off);
+        b ^= __shfl_xor_sync(0xffffffffu, b, off);
+    }
+    __device__ __forceinline__ u64 get(int i) const { return i ? b : a; }
+};
+
+// exclusive or of the pieces that quads k, k + step, ... below end name
+template <int E>
+__device__ __forceinline__ void gf2_quads(Gf2Piece<E> &acc, const Gf2Args &a, u32 k, u32 end, u32 step, const u64 *xb, bool on)
 {
-    const int lane = threadIdx.x & (G - 1);
-    const int grp = (threadIdx.x & 31) / G, gpw = 32 / G;
-    const long long wid = ((long long)blockIdx.x * kGf2Threads + threadIdx.x) >> 5;
-    const long long nw = (long long)gridDim.x * kGf2Threads / 32;
-    // warp-uniform loop: every lane takes part in the shuffles
-    for (long long base = wid * gpw; base < n; base += nw * gpw) {
-        const long long row = base + grp;
-        u64 a[W];
+    constexpr u32 kNone = 0xffffffffu;
+    uint4 j = make_uint4(kNone, kNone, kNone, kNone);
+    if (k < end) j = __ldcs(reinterpret_cast<const uint4 *>(a.col) + k);
+    while (k < end) {
+        Gf2Piece<E> x[4];
+        const u32 c[4] = {j.x, j.y, j.z, j.w};
 #pragma unroll
-        for (int v = 0; v < W; ++v) a[v] = 0;
-        bool mine = false;
-        if (row < n) {
-            const long long s = __ldg(ptr + row), e = __ldg(ptr + row + 1);
-            mine = e - s <= kGf2Long;  // longer rows: the warp kernel
-            if (mine) {
-                for (long long k = s + lane; k < e; k += 4LL * G) {
-                    u32 c[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) c[u] = k + u * G < e ? __ldg(col + k + u * G) : 0xffffffffu;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (c[u] != 0xffffffffu)
-#pragma unroll
-                            for (int v = 0; v < W; ++v) a[v] ^= __ldg(X + (size_t)c[u] * w + w0 + v);
-                }
-            }
+        for (int u = 0; u < 4; ++u) {
+            x[u].zero();
+            if (on && c[u] != kNone) x[u].load(xb + (u64)c[u] * (u32)a.w);
         }
-        for (int off = G >> 1; off > 0; off >>= 1)
-#pragma unroll
-            for (int v = 0; v < W; ++v) a[v] ^= __shfl_xor_sync(0xffffffffu, a[v], off);
-        if (row < n && lane == 0) {
-#pragma unroll
-            for (int v = 0; v < W; ++v) {
-                u64 *yp = Y + (size_t)row * w + w0 + v;
-                if (mine) *yp = accumulate ? (*yp ^ a[v]) : a[v];
-                else if (!accumulate) *yp = 0;  // the chunks of a long row xor into it
-            }
-        }
+        k += step;
+        if (k < end) j = __ldcs(reinterpret_cast<const uint4 *>(a.col) + k);
+        x[0].add(x[1]);
+        x[2].add(x[3]);
+        x[0].add(x[2]);
+        acc.add(x[0]);
     }
 }
 
-template <int W>
-__global__ void __launch_bounds__(kGf2Threads)
-k_gf2_long(const u32 *__restrict__ col, const long long *__restrict__ chunks, long long nchunks,
-           const u64 *__restrict__ X, u64 *__restrict__ Y, int w, int w0)
+// The rows of Y that chunks add to.
+__global__ void __launch_bounds__(kBlockThreads) k_gf2_clear(const u32 *__restrict__ lrow, u32 nlong, int w, u64 *Y)
 {
-    const int lane = threadIdx.x & 31;
-    const long long wid = ((long long)blockIdx.x * kGf2Threads + threadIdx.x) >> 5;
-    const long long nw = (long long)gridDim.x * kGf2Threads / 32;
-    for (long long r = wid; r < nchunks; r += nw) {  // warp-uniform
-        const long long row = __ldg(chunks + 3 * r), s = __ldg(chunks + 3 * r + 1), e = __ldg(chunks + 3 * r + 2);
-        u64 a[W];
-#pragma unroll
-        for (int v = 0; v < W; ++v) a[v] = 0;
-        for (long long k = s + lane; k < e; k += 128) {
-            u32 c[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) c[u] = k + 32 * u < e ? __ldg(col + k + 32 * u) : 0xffffffffu;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c[u] != 0xffffffffu)
-#pragma unroll
-                    for (int v = 0; v < W; ++v) a[v] ^= __ldg(X + (size_t)c[u] * w + w0 + v);
-        }
-        for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-            for (int v = 0; v < W; ++v) a[v] ^= __shfl_xor_sync(0xffffffffu, a[v], off);
-        if (lane == 0)
-#pragma unroll
-            for (int v = 0; v < W; ++v) atomicXor(reinterpret_cast<unsigned long long *>(Y + (size_t)row * w + w0 + v),
-                                                  (unsigned long long)a[v]);
-    }
+    asm volatile("griddepcontrol.launch_dependents;");
+    const u64 n = (u64)nlong * (u32)w, step = (u64)gridDim.x * kBlockThreads;
+    for (u64 t = (u64)blockIdx.x * kBlockThreads + threadIdx.x; t < n; t += step)
+        Y[(size_t)__ldg(lrow + t / (u32)w) * w + t % (u32)w] = 0;
 }
 
-// The pattern of the odd entries of A (or of A^T) from the handle's host CSR.
-ffspmv_status build_gf2(ffspmv_handle *h, int transpose, Gf2Pattern *&out)
+// One warp per chunk of a long row, or per 32 / (T G) rows of a class.
+template <int E>
+__global__ void __launch_bounds__(kBlockThreads) k_gf2(const __grid_constant__ Gf2Args a)
 {
-    const long long nr = h->A.nrows, nc = h->A.ncols;
-    std::vector<long long> ptr(1, 0);
-    std::vector<int> col;
-    std::vector<u32> one;
-    ptr.reserve(nr + 1);
-    for (long long i = 0; i < nr; ++i) {
-        for (long long k = h->h_ptr[i]; k < h->h_ptr[i + 1]; ++k)
-            if (h->h_val[k] & 1u) col.push_back(h->h_col[k]);
-        ptr.push_back((long long)col.size());
-    }
-    long long n = nr, ncols = nc;
-    if (transpose) {
-        one.assign(col.size(), 1u);
-        std::vector<long long> tptr;
-        std::vector<int> tcol;
-        std::vector<u32> tval;
-        transpose_csr(nr, nc, ptr.data(), col.data(), one.data(), tptr, tcol, tval);
-        ptr.swap(tptr);
-        col.swap(tcol);
-        n = nc;
-        ncols = nr;
-    }
-    const long long nnz = (long long)col.size();
-    if (ncols >= (1LL << 32) - 1) return FFSPMV_ERR_UNSUPPORTED;
-    std::vector<long long> chunks;
-    long long short_entries = 0, short_rows = 0;
-    for (long long i = 0; i < n; ++i) {
-        const long long L = ptr[i + 1] - ptr[i];
-        if (L > kGf2Long) {
-            for (long long k = ptr[i]; k < ptr[i + 1]; k += kGf2Chunk) {
-                chunks.push_back(i);
-                chunks.push_back(k);
-                chunks.push_back(std::min(ptr[i + 1], k + kGf2Chunk));
-            }
-        } else {
-            short_entries += L;
-            ++short_rows;
+    const u32 w = blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, T = 1 << a.lgt, c = lane & (T - 1);
+    const bool on = c < a.pieces;
+    const u64 *xb = a.X + E * c;
+    Gf2Piece<E> acc;
+    acc.zero();
+    if (w < a.nchunk) {
+        const uint4 ch = __ldg(a.chunk + w);
+        gf2_quads<E>(acc, a, ch.y + (u32)(lane >> a.lgt), ch.z, 32u >> a.lgt, xb, on);
+        for (int off = T; off < 32; off <<= 1) acc.shfl(off);
+        asm volatile("griddepcontrol.wait;" ::: "memory");   // the row is cleared
+        if (lane < T && on) {
+            u64 *yp = a.Y + (size_t)__ldg(a.lrow + ch.x) * a.w + E * c;
+#pragma unroll
+            for (int i = 0; i < E; ++i)
+                atomicXor(reinterpret_cast<unsigned long long *>(yp + i), (unsigned long long)acc.get(i));
         }
+        return;
     }
-    Gf2Pattern *g = new Gf2Pattern();
-    g->n = n;
-    g->ncols = ncols;
-    g->nnz = nnz;
-    g->nlong = (long long)chunks.size() / 3;
-    // lanes per short row: about four entries each
-    const double mean = short_rows ? (double)short_entries / (double)short_rows : 1.0;
-    while (g->G < 32 && 4.0 * g->G < mean) g->G <<= 1;
-    const size_t b_ptr = (size_t)(n + 1) * 8, b_col = (size_t)std::max<long long>(nnz, 1) * 4;
-    const size_t o_col = (b_ptr + 255) / 256 * 256, o_long = o_col + (b_col + 255) / 256 * 256;
-    const size_t bytes = o_long + (size_t)std::max<long long>(g->nlong, 1) * 24;
-    if (cudaMalloc(&g->arena, bytes) != cudaSuccess) {
-        delete g;
-        return FFSPMV_ERR_OOM;
+    int b = 0;
+#pragma unroll
+    for (int i = 1; i < kBlockClasses; ++i)
+        if (w >= a.warp0[i]) b = i;
+    if (w >= a.warp0[kBlockClasses]) return;
+    const int lgg = a.lgg[b], lgr = a.lgt + lgg;
+    const u64 r64 = a.row0[b] + ((u64)(w - a.warp0[b]) << (5 - lgr)) + (u64)(lane >> lgr);
+    const bool ok = r64 < a.row0[b + 1];
+    const u32 r = (u32)r64;
+    u32 s = 0, e = 0, row = 0;
+    if (ok) {
+        const bool one = b == kBlockClasses - 2;
+        s = one ? a.quad1 + r : __ldg(a.ptr + r);
+        e = one ? s + 1u : __ldg(a.ptr + r + 1);
+        row = __ldg(a.row + r);
     }
-    char *base = (char *)g->arena;
-    cudaMemcpy(base, ptr.data(), b_ptr, cudaMemcpyHostToDevice);
-    if (nnz) cudaMemcpy(base + o_col, col.data(), (size_t)nnz * 4, cudaMemcpyHostToDevice);
-    if (g->nlong) cudaMemcpy(base + o_long, chunks.data(), (size_t)g->nlong * 24, cudaMemcpyHostToDevice);
-    if (cudaGetLastError() != cudaSuccess) {
-        cudaFree(g->arena);
-        delete g;
-        return FFSPMV_ERR_CUDA;
+    gf2_quads<E>(acc, a, s + (u32)((lane >> a.lgt) & ((1 << lgg) - 1)), e, 1u << lgg, xb, on);
+    for (int off = T; off < 1 << lgr; off <<= 1) acc.shfl(off);
+    if (ok && on && (lane & ((1 << lgr) - 1)) < T) {
+        u64 *yp = a.Y + (size_t)row * a.w + E * c;
+#pragma unroll
+        for (int i = 0; i < E; ++i) yp[i] = a.accumulate ? yp[i] ^ acc.get(i) : acc.get(i);
     }
-    g->ptr = (const long long *)base;
-    g->col = (const u32 *)(base + o_col);
-    g->chunks = (const long long *)(base + o_long);
-    out = g;
-    return FFSPMV_OK;
-}
-
-template <int W>
-ffspmv_status launch_gf2(const Gf2Pattern &g, const u64 *X, u64 *Y, int w, int w0, int acc, int nsm,
-                         cudaStream_t st)
-{
-    if (g.n > 0) {
-        const long long want = (g.n * g.G + kGf2Threads - 1) / kGf2Threads;
-        const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>(want, 16LL * nsm));
-        k_gf2_rows<W><<<blocks, kGf2Threads, 0, st>>>(g.ptr, g.col, g.n, g.G, X, Y, w, w0, acc);
-        FF_CUDA(cudaGetLastError());
-    }
-    if (g.nlong > 0) {
-        const long long want = (g.nlong * 32 + kGf2Threads - 1) / kGf2Threads;
-        const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>(want, 16LL * nsm));
-        k_gf2_long<W><<<blocks, kGf2Threads, 0, st>>>(g.col, g.chunks, g.nlong, X, Y, w, w0);
-        FF_CUDA(cudaGetLastError());
-    }
-    return FFSPMV_OK;
 }
 
 }  // namespace
@@ -230,28 +178,65 @@ extern "C" ffspmv_status spmv_apply_gf2(ffspmv_t h, int32_t transpose, const uin
     const long long in_rows = transpose ? h->A.nrows : h->A.ncols;
     const long long out_rows = transpose ? h->A.ncols : h->A.nrows;
     if ((in_rows > 0 && !d_X) || (out_rows > 0 && !d_Y)) return FFSPMV_ERR_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
     if (!h->gf2[transpose]) {
-        Gf2Pattern *g = nullptr;
-        ffspmv_status r = build_gf2(h, transpose, g);
-        if (r != FFSPMV_OK) return r;
+        BlockPlan *g = nullptr;
+        const ffspmv_status r = make_block(h, transpose != 0, true, nullptr, &g);
+        if (r != FFSPMV_OK) {
+            free_block_plan(g);
+            return r;
+        }
         h->gf2[transpose] = g;
     }
-    const Gf2Pattern &g = *h->gf2[transpose];
+    const BlockPlan &B = *h->gf2[transpose];
     if (out_rows == 0) return FFSPMV_OK;
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    nsm = std::max(nsm, 1);
-    cudaStream_t st = (cudaStream_t)stream;
-    const u64 *X = (const u64 *)d_X;
-    u64 *Y = (u64 *)d_Y;
-    for (int w0 = 0; w0 < words; w0 += 4) {
-        const int W = std::min(4, words - w0);
-        ffspmv_status r = W == 4   ? launch_gf2<4>(g, X, Y, words, w0, accumulate ? 1 : 0, nsm, st)
-                          : W == 3 ? launch_gf2<3>(g, X, Y, words, w0, accumulate ? 1 : 0, nsm, st)
-                          : W == 2 ? launch_gf2<2>(g, X, Y, words, w0, accumulate ? 1 : 0, nsm, st)
-                                   : launch_gf2<1>(g, X, Y, words, w0, accumulate ? 1 : 0, nsm, st);
-        if (r != FFSPMV_OK) return r;
+    const bool clear = !accumulate && B.nchunk > 0;
+    if (clear) {
+        const long long n = B.nlong * words;
+        k_gf2_clear<<<(unsigned)std::min<long long>((n + kBlockThreads - 1) / kBlockThreads, 4096), kBlockThreads, 0, st>>>(
+            B.lrow, (u32)B.nlong, words, (u64 *)d_Y);
+        FF_CUDA(cudaGetLastError());
+    }
+    // two words per lane where every row of X starts on 16 bytes
+    const int E = words % 2 == 0 && ((uintptr_t)d_X & 15u) == 0 ? 2 : 1;
+    for (int w0 = 0; w0 < words; w0 += E * kGf2Lanes) {
+        Gf2Args a;
+        memset(&a, 0, sizeof(a));
+        a.ptr = B.ptr;
+        a.row = B.row;
+        a.col = B.col;
+        a.lrow = B.lrow;
+        a.chunk = B.chunk;
+        a.quad1 = B.quad1;
+        a.X = (const u64 *)d_X + w0;
+        a.Y = (u64 *)d_Y + w0;
+        a.w = words;
+        a.pieces = std::min(kGf2Lanes, (words - w0) / E);
+        while ((1 << a.lgt) < a.pieces) ++a.lgt;
+        a.accumulate = accumulate ? 1 : 0;
+        a.nchunk = (u32)B.nchunk;
+        long long warps = B.nchunk;
+        for (int c = 0; c < kBlockClasses; ++c) {
+            a.lgg[c] = block_lgg(c, a.lgt);
+            a.row0[c] = (u32)B.cls_row[c];
+            a.warp0[c] = (u32)warps;
+            const int rpw = 32 >> (a.lgt + a.lgg[c]);
+            warps += (B.cls_row[c + 1] - B.cls_row[c] + rpw - 1) / rpw;
+        }
+        a.row0[kBlockClasses] = (u32)B.cls_row[kBlockClasses];
+        a.warp0[kBlockClasses] = (u32)warps;
+        if (warps >= (1LL << 32) - 1) return FFSPMV_ERR_UNSUPPORTED;
+        // the first pass starts while the rows are cleared
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((warps * 32 + kBlockThreads - 1) / kBlockThreads));
+        cfg.blockDim = dim3(kBlockThreads);
+        cfg.stream = st;
+        cfg.attrs = &attr;
+        cfg.numAttrs = clear && w0 == 0 ? 1 : 0;
+        FF_CUDA(cudaLaunchKernelEx(&cfg, E == 2 ? k_gf2<2> : k_gf2<1>, a));
     }
     return FFSPMV_OK;
 }
