@@ -10,7 +10,8 @@ namespace ff {
 // its basis, the bound e on its degree, the largest delta and the least input
 // shift.
 struct SbSlot {
-    int e, smin, dmax, pad;
+    int e, smin, dmax;
+    int bad;             // a bounded wait of a leaf below ran out
     int delta[32];
 };
 
@@ -44,6 +45,7 @@ __device__ __forceinline__ void pm_node(const PmNode &n, int t)
         n.out->e = max(0, e);
         n.out->smin = n.s1->smin;
         n.out->dmax = n.s2->dmax;
+        n.out->bad = n.s1->bad | n.s2->bad;
     }
 }
 

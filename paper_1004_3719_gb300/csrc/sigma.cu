@@ -4,14 +4,14 @@
 // work is polynomial-matrix products on the GPU (polymat.cu, Sec. 3.2.1's
 // evaluation / pointwise / interpolation scheme, and products by definition
 // for short operands), and M-Basis, the iterative algorithm Sec. 3.2.2
-// recommends at small orders, as one CTA per leaf.
+// recommends at small orders, as one cluster of CTAs per leaf.
 //
 // The recursion.  An order-d basis is P2 P1 with P1 of order d1 = ceil(d/2)
 // and P2 of the residual, the coefficients d1..d-1 of P1 F, with P1's degrees
 // as its shift.  M-Basis itself is the recursion's limit (order k's operations
 // depend only on that order's residual and the current degrees), so the
 // result is the same matrix wherever the leaves are cut; the leaves here take
-// at most kSbLeaf orders.  Up to order kSbAsync a node needs nothing from the
+// at most sb_leaf_max orders.  Up to order kSbAsync a node needs nothing from the
 // host: degrees and degree bounds stay in device slots, the products are
 // direct (one launch each) and the launches queue up.  Above it the host
 // reads each half's degree bound to size the transforms, of exactly the
@@ -26,30 +26,29 @@
 // divides out its multipliers, which makes the result the plain algorithm's.
 // It is the serial part: four warps of the leaf's first CTA do nothing else,
 // a lane per row in pivot order, a panel of a quarter of the columns each in
-// registers.  Panel by panel, its owner shares the panel's columns, and every
-// warp eliminates them (the same few operations, redundantly) while it applies
-// each step to its own columns, so that a step needs no exchange between
-// warps.  Nearly always the pivots are the rows in order, so a panel first
-// takes them as known: a step is then a shuffle and a multiply-add long, with
-// no vote on the way; it is done again with votes if one of them turns out
-// zero.  A column's register turns from R_k's entry into the coefficient of
-// its pivot once its step is done, so what comes out is a matrix: every row
-// becomes c r plus a combination of the *original* pivot rows.  Eight other
-// warps apply it to R's later coefficients as independent multiply-adds, the
-// coefficient that the next elimination waits for first; two more CTAs of
-// the cluster, which get the matrix through distributed shared memory, apply
-// it to P.
+// registers.  Panel by panel, its owner shares the panel's columns; every warp
+// eliminates these first (the same few operations, redundantly: the chain of
+// dependent steps), then applies the steps to its own columns, so that no step
+// needs an exchange between warps.  Nearly always the pivots are the rows in
+// order, so a panel first takes them as known: a step is then a shuffle and a
+// multiply-add long, with no vote on the way; it is done again with votes if
+// one of them turns out zero.  The owner's columns turn into the coefficients
+// of the pivots, so what comes out is a matrix: every row becomes c r plus a
+// combination of the *original* pivot rows.  Eight warps of the first CTA apply
+// it to what R_{k+1} needs, and six other CTAs of the cluster, a few columns of
+// R and of P each, to all the rest: R's coefficient k + 2 first, which they send
+// back for the order after.  So the first CTA does nothing but eliminate, and
+// nobody waits for a CTA that falls behind for some orders.
 //
-// What bounds it: 64-bit multiply-adds, at 32 per clock and SM, and the chain
-// of n dependent steps.  One order of R and P (about 7 500 clocks of one SM
-// at order 16, 32 x 16) is therefore spread over three SMs and mostly off the
-// elimination's path (about 180 clocks per step).  Measured, order 12 502,
-// 32 x 16, p = 65521: one cluster of eight CTAs per leaf of order 24-25 that
-// exchanged every row operation took about 20 us per order and 293 ms for
-// the whole basis (with the transforms of polymat.cu); one warp eliminating
-// beside sixteen that apply, on one SM, 10 us; four warps and three CTAs, a
-// vote and an exchange per column, 5.7 us (98 ms); as it is here 4.4 us and
-// 81 ms.
+// What bounds it: the elimination's chain (about 5 000 clocks per order of a 32
+// x 16 leaf: 120 per dependent step, 100 per step to apply, 180 per exchange of
+// a panel, 900 for R_{k+1}); the other CTAs take 4 000.  Measured, order
+// 12 502, 32 x 16, p = 65521: one cluster of eight CTAs per leaf of order 24-25
+// that exchanged every row operation took about 20 us per order and 293 ms for
+// the whole basis (with the transforms of polymat.cu); four eliminating warps
+// beside eight that apply to R, two CTAs for P, leaves of at most 16 orders, 4.3
+// us and 81 ms; R in CTAs of its own 3.5 us and 64 ms; columns of R and P mixed,
+// panels before the rest, as it is here, 3.0 us and 58 ms.
 #include <algorithm>
 #include <climits>
 #include <cstddef>
@@ -66,14 +65,16 @@ namespace {
 
 constexpr int kSbMaxM = 32;                 // rows of F and of P (the polynomial-matrix product's limit)
 constexpr int kSbMaxBase = 32;              // largest leaf order a caller may name
-constexpr int kSbLeaf = 16;                 // largest order of one M-Basis launch
 constexpr long long kSbAsync = 200;         // largest order whose nodes run without the host
-constexpr int kSbUpd = 16;                  // warps that apply the operations
 constexpr int kSbElim = 4;                  // warps that eliminate (first CTA)
-constexpr int kSbRes = 8;                   // of kSbUpd, in the first CTA: two per scheduler, which each leave it to its eliminating warp most of the time
-constexpr int kSbFirst = 32 * (kSbRes + kSbElim);   // threads that work in the first CTA
-constexpr int kSbThreads = 32 * (kSbUpd + kSbElim);
-constexpr int kSbCtas = 3;                  // the first CTA: elimination and R; the others: P
+constexpr int kSbRes = 8;                   // warps that bring R's next coefficient up to date (first CTA)
+constexpr int kSbWarps = 20;
+constexpr int kSbFirst = 32 * (kSbRes + kSbElim);
+constexpr int kSbThreads = 32 * kSbWarps;
+constexpr int kSbSend = 32 * (kSbWarps - kSbElim);
+constexpr int kSbApply = 6;                 // CTAs that apply the operations to P and to R's later coefficients
+constexpr int kSbCtas = 1 + kSbApply;
+constexpr int kSbSpin = 1 << 20;            // tries of a bounded wait
 constexpr size_t kSbSmemMax = 227 * 1024;
 constexpr size_t kSbAlign = 256;
 constexpr int kSbMaxShift = 1 << 24;
@@ -84,41 +85,60 @@ struct SbLeaf {
     const int *shift;    // m
     SbSlot *out;
     int m, n, d;
-    int rs, ps;          // words per row of R and of P in shared memory
+    int stride;          // words per row of R and of P in shared memory
     u32 pinv;            // p^-1 mod 2^32 (odd p)
+    u32 one;             // 2^32 mod p (p = 2: 1): x -> x under sb_red
     Mod M;
 };
 
-// Shared memory of a leaf's CTA: the operations of an order (two copies, by
-// order parity), the final row scales, the elimination's exchange; then in
-// the first CTA R twice (an order reads one copy and writes the other), in
-// the others P, row by row: word t n4 + c of a row of R is coefficient t,
-// column c (n4 = n rounded up to 4), the same for P with m4.  Row strides are
-// 4 mod 32 words: the rows a quarter warp reads 16 bytes from lie in distinct
-// banks.
+// Shared memory of a leaf's CTA: the operations of every order, so that none
+// is ever waited for to be read before the next is written; then rows, one of
+// the matrix every `stride` words (2 mod 32: the 8-byte pieces that half a warp
+// reads of 16 rows lie in distinct banks), a coefficient after the other.  First
+// CTA: slot t holds R's coefficient t with the operations of orders 0..t-2
+// applied, slots yb and yb + 1 (yb = d, or d + 1 if odd) R_k, all columns (n4 =
+// n rounded up to 4).  The
+// others: two copies of their columns of R, then of P (an order reads one and
+// writes the other).
+template <int N>
 struct SbOps {
-    u32 T[kSbMaxM][kSbMaxM];   // [column][row]: what row gets of the column's pivot row
+    u32 T[N][kSbMaxM];         // [column][row]: what row gets of the column's pivot row
     u32 c[kSbMaxM];            // [row]: what it keeps of itself
     u32 q[kSbMaxM];            // [column]: byte offset of the pivot row (any row, with T = 0, when there is none)
-    u32 qp[kSbMaxM];           // [column]: the same offset in P
-    int isp[kSbMaxM];          // [row]: 1 for the pivot rows
+    u32 isp[kSbMaxM];          // [row]: 1 for the pivot rows
 };
 typedef u32 SbPanel[2][8][32];   // a panel's columns, by lane of the eliminating warps; two copies
-constexpr size_t kSbOpsBytes = sizeof(SbOps);
-constexpr size_t kSbScaleOff = 2 * kSbOpsBytes;
+constexpr size_t kSbScaleOff = 0;                                       // the final row scales
 constexpr size_t kSbOrdOff = kSbScaleOff + kSbMaxM * 4;                 // [kSbElim][32]
 constexpr size_t kSbXOff = kSbOrdOff + kSbElim * 32 * 4;                // SbPanel
-constexpr size_t kSbRowOff = kSbXOff + sizeof(SbPanel);
-static_assert(kSbRowOff % 16 == 0, "16-byte rows");
+constexpr size_t kSbCOff = kSbXOff + sizeof(SbPanel);                   // what rows keep, between panels
+constexpr size_t kSbBarOff = kSbCOff + 32 * 4;                         // mbarriers: operations of order k, R's coefficient t
+constexpr size_t kSbOpsOff = kSbBarOff + 2 * kSbMaxBase * 8;
+static_assert(kSbOpsOff % 16 == 0 && sizeof(SbOps<8>) % 16 == 0, "16-byte pieces");
 
-int sb_stride(int words) { return (words + 27) / 32 * 32 + 4; }
-int sb_rstride(int n, long long d) { return sb_stride((int)d * ((n + 3) / 4 * 4)); }
-int sb_pstride(int m, long long d) { return sb_stride((int)(d + 1) * ((m + 3) / 4 * 4)); }
-
-size_t sb_leaf_smem(int m, int n, long long d)
+// The column pairs of R or of P (`cols` columns) that CTA h of kSbApply holds:
+// their number and the first.
+__host__ __device__ inline int sb_share(int cols, int h, int *first)
 {
-    return kSbRowOff + (size_t)std::max(2 * sb_rstride(n, d), sb_pstride(m, d)) * m * 4;
+    const int pairs = (cols + 3) / 4 * 2, q = pairs / kSbApply, r = pairs % kSbApply;
+    *first = h * q + (h < r ? h : r);
+    return q + (h < r ? 1 : 0);
 }
+
+int sb_stride(int m, int n, int d)
+{
+    int words = (d + 3) * ((n + 3) / 4 * 4), first;
+    for (int h = 0; h < kSbApply; ++h)
+        words = std::max(words, 4 * d * sb_share(n, h, &first) + 4 * (d + 1) * sb_share(m, kSbApply - 1 - h, &first));
+    return (words + 29) / 32 * 32 + 2;
+}
+
+size_t sb_leaf_smem(int m, int n, int d, size_t ops) { return kSbOpsOff + d * ops + (size_t)sb_stride(m, n, d) * m * 4; }
+
+// Largest order of one launch: what fits the shared memory, and beyond which
+// what the products beside it take is small (order 12 502, 32 x 16: 67 ms at 16,
+// 61 at 24, 58 at 32).
+int sb_leaf_max(int n) { return n <= 16 ? 32 : 24; }
 
 __device__ u32 sb_pow(u32 a, u32 e, const Mod &M)
 {
@@ -142,6 +162,15 @@ __device__ __forceinline__ u32 sb_red(u64 x, const SbLeaf &a)
     return min(r, r - p);
 }
 
+// The same without the last step, in [0, 2p), where the sums of four such
+// products stay below p 2^32 (LAZY: p <= 2^26).  Zero is 0 or p.
+template <bool LAZY, bool EVEN>
+__device__ __forceinline__ u32 sb_lazy(u64 x, const SbLeaf &a)
+{
+    if constexpr (LAZY) return (u32)(x >> 32) + a.M.m - __umulhi((u32)x * a.pinv, a.M.m);
+    return sb_red<EVEN>(x, a);
+}
+
 __device__ __forceinline__ u64 sb_fold(u64 x, u32 p)   // x < 2 p 2^32 -> x mod p 2^32
 {
     const u32 h = (u32)(x >> 32);
@@ -161,15 +190,46 @@ __device__ __forceinline__ void sb_st_remote(u32 addr, u32 v)
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ void sb_st_remote_v4(u32 addr, uint4 v)
+__device__ __forceinline__ u32 sb_shared(const void *ptr) { return (u32)__cvta_generic_to_shared(ptr); }
+
+// 8 or 16 bytes into another CTA, counted by the mbarrier `bar` there.
+__device__ __forceinline__ void sb_send(u32 addr, uint2 v, u32 bar)
 {
-    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v.x),
+                 "r"(v.y), "r"(bar)
                  : "memory");
 }
 
+__device__ __forceinline__ void sb_send(u32 addr, uint4 v, u32 bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+                 : "memory");
+}
+
+__device__ __forceinline__ void sb_bar_init(u32 bar, u32 bytes)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// Every mbarrier is used once.  False when the wait ran out.
+__device__ __forceinline__ bool sb_bar_wait(u32 bar)
+{
+    for (int i = 0; i < kSbSpin; ++i) {
+        u32 ok;
+        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n"
+                     "selp.u32 %0, 1, 0, q;\n}"
+                     : "=r"(ok)
+                     : "r"(bar)
+                     : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
 __device__ __forceinline__ void sb_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-// ... by a thread whose writes no other CTA reads
-__device__ __forceinline__ void sb_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void sb_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ u32 sb_rank()
@@ -179,27 +239,13 @@ __device__ __forceinline__ u32 sb_rank()
     return r;
 }
 
-// The operations applied to W (1 or 2) adjacent columns of one coefficient:
+// The operations applied to two adjacent columns of one coefficient:
 // lane r gets row r's new values.  `row0` points at the columns in row 0.
 // FOLD (p > 2^26): two products below p^2 are added to a sum below p 2^32,
 // then the sum is brought back below that; else all 33 fit.
-template <int W>
-struct SbVec;
-template <>
-struct SbVec<1> {
-    typedef u32 V;
-    static __device__ __forceinline__ u32 get(u32 v, int) { return v; }
-};
-template <>
-struct SbVec<2> {
-    typedef uint2 V;
-    static __device__ __forceinline__ u32 get(const uint2 &v, int i) { return i ? v.y : v.x; }
-};
-
-template <class V>
-__device__ __forceinline__ V sb_at(const u32 *row0, u32 bytes)
+__device__ __forceinline__ uint2 sb_at(const u32 *row0, u32 bytes)
 {
-    return *reinterpret_cast<const V *>(reinterpret_cast<const char *>(row0) + bytes);
+    return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(row0) + bytes);
 }
 
 // The offsets of the pivot rows: in registers while there is room for them.
@@ -226,70 +272,84 @@ struct SbPiv {
 
 // All N columns, without a branch on n: columns without a pivot bring T = 0
 // and the loads of all the pivot rows are in flight together.
-template <int N, int W, bool FOLD, bool EVEN>
-__device__ __forceinline__ void sb_apply(u32 (&out)[W], const SbLeaf &a, const u32 *row0, u32 own_off, const SbPiv<N> &Q, u32 c,
-                                         const u32 (&T)[N])
+template <int N, bool FOLD, bool EVEN>
+__device__ __forceinline__ uint2 sb_apply(const SbLeaf &a, const u32 *row0, u32 own_off, const SbPiv<N> &Q, u32 c, const u32 (&T)[N])
 {
-    typedef typename SbVec<W>::V V;
     const u32 p = a.M.m;
-    const V own = sb_at<V>(row0, own_off);
-    u64 x[W];
-#pragma unroll
-    for (int i = 0; i < W; ++i) x[i] = (u64)c * SbVec<W>::get(own, i);
+    const uint2 own = sb_at(row0, own_off);
+    u64 x = (u64)c * own.x, y = (u64)c * own.y;
 #pragma unroll
     for (int j = 0; j < N; j += 2) {
-        const V v0 = sb_at<V>(row0, Q.at(j)), v1 = sb_at<V>(row0, Q.at(j + 1));
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            x[i] += (u64)T[j] * SbVec<W>::get(v0, i);
-            x[i] += (u64)T[j + 1] * SbVec<W>::get(v1, i);
-            if (FOLD) x[i] = sb_fold(x[i], p);
+        const uint2 v0 = sb_at(row0, Q.at(j)), v1 = sb_at(row0, Q.at(j + 1));
+        x += (u64)T[j] * v0.x;
+        y += (u64)T[j] * v0.y;
+        x += (u64)T[j + 1] * v1.x;
+        y += (u64)T[j + 1] * v1.y;
+        if (FOLD) {
+            x = sb_fold(x, p);
+            y = sb_fold(y, p);
         }
     }
-#pragma unroll
-    for (int i = 0; i < W; ++i) out[i] = sb_red<EVEN>(x[i], a);
+    return make_uint2(sb_red<EVEN>(x, a), sb_red<EVEN>(y, a));
 }
 
-// N: 8, 16 or 32, at least n.  One cluster of kSbCtas CTAs.  The cluster
-// barrier has one phase per order: a thread of the first CTA arrives once
-// order k's operations are in every CTA and waits before the next order's are
-// written; one of the others arrives when it is done with order k - 1 and
-// waits for order k's operations.
+// N: 8, 16 or 32, at least n.  One cluster of kSbCtas CTAs: the first
+// eliminates, the others hold P and R's later coefficients, a few columns each.
+// All that moves between them is counted by mbarriers, each used once, in the
+// CTA that waits for it: the operations of an order (to all the others), and a
+// coefficient of R (to the first) one order before it is needed.
 template <int N, bool FOLD, bool EVEN>
 __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_constant__ SbLeaf a)
 {
     extern __shared__ __align__(16) unsigned char sb_sm[];
-    const int m = a.m, n = a.n, d = a.d;
+    const int m = a.m, n = a.n, d = a.d, S = a.stride;
     const u32 p = a.M.m;
-    const int n4 = (n + 3) & ~3, m4 = (m + 3) & ~3;
-    SbOps *ops = reinterpret_cast<SbOps *>(sb_sm);
+    const int n4 = (n + 3) & ~3, yb = d + (d & 1);
+    SbOps<N> *ops = reinterpret_cast<SbOps<N> *>(sb_sm + kSbOpsOff);
     u32 *scale = reinterpret_cast<u32 *>(sb_sm + kSbScaleOff);
-    u32 *rows = reinterpret_cast<u32 *>(sb_sm + kSbRowOff);
+    u32 *rows = reinterpret_cast<u32 *>(ops + d);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const u32 cta = sb_rank();
+    const u32 bar_ops = sb_shared(sb_sm + kSbBarOff), bar_R = bar_ops + 8 * kSbMaxBase;
+    // this CTA's columns: those of R, then those of P (where R's are more, fewer)
+    const int h = cta ? (int)cta - 1 : 0;
+    int r_first, p_first;
+    const int rp = sb_share(n, h, &r_first), pp = sb_share(m, kSbApply - 1 - h, &p_first);
+    u32 *P0 = rows + 4 * d * rp;   // (the two copies of R before it)
 
-    for (int i = tid; i < (int)(2 * kSbOpsBytes / 4); i += kSbThreads) reinterpret_cast<u32 *>(ops)[i] = 0u;
-    const int words = (cta == 0 ? 2 * a.rs : a.ps) * m;
-    for (int i = tid; i < words; i += kSbThreads) rows[i] = 0u;
-    __syncthreads();
+    if (tid < d) {
+        if (cta) sb_bar_init(bar_ops + 8 * tid, (u32)sizeof(SbOps<N>));
+        else sb_bar_init(bar_R + 8 * tid, (u32)(m * n4 * 4));
+    }
+    if (cta == 0 && tid == 0) a.out->bad = 0;
+    __syncwarp();
+    sb_arrive();
     if (cta == 0) {
-        for (int i = tid; i < d * m * n; i += kSbThreads) {
-            const int c = i % n, tr = i / n, t = tr / m, r = tr - t * m;
-            rows[r * a.rs + t * n4 + c] = __ldg(a.F + i);
+        // R's coefficients 0 (as R_0) and 1
+        for (int i = tid; i < min(d, 2) * m * n4; i += kSbThreads) {
+            const int c = i % n4, tr = i / n4, t = tr / m, r = tr - t * m;
+            rows[r * S + (t ? 1 : yb) * n4 + c] = c < n ? __ldg(a.F + ((size_t)t * m + r) * n + c) : 0u;
         }
-    } else if (tid < m) {
-        rows[tid * a.ps + tid] = 1u;   // P = identity
+    } else if (lane < m) {
+        for (int t = 1 + warp; t < d; t += kSbWarps)
+            for (int c = 0; c < 2 * rp; ++c)
+                rows[lane * S + t * 2 * rp + c] =
+                    2 * r_first + c < n ? __ldg(a.F + ((size_t)t * m + lane) * n + 2 * r_first + c) : 0u;
+        if (warp < 2 * pp) P0[lane * S + warp] = 2 * p_first + warp == lane ? 1u : 0u;   // P = identity
     }
     __syncthreads();
-    sb_arrive();
-    sb_wait();   // every CTA's operations are cleared before any remote store
+    sb_wait();   // every CTA's mbarriers are ready
+    bool ok = true;
 
-    if (cta == 0 && warp >= kSbUpd) {
+    if (cta == 0 && warp >= kSbWarps - kSbElim) {
         // the eliminating warps: each keeps row r's degree and scale in lane r
         constexpr int NC = N / kSbElim;   // columns per warp: ew NC ...
-        const int ew = warp - kSbUpd, col0 = ew * NC;
+        const int ew = warp - (kSbWarps - kSbElim), col0 = ew * NC;
         int *ord = reinterpret_cast<int *>(sb_sm + kSbOrdOff) + ew * 32;
         auto &X = *reinterpret_cast<SbPanel *>(sb_sm + kSbXOff);
+        u32 *xc = reinterpret_cast<u32 *>(sb_sm + kSbCOff);
+        constexpr bool LAZY = !FOLD && !EVEN;
+        const int last = (n - 1) / NC;    // the last panel; its warp ends with c and keeps the scales
         int dl = lane < m ? __ldg(a.shift + lane) : INT_MAX;
         int smin = dl;
         u32 tot = 1u;
@@ -312,120 +372,119 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
             // R_k, once the other warps have it
             if (k) asm volatile("bar.sync 1, %0;" ::"n"(kSbFirst) : "memory");
             u32 R[NC];
-            const u32 *src = rows + (k & 1) * (a.rs * m) + (live ? row : 0) * a.rs + k * n4 + col0;
+            const u32 *src = rows + (live ? row : 0) * S + (yb + (k & 1)) * n4 + col0;
 #pragma unroll
             for (int s = 0; s < NC; ++s) R[s] = live && col0 + s < n ? src[s] : 0u;
             u32 c = 1u;
             bool isp = false;
             int q_of = 31;   // lane j: lane of column j's pivot row (31: the first row, for columns without one)
+#pragma unroll 1
+            for (int w = 0; w <= last; ++w) {
+                const bool mine = ew == w;
+                u32 *xs = &X[w & 1][0][0];
+                if (mine) {
 #pragma unroll
-            for (int w = 0; w < kSbElim; ++w) {
-                if (w * NC < n) {
-                    const bool mine = ew == w;
-                    u32 *xs = &X[w & 1][0][0];
-                    if (mine) {
+                    for (int j = 0; j < NC; ++j) xs[j * 32 + lane] = R[j];
+                }
+                if (ew == w - 1) xc[lane] = c;
+                asm volatile("bar.sync 3, %0;" ::"n"(kSbElim * 32) : "memory");
+                u32 pc[NC];   // the panel's columns
 #pragma unroll
-                        for (int j = 0; j < NC; ++j) xs[j * 32 + lane] = R[j];
+                for (int j = 0; j < NC; ++j) pc[j] = xs[j * 32 + lane];
+                if (mine && w) c = xc[lane];
+                // Step j with pivot lane q[j]: row <- av row - x pivot row
+                // (times 2^-32) for some rows, the others as they are: row <-
+                // A row + G pivot row.  The panel's own columns first, in which
+                // the pivots are found; everything else follows.
+                u32 A[NC], G[NC];
+                int q[NC];
+                auto step = [&](int j, bool act, u32 av) {
+                    A[j] = act ? av : a.one;
+                    G[j] = act ? (LAZY ? 2 * p : p) - pc[j] : 0u;
+#pragma unroll
+                    for (int i = 0; i < NC; ++i)
+                        if (i > j)
+                            pc[i] = sb_lazy<LAZY, EVEN>((u64)G[j] * __shfl_sync(0xffffffffu, pc[i], q[j]) + (u64)A[j] * pc[i], a);
+                };
+                // first with the rows in order as pivots, lanes 31 - w NC,
+                // 30 - w NC ..: right if the panels before took the lanes
+                // above and no pivot is zero
+                const u32 above = w == 0 ? 0u : ~0u << (32 - NC * w);
+                bool good = w * NC + NC <= n && __ballot_sync(0xffffffffu, isp) == above;
+                if (good) {
+                    bool zero = false;
+#pragma unroll
+                    for (int j = 0; j < NC; ++j) {
+                        q[j] = 31 - w * NC - j;
+                        const u32 av = __shfl_sync(0xffffffffu, pc[j], q[j]);
+                        zero = zero || av == 0u || (LAZY && av == p);
+                        step(j, lane < q[j], av);
                     }
-                    asm volatile("bar.sync 3, %0;" ::"n"(kSbElim * 32) : "memory");
-                    u32 pc[NC];   // the panel's columns
-#pragma unroll
-                    for (int j = 0; j < NC; ++j) pc[j] = xs[j * 32 + lane];
-                    // step j with pivot lane q: row <- av row - x pivot row
-                    // (times 2^-32) for the rows in `act`; the others compute
-                    // it too and drop it.  The panel's next column first: the
-                    // next step waits for it
-                    auto step = [&](int j, int q, bool act, u32 av) {
-                        const u32 g = p - pc[j];
-#pragma unroll
-                        for (int i = 0; i < NC; ++i) {
-                            if (i > j) {
-                                const u32 o = __shfl_sync(0xffffffffu, pc[i], q);
-                                const u32 v = sb_red<EVEN>((u64)av * pc[i] + (u64)g * o, a);
-                                pc[i] = act ? v : pc[i];
-                            }
-                        }
-                        const u32 cq = __shfl_sync(0xffffffffu, c, q);
-#pragma unroll
-                        for (int i = 0; i < NC; ++i) {
-                            // the owner's column j is done: the coefficient of its pivot begins
-                            const bool here = mine && i == j;
-                            const u32 old = here ? 0u : R[i], o = __shfl_sync(0xffffffffu, R[i], q);
-                            const u32 v = sb_red<EVEN>((u64)av * old + (u64)g * (here ? cq : o), a);
-                            R[i] = act ? v : old;
-                        }
-                        const u32 cv = sb_red<EVEN>((u64)av * c, a);
-                        c = act ? cv : c;
-                    };
-                    // first with the rows in order as pivots, lanes 31 - w NC,
-                    // 30 - w NC ..: right if the panels before took the lanes
-                    // above and no pivot is zero
-                    const u32 above = w == 0 ? 0u : ~0u << (32 - NC * w);
-                    bool good = w * NC + NC <= n && __ballot_sync(0xffffffffu, isp) == above;
+                    good = !zero;
                     if (good) {
-                        u32 keep[NC], z = 0xffffffffu;
-                        const u32 ckeep = c;
-#pragma unroll
-                        for (int j = 0; j < NC; ++j) keep[j] = R[j];
-#pragma unroll
-                        for (int j = 0; j < NC; ++j) {
-                            const int q = 31 - w * NC - j;
-                            const u32 av = __shfl_sync(0xffffffffu, pc[j], q);
-                            z = min(z, av);
-                            step(j, q, lane < q, av);
-                        }
-                        good = z != 0u;
-                        if (good) {
-                            isp = lane >= 32 - w * NC - NC;
-                            if (lane >= w * NC && lane < w * NC + NC) q_of = 31 - lane;
-                        } else {
-                            c = ckeep;
-#pragma unroll
-                            for (int j = 0; j < NC; ++j) {
-                                R[j] = keep[j];
-                                pc[j] = xs[j * 32 + lane];
-                            }
-                        }
-                    }
-                    if (!good) {
-#pragma unroll
-                        for (int j = 0; j < NC; ++j) {
-                            const bool cand = !isp && pc[j] != 0u;
-                            const u32 b = __ballot_sync(0xffffffffu, cand);
-                            // (no candidate: the column is zero in every row left,
-                            // nothing is taken over and the coefficients are 0)
-                            const int q = b ? 31 - __clz(b) : 31;
-                            step(j, q, cand && lane != q, __shfl_sync(0xffffffffu, pc[j], q));
-                            isp = isp || (cand && lane == q);
-                            if (lane == w * NC + j) q_of = q;
-                        }
+                        isp = lane >= 32 - w * NC - NC;
+                        if (lane >= w * NC && lane < w * NC + NC) q_of = 31 - lane;
                     }
                 }
+                if (!good) {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j) pc[j] = xs[j * 32 + lane];
+#pragma unroll
+                    for (int j = 0; j < NC; ++j) {
+                        const bool cand = !isp && pc[j] != 0u && !(LAZY && pc[j] == p);
+                        const u32 b = __ballot_sync(0xffffffffu, cand);
+                        // (no candidate: the column is zero in every row left,
+                        // nothing is taken over and the coefficients are 0)
+                        q[j] = b ? 31 - __clz(b) : 31;
+                        step(j, cand && lane != q[j], __shfl_sync(0xffffffffu, pc[j], q[j]));
+                        isp = isp || (cand && lane == q[j]);
+                        if (lane == w * NC + j) q_of = q[j];
+                    }
+                }
+                // the other columns; the owner's turn into the coefficients of
+                // the pivots, one with each step
+                if (mine) {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j) {
+                        const u32 cq = __shfl_sync(0xffffffffu, c, q[j]);
+#pragma unroll
+                        for (int i = 0; i < j; ++i)
+                            R[i] = sb_lazy<LAZY, EVEN>((u64)G[j] * __shfl_sync(0xffffffffu, R[i], q[j]) + (u64)A[j] * R[i], a);
+                        R[j] = sb_lazy<LAZY, EVEN>((u64)G[j] * cq, a);
+                        c = sb_lazy<LAZY, EVEN>((u64)A[j] * c, a);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+#pragma unroll
+                        for (int i = 0; i < NC; ++i)
+                            R[i] = sb_lazy<LAZY, EVEN>((u64)G[j] * __shfl_sync(0xffffffffu, R[i], q[j]) + (u64)A[j] * R[i], a);
+                }
             }
-            SbOps &O = ops[k & 1];
+            if (LAZY) {
+#pragma unroll
+                for (int s = 0; s < NC; ++s) R[s] = min(R[s], R[s] - p);
+                c = min(c, c - p);
+            }
+            SbOps<N> &O = ops[k];
             const int qrow = ord[q_of];   // always a row below m: candidates are, and so is the first in the order
             const u32 pb = __ballot_sync(0xffffffffu, isp);
-            if (live) {
+            // rows past m too: zeros
 #pragma unroll
-                for (int s = 0; s < NC; ++s) O.T[col0 + s][row] = R[s];
-                if (ew == 0) O.c[row] = c;
-                if (ew == 1) O.isp[row] = isp ? 1 : 0;
-            }
-            if (ew == 2) O.q[lane] = (u32)(qrow * a.rs * 4);
-            if (ew == 3) O.qp[lane] = (u32)(qrow * a.ps * 4);
+            for (int s = 0; s < NC; ++s) O.T[col0 + s][row] = R[s];
+            if (ew == last) O.c[row] = c;
+            if (ew == 1) O.isp[row] = isp ? 1u : 0u;
+            if (ew == 2) O.q[lane] = (u32)(qrow * S * 4);
             // the operations of order k are complete: the other warps go on
             // (this one meets them again when it has to have R)
             asm volatile("bar.arrive 2, %0;" ::"n"(kSbThreads) : "memory");
-            if (k) sb_wait();
-            sb_arrive_relaxed();
             const u32 cr = __shfl_sync(0xffffffffu, c, rank);
             if (lane < m) {
                 dl += (int)((pb >> rank) & 1u);
                 tot = sb_red<EVEN>((u64)tot * cr, a);
             }
         }
-        sb_wait();
-        if (ew == 0) {
+        if (ew == last) {
             const u32 inv = lane < m ? sb_pow(tot, p - 2u, a.M) : 0u;   // tot is not 0 in the field F_p
             for (u32 r = 1; r < kSbCtas; ++r) sb_st_remote(sb_remote(scale + lane, r), inv);
             int dmax = lane < m ? dl : INT_MIN;
@@ -440,109 +499,99 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
         }
     } else if (cta == 0 && warp >= kSbRes) {
         // the warps between: an order's operations into the other CTAs, once
-        // these read the operations of two orders ago no more
+        // R_{k+1} is there (which is urgent, and as busy with shared memory)
+        constexpr int kPieces = (int)(sizeof(SbOps<N>) / 16), kSend = kSbSend - 32 * kSbRes;
         for (int k = 0; k < d; ++k) {
             asm volatile("bar.sync 2, %0;" ::"n"(kSbThreads) : "memory");
-            if (k) sb_wait();
-            const uint4 *src = reinterpret_cast<const uint4 *>(&ops[k & 1]);
-            for (int e = tid - 32 * kSbRes; e < (int)(kSbOpsBytes / 16); e += 32 * (kSbUpd - kSbRes)) {
-                // columns past n of T stay zero everywhere
-                if (e >= n * 8 && e < kSbMaxM * 8) continue;
-                const uint4 v = src[e];
-                for (u32 r = 1; r < kSbCtas; ++r) sb_st_remote_v4(sb_remote(src + e, r), v);
+            asm volatile("bar.sync 4, %0;" ::"n"(kSbSend) : "memory");
+            const uint4 *src = reinterpret_cast<const uint4 *>(ops + k);
+            for (int i = tid - 32 * kSbRes; i < kPieces * (kSbCtas - 1); i += kSend) {
+                const u32 r = 1 + i / kPieces, e = i % kPieces;
+                sb_send(sb_remote(src + e, r), src[e], sb_remote(sb_sm + kSbBarOff + 8 * k, r));
             }
-            __syncwarp();
-            sb_arrive();
         }
-        sb_wait();
     } else if (cta == 0) {
-        const int np = n4 / 2;   // column pairs of R
+        // R_{k+1} from R_k (the pivot rows, which move up by one coefficient)
+        // and from coefficient k + 1 (the others)
+        const u32 own = (u32)(min(lane, m - 1) * S * 4);
         for (int k = 0; k < d; ++k) {
+            if (k && k + 1 < d) ok = sb_bar_wait(bar_R + 8 * (k + 1)) && ok;
             asm volatile("bar.sync 2, %0;" ::"n"(kSbThreads) : "memory");
-            sb_arrive_relaxed();
-            const SbOps &O = ops[k & 1];
-            const u32 *R0 = rows + (k & 1) * (a.rs * m);
-            u32 *R1 = rows + ((k + 1) & 1) * (a.rs * m);
+            if (k + 1 == d) {
+                asm volatile("bar.arrive 4, %0;" ::"n"(kSbSend) : "memory");
+                break;
+            }
+            const SbOps<N> &O = ops[k];
             const u32 c = O.c[lane];
-            const int up = O.isp[lane];   // pivot rows move up by one coefficient
+            const u32 *at = rows + (O.isp[lane] ? yb + (k & 1) : k + 1) * n4;
             u32 T[N];
 #pragma unroll
             for (int j = 0; j < N; ++j) T[j] = O.T[j][lane];
             const SbPiv<N> Q(O.q);
-            const u32 own = (u32)(min(lane, m - 1) * a.rs * 4);
-            auto r_unit = [&](const u32 *at, int t, int pr) {   // lane r: coefficient t of R, column pair pr, at `at`
-                u32 v[2];
-                sb_apply<N, 2, FOLD, EVEN>(v, a, at, own, Q, c, T);
-                if (lane < m && t + up < d)
-                    *reinterpret_cast<uint2 *>(R1 + lane * a.rs + (t + up) * n4 + 2 * pr) = make_uint2(v[0], v[1]);
-            };
-            if (k + 1 < d) {
-                // coefficient k + 1 first: from k for the pivot rows, from k + 1 for the others
-                for (int u = warp; u < np; u += kSbRes) r_unit(R0 + (k + 1 - up) * n4 + 2 * u, k + 1 - up, u);
-                asm volatile("bar.arrive 1, %0;" ::"n"(kSbFirst) : "memory");
-                // coefficients k + 1 (pivot rows: to k + 2) .. d - 1
-                for (int pr = warp; pr < np; pr += kSbRes) {
-                    u32 *to = R1 + lane * a.rs + 2 * pr;
-                    for (int t = k + 1; t < d; ++t) {
-                        u32 v[2];
-                        sb_apply<N, 2, FOLD, EVEN>(v, a, R0 + t * n4 + 2 * pr, own, Q, c, T);
-                        if (lane < m && t + up < d && t + up > k + 1)
-                            *reinterpret_cast<uint2 *>(to + (t + up) * n4) = make_uint2(v[0], v[1]);
-                    }
-                }
+            for (int u = 2 * warp; u < n4; u += 2 * kSbRes) {
+                const uint2 v = sb_apply<N, FOLD, EVEN>(a, at + u, own, Q, c, T);
+                if (lane < m) *reinterpret_cast<uint2 *>(rows + lane * S + (yb + ((k + 1) & 1)) * n4 + u) = v;
             }
-            sb_wait();
+            asm volatile("bar.arrive 1, %0;" ::"n"(kSbFirst) : "memory");
+            asm volatile("bar.arrive 4, %0;" ::"n"(kSbSend) : "memory");
         }
     } else {
-        // P in place: a column belongs to one warp, top coefficient first
-        const int per = (kSbCtas - 1) * kSbUpd;
+        // The operations of order k applied to this CTA's columns, a column
+        // pair of a coefficient per warp and turn: of R from coefficient k + 1
+        // on, the new k + 2 first, for which the first CTA waits; of P up to k.
+        const u32 own = (u32)(min(lane, m - 1) * S * 4);
+        const u32 rdiv = rp ? (65536u + rp - 1) / rp : 0u, pdiv = pp ? (65536u + pp - 1) / pp : 0u;   // u / rp: u rdiv >> 16
         for (int k = 0; k < d; ++k) {
-            sb_arrive();
-            sb_wait();
-            if (warp >= kSbUpd) continue;
-            const SbOps &O = ops[k & 1];
+            ok = sb_bar_wait(bar_ops + 8 * k) && ok;
+            const SbOps<N> &O = ops[k];
             const u32 c = O.c[lane];
-            const int up = O.isp[lane];
+            const int up = O.isp[lane] ? 1 : 0;   // pivot rows move up by one coefficient
             u32 T[N];
 #pragma unroll
             for (int j = 0; j < N; ++j) T[j] = O.T[j][lane];
-            const SbPiv<N> Q(O.qp);
-            const u32 own = (u32)(min(lane, m - 1) * a.ps * 4);
-            for (int w = ((int)cta - 1) * kSbUpd + warp; w < m; w += per) {
-                u32 *at = rows + k * m4 + w, *to = at + lane * a.ps + up * m4;
-                int t = k;
-                for (; t > 0; t -= 2, at -= 2 * m4, to -= 2 * m4) {   // two coefficients at a time
-                    u32 v[1], u[1];
-                    sb_apply<N, 1, FOLD, EVEN>(v, a, at, own, Q, c, T);
-                    sb_apply<N, 1, FOLD, EVEN>(u, a, at - m4, own, Q, c, T);
-                    __syncwarp();   // every lane has read them
-                    if (lane < m) {
-                        to[0] = v[0];
-                        to[-m4] = u[0];
-                    }
+            const SbPiv<N> Q(O.q);
+            const u32 *Rf = rows + (k & 1) * (2 * d * rp), *Pf = P0 + (k & 1) * (2 * (d + 1) * pp);
+            u32 *Rt = rows + ((k + 1) & 1) * (2 * d * rp) + lane * S, *Pt = P0 + ((k + 1) & 1) * (2 * (d + 1) * pp) + lane * S;
+            const int nr = k + 2 < d ? (d - 2 - k) * rp : 0, nu = nr + (k + 1) * pp, urgent = nr ? rp : 0;
+            if (warp < urgent) {
+                const uint2 v = sb_apply<N, FOLD, EVEN>(a, Rf + ((k + 2 - up) * rp + warp) * 2, own, Q, c, T);
+                if (lane < m) {
+                    *reinterpret_cast<uint2 *>(Rt + ((k + 2) * rp + warp) * 2) = v;
+                    sb_send(sb_remote(rows + lane * S + (k + 2) * n4 + 2 * (r_first + warp), 0), v,
+                            sb_remote(sb_sm + kSbBarOff + 8 * (kSbMaxBase + k + 2), 0));
                 }
-                if (t == 0) {
-                    u32 v[1];
-                    sb_apply<N, 1, FOLD, EVEN>(v, a, at, own, Q, c, T);
-                    __syncwarp();
-                    if (lane < m) to[0] = v[0];
-                }
-                if (lane < m && up) rows[lane * a.ps + w] = 0u;
-                __syncwarp();
             }
+            for (int u = warp < urgent ? warp + kSbWarps - urgent : warp - urgent; u < nu; u += kSbWarps) {
+                const bool is_R = u < nr;
+                const int e = is_R ? u : u - nr, t0 = (int)((u32)e * (is_R ? rdiv : pdiv) >> 16), pr = e - t0 * (is_R ? rp : pp);
+                const int t = is_R ? k + 2 + t0 : t0, step = 2 * (is_R ? rp : pp);
+                const uint2 v = sb_apply<N, FOLD, EVEN>(a, (is_R ? Rf : Pf) + t * step + 2 * pr, own, Q, c, T);
+                u32 *to = (is_R ? Rt : Pt) + 2 * pr;
+                if (lane < m) {
+                    const uint2 zero = make_uint2(0u, 0u);
+                    if (!is_R || (t + up < d && t + up > k + 2)) *reinterpret_cast<uint2 *>(to + (t + up) * step) = v;
+                    // P: what no coefficient moves to
+                    if (!is_R && t == 0 && up) *reinterpret_cast<uint2 *>(to) = zero;
+                    if (!is_R && t == k && !up) *reinterpret_cast<uint2 *>(to + (k + 1) * step) = zero;
+                }
+            }
+            __syncthreads();
         }
     }
+    if (!ok) a.out->bad = 1;
     __syncwarp();
     sb_arrive();
-    sb_wait();   // the scales are in every CTA, and P is complete; no remote access after this
-    if (cta == 0) return;
+    sb_wait();   // the scales are in every CTA; no remote access after this
+    if (cta == 0 || lane >= m) return;
     // this CTA's columns of P
-    for (int i = tid; i < (d + 1) * m * kSbUpd; i += kSbThreads) {
-        const int w = ((int)cta - 1) * kSbUpd + (i & (kSbUpd - 1)), tr = i / kSbUpd, t = tr / m, r = tr - t * m;
-        if (w < m) a.P[((size_t)t * m + r) * m + w] = red64((u64)rows[r * a.ps + t * m4 + w] * scale[r], a.M);
-    }
+    const u32 *Pd = P0 + (d & 1) * (2 * (d + 1) * pp) + lane * S;
+    const u32 sc = scale[lane];
+    for (int t = warp; t <= d; t += kSbWarps)
+        for (int c = 0; c < 2 * pp; ++c)
+            if (2 * p_first + c < m) a.P[((size_t)t * m + lane) * m + 2 * p_first + c] = red64((u64)Pd[t * 2 * pp + c] * sc, a.M);
 }
-static_assert((kSbCtas - 1) * kSbUpd >= kSbMaxM, "one column of P per warp");
+static_assert(kSbMaxM / 2 <= kSbWarps * kSbApply, "a warp per column pair of R's next coefficient");
+static_assert(2 * ((kSbMaxM / 2 + kSbApply - 1) / kSbApply) <= kSbWarps, "a warp per column of P's first coefficient");
 
 __global__ void k_sb_node(const PmNode n) { pm_node(n, (int)threadIdx.x); }
 
@@ -653,12 +702,12 @@ u32 *sb_alloc(SbRun &R, size_t elems)
 }
 
 template <int N>
-ffspmv_status sb_launch(const SbLeaf &a, size_t smem, cudaStream_t st)
+ffspmv_status sb_launch(const SbLeaf &a, cudaStream_t st)
 {
+    const size_t smem = sb_leaf_smem(a.m, a.n, a.d, sizeof(SbOps<N>));
     // p <= 2^26: all 33 products of a sum stay below p 2^32
     auto *k = a.M.m <= (1u << 26) ? k_sb_mbasis<N, false, false> : k_sb_mbasis<N, true, false>;
-    if constexpr (N == 32)
-        if (a.M.m == 2u) k = k_sb_mbasis<32, false, true>;
+    if (a.M.m == 2u) k = k_sb_mbasis<N, false, true>;
     FF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSbSmemMax));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kSbCtas);
@@ -687,15 +736,13 @@ ffspmv_status sb_leaf(SbRun &R, const u32 *F, long long d, const int *shift, u32
     a.m = R.m;
     a.n = R.n;
     a.d = (int)d;
-    a.rs = sb_rstride(R.n, d);
-    a.ps = sb_pstride(R.m, d);
+    a.stride = sb_stride(R.m, R.n, a.d);
     u32 y = R.p;   // p^-1 mod 2^32 for odd p (Newton)
     for (int i = 0; i < 4; ++i) y *= 2u - R.p * y;
     a.pinv = y;
+    a.one = R.p == 2u ? 1u : (u32)((1ull << 32) % R.p);
     a.M = R.M;
-    const size_t smem = sb_leaf_smem(R.m, R.n, d);
-    if (R.p == 2u) return sb_launch<32>(a, smem, R.st);
-    return R.n <= 8 ? sb_launch<8>(a, smem, R.st) : R.n <= 16 ? sb_launch<16>(a, smem, R.st) : sb_launch<32>(a, smem, R.st);
+    return R.n <= 8 ? sb_launch<8>(a, R.st) : R.n <= 16 ? sb_launch<16>(a, R.st) : sb_launch<32>(a, R.st);
 }
 
 // Order-d basis of F (d coefficients of m x n) for the shift at `shift` (device)
@@ -761,9 +808,9 @@ ffspmv_status sb_layout(int32_t m, int32_t n, int64_t d, int32_t base, SbLayout 
     if (m < 1 || m > kSbMaxM || n < 1 || n > m || d < 1 || base < 0 || base > kSbMaxBase) return FFSPMV_ERR_ARG;
     SbLayout L;
     L.base = base ? base : kSbMaxBase;
-    L.leaf = std::min(L.base, kSbLeaf);
+    L.leaf = std::min(L.base, sb_leaf_max(n));
     L.async = kSbAsync;
-    if (sb_leaf_smem(m, n, L.leaf) > kSbSmemMax) return FFSPMV_ERR_UNSUPPORTED;
+    if (sb_leaf_smem(m, n, L.leaf, n <= 16 ? sizeof(SbOps<16>) : sizeof(SbOps<32>)) > kSbSmemMax) return FFSPMV_ERR_UNSUPPORTED;
     // the recursion's largest product, ceil(d/2) + d coefficients, must fit the transforms
     if (d > L.base && (d + 1) / 2 + d > (1LL << 15)) return FFSPMV_ERR_UNSUPPORTED;
     L.nodes = sb_nodes(d, L.leaf);
@@ -838,6 +885,7 @@ extern "C" ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d
     const cudaError_t sync = cudaStreamSynchronize(R.st);
     if (st != FFSPMV_OK) return st;
     FF_CUDA(sync);
+    if (h.bad) return FFSPMV_ERR_TIMEOUT;
     for (int i = 0; i < m; ++i) h_delta[i] = h.delta[i];
     if (h_degree) *h_degree = h.e;
     return FFSPMV_OK;
