@@ -48,7 +48,8 @@
 // the whole basis (with the transforms of polymat.cu); four eliminating warps
 // beside eight that apply to R, two CTAs for P, leaves of at most 16 orders, 4.3
 // us and 81 ms; R in CTAs of its own 3.5 us and 64 ms; columns of R and P mixed,
-// panels before the rest, as it is here, 3.0 us and 58 ms.
+// panels before the rest, as it is here, 3.0 us and 58 ms (56 with the products
+// of 16-bit pairs, polymat.cu).
 #include <algorithm>
 #include <climits>
 #include <cstddef>
@@ -137,7 +138,7 @@ size_t sb_leaf_smem(int m, int n, int d, size_t ops) { return kSbOpsOff + d * op
 
 // Largest order of one launch: what fits the shared memory, and beyond which
 // what the products beside it take is small (order 12 502, 32 x 16: 67 ms at 16,
-// 61 at 24, 58 at 32).
+// 61 at 24, 58 at 32, before the products took 16-bit pairs).
 int sb_leaf_max(int n) { return n <= 16 ? 32 : 24; }
 
 __device__ u32 sb_pow(u32 a, u32 e, const Mod &M)
