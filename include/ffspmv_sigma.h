@@ -60,7 +60,8 @@ ffspmv_status sigma_basis_workspace(int32_t m, int32_t n, int64_t d, int32_t bas
  * owned by the caller and not used by another call at the same time.
  * Synchronous: the recursion reads the larger halves' degrees back to size
  * the next products, so the call returns after the stream has finished the
- * work.
+ * work.  FFSPMV_ERR_TIMEOUT when a bounded device wait of a leaf ran out (the
+ * outputs are then undefined).
  */
 ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
                           const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,

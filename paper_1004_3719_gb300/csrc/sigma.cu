@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
         // and from coefficient k + 1 (the others)
         const u32 own = (u32)(min(lane, m - 1) * S * 4);
         for (int k = 0; k < d; ++k) {
-            if (k && k + 1 < d) ok = sb_bar_wait(bar_R + 8 * (k + 1)) && ok;
+            if (k && k + 1 < d) ok = __all_sync(0xffffffffu, ok && sb_bar_wait(bar_R + 8 * (k + 1)));
             asm volatile("bar.sync 2, %0;" ::"n"(kSbThreads) : "memory");
             if (k + 1 == d) {
                 asm volatile("bar.arrive 4, %0;" ::"n"(kSbSend) : "memory");
@@ -543,7 +543,10 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
         const u32 own = (u32)(min(lane, m - 1) * S * 4);
         const u32 rdiv = rp ? (65536u + rp - 1) / rp : 0u, pdiv = pp ? (65536u + pp - 1) / pp : 0u;   // u / rp: u rdiv >> 16
         for (int k = 0; k < d; ++k) {
-            ok = sb_bar_wait(bar_ops + 8 * k) && ok;
+            // without the operations nothing is done (their offsets are not there)
+            ok = __all_sync(0xffffffffu, sb_bar_wait(bar_ops + 8 * k));
+            ok = __syncthreads_and(ok) != 0;
+            if (!ok) break;
             const SbOps<N> &O = ops[k];
             const u32 c = O.c[lane];
             const int up = O.isp[lane] ? 1 : 0;   // pivot rows move up by one coefficient
@@ -576,7 +579,6 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
                     if (!is_R && t == k && !up) *reinterpret_cast<uint2 *>(to + (k + 1) * step) = zero;
                 }
             }
-            __syncthreads();
         }
     }
     if (!ok) a.out->bad = 1;
