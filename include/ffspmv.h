@@ -284,7 +284,8 @@ ffspmv_status spmv_get_info(ffspmv_t h, int64_t *nrows, int64_t *ncols,
  * add up, so an even number of odd copies cancels.  The first call for A (or
  * A^T) builds the pattern of the odd entries on the device (synchronous);
  * later calls are stream-ordered and asynchronous.  d_X and d_Y must not
- * overlap.  Not in the paper as a kernel.
+ * overlap; calls on one handle may, once its pattern is built.  Not in the
+ * paper as a kernel.
  */
 ffspmv_status spmv_apply_gf2(ffspmv_t h, int32_t transpose, const uint64_t *d_X,
                              uint64_t *d_Y, int32_t words, int32_t accumulate,

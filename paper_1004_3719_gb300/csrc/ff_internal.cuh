@@ -199,8 +199,8 @@ struct Phase {
 // (general lanes only) are lane by lane for u16, interleaved the same way
 // for u32.  Entry word: (row in group << 16) | (sign << 15) | x element of
 // the panel.  Row sums stay in shared memory (u32 sums of terms below 2m when
-// m <= 2^16 -- at most kPanelLong of them, so below 2^32 -- u64 sums of terms
-// below 2^32 otherwise); the q CTAs of a cluster add their partial sums
+// m <= 2^16 -- at most kPanelLong of them, so below 2^32 -- else a pair of u32
+// sums, of the terms' low 16 bits and of the rest); the q CTAs of a cluster add their partial sums
 // through distributed shared memory.
 constexpr int kPanelConsumers = 512;          // 16 warps sum entries
 constexpr int kPanelStages = 3;
