@@ -97,8 +97,9 @@ typedef struct {
                                   sequence kernel never arrives at its first grid barrier, so the
                                   bounded wait of every other CTA runs out (FFSPMV_ERR_TIMEOUT);
                                   bit 1 = the x-panel kernel never issues the copies of the second
-                                  stage of each CTA, so the waits for it run out (the status word
-                                  read by spmv_check_status); bit 2 = x-panel blocks always take
+                                  and later stages of each CTA, so a wait for them runs out and the
+                                  launch ends within a second (the status word read by
+                                  spmv_check_status); bit 2 = x-panel blocks always take
                                   the 2- and 4-vector passes, without the timing that decides it;
                                   bit 3 = x-panel blocks never take them (one-vector passes) */
     int32_t panel_cluster;     /* x-panel layout: CTAs per cluster (column groups); 0 = chosen by

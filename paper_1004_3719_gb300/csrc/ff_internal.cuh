@@ -210,16 +210,21 @@ constexpr int kPanelBarBytes = 128;           // full and empty mbarrier of each
 constexpr int kPanelDescBytes = 128;          // (entries, general, packs, x slot) of each buffer
 constexpr u32 kPanelSlotMask = 7u;            // PanelStage::xs: x slot
 constexpr u32 kPanelNewX = 8u;                // PanelStage::xs: the panel is copied in with this stage
-static_assert(16 * kPanelStages + 8 <= kPanelBarBytes && kPanelStages <= 7,
-              "full and empty mbarriers of the stage buffers, the epilogue's receive mbarrier, x slots");
-constexpr unsigned kPanelSpin = 1u << 20;     // polls of an mbarrier before giving up
-constexpr unsigned kPanelGridSpin = 1u << 20; // polls of the grid barrier before giving up
+constexpr int kPanelAskOff = 64;              // in the mbarriers' block: a word per consumer warp
+static_assert(16 * kPanelStages + 8 <= kPanelAskOff && kPanelAskOff + kPanelConsumers / 8 <= kPanelBarBytes && kPanelStages <= 7,
+              "full and empty mbarriers of the stage buffers, the consumer warps' words, x slots");
+// A wait gives up after kPanelPolls polls and then kPanelWaitNs on the clock;
+// the first one of a CTA that does ends the others, so that a CTA whose copies
+// stop coming ends within a second, the copies still in flight included.
+constexpr int kPanelPolls = 128;
+constexpr unsigned long long kPanelWaitNs = 700ull * 1000 * 1000, kPanelDrainNs = 50ull * 1000 * 1000;
 constexpr u32 kPanelIdxMask = 0x7fffu;        // x element of the panel
 constexpr u32 kPanelNeg = 0x8000u;            // a -1 entry (+-1 sections)
 constexpr long long kPanelLong = 32768;       // longer rows go to split CSR segments
 constexpr int kPanelSmemMax = 227 * 1024;
 constexpr int kPanelMaxPe = 32760;            // stage entries (fits the 16-bit pack counts)
-static_assert(16 * kPanelStages + 4 <= kPanelDescBytes, "stage descriptors and the grid generation word");
+static_assert(16 * kPanelStages + 8 + 4 * kPanelStages <= kPanelDescBytes,
+              "stage descriptors, the grid generation word, the flag of a wait that ran out, stages issued");
 
 struct PanelStage {
     u32 xoff;  // first staged-x element of the panel (16-byte aligned)
@@ -333,7 +338,7 @@ void free_plan(Plan &P);
 // Run-time controls of the x-panel kernel's bounded waits.
 struct PanelCtl {
     int *status = nullptr;  // device word: bit 0 set when a wait ran out
-    int skip_stage = -1;    // testing only: the copies of this stage of every CTA are never issued
+    int skip_stage = -1;    // testing only: the copies of this stage of every CTA and of the later ones are never issued
 };
 
 ffspmv_status run_plan(const Plan &P, const u32 *x, long long ldx, u32 *y,

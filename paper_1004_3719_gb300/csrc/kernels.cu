@@ -639,6 +639,13 @@ __device__ __forceinline__ void mbar_expect_tx(u32 bar, u32 bytes)
                  : "memory");
 }
 
+__device__ __forceinline__ u64 global_ns()
+{
+    u64 t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // Bulk copy global -> this CTA's shared memory, completing on mbarrier `bar`.
 __device__ __forceinline__ void bulk_g2s(u32 dst, const void *src, u32 bytes, u32 bar)
 {
@@ -647,20 +654,76 @@ __device__ __forceinline__ void bulk_g2s(u32 dst, const void *src, u32 bytes, u3
                  : "memory");
 }
 
-// Wait for the phase of `bar` with parity `parity`; false after POLLS polls.
-template <unsigned POLLS = kPanelSpin>
-__device__ __forceinline__ bool mbar_wait(u32 bar, u32 parity)
+// Has the phase of `bar` with parity `parity` ended?  (SUSPEND: the hardware
+// may hold the thread for a while before it says no.)
+template <bool SUSPEND>
+__device__ __forceinline__ bool mbar_poll(u32 bar, u32 parity)
 {
-    for (unsigned i = 0; i < POLLS; ++i) {
-        u32 done;
+    u32 done;
+    if constexpr (SUSPEND)
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done)
                      : "r"(bar), "r"(parity)
                      : "memory");
-        if (done) return true;
-    }
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+    return done != 0;
+}
+
+// The same, waited for: kPanelPolls polls, the rare rest in mbar_wait_on.
+__device__ __forceinline__ bool mbar_wait(u32 bar, u32 parity)
+{
+    for (int i = 0; i < kPanelPolls; ++i)
+        if (mbar_poll<true>(bar, parity)) return true;
     return false;
+}
+
+// A wait that has taken long: on with polls that return at once, until the
+// phase ends, `ns` nanoseconds have passed, or the CTA has given up (*dead).
+__device__ __forceinline__ bool mbar_wait_on(u32 bar, u32 parity, const volatile u32 *dead, u64 ns)
+{
+    const u64 t0 = global_ns();
+    for (;;) {
+        if (mbar_poll<false>(bar, parity)) return true;
+        if (*dead != 0u || global_ns() - t0 > ns) return false;
+        __nanosleep(64);
+    }
+}
+
+// The same for a warp whose 32 lanes wait for one phase: all of them get the
+// same answer.  A lane that would give up asks for it in `*ask` (a bit per
+// lane, zero before) and does once all the lanes have asked; until then the
+// phase may still end, and the lane takes its bit back.  Where some lanes
+// have seen the phase end the others do so too.  (No vote: that would be paid
+// for by every wait, 1% of a product.)
+__device__ __forceinline__ bool mbar_wait_on_warp(u32 bar, u32 parity, const volatile u32 *dead, u64 ns, u32 *ask)
+{
+    const u32 bit = 1u << (threadIdx.x & 31u);
+    const u64 t0 = global_ns();
+    bool asked = false;
+    for (;;) {
+        const bool ended = mbar_poll<false>(bar, parity);
+        if (asked) {
+            u32 m = *reinterpret_cast<volatile u32 *>(ask);
+            while (ended && m != 0xffffffffu) {
+                const u32 o = atomicCAS(ask, m, m & ~bit);
+                if (o == m) return true;
+                m = o;
+            }
+            if (m == 0xffffffffu) return false;
+        } else if (ended) {
+            return true;
+        } else if (*dead != 0u || global_ns() - t0 > ns) {
+            atomicOr(ask, bit);
+            asked = true;
+        }
+        __nanosleep(64);
+    }
 }
 
 __device__ __forceinline__ void mbar_arrive(u32 bar)
@@ -748,6 +811,10 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
     unsigned char *bars = ebuf + kPanelStages * EB;
     uint4 *desc = reinterpret_cast<uint4 *>(bars + kPanelBarBytes);  // (entries, general, packs, x slot)
     u32 &s_gen = *reinterpret_cast<u32 *>(bars + kPanelBarBytes + 16 * kPanelStages);  // grid barrier generation
+    // a wait of this CTA ran out; stages issued into each buffer
+    volatile u32 *dead = reinterpret_cast<volatile u32 *>(bars + kPanelBarBytes + 16 * kPanelStages + 4);
+    u32 *issued = reinterpret_cast<u32 *>(bars + kPanelBarBytes + 16 * kPanelStages + 8);
+    u32 *ask = reinterpret_cast<u32 *>(bars + kPanelAskOff);   // lanes of each consumer warp that would give up
     AT *acc = reinterpret_cast<AT *>(bars + kPanelBarBytes + kPanelDescBytes);
     const int q = P.q;
     const int cta = blockIdx.x, g = cta / q, rank = cta % q;
@@ -835,8 +902,10 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
         fence_proxy_async_global();
     }
     for (u32 r = t; r < nr * NV; r += kPanelThreads) acc[r] = 0;
+    if (t < kWarps) ask[t] = 0u;
     __syncthreads();
     if (t == 0) {
+        *dead = 0u;
         for (int b = 0; b < kPanelStages; ++b) {
             mbar_init(full0 + 8u * b, 1);
             mbar_init(empty0 + 8u * b, kWarps);
@@ -855,6 +924,12 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
         }
     }
     __syncthreads();
+    // A wait that runs out ends the CTA's work: the flag *dead ends the other
+    // waits, copy warps issue nothing more, consumers leave the stage loop
+    // without reading a descriptor or a buffer whose copies they have not
+    // seen, and without releasing it.  So no buffer is filled twice, and no
+    // phase of its mbarriers passes by unseen: each stage that was issued is
+    // one phase of its buffer, in order.
     bool timed_out = false;
     if (warp >= kWarps) {
         // Copy warps.  Warp kWarps + b fills stage buffer b: stages b,
@@ -871,18 +946,22 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
         const unsigned char *ev = reinterpret_cast<const unsigned char *>(P.ent);
         const unsigned char *vv = reinterpret_cast<const unsigned char *>(P.val);
         bool xready = !fused;
+        u32 nissued = 0;
         for (u32 s = b; s < ns; s += kPanelStages) {
+            if (s >= (u32)skip_stage) break;  // testing: this stage and the later ones are never issued
             const PanelStage a = P.stage[s0 + s];
             if (s >= kPanelStages) {
                 // stage s - kPanelStages of this buffer must be done with
                 u32 ok = 1;
                 if (lane == 0) {
                     const u32 ep = (s / kPanelStages - 1) & 1u;
-                    ok = (timed_out ? mbar_wait<1>(ebar, ep) : mbar_wait(ebar, ep)) ? 1u : 0u;
+                    ok = mbar_wait(ebar, ep) || mbar_wait_on(ebar, ep, dead, kPanelWaitNs) ? 1u : 0u;
                 }
-                if (!__shfl_sync(0xffffffffu, ok, 0)) timed_out = true;
+                if (!__shfl_sync(0xffffffffu, ok, 0)) {
+                    timed_out = true;
+                    break;
+                }
             }
-            if ((int)s == skip_stage) continue;  // testing: this stage is never issued
             // values: u8 ones are copied in whole 16-byte blocks (the layout pads them)
             const u32 vbytes = TINY ? (a.ngen + 15u) & ~15u : a.ngen * (u32)VB;
             const u32 dbytes = a.nent * 4u + vbytes;
@@ -896,32 +975,42 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
                 if (!xready) {
                     // every CTA's share of x is staged before the first panel copy
                     unsigned spin = 0;
-                    while (ld_acquire_gpu(P.gbar + 1) == s_gen)
-                        if (++spin >= kPanelGridSpin) {
+                    u64 t0 = 0;
+                    while (ld_acquire_gpu(P.gbar + 1) == s_gen) {
+                        if (++spin < (unsigned)kPanelPolls) continue;
+                        if (t0 == 0) t0 = global_ns();
+                        if (*dead != 0u || global_ns() - t0 > kPanelWaitNs) {
                             timed_out = true;
                             break;
                         }
+                    }
                     fence_proxy_async_global();
                     xready = true;
                 }
-                const bool newx = (a.xs & kPanelNewX) != 0;
-                desc[b] = make_uint4(a.nent, a.ngen, a.npg | (a.npp << 16), a.xs & kPanelSlotMask);  // published by the arrive
+                // (without x: a stage of no entries, so that lane 1's copies end a phase)
+                const bool newx = (a.xs & kPanelNewX) != 0 && !timed_out;
+                desc[b] = timed_out ? make_uint4(0u, 0u, 0u, 0u)
+                                    : make_uint4(a.nent, a.ngen, a.npg | (a.npp << 16), a.xs & kPanelSlotMask);  // published by the arrive
                 mbar_expect_tx(bar, newx ? (u32)PX : 0u);
                 if (newx) bulk_g2s(sbase + (a.xs & kPanelSlotMask) * PX, xh + (size_t)a.xoff * sizeof(XW), (u32)PX, bar);
             }
-            __syncwarp();
+            ++nissued;
+            if (__any_sync(0xffffffffu, timed_out)) {
+                timed_out = true;
+                break;
+            }
         }
+        if (timed_out) *dead = 1u;
+        if (lane == 0) issued[b] = nissued;
     } else {
         const u32 mu32 = (u32)(M.mu >> 32);  // floor(2^32 / m)
         const u32 mneg = MONT ? neg_inv32(M.m) : 0u;
         const u32 rot = ((u32)P.pe / 8u + 31u) / 32u;  // blocks of a full stage
         for (u32 s = 0; s < ns; ++s) {
             const u32 b = s % kPanelStages;
-            // after one wait has run out, the others poll once: a CTA whose
-            // copies stopped coming ends in bounded time
             const u32 fb = full0 + 8u * b, fp = (s / kPanelStages) & 1u;
             bool released = false;
-            if (timed_out ? mbar_wait<1>(fb, fp) : mbar_wait(fb, fp)) {
+            if (mbar_wait(fb, fp) || mbar_wait_on_warp(fb, fp, dead, kPanelWaitNs, ask + warp)) {
                 const uint4 st = desc[b];
                 const u32 nl = st.x >> 3, nlg = st.y >> 3, lpg = (st.z & 0xffffu) >> 3, lpp = (st.z >> 16) >> 3;
                 const unsigned char *sb = ebuf + b * EB;
@@ -1118,22 +1207,27 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
                         }
                     }
                 }
+                if (!released) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty0 + 8u * b);
+                }
             } else {
                 timed_out = true;
-            }
-            if (!released) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(empty0 + 8u * b);
+                *dead = 1u;
+                s = ns;
             }
         }
     }
     if (__syncthreads_or(timed_out)) {
-        // a copy, a buffer or the grid barrier never came: report, and give
-        // the last copies a bounded chance to land before the CTA leaves
-        if (t == 0) {
-            if (status) atomicOr(status, 1);
-            for (u32 s = ns > kPanelStages ? ns - kPanelStages : 0; s < ns; ++s)
-                if ((int)s != skip_stage) mbar_wait(full0 + 8u * (s % kPanelStages), (s / kPanelStages) & 1u);
+        // a copy, a buffer or the grid barrier never came: report, and let the
+        // copies that were issued land before the CTA leaves.  A buffer's last
+        // stage but one had ended when its last was issued, so the last one's
+        // parity is the one to wait for
+        if (t < kPanelStages) {
+            if (t == 0 && status) atomicOr(status, 1);
+            const u32 n = issued[t];
+            *dead = 0u;   // these waits end by their own limit
+            if (n) mbar_wait_on(full0 + 8u * t, (n - 1u) & 1u, dead, kPanelDrainNs);
         }
         __syncthreads();
     }
