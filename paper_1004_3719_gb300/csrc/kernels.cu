@@ -551,9 +551,12 @@ __global__ void __launch_bounds__(256) k_x_stage(const u32 *__restrict__ x, long
     for (long long i = done + t; i < n; i += nth) xs[i] = (XT)x[i * ldx];
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 // The shared::cluster address of `local` in CTA `rank` of the cluster.
@@ -924,6 +927,10 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
         }
     }
     __syncthreads();
+    // The other CTAs of the cluster add into this one's row sums: not before
+    // they are zeroed.  (After a grid barrier they are.)
+    const bool pair_up = q > 1 && !fused;
+    if (pair_up) cluster_arrive();
     // A wait that runs out ends the CTA's work: the flag *dead ends the other
     // waits, copy warps issue nothing more, consumers leave the stage loop
     // without reading a descriptor or a buffer whose copies they have not
@@ -1241,6 +1248,7 @@ k_panel(const PanelPart P, const u32 *__restrict__ x, long long ldx, u32 *__rest
     constexpr u32 G = 16 / sizeof(AT);
     const u32 nf = nr * NV;
     const u32 share = ((nf + q - 1) / q + G - 1) / G * G;
+    if (pair_up) cluster_wait();
     if (q > 1) {
         for (int j = 0; j < q; ++j) {
             if (j == rank) continue;

@@ -1,5 +1,6 @@
-"""x-panel products whose copies stop coming: every kernel instance gives up
-within its bound, says so in the status word, and leaves the device usable."""
+"""What the CTAs of an x-panel product wait for: copies that stop coming (every
+kernel instance gives up within its bound, says so in the status word, and
+leaves the device usable), and each other's row sums."""
 import time
 
 import numpy as np
@@ -31,3 +32,30 @@ def test_products_without_their_copies_end_within_the_bound(lib, m, q, nvec):
     N.apply(xd, yd)
     N.check_status()
     assert np.array_equal(to_host(yd), oracle.csr_spmv(A, x).reshape(A.nrows, nvec))
+
+
+@pytest.mark.parametrize("m,q,n", [(65521, 2, 4_000_000), (2**31 - 1, 2, 2_000_000), (2**31 - 1, 4, 1_200_000)])
+def test_ctas_of_a_cluster_with_uneven_work(lib, m, q, n):
+    """More row groups than fit the GPU at once (x staged by a launch before, so
+    no grid barrier), and rows whose entries lie in one column group but for one
+    in a hundred: one CTA of a cluster is done long before the others and adds
+    its few terms into their row sums."""
+    nc = 200_000
+    rng = np.random.default_rng(q)
+    # rows in q bands, each with the columns of one q-th
+    lo = np.arange(n) * q // n * (nc // q)
+    cols = lo[:, None] + rng.integers(0, nc // q, (n, 3))
+    far = rng.random(n) < 0.01
+    cols[far, 0] = rng.integers(0, nc, int(far.sum()))
+    A = gen.CSR(n, nc, np.arange(n + 1, dtype=np.int64) * 3, np.sort(cols, axis=1).reshape(-1).astype(np.int32),
+                rng.integers(0, m, 3 * n, dtype=np.uint64).astype(np.uint32), m)
+    M = lib.Matrix.from_csr(A, priority_format=lib.FMT.PANEL, panel_cluster=q, transpose_mode=lib.TRANSPOSE.NONE)
+    assert M.launches(False, 1) == 2     # staging, product
+    for k in range(3):
+        x = rand_block(k, nc, 1, m)
+        xd = to_dev(x)
+        ys = [M.apply(xd) for _ in range(4)]
+        M.check_status()
+        want = oracle.csr_spmv(A, x)
+        for y in ys:
+            assert np.array_equal(to_host(y).reshape(want.shape), want)
