@@ -60,13 +60,24 @@ ffspmv_status sigma_basis_workspace(int32_t m, int32_t n, int64_t d, int32_t bas
  * owned by the caller and not used by another call at the same time.
  * Synchronous: the recursion reads the larger halves' degrees back to size
  * the next products, so the call returns after the stream has finished the
- * work.  FFSPMV_ERR_TIMEOUT when a bounded device wait of a leaf ran out (the
- * outputs are then undefined).
+ * work.  FFSPMV_ERR_TIMEOUT when a device wait of a leaf (0.7 s at most) ran
+ * out (the outputs are then undefined).
  */
 ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
                           const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,
                           int32_t *h_delta, int64_t *h_degree, void *d_work, int64_t work_bytes,
                           ffspmv_stream_t stream);
+
+/*
+ * Testing only: sigma_basis whose first leaf's eliminating CTA keeps the
+ * operations of order `hold` (>= 0) and of the later ones from the other CTAs,
+ * whose waits for them run out: FFSPMV_ERR_TIMEOUT within a second or two, the
+ * device usable as before.  A leaf of at most `hold` orders is not affected.
+ */
+ffspmv_status ffspmv_sigma_basis_hold(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
+                                      const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,
+                                      int32_t *h_delta, int64_t *h_degree, void *d_work, int64_t work_bytes,
+                                      int32_t hold, ffspmv_stream_t stream);
 
 /*
  * The block-Wiedemann input of sigma_basis: d_F (device, L x 2s x s) =

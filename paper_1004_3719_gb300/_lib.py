@@ -94,6 +94,8 @@ def _declare(L):
     L.sigma_basis_workspace.restype = ctypes.c_int
     L.sigma_basis.argtypes = [_U32, _I32, _I32, _I64, _I32, _P, _P, _P, _P, _P, _P, _I64, _P]
     L.sigma_basis.restype = ctypes.c_int
+    L.ffspmv_sigma_basis_hold.argtypes = [_U32, _I32, _I32, _I64, _I32, _P, _P, _P, _P, _P, _P, _I64, _I32, _P]
+    L.ffspmv_sigma_basis_hold.restype = ctypes.c_int
     L.sigma_wiedemann_input.argtypes = [_U32, _I32, _I64, _P, _P, _P]
     L.sigma_wiedemann_input.restype = ctypes.c_int
     L.sigma_generator_degrees.argtypes = [_U32, _I32, _I32, _I64, _P, _P, _I32, ctypes.POINTER(_I64),

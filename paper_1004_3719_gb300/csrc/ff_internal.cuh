@@ -61,6 +61,14 @@ __device__ __forceinline__ u32 combine(u32 r, const u32 *yp, bool accum,
     return addmod(a, b, M.m);
 }
 
+// Nanoseconds of the device's clock, for the limits of waits.
+__device__ __forceinline__ u64 global_ns()
+{
+    u64 t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // ---------------------------------------------------------------------------
 // Accumulators.  AccSmall is one 64-bit word and is used when the plan has
 // checked that no output sums more than floor((2^64-1)/B) terms, B the

@@ -642,13 +642,6 @@ __device__ __forceinline__ void mbar_expect_tx(u32 bar, u32 bytes)
                  : "memory");
 }
 
-__device__ __forceinline__ u64 global_ns()
-{
-    u64 t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // Bulk copy global -> this CTA's shared memory, completing on mbarrier `bar`.
 __device__ __forceinline__ void bulk_g2s(u32 dst, const void *src, u32 bytes, u32 bar)
 {

@@ -75,7 +75,8 @@ constexpr int kSbThreads = 32 * kSbWarps;
 constexpr int kSbSend = 32 * (kSbWarps - kSbElim);
 constexpr int kSbApply = 6;                 // CTAs that apply the operations to P and to R's later coefficients
 constexpr int kSbCtas = 1 + kSbApply;
-constexpr int kSbSpin = 1 << 20;            // tries of a bounded wait
+constexpr int kSbPolls = 256;               // tries of a wait before it looks at the clock
+constexpr u64 kSbWaitNs = 700ull * 1000 * 1000, kSbDrainNs = 50ull * 1000 * 1000;   // its limit; that of messages in flight
 constexpr size_t kSbSmemMax = 227 * 1024;
 constexpr size_t kSbAlign = 256;
 constexpr int kSbMaxShift = 1 << 24;
@@ -87,6 +88,7 @@ struct SbLeaf {
     SbSlot *out;
     int m, n, d;
     int stride;          // words per row of R and of P in shared memory
+    int hold;            // testing: the operations of this order and of the later ones are not sent (else INT_MAX)
     u32 pinv;            // p^-1 mod 2^32 (odd p)
     u32 one;             // 2^32 mod p (p = 2: 1): x -> x under sb_red
     Mod M;
@@ -215,11 +217,29 @@ __device__ __forceinline__ void sb_bar_init(u32 bar, u32 bytes)
     asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// Every mbarrier is used once.  False when the wait ran out.
-__device__ __forceinline__ bool sb_bar_wait(u32 bar)
+// The rare rest of sb_bar_wait: `ns` nanoseconds of tries that return at once.
+__device__ __noinline__ bool sb_bar_wait_on(u32 bar, u64 ns)
 {
-    for (int i = 0; i < kSbSpin; ++i) {
-        u32 ok;
+    u32 ok;
+    const u64 t0 = global_ns();
+    do {
+        asm volatile("{\n.reg .pred q;\nmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n"
+                     "selp.u32 %0, 1, 0, q;\n}"
+                     : "=r"(ok)
+                     : "r"(bar)
+                     : "memory");
+        if (ok) return true;
+        __nanosleep(64);
+    } while (global_ns() - t0 < ns);
+    return false;
+}
+
+// Every mbarrier is used once.  False when the wait ran out: after kSbPolls
+// tries, which the hardware may draw out, and `ns` nanoseconds.
+__device__ __forceinline__ bool sb_bar_wait(u32 bar, u64 ns = kSbWaitNs)
+{
+    u32 ok;
+    for (int i = 0; i < kSbPolls; ++i) {
         asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n"
                      "selp.u32 %0, 1, 0, q;\n}"
                      : "=r"(ok)
@@ -227,11 +247,28 @@ __device__ __forceinline__ bool sb_bar_wait(u32 bar)
                      : "memory");
         if (ok) return true;
     }
-    return false;
+    return sb_bar_wait_on(bar, ns);
 }
 
 __device__ __forceinline__ void sb_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void sb_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// The end of a warp whose wait ran out.  A CTA that gave up at order k sends
+// zeros for the coefficients that it owes the first CTA, so that this one ends
+// without waiting; and no CTA leaves before what was sent to it has landed.
+__device__ __noinline__ void sb_give_up(int *bad, u32 bar, int k0, int k1, u32 to, u32 to_bar, u32 step, int t0)
+{
+    *bad = 1;
+    for (int t = t0; t < k1; ++t) sb_send(to + t * step, make_uint2(0u, 0u), to_bar + 8 * t);
+    __syncwarp();
+    sb_arrive();
+    sb_wait();
+    const u64 since = global_ns();
+    for (int k = k0; k < k1; ++k) {
+        const u64 spent = global_ns() - since;
+        sb_bar_wait(bar + 8 * k, spent < kSbDrainNs ? kSbDrainNs - spent : 0);
+    }
+}
 
 __device__ __forceinline__ u32 sb_rank()
 {
@@ -341,6 +378,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
     __syncthreads();
     sb_wait();   // every CTA's mbarriers are ready
     bool ok = true;
+    int kf = 0;   // the order at which this CTA gave up
 
     if (cta == 0 && warp >= kSbWarps - kSbElim) {
         // the eliminating warps: each keeps row r's degree and scale in lane r
@@ -506,6 +544,7 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
             asm volatile("bar.sync 2, %0;" ::"n"(kSbThreads) : "memory");
             asm volatile("bar.sync 4, %0;" ::"n"(kSbSend) : "memory");
             const uint4 *src = reinterpret_cast<const uint4 *>(ops + k);
+            if (k >= a.hold) continue;
             for (int i = tid - 32 * kSbRes; i < kPieces * (kSbCtas - 1); i += kSend) {
                 const u32 r = 1 + i / kPieces, e = i % kPieces;
                 sb_send(sb_remote(src + e, r), src[e], sb_remote(sb_sm + kSbBarOff + 8 * k, r));
@@ -546,7 +585,10 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
             // without the operations nothing is done (their offsets are not there)
             ok = __all_sync(0xffffffffu, sb_bar_wait(bar_ops + 8 * k));
             ok = __syncthreads_and(ok) != 0;
-            if (!ok) break;
+            if (!ok) {
+                kf = k;
+                break;
+            }
             const SbOps<N> &O = ops[k];
             const u32 c = O.c[lane];
             const int up = O.isp[lane] ? 1 : 0;   // pivot rows move up by one coefficient
@@ -581,10 +623,15 @@ __global__ void __launch_bounds__(kSbThreads, 1) k_sb_mbasis(const __grid_consta
             }
         }
     }
-    if (!ok) a.out->bad = 1;
-    __syncwarp();
-    sb_arrive();
-    sb_wait();   // the scales are in every CTA; no remote access after this
+    if (!ok) {
+        const bool owes = cta && warp < rp && lane < m;
+        sb_give_up(&a.out->bad, cta ? bar_ops : bar_R, cta ? 0 : 2, d, sb_remote(rows + lane * S + 2 * (r_first + warp), 0),
+                   sb_remote(sb_sm + kSbBarOff + 8 * kSbMaxBase, 0), 4 * n4, owes ? kf + 2 : d);
+    } else {
+        __syncwarp();
+        sb_arrive();
+        sb_wait();   // the scales are in every CTA; no remote access is begun after this
+    }
     if (cta == 0 || lane >= m) return;
     // this CTA's columns of P
     const u32 *Pd = P0 + (d & 1) * (2 * (d + 1) * pp) + lane * S;
@@ -693,6 +740,7 @@ struct SbRun {
     size_t pm_bytes;
     SbSlot *slots;
     long long nslot, cslot;
+    int hold;
 };
 
 u32 *sb_alloc(SbRun &R, size_t elems)
@@ -740,6 +788,8 @@ ffspmv_status sb_leaf(SbRun &R, const u32 *F, long long d, const int *shift, u32
     a.n = R.n;
     a.d = (int)d;
     a.stride = sb_stride(R.m, R.n, a.d);
+    a.hold = R.hold;
+    R.hold = INT_MAX;   // (the first leaf's only)
     u32 y = R.p;   // p^-1 mod 2^32 for odd p (Newton)
     for (int i = 0; i < 4; ++i) y *= 2u - R.p * y;
     a.pinv = y;
@@ -780,6 +830,7 @@ ffspmv_status sb_rec(SbRun &R, const u32 *F, long long d, const int *shift, u32 
         SbSlot h1, h2;
         FF_CUDA(cudaMemcpyAsync(&h1, s1, sizeof(SbSlot), cudaMemcpyDeviceToHost, R.st));
         FF_CUDA(cudaStreamSynchronize(R.st));
+        if (h1.bad) return FFSPMV_ERR_TIMEOUT;
         const long long e1 = h1.e;
         if (e1 < 0 || e1 > d1) return FFSPMV_ERR_CUDA;
         st = pm_product(R.p, R.m, R.m, R.n, e1, d - 1, P1, F, C, d1, d - 1, R.pm_work, R.pm_bytes, R.st);
@@ -787,6 +838,7 @@ ffspmv_status sb_rec(SbRun &R, const u32 *F, long long d, const int *shift, u32 
         if ((st = sb_rec(R, C, d2, s1->delta, P2, &s2)) != FFSPMV_OK) return st;
         FF_CUDA(cudaMemcpyAsync(&h2, s2, sizeof(SbSlot), cudaMemcpyDeviceToHost, R.st));
         FF_CUDA(cudaStreamSynchronize(R.st));
+        if (h2.bad) return FFSPMV_ERR_TIMEOUT;
         const long long e2 = h2.e;
         if (e2 < 0 || e2 > d2) return FFSPMV_ERR_CUDA;
         st = pm_product(R.p, R.m, R.m, R.m, e2, e1, P2, P1, P, 0, e1 + e2, R.pm_work, R.pm_bytes, R.st);
@@ -841,10 +893,9 @@ extern "C" ffspmv_status sigma_basis_workspace(int32_t m, int32_t n, int64_t d, 
     return FFSPMV_OK;
 }
 
-extern "C" ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
-                                     const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,
-                                     int32_t *h_delta, int64_t *h_degree, void *d_work, int64_t work_bytes,
-                                     ffspmv_stream_t stream)
+static ffspmv_status sb_basis(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base, const uint32_t *d_F,
+                              const int32_t *h_shift, uint32_t *d_P, int32_t *h_delta, int64_t *h_degree, void *d_work,
+                              int64_t work_bytes, int hold, ffspmv_stream_t stream)
 {
     if (p < 2 || p > (1u << 31) || !sb_is_prime(p) || !d_F || !d_P || !h_delta || !d_work) return FFSPMV_ERR_ARG;
     SbLayout L;
@@ -866,6 +917,7 @@ extern "C" ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d
     R.base = L.base;
     R.leaf = L.leaf;
     R.async = L.async;
+    R.hold = hold;
     R.M = make_mod(p, 1, 0);
     R.st = (cudaStream_t)stream;
     char *w = static_cast<char *>(d_work);
@@ -892,6 +944,23 @@ extern "C" ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d
     for (int i = 0; i < m; ++i) h_delta[i] = h.delta[i];
     if (h_degree) *h_degree = h.e;
     return FFSPMV_OK;
+}
+
+extern "C" ffspmv_status sigma_basis(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
+                                     const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,
+                                     int32_t *h_delta, int64_t *h_degree, void *d_work, int64_t work_bytes,
+                                     ffspmv_stream_t stream)
+{
+    return sb_basis(p, m, n, d, base, d_F, h_shift, d_P, h_delta, h_degree, d_work, work_bytes, INT_MAX, stream);
+}
+
+extern "C" ffspmv_status ffspmv_sigma_basis_hold(uint32_t p, int32_t m, int32_t n, int64_t d, int32_t base,
+                                                 const uint32_t *d_F, const int32_t *h_shift, uint32_t *d_P,
+                                                 int32_t *h_delta, int64_t *h_degree, void *d_work, int64_t work_bytes,
+                                                 int32_t hold, ffspmv_stream_t stream)
+{
+    if (hold < 0) return FFSPMV_ERR_ARG;
+    return sb_basis(p, m, n, d, base, d_F, h_shift, d_P, h_delta, h_degree, d_work, work_bytes, hold, stream);
 }
 
 extern "C" ffspmv_status sigma_wiedemann_input(uint32_t p, int32_t s, int64_t L, const uint32_t *d_S, uint32_t *d_F,
