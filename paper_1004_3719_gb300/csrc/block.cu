@@ -218,13 +218,15 @@ struct BlockAcc<false> {
     static __device__ __forceinline__ u32 get(const AccWide &s, const Mod &M) { return (u32)s.partial(M); }
 };
 
-// COH: X is a buffer that earlier kernels of the stream wrote (L2 only), else
-// the read-only path.
+// X is what the kernel before wrote, which may still run when this one starts
+// (programmatic dependence): ordinary loads after the wait, never the read-only
+// path, which is for data that nothing writes while the kernel runs.  COH: by
+// way of L2 alone.
 template <bool COH>
 __device__ __forceinline__ uint4 block_gather(const char *p)
 {
     if constexpr (COH) return __ldcg(reinterpret_cast<const uint4 *>(p));
-    else return __ldg(reinterpret_cast<const uint4 *>(p));
+    else return *reinterpret_cast<const uint4 *>(p);
 }
 
 // acc += quads k, k + step, ... below end; xb: this lane's piece of the rows
