@@ -134,18 +134,20 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
  * d_y ("apply": y <- A x).  d_x and d_y must not overlap.  On a handle whose
  * format the library chose (FFSPMV_FMT_AUTO) most blocks run on a layout of
  * their own, up to 32 vectors per pass, with the rows of X packed next to
- * each other: the first such block (the second, unless the plan is the x-panel
- * layout) builds it on the device (synchronous, one allocation per handle and
- * direction); before that, while the stream is captured before that, and when
- * it cannot be built, the block runs as follows.  On a
- * handle whose plan is the x-panel layout, a block runs in passes of 4 vectors (m <=
- * 2^16) or 2, then 1: each pass reads the matrix once for all its vectors
+ * each other.  The first such block (on a handle whose plan is not the x-panel
+ * layout the second) builds it on the device: synchronous, one allocation per
+ * handle and direction, and one for the packed rows of X where a wider block
+ * than before needs it.  A block runs by the handle's plan instead until the
+ * layout is built, while its stream is captured without it, and where there is
+ * no memory for it.
+ * On a handle whose plan is the x-panel layout that is: passes of 4 vectors (m
+ * <= 2^16) or 2, then 1.  Each pass reads the matrix once for all its vectors
  * (Sec. 2.5.1) on an x-panel layout built for that width; the first block
  * that needs a width builds its layout and times one pass of it against the
  * same vectors one at a time (synchronous, host work plus one allocation
- * per handle, direction and width), and keeps it only if it is faster.  Calls on one handle must not
- * overlap on the GPU (x-panel plans and blocks stage x in buffers of the
- * handle).
+ * per handle, direction and width), and keeps it only if it is faster.
+ * Calls on one handle must not overlap on the GPU (x-panel plans and blocks
+ * stage x in buffers of the handle).
  */
 ffspmv_status spmv_apply(ffspmv_t h, const uint32_t *d_x, int64_t ldx,
                          uint32_t *d_y, int64_t ldy, int32_t nvec,

@@ -418,7 +418,8 @@ static ffspmv_status next_pass(ffspmv_t h, bool transpose, const Plan *P, int le
 //     block still takes the plan: building the layout costs 0.1 to 2 ms,
 //     which a single product would not earn back (a panel plan's first block
 //     would build panel layouts instead, which takes longer).
-static const BlockPlan *block_path(ffspmv_t h, bool transpose, int nvec, cudaStream_t st, bool counting = false)
+static BlockPlan *block_path(ffspmv_t h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st,
+                             bool counting = false)
 {
     if (h->opt.priority_format != FFSPMV_FMT_AUTO || nvec < 2 || (h->opt.test_hooks & 12)) return nullptr;
     const Plan &P = transpose ? h->AT : h->A;
@@ -430,7 +431,7 @@ static const BlockPlan *block_path(ffspmv_t h, bool transpose, int nvec, cudaStr
         h->block_seen[transpose ? 1 : 0] = true;
         if (!h->block[transpose ? 1 : 0]) return nullptr;
     }
-    return ensure_block(h, transpose, st);
+    return ensure_block(h, transpose, x, ldx, nvec, st);
 }
 
 static ffspmv_status apply_common(ffspmv_t h, bool transpose, const uint32_t *d_x,
@@ -457,8 +458,10 @@ static ffspmv_status apply_common(ffspmv_t h, bool transpose, const uint32_t *d_
     PanelCtl ctl;
     ctl.status = h->d_status + 2;
     ctl.skip_stage = (h->opt.test_hooks & 2) ? 1 : -1;
-    if (const BlockPlan *B = block_path(h, transpose, nvec, st))
-        return run_block(*B, d_x, ldx, d_y, ldy, nvec, h->m, alpha % h->m, beta % h->m, st);
+    BlockPlan *B = block_path(h, transpose, d_x, ldx, nvec, st);
+    uint4 *xs = nullptr;
+    if (B && block_staging(*B, d_x, ldx, nvec, st, &xs))
+        return run_block(*B, xs, d_x, ldx, d_y, ldy, nvec, h->m, alpha % h->m, beta % h->m, st);
     if (!P->panel.on || nvec == 1)
         return run_plan(*P, d_x, ldx, d_y, ldy, nvec, h->m, alpha % h->m, beta % h->m, st, &ctl);
     // x-panel blocks: passes of 4 or 2 vectors read the matrix once for all
@@ -532,8 +535,8 @@ ffspmv_status spmv_destroy(ffspmv_t h)
 ffspmv_status spmv_describe_plan(ffspmv_t h, char *buf, size_t len)
 {
     if (!h || !buf || len == 0) return FFSPMV_ERR_ARG;
-    std::string s = "A  " + h->A.summary;
-    if (h->has_T && h->transpose_mode == FFSPMV_TRANSPOSE_EXPLICIT) s += "A^T " + h->AT.summary;
+    std::string s = "A  " + h->A.summary + block_summary(h->block[0]);
+    if (h->has_T && h->transpose_mode == FFSPMV_TRANSPOSE_EXPLICIT) s += "A^T " + h->AT.summary + block_summary(h->block[1]);
     else if (h->transpose_mode == FFSPMV_TRANSPOSE_ATOMIC) s += "A^T by 64-bit atomic scatter\n";
     size_t n = s.size() < len - 1 ? s.size() : len - 1;
     memcpy(buf, s.data(), n);
@@ -552,8 +555,9 @@ ffspmv_status spmv_count_launches(ffspmv_t h, int32_t transpose, int32_t nvec, i
         n += 2LL * ((nvec + chunk - 1) / chunk);
     } else {
         const Plan &P = transpose ? h->AT : h->A;
-        const BlockPlan *B = block_path(h, transpose != 0, nvec, nullptr, true);
-        if (B) {
+        BlockPlan *B = block_path(h, transpose != 0, nullptr, nvec, nvec, nullptr, true);
+        uint4 *xs = nullptr;
+        if (B && block_staging(*B, nullptr, nvec, nvec, nullptr, &xs)) {
             n += block_launches(*B, nvec);
         } else if (!P.panel.on || nvec == 1) {
             n += count_plan_launches(P, nvec);

@@ -31,18 +31,21 @@ static ffspmv_status batch_apply(int32_t count, const ffspmv_t *hs, const uint32
     for (int i = 1; i < count; ++i)
         if (hs[by[i]] == hs[by[i - 1]]) rounds = std::max(rounds, (turn[by[i]] = turn[by[i - 1]] + 1) + 1);
     std::vector<const BlockPlan *> B;
+    std::vector<uint4 *> xs;
     std::vector<const u32 *> x;
     std::vector<u32 *> y;
     std::vector<int> nv;
     for (int r = 0; r < rounds; ++r) {
         B.clear();
+        xs.clear();
         x.clear();
         y.clear();
         nv.clear();
         for (int j = 0; j < count; ++j) {
             if (turn[j] != r || hs[j]->A.nrows == 0) continue;
-            const BlockPlan *b = ensure_block(hs[j], false, st);
-            if (!b) {
+            BlockPlan *b = ensure_block(hs[j], false, d_x[j], nvec[j], nvec[j], st);
+            uint4 *xj = nullptr;
+            if (!b || !block_staging(*b, d_x[j], nvec[j], nvec[j], st, &xj)) {
                 // no block layout (no memory for it, or the stream is being
                 // captured before it exists): the matrix's own plan
                 const ffspmv_status s = run_plan(hs[j]->A, d_x[j], nvec[j], d_y[j], nvec[j], nvec[j], hs[j]->m, 1, 0, st);
@@ -50,11 +53,12 @@ static ffspmv_status batch_apply(int32_t count, const ffspmv_t *hs, const uint32
                 continue;
             }
             B.push_back(b);
+            xs.push_back(xj);
             x.push_back(d_x[j]);
             y.push_back(d_y[j]);
             nv.push_back(nvec[j]);
         }
-        const ffspmv_status s = run_block_many((int)B.size(), B.data(), x.data(), y.data(), nv.data(), st);
+        const ffspmv_status s = run_block_many((int)B.size(), B.data(), xs.data(), x.data(), y.data(), nv.data(), st);
         if (s != FFSPMV_OK) return s;
     }
     return FFSPMV_OK;

@@ -20,8 +20,10 @@
 // are cut into chunks of that many, one warp each; the chunks add reduced
 // sums into 64-bit words and the last one to arrive writes the row.
 #include <algorithm>
+#include <cstdio>
 #include <cstring>
 #include <new>
+#include <string>
 #include <type_traits>
 
 #include "ff_internal.cuh"
@@ -42,7 +44,6 @@ struct BlockDev {
     const u32 *ptr, *row, *col, *lrow;
     const uint4 *chunk;
     const void *val;
-    uint4 *xs;
     u64 *carry;
     u32 *count;
     long long ncols;
@@ -511,9 +512,10 @@ constexpr int kMany = 512;
 struct BlockMany {
     const BlockDev *dev[kMany];
     const u32 *x[kMany];
+    uint4 *xs[kMany];
     u32 *y[kMany];
     u32 first[kMany + 1];
-    unsigned char nvec[kMany], place[kMany];  // place: x is read where it lies
+    unsigned char nvec[kMany], place[kMany];  // place: x is read where it lies, else packed in xs
     int count;
 };
 static_assert(sizeof(BlockMany) < 32000, "launch parameters");
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_stage_many(const __grid
     const int vec4 = nvec % 4 == 0 && ((uintptr_t)x & 15u) == 0;
     const long long t = (long long)(blockIdx.x - P.first[j]) * kBlockThreads + threadIdx.x;
     if (t >= D.ncols * pieces) return;
-    D.xs[t] = D.small ? block_pack<true>(x, nvec, t, nvec, pieces, vec4) : block_pack<false>(x, nvec, t, nvec, pieces, vec4);
+    P.xs[j][t] = D.small ? block_pack<true>(x, nvec, t, nvec, pieces, vec4) : block_pack<false>(x, nvec, t, nvec, pieces, vec4);
 }
 
 __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_constant__ BlockMany P)
@@ -563,7 +565,7 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_co
     const int C = D.small ? 8 : 4;
     a.pieces = (a.nvec + C - 1) / C;
     a.lgt = a.pieces > 1 ? 32 - __clz(a.pieces - 1) : 0;
-    a.xs = P.place[j] ? reinterpret_cast<const uint4 *>(P.x[j]) : D.xs;
+    a.xs = P.place[j] ? reinterpret_cast<const uint4 *>(P.x[j]) : P.xs[j];
     a.pitch = a.pieces;
     a.vec4 = a.nvec % 4 == 0 && ((uintptr_t)a.y & 15u) == 0;
     a.quad1 = D.quad1;
@@ -593,6 +595,25 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_co
     if (b == kBlockClasses) return;
     if (D.small) block_rows<true>(a, r0, rend, lgg, b == kBlockClasses - 2, lane);
     else block_rows<false>(a, r0, rend, lgg, b == kBlockClasses - 2, lane);
+}
+
+// x is read in place where its rows already are whole aligned 16-byte pieces of
+// u32, else packed by a launch before.
+bool block_in_place(bool small, const u32 *x, long long ldx, int nv)
+{
+    return !small && nv % 4 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15u) == 0 && ldx / 4 < (1LL << 28);
+}
+
+// log2 of the 16-byte pieces per packed row that a block's widest packed pass
+// takes, rounded up; -1 when all of it is read in place
+int staging_width(bool small, const u32 *x, long long ldx, int nvec)
+{
+    const int C = small ? 8 : 4, last = (nvec - 1) % kBlockVecs + 1;   // vectors of the last pass
+    int pieces = 0, lg = -1;
+    if (nvec > kBlockVecs && !block_in_place(small, x, ldx, kBlockVecs)) pieces = kBlockVecs / C;
+    else if (!block_in_place(small, x + (nvec - last), ldx, last)) pieces = (last + C - 1) / C;
+    for (; pieces; pieces = pieces > 1 ? (pieces + 1) / 2 : 0) ++lg;
+    return lg;
 }
 
 // ---------------------------------------------------------------------------
@@ -700,9 +721,10 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild b
     }
 }
 
-// The block layout of A (nr x nc, values below m), or of A^T.
+// The block layout of A (nr x nc, values below m), or of A^T, with a buffer for
+// packed rows of 2^lgx pieces (lgx = -1: none).
 ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long nc, const long long *ptr, const int *col,
-                          const u32 *val, u32 m, bool odd, cudaStream_t st, void *&tmp)
+                          const u32 *val, u32 m, bool odd, int lgx, cudaStream_t st, void *&tmp)
 {
     const long long nnz = ptr[nr], n = transpose ? nc : nr, ncols = transpose ? nr : nc;
     // offsets in quads and lengths of rows are 32-bit; with values, 32-bit row numbers are rounded up to a warp's
@@ -781,13 +803,14 @@ ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long 
     const size_t o_ptr = put((size_t)(rows + 1) * 4), o_row = put((size_t)rows * 4), o_chunk = put((size_t)B.nchunk * 16),
                  o_lrow = put((size_t)B.nlong * 4), o_col = put((size_t)quads * 16), o_val = put((size_t)quads * 4 * vb),
                  o_carry = put((size_t)(odd ? 0 : B.nlong) * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
-                 o_dev = put(sizeof(BlockDev)), o_xs = put((size_t)ncols * kBlockVecs * vb);
+                 o_dev = put(sizeof(BlockDev)), o_xs = put(lgx < 0 ? 0 : ((size_t)ncols << lgx) * sizeof(uint4));
     if (cudaMalloc(&B.arena, o) != cudaSuccess) {
         cudaGetLastError();
         B.arena = nullptr;
         return FFSPMV_ERR_OOM;
     }
     char *base = (char *)B.arena;
+    if (lgx >= 0) B.xs[B.lgx = lgx] = (uint4 *)(base + o_xs);
     BlockDev D;
     memset(&D, 0, sizeof(D));
     D.ptr = B.ptr = (const u32 *)(base + o_ptr);
@@ -798,7 +821,6 @@ ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long 
     D.val = B.val = base + o_val;
     D.carry = B.carry = (u64 *)(base + o_carry);
     D.count = B.count = (u32 *)(base + o_count);
-    D.xs = B.xs = (uint4 *)(base + o_xs);
     D.ncols = ncols;
     for (int c = 0; c <= kBlockClasses; ++c) D.row0[c] = (u32)B.cls_row[c];
     D.nchunk = (u32)B.nchunk;
@@ -837,7 +859,7 @@ static bool capturing(cudaStream_t st)
     return true;
 }
 
-ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, cudaStream_t st, BlockPlan **out)
+ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, int lgx, cudaStream_t st, BlockPlan **out)
 {
     *out = nullptr;
     if (capturing(st)) return FFSPMV_ERR_CUDA;  // nothing can be allocated or copied now
@@ -845,7 +867,7 @@ ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, cudaS
     if (!nb) return FFSPMV_ERR_OOM;
     void *tmp = nullptr;
     const ffspmv_status r = build_block(*nb, transpose, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(),
-                                        h->h_val.data(), h->m, odd, st, tmp);
+                                        h->h_val.data(), h->m, odd, lgx, st, tmp);
     if (tmp) cudaFree(tmp);
     if (r != FFSPMV_OK && nb->arena) {
         cudaFree(nb->arena);
@@ -858,30 +880,58 @@ ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, cudaS
 
 void free_block_plan(BlockPlan *b)
 {
-    if (b && b->arena) cudaFree(b->arena);
+    if (!b) return;
+    if (b->arena) cudaFree(b->arena);
+    for (int k = 0; k < kBlockStagings; ++k)
+        if (b->xs[k] && k != b->lgx) cudaFree(b->xs[k]);
     delete b;
 }
 
-const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st)
+BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st)
 {
     BlockPlan *&b = h->block[transpose ? 1 : 0];
-    if (!b) make_block(h, transpose, false, st, &b);   // a layout that could not be made is not tried again
+    // a layout that could not be made is not tried again
+    if (!b) make_block(h, transpose, false, nvec ? staging_width(h->m <= 65536u, x, ldx, nvec) : -1, st, &b);
     return b && b->ok ? b : nullptr;
 }
 
-// Launches of one block of nvec vectors: a staging pass and the product per
-// kBlockVecs vectors; x is read in place where its rows already are whole
-// aligned 16-byte pieces of u32.
-static bool block_in_place(const BlockPlan &B, const u32 *x, long long ldx, int nv)
+std::string block_summary(const BlockPlan *b)
 {
-    return !B.small && nv % 4 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15u) == 0 && ldx / 4 < (1LL << 28);
+    if (!b || !b->ok) return "";
+    size_t staged = 0;
+    for (int k = 0; k < kBlockStagings; ++k)
+        if (b->xs[k]) staged += ((size_t)b->ncols << k) * sizeof(uint4);
+    char buf[160];
+    snprintf(buf, sizeof buf, "  blocks: rows in length classes, %lld in %lld chunks, %s values, %zu bytes of staged rows of X\n",
+             b->nlong, b->nchunk, b->small ? "u16" : "u32", staged);
+    return buf;
+}
+
+bool block_staging(BlockPlan &B, const u32 *x, long long ldx, int nvec, cudaStream_t st, uint4 **xs)
+{
+    *xs = nullptr;
+    const int lg = staging_width(B.small, x, ldx, nvec);
+    if (lg < 0 || B.ncols == 0) return true;
+    for (int k = lg; k < kBlockStagings; ++k)
+        if (B.xs[k]) {
+            *xs = B.xs[k];
+            return true;
+        }
+    if (capturing(st)) return false;
+    if (cudaMalloc((void **)&B.xs[lg], ((size_t)B.ncols << lg) * sizeof(uint4)) != cudaSuccess) {
+        cudaGetLastError();
+        B.xs[lg] = nullptr;
+        return false;
+    }
+    *xs = B.xs[lg];
+    return true;
 }
 
 long long block_launches(const BlockPlan &B, int nvec)
 {
     long long n = 0;
     for (int v0 = 0; v0 < nvec; v0 += kBlockVecs)
-        n += block_in_place(B, nullptr, nvec, std::min(kBlockVecs, nvec - v0)) ? 1 : 2;
+        n += block_in_place(B.small, nullptr, nvec, std::min(kBlockVecs, nvec - v0)) ? 1 : 2;
     return n;
 }
 
@@ -936,8 +986,8 @@ static long long block_warps(const BlockPlan &B, BlockArgs &a)
     return warps;
 }
 
-ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec, u32 m,
-                        u32 alpha, u32 beta, cudaStream_t st)
+ffspmv_status run_block(const BlockPlan &B, uint4 *xs, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec,
+                        u32 m, u32 alpha, u32 beta, cudaStream_t st)
 {
     const int C = B.small ? 8 : 4;
     for (int v0 = 0; v0 < nvec; v0 += kBlockVecs) {
@@ -946,21 +996,21 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
         u32 *yv = y + v0;
         BlockArgs a = block_args(B, yv, ldy, nv, m, alpha, beta);
         const int pieces = (nv + C - 1) / C;
-        const bool in_place = block_in_place(B, xv, ldx, nv);
+        const bool in_place = block_in_place(B.small, xv, ldx, nv);
         if (in_place) {
             a.m.xs = reinterpret_cast<const uint4 *>(xv);
             a.m.pitch = (int)(ldx / 4);
         } else {
-            a.m.xs = B.xs;
+            a.m.xs = xs;
             a.m.pitch = pieces;
             const long long words = B.ncols * pieces;
             const int vec4 = (ldx % 4 == 0 && ((uintptr_t)xv & 15u) == 0) ? 1 : 0;
             if (words > 0) {
                 const unsigned blocks = (unsigned)((words + kBlockThreads - 1) / kBlockThreads);
                 if (B.small)
-                    k_block_stage<true><<<blocks, kBlockThreads, 0, st>>>(xv, ldx, B.ncols, nv, pieces, vec4, B.xs);
+                    k_block_stage<true><<<blocks, kBlockThreads, 0, st>>>(xv, ldx, B.ncols, nv, pieces, vec4, xs);
                 else
-                    k_block_stage<false><<<blocks, kBlockThreads, 0, st>>>(xv, ldx, B.ncols, nv, pieces, vec4, B.xs);
+                    k_block_stage<false><<<blocks, kBlockThreads, 0, st>>>(xv, ldx, B.ncols, nv, pieces, vec4, xs);
                 FF_CUDA(cudaGetLastError());
             }
         }
@@ -983,8 +1033,8 @@ ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y,
 
 // Y_j = A_j X_j for `count` (at most kMany) different plans, contiguous blocks
 // of nvec[j] <= kBlockVecs vectors.
-static ffspmv_status block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
-                                cudaStream_t st)
+static ffspmv_status block_many(int count, const BlockPlan *const *B, uint4 *const *xs, const u32 *const *x, u32 *const *y,
+                                const int *nvec, cudaStream_t st)
 {
     BlockMany P, S;   // the products, and the staging of the X that are not read in place
     memset(&P, 0, sizeof(P));
@@ -996,10 +1046,11 @@ static ffspmv_status block_many(int count, const BlockPlan *const *B, const u32 
         int lgt = 0;
         while ((1 << lgt) < pieces) ++lgt;
         P.dev[j] = b.dev;
+        P.place[j] = block_in_place(b.small, x[j], nvec[j], nvec[j]) ? 1 : 0;
         P.x[j] = x[j];
+        P.xs[j] = xs[j];
         P.y[j] = y[j];
         P.nvec[j] = (unsigned char)nvec[j];
-        P.place[j] = block_in_place(b, x[j], nvec[j], nvec[j]) ? 1 : 0;
         P.first[j] = (u32)warps;
         warps += b.nchunk;
         for (int c = 0; c < kBlockClasses; ++c) {
@@ -1009,6 +1060,7 @@ static ffspmv_status block_many(int count, const BlockPlan *const *B, const u32 
         if (!P.place[j] && b.ncols > 0) {
             S.dev[S.count] = b.dev;
             S.x[S.count] = x[j];
+            S.xs[S.count] = xs[j];
             S.nvec[S.count] = (unsigned char)nvec[j];
             S.first[S.count++] = (u32)stage;
             stage += (b.ncols * pieces + kBlockThreads - 1) / kBlockThreads;
@@ -1036,11 +1088,11 @@ static ffspmv_status block_many(int count, const BlockPlan *const *B, const u32 
     return FFSPMV_OK;
 }
 
-ffspmv_status run_block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
-                             cudaStream_t st)
+ffspmv_status run_block_many(int count, const BlockPlan *const *B, uint4 *const *xs, const u32 *const *x, u32 *const *y,
+                             const int *nvec, cudaStream_t st)
 {
     for (int c0 = 0; c0 < count; c0 += kMany) {
-        const ffspmv_status r = block_many(std::min(kMany, count - c0), B + c0, x + c0, y + c0, nvec + c0, st);
+        const ffspmv_status r = block_many(std::min(kMany, count - c0), B + c0, xs + c0, x + c0, y + c0, nvec + c0, st);
         if (r != FFSPMV_OK) return r;
     }
     return FFSPMV_OK;

@@ -25,6 +25,8 @@ __host__ __device__ inline int block_lgg(int i, int lgt)
 
 struct BlockDev;   // what a launch over many matrices reads of each (block.cu)
 
+constexpr int kBlockStagings = 4;       // of 1, 2, 4 and 8 16-byte pieces per row of X
+
 struct BlockPlan {
     bool ok = false;
     const BlockDev *dev = nullptr;
@@ -39,7 +41,11 @@ struct BlockPlan {
     const u32 *lrow = nullptr;         // [nlong] matrix rows
     const u32 *col = nullptr;
     const void *val = nullptr;
-    uint4 *xs = nullptr;               // staged rows of X
+    // Packed rows of X: buffer k holds rows of up to 2^k pieces.  Each is made
+    // for the first block that needs it and kept (a captured graph may name it):
+    // buffer lgx with the layout, in its allocation.
+    uint4 *xs[kBlockStagings] = {};
+    int lgx = -1;
     u32 quad1 = 0;                     // the one-quad class: row r at quad quad1 + r (mod 2^32)
     u64 *carry = nullptr;              // [nlong][kBlockVecs], zero between calls
     u32 *count = nullptr;              // [nlong] chunks arrived, zero between calls
@@ -47,26 +53,32 @@ struct BlockPlan {
 
 // A block layout of A or A^T, made on the device (synchronous); `odd`: of the
 // pattern of the odd values, padded with columns 2^32 - 1, without values and
-// without sums of long rows.  On
+// without sums of long rows; lgx: with packed rows of 2^lgx pieces (-1: none).  On
 // an error other than a stream under capture or no host memory *out is a plan
 // with ok = false.
-ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, cudaStream_t st, BlockPlan **out);
+ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, int lgx, cudaStream_t st, BlockPlan **out);
 void free_block_plan(BlockPlan *b);
 
 // The block layout of A (or A^T), built on first use from the handle's host
 // copy of the matrix (synchronous, one allocation); null while `st` is being
 // captured into a graph before that, or when the layout cannot be made (2^32
-// entries, no memory): the caller then takes the plan's own path.
-const BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, cudaStream_t st);
+// entries, no memory): the caller then takes the plan's own path.  A new layout comes with the staging for the block x (nvec
+// = 0: none).
+BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st);
 void free_block(ffspmv_handle *h);
+std::string block_summary(const BlockPlan *b);   // a line of spmv_describe_plan
+// The buffer for the packed rows of a block (null where all its rows are read
+// in place), allocated for the first block of that width.  False when it is not
+// there and cannot be made now (a capture, no memory): the plan's own path.
+bool block_staging(BlockPlan &B, const u32 *x, long long ldx, int nvec, cudaStream_t st, uint4 **xs);
 long long block_launches(const BlockPlan &B, int nvec);  // of a contiguous, 16-byte aligned block
-ffspmv_status run_block(const BlockPlan &B, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec, u32 m,
-                        u32 alpha, u32 beta, cudaStream_t st);
+ffspmv_status run_block(const BlockPlan &B, uint4 *xs, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec,
+                        u32 m, u32 alpha, u32 beta, cudaStream_t st);
 
 // Y_j = A_j X_j of different plans, one product launch per 512 of them:
-// contiguous blocks of nvec[j] <= 32 vectors.
-ffspmv_status run_block_many(int count, const BlockPlan *const *B, const u32 *const *x, u32 *const *y, const int *nvec,
-                             cudaStream_t st);
+// contiguous blocks of nvec[j] <= 32 vectors, each with its staging.
+ffspmv_status run_block_many(int count, const BlockPlan *const *B, uint4 *const *xs, const u32 *const *x, u32 *const *y,
+                             const int *nvec, cudaStream_t st);
 
 // nsteps >= 1 steps of a block sequence at m > 2^16, one launch each and one
 // more: S_i = X^T V_i (at S + i s s) and V_{i+1} = A V_i between V0 and V1 (n

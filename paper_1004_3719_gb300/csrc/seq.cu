@@ -683,7 +683,7 @@ ffspmv_status sequence_per_launch(ffspmv_handle *h, SeqState &q, const u32 *X, c
     const BlockPlan *B = nullptr;
     if (h->m > 65536u && n > 0 && h->opt.sequence_mode == 0 && h->opt.priority_format == FFSPMV_FMT_AUTO &&
         nsteps > 0 && !(h->opt.test_hooks & 12) && (h->block[0] || nsteps >= 16))
-        B = ensure_block(h, false, st);
+        B = ensure_block(h, false, nullptr, 0, 0, st);
     const int ldv = B ? (s + 3) / 4 * 4 : s;
     size_t vb = ((size_t)n * ldv * 4 + 255) / 256 * 256 + 256;
     size_t need = 2 * vb + std::max((size_t)s * s * 8, B ? block_steps_bytes(n, s) : 0) + 256;
