@@ -101,7 +101,9 @@ typedef struct {
                                   launch ends within a second (the status word read by
                                   spmv_check_status); bit 2 = x-panel blocks always take
                                   the 2- and 4-vector passes, without the timing that decides it;
-                                  bit 3 = x-panel blocks never take them (one-vector passes) */
+                                  bit 3 = x-panel blocks never take them (one-vector passes);
+                                  bit 4 = the first attempt at a block layout of A, and of A^T,
+                                  finds no device memory */
     int32_t panel_cluster;     /* x-panel layout: CTAs per cluster (column groups); 0 = chosen by
                                   the builder, 1, 2 or 4 to force one */
 } ffspmv_options;
@@ -139,7 +141,7 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
  * handle and direction, and one for the packed rows of X where a wider block
  * than before needs it.  A block runs by the handle's plan instead until the
  * layout is built, while its stream is captured without it, and where there is
- * no memory for it.
+ * no memory for it (which is asked for again by later blocks).
  * On a handle whose plan is the x-panel layout that is: passes of 4 vectors (m
  * <= 2^16) or 2, then 1.  Each pass reads the matrix once for all its vectors
  * (Sec. 2.5.1) on an x-panel layout built for that width; the first block

@@ -866,14 +866,20 @@ ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, int l
     BlockPlan *nb = new (std::nothrow) BlockPlan();
     if (!nb) return FFSPMV_ERR_OOM;
     void *tmp = nullptr;
-    const ffspmv_status r = build_block(*nb, transpose, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(),
-                                        h->h_val.data(), h->m, odd, lgx, st, tmp);
+    ffspmv_status r = FFSPMV_ERR_OOM;
+    if (!odd && (h->opt.test_hooks & 16) && !h->block[transpose ? 1 : 0]) {
+        // testing: the first attempt finds no memory
+    } else {
+        r = build_block(*nb, transpose, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(), h->h_val.data(), h->m,
+                        odd, lgx, st, tmp);
+    }
     if (tmp) cudaFree(tmp);
     if (r != FFSPMV_OK && nb->arena) {
         cudaFree(nb->arena);
         nb->arena = nullptr;
     }
     nb->ok = r == FFSPMV_OK;
+    nb->memory.short_of = r == FFSPMV_ERR_OOM;
     *out = nb;
     return r;
 }
@@ -890,9 +896,15 @@ void free_block_plan(BlockPlan *b)
 BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st)
 {
     BlockPlan *&b = h->block[transpose ? 1 : 0];
-    // a layout that could not be made is not tried again
-    if (!b) make_block(h, transpose, false, nvec ? staging_width(h->m <= 65536u, x, ldx, nvec) : -1, st, &b);
-    return b && b->ok ? b : nullptr;
+    if (b && b->ok) return b;
+    if (b && !b->memory.again()) return nullptr;   // cannot be made, or no memory a while ago
+    BlockPlan *nb = nullptr;
+    make_block(h, transpose, false, nvec ? staging_width(h->m <= 65536u, x, ldx, nvec) : -1, st, &nb);
+    if (!nb) return nullptr;
+    if (b) nb->memory.next(b->memory);
+    free_block_plan(b);
+    b = nb;
+    return b->ok ? b : nullptr;
 }
 
 std::string block_summary(const BlockPlan *b)
@@ -917,12 +929,15 @@ bool block_staging(BlockPlan &B, const u32 *x, long long ldx, int nvec, cudaStre
             *xs = B.xs[k];
             return true;
         }
-    if (capturing(st)) return false;
+    if (capturing(st) || (B.staging.short_of && !B.staging.again())) return false;
     if (cudaMalloc((void **)&B.xs[lg], ((size_t)B.ncols << lg) * sizeof(uint4)) != cudaSuccess) {
         cudaGetLastError();
         B.xs[lg] = nullptr;
+        B.staging.next(B.staging);
+        B.staging.short_of = true;
         return false;
     }
+    B.staging = BlockMemory();
     *xs = B.xs[lg];
     return true;
 }

@@ -27,8 +27,22 @@ struct BlockDev;   // what a launch over many matrices reads of each (block.cu)
 
 constexpr int kBlockStagings = 4;       // of 1, 2, 4 and 8 16-byte pieces per row of X
 
+// When to ask again for device memory that was not there: after 1, 2, 4, ...
+// (at most 1024) more calls.
+struct BlockMemory {
+    bool short_of = false;
+    int calls = 0, wait = 1;
+    bool again() { return short_of && ++calls >= wait; }
+    void next(const BlockMemory &before)   // asked again, in vain if short_of
+    {
+        calls = 0;
+        wait = before.wait < 1024 ? 2 * before.wait : before.wait;
+    }
+};
+
 struct BlockPlan {
     bool ok = false;
+    BlockMemory memory, staging;
     const BlockDev *dev = nullptr;
     void *arena = nullptr;
     long long n = 0, ncols = 0;
@@ -62,7 +76,8 @@ void free_block_plan(BlockPlan *b);
 // The block layout of A (or A^T), built on first use from the handle's host
 // copy of the matrix (synchronous, one allocation); null while `st` is being
 // captured into a graph before that, or when the layout cannot be made (2^32
-// entries, no memory): the caller then takes the plan's own path.  A new layout comes with the staging for the block x (nvec
+// entries; no memory, which is asked for again later): the caller then takes
+// the plan's own path.  A new layout comes with the staging for the block x (nvec
 // = 0: none).
 BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st);
 void free_block(ffspmv_handle *h);

@@ -1,5 +1,6 @@
 """Device memory of block layouts: what the packed rows of X take for the widths
-in use, widths that grow, and which blocks run on the layout at all."""
+in use, widths that grow, layouts that find no memory at first, and which blocks
+run on the layout at all."""
 import numpy as np
 import pytest
 
@@ -72,6 +73,23 @@ def test_captured_width_outlives_a_wider_block(lib):
     torch.cuda.synchronize()
     for v in X:
         assert np.array_equal(to_host(y[v]), oracle.csr_spmv(A, X[v])), v
+
+
+@pytest.mark.parametrize("m", [65521, 2**31 - 1])
+def test_no_memory_at_first(lib, m):
+    # test hook 16: the first attempt at each layout fails
+    A = gen.uniform_matrix(4, 3000, 2500, np.full(3000, 9), m)
+    M = lib.Matrix.from_csr(A, test_hooks=16)
+    B = lib.Matrix.from_csr(A, test_hooks=16, transpose_mode=lib.TRANSPOSE.NONE)
+    for k in range(4):
+        for transpose in (False, True):
+            check_apply(lib, M, A, nvec=9, alpha=3, beta=2, seed=k, transpose=transpose)
+        x, y = rand_block(k, A.ncols, 5, m), to_dev(np.zeros((A.nrows, 5), dtype=np.uint32))
+        lib.spmv_batch_apply([B.handle], [to_dev(x)], [y], [5])
+        assert np.array_equal(to_host(y), oracle.csr_spmv(A, x))
+        if k == 0:
+            assert not _staged(M) and not _staged(B)
+    assert len(_staged(M)) == 2 and len(_staged(B)) == 1
 
 
 @pytest.mark.parametrize("m", [251, 65521, 2**31 - 1, 2**32 - 5])
