@@ -137,9 +137,10 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
  * format the library chose (FFSPMV_FMT_AUTO) most blocks run on a layout of
  * their own, up to 32 vectors per pass, with the rows of X packed next to
  * each other.  The first such block (on a handle whose plan is not the x-panel
- * layout the second) builds it on the device: synchronous, one allocation per
- * handle and direction, and one for the packed rows of X where a wider block
- * than before needs it.  A block runs by the handle's plan instead until the
+ * layout the second) builds it on the device: the host waits for that, but for
+ * nothing else (the build has a stream of its own); one allocation per handle
+ * and direction, and one for the packed rows of X where a wider block than
+ * before needs it.  A block runs by the handle's plan instead until the
  * layout is built, while its stream is captured without it, and where there is
  * no memory for it (which is asked for again by later blocks).
  * On a handle whose plan is the x-panel layout that is: passes of 4 vectors (m

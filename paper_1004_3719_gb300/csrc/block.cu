@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <new>
 #include <string>
 #include <type_traits>
@@ -617,11 +618,12 @@ int staging_width(bool small, const u32 *x, long long ldx, int nvec)
 }
 
 // ---------------------------------------------------------------------------
-// The layout is made on the device from the CSR arrays: the lengths of the
-// output rows (of A: row offsets; of A^T: a histogram of the columns), the
-// rows and quads of each class, each row's place (a warp's rows of a class
-// take consecutive places, so rows stay nearly in order), then the entries.
-// The order of the entries of a row is free: sums mod m are exact.
+// Layouts are made on the device from the CSR arrays, any number at a time (a
+// job each, blockIdx.y): the lengths of the output rows (of A: row offsets; of
+// A^T: a histogram of the columns), the rows and quads of each class, each
+// row's place (a warp's rows of a class take consecutive places, so rows stay
+// nearly in order) with its padding, then the entries.  The order of the
+// entries of a row is free: sums mod m are exact.
 struct BlockBuild {
     const long long *ptr;   // CSR of A
     const u32 *col, *val;
@@ -631,15 +633,19 @@ struct BlockBuild {
     u32 *orow, *optr, *lrow, *ocol;
     uint4 *chunk;
     void *oval;
-    int small, odd;         // odd: the pattern of the odd values only, without values
+    int small, odd, transpose;   // odd: the pattern of the odd values only, without values
+    u32 rows, quads;        // of the layout, without and with the long rows
+    BlockDev dev, *dev_out;
 };
 
-__global__ void __launch_bounds__(kBlockThreads) k_block_lengths(const BlockBuild b, int transpose)
+__global__ void __launch_bounds__(kBlockThreads) k_block_lengths(const BlockBuild *__restrict__ jobs)
 {
+    const BlockBuild &b = jobs[blockIdx.y];
     const long long nth = (long long)gridDim.x * kBlockThreads, t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
-    if (!transpose && !b.odd) {
+    const int odd = b.odd;
+    if (!b.transpose && !odd) {
         for (long long i = t; i < b.nr; i += nth) b.len[i] = (u32)(b.ptr[i + 1] - b.ptr[i]);
-    } else if (!transpose) {
+    } else if (!b.transpose) {
         for (long long w = t >> 5; w < b.nr; w += nth >> 5) {   // a warp per row
             const long long e = b.ptr[w + 1];
             u32 c = 0;
@@ -650,20 +656,21 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_lengths(const BlockBuil
     } else {
         const long long nnz = b.ptr[b.nr];
         for (long long k = t; k < nnz; k += nth)
-            if (!b.odd || (b.val[k] & 1u)) atomicAdd(b.len + b.col[k], 1u);
+            if (!odd || (b.val[k] & 1u)) atomicAdd(b.len + b.col[k], 1u);
     }
 }
 
 // place = 0: the totals of every class into the cursors; place = 1: every row
 // to its place, the cursors holding the first places.
-__global__ void __launch_bounds__(kBlockThreads) k_block_place(const BlockBuild b, int place)
+__global__ void __launch_bounds__(kBlockThreads) k_block_place(const BlockBuild *__restrict__ jobs, int place)
 {
+    const BlockBuild &b = jobs[blockIdx.y];
     const int lane = threadIdx.x & 31;
-    const long long nw = (b.n + 31) / 32, step = (long long)gridDim.x * (kBlockThreads / 32);
+    const long long n = b.n, nw = (n + 31) / 32, step = (long long)gridDim.x * (kBlockThreads / 32);
     for (long long w = (long long)blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5); w < nw; w += step) {
         const long long i = w * 32 + lane;
-        const u32 len = i < b.n ? b.len[i] : 0u, quads = (u32)(((u64)len + 3u) / 4u);
-        const int c = i >= b.n ? -1 : len > (u32)kBlockLong ? kBlockClasses : block_class(quads);
+        const u32 len = i < n ? b.len[i] : 0u, quads = (u32)(((u64)len + 3u) / 4u);
+        const int c = i >= n ? -1 : len > (u32)kBlockLong ? kBlockClasses : block_class(quads);
         const u32 parts = c == kBlockClasses ? (u32)(((u64)len + kBlockLong - 1) / kBlockLong) : 0u;
         for (int k = 0; k <= kBlockClasses; ++k) {
             const u32 same = __ballot_sync(0xffffffffu, c == k);
@@ -687,8 +694,18 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_place(const BlockBuild 
             const u64 at = base + sum - mine;
             const u32 slot = (u32)(at >> 32), q = (u32)at;
             b.start[i] = q;
+            // padding entries (value 0, or no column)
+            for (size_t e = (size_t)q * 4 + len, end = ((size_t)q + quads) * 4; e < end; ++e) {
+                b.ocol[e] = b.odd ? 0xffffffffu : 0u;
+                if (b.odd) continue;
+                if (b.small) reinterpret_cast<unsigned short *>(b.oval)[e] = 0;
+                else reinterpret_cast<u32 *>(b.oval)[e] = 0u;
+            }
             if (k == kBlockClasses) {
                 b.lrow[slot] = (u32)i;
+                b.dev.count[slot] = 0u;
+                if (!b.odd)
+                    for (int v = 0; v < kBlockVecs; ++v) b.dev.carry[(size_t)slot * kBlockVecs + v] = 0;
                 const u64 c0 = atomicAdd(b.cursor + kBlockClasses + 1, (u64)parts);
                 for (u32 p = 0; p < parts; ++p)
                     b.chunk[c0 + p] = make_uint4(slot, q + p * (u32)(kBlockLong / 4),
@@ -701,157 +718,33 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_place(const BlockBuild 
     }
 }
 
-__global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild b, int transpose)
+__global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild *__restrict__ jobs)
 {
+    const BlockBuild &b = jobs[blockIdx.y];
     const int lane = threadIdx.x & 31;
+    const int transpose = b.transpose, odd = b.odd, small = b.small;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && b.dev_out) {
+        *b.dev_out = b.dev;
+        b.optr[b.rows] = b.quads;
+    }
     const long long step = (long long)gridDim.x * (kBlockThreads / 32);
     for (long long i = (long long)blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5); i < b.nr; i += step) {
         const long long s = b.ptr[i], e = b.ptr[i + 1];
         for (long long k = s + lane; k < e; k += 32) {
             const u32 j = b.col[k], v = b.val[k];
-            if (b.odd && !(v & 1u)) continue;
+            if (odd && !(v & 1u)) continue;
             const u32 r = transpose ? j : (u32)i;
             const size_t to = (size_t)b.start[r] * 4 +
-                              (transpose || b.odd ? (size_t)(atomicSub(b.len + r, 1u) - 1u) : (size_t)(k - s));
+                              (transpose || odd ? (size_t)(atomicSub(b.len + r, 1u) - 1u) : (size_t)(k - s));
             b.ocol[to] = transpose ? (u32)i : j;
-            if (b.odd) continue;
-            if (b.small) reinterpret_cast<unsigned short *>(b.oval)[to] = (unsigned short)v;
+            if (odd) continue;
+            if (small) reinterpret_cast<unsigned short *>(b.oval)[to] = (unsigned short)v;
             else reinterpret_cast<u32 *>(b.oval)[to] = v;
         }
     }
 }
 
-// The block layout of A (nr x nc, values below m), or of A^T, with a buffer for
-// packed rows of 2^lgx pieces (lgx = -1: none).
-ffspmv_status build_block(BlockPlan &B, bool transpose, long long nr, long long nc, const long long *ptr, const int *col,
-                          const u32 *val, u32 m, bool odd, int lgx, cudaStream_t st, void *&tmp)
-{
-    const long long nnz = ptr[nr], n = transpose ? nc : nr, ncols = transpose ? nr : nc;
-    // offsets in quads and lengths of rows are 32-bit; with values, 32-bit row numbers are rounded up to a warp's
-    constexpr long long kLim = (1LL << 32) - 1;
-    if (nnz / 4 + std::min(n, nnz) >= kLim || (!odd && (nnz >= kLim || n >= kLim - 63))) return FFSPMV_ERR_UNSUPPORTED;
-    if (nnz >= kLim) {
-        std::vector<long long> len((size_t)n, 0);
-        for (long long i = 0; i < nr; ++i)
-            for (long long k = ptr[i]; k < ptr[i + 1]; ++k) ++len[transpose ? (size_t)col[k] : (size_t)i];
-        for (long long l : len)
-            if (l >= kLim) return FFSPMV_ERR_UNSUPPORTED;
-    }
-    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    size_t o = 0;
-    auto put = [&](size_t bytes) {
-        const size_t here = o;
-        o += al(std::max<size_t>(bytes, 16));
-        return here;
-    };
-    constexpr int kCur = kBlockClasses + 2;
-    const size_t t_ptr = put((size_t)(nr + 1) * 8), t_col = put((size_t)nnz * 4), t_val = put((size_t)nnz * 4),
-                 t_len = put((size_t)n * 4), t_start = put((size_t)n * 4), t_cur = put(kCur * 8);
-    if (cudaMalloc(&tmp, o) != cudaSuccess) {
-        cudaGetLastError();
-        tmp = nullptr;
-        return FFSPMV_ERR_OOM;
-    }
-    char *t = (char *)tmp;
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned grid = (unsigned)(8 * std::max(nsm, 1));
-    BlockBuild b;
-    memset(&b, 0, sizeof(b));
-    b.ptr = (const long long *)(t + t_ptr);
-    b.col = (const u32 *)(t + t_col);
-    b.val = (const u32 *)(t + t_val);
-    b.nr = nr;
-    b.n = n;
-    b.len = (u32 *)(t + t_len);
-    b.start = (u32 *)(t + t_start);
-    b.cursor = (u64 *)(t + t_cur);
-    b.small = m <= 65536u ? 1 : 0;
-    b.odd = odd ? 1 : 0;
-    u64 cur[kCur] = {};
-    FF_CUDA(cudaMemcpyAsync(t + t_ptr, ptr, (size_t)(nr + 1) * 8, cudaMemcpyHostToDevice, st));
-    if (nnz) {
-        FF_CUDA(cudaMemcpyAsync(t + t_col, col, (size_t)nnz * 4, cudaMemcpyHostToDevice, st));
-        FF_CUDA(cudaMemcpyAsync(t + t_val, val, (size_t)nnz * 4, cudaMemcpyHostToDevice, st));
-    }
-    FF_CUDA(cudaMemsetAsync(t + t_len, 0, o - t_len, st));
-    k_block_lengths<<<grid, kBlockThreads, 0, st>>>(b, transpose ? 1 : 0);
-    k_block_place<<<grid, kBlockThreads, 0, st>>>(b, 0);
-    FF_CUDA(cudaGetLastError());
-    FF_CUDA(cudaMemcpyAsync(cur, b.cursor, sizeof(cur), cudaMemcpyDeviceToHost, st));
-    FF_CUDA(cudaStreamSynchronize(st));
-    // the long rows' quads come first, then the classes, heaviest first
-    B.n = n;
-    B.ncols = ncols;
-    B.small = b.small != 0;
-    B.nlong = (long long)(cur[kBlockClasses] >> 32);
-    B.nchunk = (long long)cur[kBlockClasses + 1];
-    u64 quads = cur[kBlockClasses] & 0xffffffffull, rows = 0;
-    cur[kBlockClasses] = cur[kBlockClasses + 1] = 0;
-    for (int i = 0; i < kBlockClasses; ++i) {
-        const int c = kBlockClasses - 1 - i;
-        const u64 here = cur[c];
-        cur[c] = (rows << 32) + quads;
-        if (c == 1) B.quad1 = (u32)quads - (u32)rows;
-        rows += here >> 32;
-        quads += here & 0xffffffffull;
-        B.cls_row[i + 1] = (long long)rows;
-    }
-    const int vb = odd ? 0 : B.small ? 2 : 4;
-    o = 0;
-    const size_t o_ptr = put((size_t)(rows + 1) * 4), o_row = put((size_t)rows * 4), o_chunk = put((size_t)B.nchunk * 16),
-                 o_lrow = put((size_t)B.nlong * 4), o_col = put((size_t)quads * 16), o_val = put((size_t)quads * 4 * vb),
-                 o_carry = put((size_t)(odd ? 0 : B.nlong) * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
-                 o_dev = put(sizeof(BlockDev)), o_xs = put(lgx < 0 ? 0 : ((size_t)ncols << lgx) * sizeof(uint4));
-    if (cudaMalloc(&B.arena, o) != cudaSuccess) {
-        cudaGetLastError();
-        B.arena = nullptr;
-        return FFSPMV_ERR_OOM;
-    }
-    char *base = (char *)B.arena;
-    if (lgx >= 0) B.xs[B.lgx = lgx] = (uint4 *)(base + o_xs);
-    BlockDev D;
-    memset(&D, 0, sizeof(D));
-    D.ptr = B.ptr = (const u32 *)(base + o_ptr);
-    D.row = B.row = (const u32 *)(base + o_row);
-    D.chunk = B.chunk = (const uint4 *)(base + o_chunk);
-    D.lrow = B.lrow = (const u32 *)(base + o_lrow);
-    D.col = B.col = (const u32 *)(base + o_col);
-    D.val = B.val = base + o_val;
-    D.carry = B.carry = (u64 *)(base + o_carry);
-    D.count = B.count = (u32 *)(base + o_count);
-    D.ncols = ncols;
-    for (int c = 0; c <= kBlockClasses; ++c) D.row0[c] = (u32)B.cls_row[c];
-    D.nchunk = (u32)B.nchunk;
-    D.quad1 = B.quad1;
-    D.small = b.small;
-    D.fold = m <= (1u << 31) ? 1 : 0;
-    D.M = make_mod(m, 1, 0);
-    B.dev = (const BlockDev *)(base + o_dev);
-    b.optr = (u32 *)(base + o_ptr);
-    b.orow = (u32 *)(base + o_row);
-    b.chunk = (uint4 *)(base + o_chunk);
-    b.lrow = (u32 *)(base + o_lrow);
-    b.ocol = (u32 *)(base + o_col);
-    b.oval = base + o_val;
-    const u32 end = (u32)quads;
-    FF_CUDA(cudaMemcpyAsync(b.cursor, cur, sizeof(cur), cudaMemcpyHostToDevice, st));
-    FF_CUDA(cudaMemcpyAsync(b.optr + rows, &end, 4, cudaMemcpyHostToDevice, st));
-    FF_CUDA(cudaMemcpyAsync(base + o_dev, &D, sizeof(D), cudaMemcpyHostToDevice, st));
-    // padding entries (value 0, or no column), sums and counts of long rows
-    FF_CUDA(cudaMemsetAsync(base + o_col, odd ? 0xff : 0, o_val - o_col, st));
-    FF_CUDA(cudaMemsetAsync(base + o_val, 0, o_dev - o_val, st));
-    k_block_place<<<grid, kBlockThreads, 0, st>>>(b, 1);
-    k_block_fill<<<grid, kBlockThreads, 0, st>>>(b, transpose ? 1 : 0);
-    FF_CUDA(cudaGetLastError());
-    FF_CUDA(cudaStreamSynchronize(st));
-    return FFSPMV_OK;
-}
-
-}  // namespace
-
-static bool capturing(cudaStream_t st)
+bool capturing(cudaStream_t st)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) return false;
@@ -859,29 +752,268 @@ static bool capturing(cudaStream_t st)
     return true;
 }
 
+// A layout to be made: of A (nr x nc, values below m), or of A^T, with a buffer
+// for packed rows of 2^lgx pieces (lgx = -1: none).
+struct BlockJob {
+    BlockPlan *B;
+    const ffspmv_handle *h;
+    bool transpose, odd;
+    int lgx;
+    ffspmv_status st;
+};
+
+ffspmv_status block_limits(const BlockJob &J)
+{
+    const long long nr = J.h->A.nrows, *ptr = J.h->h_ptr.data(), nnz = ptr[nr], n = J.transpose ? J.h->A.ncols : nr;
+    const int *col = J.h->h_col.data();
+    // offsets in quads and lengths of rows are 32-bit; with values, 32-bit row numbers are rounded up to a warp's
+    constexpr long long kLim = (1LL << 32) - 1;
+    if (nnz / 4 + std::min(n, nnz) >= kLim || (!J.odd && (nnz >= kLim || n >= kLim - 63))) return FFSPMV_ERR_UNSUPPORTED;
+    if (nnz >= kLim) {
+        std::vector<long long> len((size_t)n, 0);
+        for (long long i = 0; i < nr; ++i)
+            for (long long k = ptr[i]; k < ptr[i + 1]; ++k) ++len[J.transpose ? (size_t)col[k] : (size_t)i];
+        for (long long l : len)
+            if (l >= kLim) return FFSPMV_ERR_UNSUPPORTED;
+    }
+    return FFSPMV_OK;
+}
+
+// What a build holds: a stream of its own, so that nothing waits for the
+// caller's, temporary memory in that stream's order (a cudaFree would wait for
+// all of them), and this thread's leave to allocate while another stream is
+// being captured.
+struct BlockScope {
+    cudaStream_t st = nullptr;
+    void *tmp = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BlockScope() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BlockScope()
+    {
+        if (tmp) cudaFreeAsync(tmp, st);
+        if (st) {
+            cudaStreamSynchronize(st);
+            cudaStreamDestroy(st);
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+};
+
+constexpr int kBlockCursors = kBlockClasses + 2;
+constexpr size_t kBlockAlign = 256;
+size_t block_round(size_t b) { return (std::max<size_t>(b, 16) + kBlockAlign - 1) / kBlockAlign * kBlockAlign; }
+
+// The layouts of all the jobs (within the limits), with two synchronisations of
+// the build's stream in all.  Arrays below kPack bytes go up together.
+ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
+{
+    constexpr size_t kPack = 256 * 1024;
+    FF_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
+    cudaStream_t st = S.st;
+    std::vector<BlockBuild> b((size_t)count);
+    memset(b.data(), 0, sizeof(BlockBuild) * b.size());
+    // [jobs][cursors][small arrays] (one copy), [large arrays], [lengths], [first quads]
+    const size_t o_cur = block_round(sizeof(BlockBuild) * b.size()),
+                 head = o_cur + block_round(sizeof(u64) * kBlockCursors * b.size());
+    struct Array {
+        const void *src;
+        size_t bytes, at;
+    };
+    std::vector<Array> arr((size_t)3 * count);
+    for (int j = 0; j < count; ++j) {
+        const ffspmv_handle &h = *jobs[j].h;
+        arr[3 * j] = {h.h_ptr.data(), h.h_ptr.size() * 8, 0};
+        arr[3 * j + 1] = {h.h_col.data(), h.h_col.size() * 4, 0};
+        arr[3 * j + 2] = {h.h_val.data(), h.h_val.size() * 4, 0};
+    }
+    size_t o = head;
+    for (Array &a : arr)
+        if (a.bytes < kPack) {
+            a.at = o;
+            o += block_round(a.bytes);
+        }
+    const size_t packed = o;
+    for (Array &a : arr)
+        if (a.bytes >= kPack) {
+            a.at = o;
+            o += block_round(a.bytes);
+        }
+    const size_t o_len = o;
+    long long most = 1;
+    std::vector<size_t> lens((size_t)count), starts((size_t)count);
+    for (int pass = 0; pass < 2; ++pass)
+        for (int j = 0; j < count; ++j) {
+            const long long n = jobs[j].transpose ? jobs[j].h->A.ncols : jobs[j].h->A.nrows;
+            (pass ? starts : lens)[j] = o;
+            o += block_round((size_t)n * 4);
+            most = std::max(most, std::max(n, jobs[j].h->A.nrows));
+        }
+    const size_t o_start = starts[0];
+    if (cudaMallocAsync(&S.tmp, o, st) != cudaSuccess) {
+        cudaGetLastError();
+        S.tmp = nullptr;
+        return FFSPMV_ERR_OOM;
+    }
+    char *t = (char *)S.tmp;
+    for (int j = 0; j < count; ++j) {
+        const BlockJob &J = jobs[j];
+        b[j].ptr = (const long long *)(t + arr[3 * j].at);
+        b[j].col = (const u32 *)(t + arr[3 * j + 1].at);
+        b[j].val = (const u32 *)(t + arr[3 * j + 2].at);
+        b[j].nr = J.h->A.nrows;
+        b[j].n = J.transpose ? J.h->A.ncols : J.h->A.nrows;
+        b[j].len = (u32 *)(t + lens[j]);
+        b[j].start = (u32 *)(t + starts[j]);
+        b[j].cursor = (u64 *)(t + o_cur) + (size_t)j * kBlockCursors;
+        b[j].small = J.h->m <= 65536u ? 1 : 0;
+        b[j].odd = J.odd ? 1 : 0;
+        b[j].transpose = J.transpose ? 1 : 0;
+    }
+    std::vector<char> up(packed, 0);
+    memcpy(up.data(), b.data(), sizeof(BlockBuild) * b.size());
+    for (const Array &a : arr)
+        if (a.bytes && a.bytes < kPack) memcpy(up.data() + a.at, a.src, a.bytes);
+    FF_CUDA(cudaMemcpyAsync(t, up.data(), packed, cudaMemcpyHostToDevice, st));
+    for (const Array &a : arr)
+        if (a.bytes >= kPack) FF_CUDA(cudaMemcpyAsync(t + a.at, a.src, a.bytes, cudaMemcpyHostToDevice, st));
+    FF_CUDA(cudaMemsetAsync(t + o_len, 0, o_start - o_len, st));
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const dim3 grid((unsigned)std::min<long long>(8 * std::max(nsm, 1), (most + 7) / 8), (unsigned)count);
+    const BlockBuild *dj = (const BlockBuild *)t;
+    k_block_lengths<<<grid, kBlockThreads, 0, st>>>(dj);
+    k_block_place<<<grid, kBlockThreads, 0, st>>>(dj, 0);
+    FF_CUDA(cudaGetLastError());
+    std::vector<u64> curs((size_t)kBlockCursors * count);
+    FF_CUDA(cudaMemcpyAsync(curs.data(), t + o_cur, sizeof(u64) * curs.size(), cudaMemcpyDeviceToHost, st));
+    FF_CUDA(cudaStreamSynchronize(st));
+    for (int j = 0; j < count; ++j) {
+        BlockJob &J = jobs[j];
+        BlockPlan &B = *J.B;
+        u64 *cur = curs.data() + (size_t)j * kBlockCursors;
+        const u32 m = J.h->m;
+        // the long rows' quads come first, then the classes, heaviest first
+        B.n = b[j].n;
+        B.ncols = J.transpose ? J.h->A.nrows : J.h->A.ncols;
+        B.small = b[j].small != 0;
+        B.nlong = (long long)(cur[kBlockClasses] >> 32);
+        B.nchunk = (long long)cur[kBlockClasses + 1];
+        u64 quads = cur[kBlockClasses] & 0xffffffffull, rows = 0;
+        cur[kBlockClasses] = cur[kBlockClasses + 1] = 0;
+        for (int i = 0; i < kBlockClasses; ++i) {
+            const int c = kBlockClasses - 1 - i;
+            const u64 here = cur[c];
+            cur[c] = (rows << 32) + quads;
+            if (c == 1) B.quad1 = (u32)quads - (u32)rows;
+            rows += here >> 32;
+            quads += here & 0xffffffffull;
+            B.cls_row[i + 1] = (long long)rows;
+        }
+        const int vb = J.odd ? 0 : B.small ? 2 : 4;
+        size_t a = 0;
+        auto put = [&](size_t bytes) {
+            const size_t here = a;
+            a += block_round(bytes);
+            return here;
+        };
+        const size_t o_ptr = put((size_t)(rows + 1) * 4), o_row = put((size_t)rows * 4), o_chunk = put((size_t)B.nchunk * 16),
+                     o_lrow = put((size_t)B.nlong * 4), o_col = put((size_t)quads * 16), o_val = put((size_t)quads * 4 * vb),
+                     o_carry = put((size_t)(J.odd ? 0 : B.nlong) * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
+                     o_dev = put(sizeof(BlockDev)),
+                     o_xs = put(J.lgx < 0 ? 0 : ((size_t)B.ncols << J.lgx) * sizeof(uint4));
+        if (cudaMalloc(&B.arena, a) != cudaSuccess) {
+            cudaGetLastError();
+            B.arena = nullptr;
+            J.st = FFSPMV_ERR_OOM;
+            b[j].nr = b[j].n = 0;   // (nothing to place)
+            continue;
+        }
+        char *base = (char *)B.arena;
+        if (J.lgx >= 0) B.xs[B.lgx = J.lgx] = (uint4 *)(base + o_xs);
+        BlockDev &D = b[j].dev;
+        D.ptr = B.ptr = (const u32 *)(base + o_ptr);
+        D.row = B.row = (const u32 *)(base + o_row);
+        D.chunk = B.chunk = (const uint4 *)(base + o_chunk);
+        D.lrow = B.lrow = (const u32 *)(base + o_lrow);
+        D.col = B.col = (const u32 *)(base + o_col);
+        D.val = B.val = base + o_val;
+        D.carry = B.carry = (u64 *)(base + o_carry);
+        D.count = B.count = (u32 *)(base + o_count);
+        D.ncols = B.ncols;
+        for (int c = 0; c <= kBlockClasses; ++c) D.row0[c] = (u32)B.cls_row[c];
+        D.nchunk = (u32)B.nchunk;
+        D.quad1 = B.quad1;
+        D.small = b[j].small;
+        D.fold = m <= (1u << 31) ? 1 : 0;
+        D.M = make_mod(m, 1, 0);
+        B.dev = (const BlockDev *)(base + o_dev);
+        b[j].dev_out = (BlockDev *)(base + o_dev);
+        b[j].optr = (u32 *)(base + o_ptr);
+        b[j].orow = (u32 *)(base + o_row);
+        b[j].chunk = (uint4 *)(base + o_chunk);
+        b[j].lrow = (u32 *)(base + o_lrow);
+        b[j].ocol = (u32 *)(base + o_col);
+        b[j].oval = base + o_val;
+        b[j].rows = (u32)rows;
+        b[j].quads = (u32)quads;
+    }
+    memcpy(up.data(), b.data(), sizeof(BlockBuild) * b.size());
+    memcpy(up.data() + o_cur, curs.data(), sizeof(u64) * curs.size());
+    FF_CUDA(cudaMemcpyAsync(t, up.data(), head, cudaMemcpyHostToDevice, st));
+    k_block_place<<<grid, kBlockThreads, 0, st>>>(dj, 1);
+    k_block_fill<<<grid, kBlockThreads, 0, st>>>(dj);
+    FF_CUDA(cudaGetLastError());
+    FF_CUDA(cudaStreamSynchronize(st));
+    return FFSPMV_OK;
+}
+
+// The jobs' layouts; every job's status, and that of its plan, set.
+void run_jobs(BlockJob *jobs, int count)
+{
+    for (int j = 0; j < count; ++j) jobs[j].st = FFSPMV_OK;
+    try {
+        BlockScope S;
+        const ffspmv_status r = build_blocks(jobs, count, S);
+        for (int j = 0; j < count && r != FFSPMV_OK; ++j) jobs[j].st = r;
+    } catch (const std::exception &) {
+        for (int j = 0; j < count; ++j) jobs[j].st = FFSPMV_ERR_OOM;
+    }
+    for (int j = 0; j < count; ++j) {
+        BlockPlan &B = *jobs[j].B;
+        B.ok = jobs[j].st == FFSPMV_OK;
+        B.memory.short_of = jobs[j].st == FFSPMV_ERR_OOM;
+        if (B.ok || !B.arena) continue;
+        cudaFree(B.arena);
+        B.arena = nullptr;
+        B.xs[B.lgx < 0 ? 0 : B.lgx] = nullptr;
+        B.lgx = -1;
+    }
+}
+
+}  // namespace
+
 ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, int lgx, cudaStream_t st, BlockPlan **out)
 {
     *out = nullptr;
     if (capturing(st)) return FFSPMV_ERR_CUDA;  // nothing can be allocated or copied now
     BlockPlan *nb = new (std::nothrow) BlockPlan();
     if (!nb) return FFSPMV_ERR_OOM;
-    void *tmp = nullptr;
-    ffspmv_status r = FFSPMV_ERR_OOM;
+    BlockJob J = {nb, h, transpose, odd, lgx, FFSPMV_OK};
+    try {
+        J.st = block_limits(J);
+    } catch (const std::exception &) {
+        J.st = FFSPMV_ERR_OOM;
+    }
     if (!odd && (h->opt.test_hooks & 16) && !h->block[transpose ? 1 : 0]) {
         // testing: the first attempt finds no memory
-    } else {
-        r = build_block(*nb, transpose, h->A.nrows, h->A.ncols, h->h_ptr.data(), h->h_col.data(), h->h_val.data(), h->m,
-                        odd, lgx, st, tmp);
+        J.st = FFSPMV_ERR_OOM;
+        nb->memory.short_of = true;
+    } else if (J.st == FFSPMV_OK) {
+        run_jobs(&J, 1);
     }
-    if (tmp) cudaFree(tmp);
-    if (r != FFSPMV_OK && nb->arena) {
-        cudaFree(nb->arena);
-        nb->arena = nullptr;
-    }
-    nb->ok = r == FFSPMV_OK;
-    nb->memory.short_of = r == FFSPMV_ERR_OOM;
     *out = nb;
-    return r;
+    return J.st;
 }
 
 void free_block_plan(BlockPlan *b)
@@ -930,6 +1062,7 @@ bool block_staging(BlockPlan &B, const u32 *x, long long ldx, int nvec, cudaStre
             return true;
         }
     if (capturing(st) || (B.staging.short_of && !B.staging.again())) return false;
+    BlockScope S;   // (another stream may be under capture)
     if (cudaMalloc((void **)&B.xs[lg], ((size_t)B.ncols << lg) * sizeof(uint4)) != cudaSuccess) {
         cudaGetLastError();
         B.xs[lg] = nullptr;
