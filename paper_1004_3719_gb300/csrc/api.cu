@@ -58,6 +58,7 @@ void destroy_handle(ffspmv_handle *h)
     free_sequence_state(h);
     free_gf2(h);
     free_block(h);
+    block_handles(-1);
     delete h;
 }
 
@@ -276,6 +277,7 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
 
     ffspmv_handle *h = new (std::nothrow) ffspmv_handle();
     if (!h) return FFSPMV_ERR_OOM;
+    block_handles(1);
     h->opt = o;
     h->m = modulus;
     h->transpose_mode = o.transpose_mode;
@@ -289,7 +291,9 @@ ffspmv_status spmv_create_hybrid(ffspmv_t *out, int64_t nrows, int64_t ncols,
     h->h_ptr.assign(ptr, ptr + nrows + 1);
     h->h_col.assign(cidx, cidx + nnz);
     h->h_val.resize((size_t)nnz);
-    for (long long k = 0; k < nnz; ++k) h->h_val[k] = vals[k] % modulus;
+    u32 odd = 1u;
+    for (long long k = 0; k < nnz; ++k) odd &= h->h_val[k] = vals[k] % modulus;
+    h->all_odd = odd != 0u;
     st = build_with_selector(h->A, nrows, ncols, ptr, cidx, vals, modulus, o);
     if (st == FFSPMV_OK && o.transpose_mode == FFSPMV_TRANSPOSE_EXPLICIT) {
         std::vector<long long> tptr;

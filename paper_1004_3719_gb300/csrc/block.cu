@@ -23,6 +23,7 @@
 #include <cstdio>
 #include <cstring>
 #include <exception>
+#include <mutex>
 #include <new>
 #include <string>
 #include <type_traits>
@@ -626,7 +627,7 @@ int staging_width(bool small, const u32 *x, long long ldx, int nvec)
 // entries of a row is free: sums mod m are exact.
 struct BlockBuild {
     const long long *ptr;   // CSR of A
-    const u32 *col, *val;
+    const u32 *col, *val;   // val null: all odd
     long long nr, n;        // rows of A, output rows
     u32 *len, *start;       // [n]: entries, first quad
     u64 *cursor;            // [kBlockClasses + 2]: (rows << 32) + quads of each class and of the long rows; chunks
@@ -642,7 +643,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_lengths(const BlockBuil
 {
     const BlockBuild &b = jobs[blockIdx.y];
     const long long nth = (long long)gridDim.x * kBlockThreads, t = (long long)blockIdx.x * kBlockThreads + threadIdx.x;
-    const int odd = b.odd;
+    const bool odd = b.odd && b.val;   // some of the values do not count
     if (!b.transpose && !odd) {
         for (long long i = t; i < b.nr; i += nth) b.len[i] = (u32)(b.ptr[i + 1] - b.ptr[i]);
     } else if (!b.transpose) {
@@ -722,7 +723,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild *
 {
     const BlockBuild &b = jobs[blockIdx.y];
     const int lane = threadIdx.x & 31;
-    const int transpose = b.transpose, odd = b.odd, small = b.small;
+    const bool transpose = b.transpose != 0, small = b.small != 0, values = b.odd == 0, odd = !values && b.val;
     if (blockIdx.x == 0 && threadIdx.x == 0 && b.dev_out) {
         *b.dev_out = b.dev;
         b.optr[b.rows] = b.quads;
@@ -731,13 +732,13 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_fill(const BlockBuild *
     for (long long i = (long long)blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5); i < b.nr; i += step) {
         const long long s = b.ptr[i], e = b.ptr[i + 1];
         for (long long k = s + lane; k < e; k += 32) {
-            const u32 j = b.col[k], v = b.val[k];
+            const u32 j = b.col[k], v = values || odd ? b.val[k] : 1u;
             if (odd && !(v & 1u)) continue;
             const u32 r = transpose ? j : (u32)i;
             const size_t to = (size_t)b.start[r] * 4 +
                               (transpose || odd ? (size_t)(atomicSub(b.len + r, 1u) - 1u) : (size_t)(k - s));
             b.ocol[to] = transpose ? (u32)i : j;
-            if (odd) continue;
+            if (!values) continue;
             if (small) reinterpret_cast<unsigned short *>(b.oval)[to] = (unsigned short)v;
             else reinterpret_cast<u32 *>(b.oval)[to] = v;
         }
@@ -778,6 +779,70 @@ ffspmv_status block_limits(const BlockJob &J)
     }
     return FFSPMV_OK;
 }
+
+// Uploads of a handle's arrays go through page-locked memory: the copy engine
+// reads pageable memory page by page, and where the host's pages are small (a
+// machine that has been up for a while) that is 3 GB/s: 126 MB of a 15.8M-entry
+// matrix took 1.6 ms to 45 ms.  Through two slots of kUpSlot bytes, filled by
+// the host while the other one is sent: 9 ms.  One buffer for the process,
+// taken in turn, given back with the last handle.
+constexpr size_t kUpSlot = 2 << 20, kUpDirect = 64 * 1024;   // smaller copies leave the host's memory at once
+
+struct BlockRing {
+    std::mutex use;
+    long long handles = 0;
+    char *buf = nullptr;
+};
+BlockRing &block_ring()
+{
+    static BlockRing *r = new BlockRing();   // (outlives the handles of a process that ends without freeing them)
+    return *r;
+}
+
+class BlockUpload {
+    std::unique_lock<std::mutex> lock;
+    cudaStream_t st;
+    cudaEvent_t sent[2] = {nullptr, nullptr};
+    char *buf = nullptr;
+    int slot = 0;
+
+public:
+    BlockUpload(cudaStream_t s, size_t bytes) : st(s)
+    {
+        if (bytes < kUpDirect) return;
+        BlockRing &R = block_ring();
+        lock = std::unique_lock<std::mutex>(R.use);
+        if (!R.buf && cudaHostAlloc((void **)&R.buf, 2 * kUpSlot, cudaHostAllocPortable) != cudaSuccess) R.buf = nullptr;
+        if (R.buf && cudaEventCreateWithFlags(&sent[0], cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventCreateWithFlags(&sent[1], cudaEventDisableTiming) == cudaSuccess)
+            buf = R.buf;
+        cudaGetLastError();   // (without it: ordinary copies)
+    }
+    ~BlockUpload()
+    {
+        if (buf) cudaStreamSynchronize(st);   // the next build may fill the slots
+        for (cudaEvent_t e : sent)
+            if (e) cudaEventDestroy(e);
+    }
+    BlockUpload(const BlockUpload &) = delete;
+    ffspmv_status copy(void *dst, const void *src, size_t bytes)
+    {
+        if (!bytes) return FFSPMV_OK;
+        if (!buf || bytes < kUpDirect) {
+            FF_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st));
+            return FFSPMV_OK;
+        }
+        for (size_t at = 0; at < bytes; at += kUpSlot, slot ^= 1) {
+            const size_t n = std::min(kUpSlot, bytes - at);
+            char *h = buf + slot * kUpSlot;
+            FF_CUDA(cudaEventSynchronize(sent[slot]));   // (never recorded: done)
+            memcpy(h, (const char *)src + at, n);
+            FF_CUDA(cudaMemcpyAsync((char *)dst + at, h, n, cudaMemcpyHostToDevice, st));
+            FF_CUDA(cudaEventRecord(sent[slot], st));
+        }
+        return FFSPMV_OK;
+    }
+};
 
 // What a build holds: a stream of its own, so that nothing waits for the
 // caller's, temporary memory in that stream's order (a cudaFree would wait for
@@ -824,7 +889,8 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
         const ffspmv_handle &h = *jobs[j].h;
         arr[3 * j] = {h.h_ptr.data(), h.h_ptr.size() * 8, 0};
         arr[3 * j + 1] = {h.h_col.data(), h.h_col.size() * 4, 0};
-        arr[3 * j + 2] = {h.h_val.data(), h.h_val.size() * 4, 0};
+        // (a pattern of odd values needs none of them when all are)
+        arr[3 * j + 2] = {h.h_val.data(), jobs[j].odd && h.all_odd ? 0 : h.h_val.size() * 4, 0};
     }
     size_t o = head;
     for (Array &a : arr)
@@ -859,7 +925,7 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
         const BlockJob &J = jobs[j];
         b[j].ptr = (const long long *)(t + arr[3 * j].at);
         b[j].col = (const u32 *)(t + arr[3 * j + 1].at);
-        b[j].val = (const u32 *)(t + arr[3 * j + 2].at);
+        b[j].val = arr[3 * j + 2].bytes ? (const u32 *)(t + arr[3 * j + 2].at) : nullptr;
         b[j].nr = J.h->A.nrows;
         b[j].n = J.transpose ? J.h->A.ncols : J.h->A.nrows;
         b[j].len = (u32 *)(t + lens[j]);
@@ -873,9 +939,11 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
     memcpy(up.data(), b.data(), sizeof(BlockBuild) * b.size());
     for (const Array &a : arr)
         if (a.bytes && a.bytes < kPack) memcpy(up.data() + a.at, a.src, a.bytes);
-    FF_CUDA(cudaMemcpyAsync(t, up.data(), packed, cudaMemcpyHostToDevice, st));
+    BlockUpload to_device(st, o);
+    ffspmv_status r = to_device.copy(t, up.data(), packed);
     for (const Array &a : arr)
-        if (a.bytes >= kPack) FF_CUDA(cudaMemcpyAsync(t + a.at, a.src, a.bytes, cudaMemcpyHostToDevice, st));
+        if (r == FFSPMV_OK && a.bytes >= kPack) r = to_device.copy(t + a.at, a.src, a.bytes);
+    if (r != FFSPMV_OK) return r;
     FF_CUDA(cudaMemsetAsync(t + o_len, 0, o_start - o_len, st));
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
@@ -1014,6 +1082,17 @@ ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, int l
     }
     *out = nb;
     return J.st;
+}
+
+void block_handles(int more)
+{
+    BlockRing &R = block_ring();
+    std::lock_guard<std::mutex> use(R.use);
+    R.handles += more;
+    if (R.handles == 0 && R.buf) {
+        cudaFreeHost(R.buf);
+        R.buf = nullptr;
+    }
 }
 
 void free_block_plan(BlockPlan *b)

@@ -81,6 +81,7 @@ void free_block_plan(BlockPlan *b);
 // = 0: none).
 BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st);
 void free_block(ffspmv_handle *h);
+void block_handles(int more);   // a handle was made (1) or freed (-1)
 std::string block_summary(const BlockPlan *b);   // a line of spmv_describe_plan
 // The buffer for the packed rows of a block (null where all its rows are read
 // in place), allocated for the first block of that width.  False when it is not

@@ -320,6 +320,7 @@ struct ffspmv_handle {
     std::vector<long long> h_ptr;
     std::vector<int> h_col;
     std::vector<ff::u32> h_val;
+    bool all_odd = true;       // every value is odd
     // block sequence state
     void *seq_state = nullptr;
     int *d_status = nullptr;   // device status word (timeouts)

@@ -181,7 +181,7 @@ extern "C" ffspmv_status spmv_apply_gf2(ffspmv_t h, int32_t transpose, const uin
     cudaStream_t st = (cudaStream_t)stream;
     if (!h->gf2[transpose]) {
         BlockPlan *g = nullptr;
-        const ffspmv_status r = make_block(h, transpose != 0, true, -1, nullptr, &g);
+        const ffspmv_status r = make_block(h, transpose != 0, true, -1, st, &g);
         if (r != FFSPMV_OK) {
             free_block_plan(g);
             return r;

@@ -86,3 +86,21 @@ def test_layouts_of_many_shapes(lib, m, rows, cols, mean):
             M.launches(False, nvec)
             check_apply(lib, M, A, nvec=nvec, seed=k)
             check_apply(lib, M, A, nvec=nvec, alpha=3, beta=4, seed=k + 5, transpose=True)
+
+
+@pytest.mark.parametrize("even", [0, 1, 1000])
+@pytest.mark.parametrize("n,mean", [(300, 7), (40_000, 60)])
+def test_patterns_with_and_without_even_values(lib, n, mean, even):
+    """GF(2) patterns whose values are all odd go up without them; one even
+    value, or many, and they go up too.  Arrays below and above the upload's
+    slots (2 MB)."""
+    from oracle import gf2
+    A = gen.uniform_matrix(n + even, n, n + 9, np.full(n, mean), 2)
+    A.val[:] = 1
+    A.val[:even] = 0
+    A.val[-1] = 0 if even else 1
+    M = lib.Matrix.from_csr(A)
+    for transpose in (False, True):
+        x = gen.uniform_block(4, n if transpose else n + 9, 4, 2**32 - 1).view(np.uint64)
+        y = M.apply_gf2(x, transpose=transpose).cpu().numpy().view(np.uint64)
+        assert np.array_equal(y, gf2.csr_gf2(A, x, transpose))
