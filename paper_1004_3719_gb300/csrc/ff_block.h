@@ -80,6 +80,9 @@ void free_block_plan(BlockPlan *b);
 // the plan's own path.  A new layout comes with the staging for the block x (nvec
 // = 0: none).
 BlockPlan *ensure_block(ffspmv_handle *h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st);
+// The same for the A of several different handles, before a batch of contiguous
+// blocks: what is missing is built together.
+void ensure_blocks(int count, ffspmv_handle *const *hs, const u32 *const *x, const int *nvec, cudaStream_t st);
 void free_block(ffspmv_handle *h);
 void block_handles(int more);   // a handle was made (1) or freed (-1)
 std::string block_summary(const BlockPlan *b);   // a line of spmv_describe_plan

@@ -104,3 +104,27 @@ def test_patterns_with_and_without_even_values(lib, n, mean, even):
         x = gen.uniform_block(4, n if transpose else n + 9, 4, 2**32 - 1).view(np.uint64)
         y = M.apply_gf2(x, transpose=transpose).cpu().numpy().view(np.uint64)
         assert np.array_equal(y, gf2.csr_gf2(A, x, transpose))
+
+
+def test_layouts_of_a_batch_are_built_together(lib):
+    """Handles with and without a layout, empty ones, one that finds no memory at
+    first, moduli and widths mixed, more than one build's temporary memory (64
+    MB), and then the same again with what is there."""
+    import torch
+    shapes = [(0, 5, 0), (40, 0, 0), (300, 200, 9)] + [(50_000 + k, 40_000, 20) for k in range(9)] + [(17, 90_000, 1500)]
+    mats, hs = [], []
+    for k, (rows, cols, mean) in enumerate(shapes):
+        m = (65521, 2**31 - 1, 251, 2**32 - 5)[k % 4]
+        mats.append(gen.uniform_matrix(k, rows, cols, np.full(rows, mean), m, pm_fraction=0.1))
+        hs.append(lib.Matrix.from_csr(mats[-1], transpose_mode=lib.TRANSPOSE.NONE, test_hooks=16 if k == 5 else 0))
+    hs[3].launches(False, 32)       # (its layout may be there already)
+    for k in range(4):
+        nv = [1 + (7 * j + 3 * k) % 32 for j in range(len(hs))]
+        xs = [rand_block(k * 100 + j, A.ncols, v, A.modulus).reshape(A.ncols, v) for j, (A, v) in enumerate(zip(mats, nv))]
+        ys = [torch.full((A.nrows, v), -1, dtype=torch.int32, device="cuda") for A, v in zip(mats, nv)]
+        lib.spmv_batch_apply([h.handle for h in hs], [to_dev(x) for x in xs], ys, nv)
+        for j, A in enumerate(mats):
+            if A.nrows:
+                want = oracle.csr_spmv(A, xs[j]).reshape(A.nrows, nv[j]) if A.ncols else np.zeros((A.nrows, nv[j]), np.uint32)
+                assert np.array_equal(to_host(ys[j]), want), (k, j)
+    assert all("blocks:" in h.describe() for h, A in zip(hs, mats) if A.nrows)
