@@ -214,11 +214,12 @@ ffspmv_status spmv_block_project_finish(uint32_t p, int32_t s, uint64_t *d_Sacc,
  * modulus); d_x / d_y: host arrays of device pointers, X_j: ncols_j x nvec[j]
  * row-major (ld = nvec[j]), Y_j: nrows_j x nvec[j]; 1 <= nvec[j] <= 32.
  * The first batched (or block) product of a handle builds its block layout
- * (synchronous, one allocation per handle); after that a call
- * with any set of handles only launches: one product kernel per 512 matrices,
- * and one that packs the X_j which are not made of whole aligned 16-byte
- * pieces.  A handle may appear several times: its products then run one after
- * another.  Like the other products, calls that share a handle must not
+ * (the host waits for that; one allocation per handle, the missing layouts of a
+ * call together); after that a call with any set of handles only launches: one
+ * product kernel per 512 products, and one that packs the X_j which are not
+ * made of whole aligned 16-byte pieces.  A handle may appear several times: as
+ * many of its products as share its buffers (64 packed pieces per row, 64 MB;
+ * 32 vectors where it has rows above 512 entries) run at a time.  Like the other products, calls that share a handle must not
  * overlap on the GPU.
  */
 ffspmv_status spmv_batch_apply(int32_t count, const ffspmv_t *hs,

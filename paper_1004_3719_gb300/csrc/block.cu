@@ -370,7 +370,8 @@ __device__ __forceinline__ void block_chunk(const BlockMat &a, u32 w, int lane)
     u32 last = 0;
     __threadfence();
     __syncwarp();
-    if (lane == 0) last = atomicAdd(a.count + ch.x, 1u) == ch.w - 1u ? 1u : 0u;
+    u32 *count = a.count + (size_t)ch.x * kBlockVecs;
+    if (lane == 0) last = atomicAdd(count, 1u) == ch.w - 1u ? 1u : 0u;
     last = __shfl_sync(0xffffffffu, last, 0);
     if (!last) return;
     __threadfence();
@@ -380,7 +381,7 @@ __device__ __forceinline__ void block_chunk(const BlockMat &a, u32 w, int lane)
         *yp = combine(red64(__ldcg(cw + lane), a.M), yp, false, a.M);
         cw[lane] = 0;
     }
-    if (lane == 0) a.count[ch.x] = 0;
+    if (lane == 0) *count = 0;
 }
 
 // A warp's 32 / (T G) rows of a class: r0 the first, below rend, G = 2^lgg.
@@ -517,7 +518,8 @@ struct BlockMany {
     uint4 *xs[kMany];
     u32 *y[kMany];
     u32 first[kMany + 1];
-    unsigned char nvec[kMany], place[kMany];  // place: x is read where it lies, else packed in xs
+    unsigned char nvec[kMany];                // bit 7: x is read where it lies, else packed in xs
+    unsigned char v0[kMany];                  // first word of each long row's sums (a matrix that is there twice)
     int count;
 };
 static_assert(sizeof(BlockMany) < 32000, "launch parameters");
@@ -559,15 +561,15 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block_many(const __grid_co
     a.lrow = D.lrow;
     a.chunk = D.chunk;
     a.val = D.val;
-    a.carry = D.carry;
-    a.count = D.count;
+    a.carry = D.carry + P.v0[j];
+    a.count = D.count + P.v0[j];
     a.y = P.y[j];
-    a.nvec = P.nvec[j];
+    a.nvec = P.nvec[j] & 127;
     a.ldy = a.nvec;
     const int C = D.small ? 8 : 4;
     a.pieces = (a.nvec + C - 1) / C;
     a.lgt = a.pieces > 1 ? 32 - __clz(a.pieces - 1) : 0;
-    a.xs = P.place[j] ? reinterpret_cast<const uint4 *>(P.x[j]) : P.xs[j];
+    a.xs = P.nvec[j] & 128 ? reinterpret_cast<const uint4 *>(P.x[j]) : P.xs[j];
     a.pitch = a.pieces;
     a.vec4 = a.nvec % 4 == 0 && ((uintptr_t)a.y & 15u) == 0;
     a.quad1 = D.quad1;
@@ -704,9 +706,10 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_place(const BlockBuild 
             }
             if (k == kBlockClasses) {
                 b.lrow[slot] = (u32)i;
-                b.dev.count[slot] = 0u;
-                if (!b.odd)
-                    for (int v = 0; v < kBlockVecs; ++v) b.dev.carry[(size_t)slot * kBlockVecs + v] = 0;
+                for (int v = 0; v < kBlockVecs && !b.odd; ++v) {
+                    b.dev.carry[(size_t)slot * kBlockVecs + v] = 0;
+                    b.dev.count[(size_t)slot * kBlockVecs + v] = 0u;
+                }
                 const u64 c0 = atomicAdd(b.cursor + kBlockClasses + 1, (u64)parts);
                 for (u32 p = 0; p < parts; ++p)
                     b.chunk[c0 + p] = make_uint4(slot, q + p * (u32)(kBlockLong / 4),
@@ -994,7 +997,8 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
         };
         const size_t o_ptr = put((size_t)(rows + 1) * 4), o_row = put((size_t)rows * 4), o_chunk = put((size_t)B.nchunk * 16),
                      o_lrow = put((size_t)B.nlong * 4), o_col = put((size_t)quads * 16), o_val = put((size_t)quads * 4 * vb),
-                     o_carry = put((size_t)(J.odd ? 0 : B.nlong) * kBlockVecs * 8), o_count = put((size_t)B.nlong * 4),
+                     o_carry = put((size_t)(J.odd ? 0 : B.nlong) * kBlockVecs * 8),
+                     o_count = put((size_t)(J.odd ? 0 : B.nlong) * kBlockVecs * 4),
                      o_dev = put(sizeof(BlockDev)),
                      o_xs = put(J.lgx < 0 ? 0 : ((size_t)B.ncols << J.lgx) * sizeof(uint4));
         if (cudaMalloc(&B.arena, a) != cudaSuccess) {
@@ -1183,28 +1187,50 @@ std::string block_summary(const BlockPlan *b)
     return buf;
 }
 
-bool block_staging(BlockPlan &B, const u32 *x, long long ldx, int nvec, cudaStream_t st, uint4 **xs)
+// The staging buffer for 2^lg pieces per row.
+static uint4 *block_buffer(BlockPlan &B, int lg, cudaStream_t st)
 {
-    *xs = nullptr;
-    const int lg = staging_width(B.small, x, ldx, nvec);
-    if (lg < 0 || B.ncols == 0) return true;
     for (int k = lg; k < kBlockStagings; ++k)
-        if (B.xs[k]) {
-            *xs = B.xs[k];
-            return true;
-        }
-    if (capturing(st) || (B.staging.short_of && !B.staging.again())) return false;
+        if (B.xs[k]) return B.xs[k];
+    if (capturing(st) || (B.staging.short_of && !B.staging.again())) return nullptr;
     BlockScope S;   // (another stream may be under capture)
     if (cudaMalloc((void **)&B.xs[lg], ((size_t)B.ncols << lg) * sizeof(uint4)) != cudaSuccess) {
         cudaGetLastError();
         B.xs[lg] = nullptr;
         B.staging.next(B.staging);
         B.staging.short_of = true;
-        return false;
+        return nullptr;
     }
     B.staging = BlockMemory();
-    *xs = B.xs[lg];
-    return true;
+    return B.xs[lg];
+}
+
+bool block_staging(BlockPlan &B, const u32 *x, long long ldx, int nvec, cudaStream_t st, uint4 **xs)
+{
+    const int lg = staging_width(B.small, x, ldx, nvec);
+    *xs = lg < 0 || B.ncols == 0 ? nullptr : block_buffer(B, lg, st);
+    return lg < 0 || B.ncols == 0 || *xs;
+}
+
+int block_pieces(const BlockPlan &B, const u32 *x, int nvec)
+{
+    const int C = B.small ? 8 : 4;
+    return block_in_place(B.small, x, nvec, nvec) || B.ncols == 0 ? 0 : (nvec + C - 1) / C;
+}
+
+uint4 *block_staging(BlockPlan &B, int most, int total, cudaStream_t st, int *room)
+{
+    constexpr long long kWords = (64LL << 20) / sizeof(uint4);   // and 64 MB, or one block's
+    const int want = (int)std::max<long long>(most, std::min<long long>(std::min(total, kBlockPieces), kWords / B.ncols));
+    for (int p : {want, most}) {
+        int lg = 0;
+        while ((1 << lg) < p) ++lg;
+        if (uint4 *xs = block_buffer(B, lg, st)) {
+            *room = 1 << lg;
+            return xs;
+        }
+    }
+    return nullptr;
 }
 
 long long block_launches(const BlockPlan &B, int nvec)
@@ -1314,7 +1340,7 @@ ffspmv_status run_block(const BlockPlan &B, uint4 *xs, const u32 *x, long long l
 // Y_j = A_j X_j for `count` (at most kMany) different plans, contiguous blocks
 // of nvec[j] <= kBlockVecs vectors.
 static ffspmv_status block_many(int count, const BlockPlan *const *B, uint4 *const *xs, const u32 *const *x, u32 *const *y,
-                                const int *nvec, cudaStream_t st)
+                                const int *nvec, const int *v0, cudaStream_t st)
 {
     BlockMany P, S;   // the products, and the staging of the X that are not read in place
     memset(&P, 0, sizeof(P));
@@ -1326,18 +1352,19 @@ static ffspmv_status block_many(int count, const BlockPlan *const *B, uint4 *con
         int lgt = 0;
         while ((1 << lgt) < pieces) ++lgt;
         P.dev[j] = b.dev;
-        P.place[j] = block_in_place(b.small, x[j], nvec[j], nvec[j]) ? 1 : 0;
+        const bool place = block_in_place(b.small, x[j], nvec[j], nvec[j]);
         P.x[j] = x[j];
         P.xs[j] = xs[j];
         P.y[j] = y[j];
-        P.nvec[j] = (unsigned char)nvec[j];
+        P.nvec[j] = (unsigned char)(nvec[j] | (place ? 128 : 0));
+        P.v0[j] = (unsigned char)v0[j];
         P.first[j] = (u32)warps;
         warps += b.nchunk;
         for (int c = 0; c < kBlockClasses; ++c) {
             const int rpw = 1 << (5 - lgt - block_lgg(c, lgt));
             warps += (b.cls_row[c + 1] - b.cls_row[c] + rpw - 1) / rpw;
         }
-        if (!P.place[j] && b.ncols > 0) {
+        if (!place && b.ncols > 0) {
             S.dev[S.count] = b.dev;
             S.x[S.count] = x[j];
             S.xs[S.count] = xs[j];
@@ -1369,10 +1396,11 @@ static ffspmv_status block_many(int count, const BlockPlan *const *B, uint4 *con
 }
 
 ffspmv_status run_block_many(int count, const BlockPlan *const *B, uint4 *const *xs, const u32 *const *x, u32 *const *y,
-                             const int *nvec, cudaStream_t st)
+                             const int *nvec, const int *v0, cudaStream_t st)
 {
     for (int c0 = 0; c0 < count; c0 += kMany) {
-        const ffspmv_status r = block_many(std::min(kMany, count - c0), B + c0, xs + c0, x + c0, y + c0, nvec + c0, st);
+        const ffspmv_status r =
+            block_many(std::min(kMany, count - c0), B + c0, xs + c0, x + c0, y + c0, nvec + c0, v0 + c0, st);
         if (r != FFSPMV_OK) return r;
     }
     return FFSPMV_OK;

@@ -25,7 +25,8 @@ __host__ __device__ inline int block_lgg(int i, int lgt)
 
 struct BlockDev;   // what a launch over many matrices reads of each (block.cu)
 
-constexpr int kBlockStagings = 4;       // of 1, 2, 4 and 8 16-byte pieces per row of X
+constexpr int kBlockStagings = 7;       // of 1, 2, 4, ... 16-byte pieces per row of X: up to 8 for a block,
+constexpr int kBlockPieces = 1 << (kBlockStagings - 1);   // ... more for several blocks of a batch
 
 // When to ask again for device memory that was not there: after 1, 2, 4, ...
 // (at most 1024) more calls.
@@ -62,7 +63,7 @@ struct BlockPlan {
     int lgx = -1;
     u32 quad1 = 0;                     // the one-quad class: row r at quad quad1 + r (mod 2^32)
     u64 *carry = nullptr;              // [nlong][kBlockVecs], zero between calls
-    u32 *count = nullptr;              // [nlong] chunks arrived, zero between calls
+    u32 *count = nullptr;              // [nlong][kBlockVecs] chunks arrived, zero between calls
 };
 
 // A block layout of A or A^T, made on the device (synchronous); `odd`: of the
@@ -94,10 +95,18 @@ long long block_launches(const BlockPlan &B, int nvec);  // of a contiguous, 16-
 ffspmv_status run_block(const BlockPlan &B, uint4 *xs, const u32 *x, long long ldx, u32 *y, long long ldy, int nvec,
                         u32 m, u32 alpha, u32 beta, cudaStream_t st);
 
-// Y_j = A_j X_j of different plans, one product launch per 512 of them:
-// contiguous blocks of nvec[j] <= 32 vectors, each with its staging.
+// Pieces per packed row of a contiguous block; 0 where it is read in place.
+int block_pieces(const BlockPlan &B, const u32 *x, int nvec);
+// A staging buffer for several blocks of one plan at a time, of at most `most`
+// pieces each and `total` in all: with room for *room pieces, as many as up to
+// kBlockPieces and 64 MB allow (null: not there and cannot be made now).
+uint4 *block_staging(BlockPlan &B, int most, int total, cudaStream_t st, int *room);
+
+// Y_j = A_j X_j, one product launch per 512 of them: contiguous blocks of nvec[j]
+// <= 32 vectors, each with its staging.  Blocks of one plan need stagings of
+// their own and, where it has long rows, words v0[j] .. v0[j] + nvec[j] - 1 of 32.
 ffspmv_status run_block_many(int count, const BlockPlan *const *B, uint4 *const *xs, const u32 *const *x, u32 *const *y,
-                             const int *nvec, cudaStream_t st);
+                             const int *nvec, const int *v0, cudaStream_t st);
 
 // nsteps >= 1 steps of a block sequence at m > 2^16, one launch each and one
 // more: S_i = X^T V_i (at S + i s s) and V_{i+1} = A V_i between V0 and V1 (n
