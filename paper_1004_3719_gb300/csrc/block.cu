@@ -438,12 +438,14 @@ __global__ void __launch_bounds__(kBlockThreads, 4) k_block(const __grid_constan
 // one launch, both read V_i.  CTAs below `spmm` multiply; each of the next
 // `proj` projects its rows (four outputs of one row of S per thread, the
 // threads in groups that take every ngrp-th row) and writes its reduced sums;
-// one more adds up the sums of the step before and writes S_{i-1}, so that no
-// CTA waits for another.  V: rows of ldv words (a multiple of four, zero past
+// the last `fin` add up the sums of the step before, kStepOuts outputs each, and
+// write S_{i-1}, so that no CTA waits for another (one CTA for all 1 024 outputs
+// of s = 32 was the longest of the launch: 59 us per step at 4 001 rows).  V: rows of ldv words (a multiple of four, zero past
 // s).  A kernel lets the next one start once the one before it is complete.
+constexpr int kStepOuts = 64;
 struct BlockStep {
     BlockArgs b;
-    unsigned spmm, proj;      // CTAs of each kind
+    unsigned spmm, proj, fin; // CTAs of each kind
     int s, tiles, ngrp;       // tiles of four outputs, groups of threads
     long long n, ldv, per;    // rows, words per row of V, rows per projecting CTA
     const u32 *X, *V;
@@ -453,7 +455,7 @@ struct BlockStep {
 
 __global__ void __launch_bounds__(kBlockThreads, 3) k_block_step(const __grid_constant__ BlockStep a)
 {
-    __shared__ u32 red[4 * kBlockThreads];
+    __shared__ __align__(8) u32 red[4 * kBlockThreads];
     const int tid = threadIdx.x;
     if (blockIdx.x < a.spmm) {
         const u32 w = blockIdx.x * (kBlockThreads / 32) + (tid >> 5);
@@ -463,14 +465,23 @@ __global__ void __launch_bounds__(kBlockThreads, 3) k_block_step(const __grid_co
     }
     const Mod &M = a.b.m.M;
     const int outs = a.s * a.s;
-    if (blockIdx.x == gridDim.x - 1) {
+    if (blockIdx.x >= gridDim.x - a.fin) {
+        // an output's sums by kBlockThreads / kStepOuts threads
+        constexpr int kParts = kBlockThreads / kStepOuts;
+        const int o = (int)(blockIdx.x - (gridDim.x - a.fin)) * kStepOuts + tid % kStepOuts;
+        u64 *part = reinterpret_cast<u64 *>(red), sum = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (!a.prev) return;
-        for (int o = tid; o < outs; o += kBlockThreads) {
-            u64 sum = 0;
+        if (o < outs) {
 #pragma unroll 8
-            for (unsigned c = 0; c < a.proj; ++c) sum += __ldcg(a.prev + (size_t)c * outs + o);
+            for (unsigned c = tid / kStepOuts; c < a.proj; c += kParts) sum += __ldcg(a.prev + (size_t)c * outs + o);
+        }
+        part[tid] = sum;
+        __syncthreads();
+        if (tid < kStepOuts && o < outs) {
+#pragma unroll
+            for (int k = 1; k < kParts; ++k) sum += part[k * kStepOuts + tid];
             a.S[o] = red64(sum, M);
         }
         return;
@@ -1431,6 +1442,7 @@ ffspmv_status run_block_steps(const BlockPlan &B, long long n, int s, u32 m, con
     a.ldv = ldv;
     a.X = X;
     a.proj = step_proj(n, s);
+    a.fin = (unsigned)((s * s + kStepOuts - 1) / kStepOuts);
     a.per = (n + a.proj - 1) / a.proj;
     u32 *parts[2] = {part, part + (size_t)a.proj * s * s};
     for (long long i = 0; i <= nsteps; ++i) {
@@ -1445,7 +1457,7 @@ ffspmv_status run_block_steps(const BlockPlan &B, long long n, int s, u32 m, con
         a.prev = i ? parts[(i + 1) & 1] : nullptr;
         a.S = i ? S + (i - 1) * s * s : nullptr;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(a.spmm + (i < nsteps ? a.proj : 0u) + 1u);
+        cfg.gridDim = dim3(a.spmm + (i < nsteps ? a.proj : 0u) + a.fin);
         cfg.blockDim = dim3(kBlockThreads);
         cfg.stream = st;
         cudaLaunchAttribute at[1];
