@@ -56,6 +56,7 @@ constexpr int kMaxEnt = 16;                       // entries per row
 constexpr int kSeqBatch = 5;                      // entry pairs gathered together per lane
 constexpr int kSeqTiles = 3;                      // groups that a warp forms before it projects them
 constexpr int kSeqBufs = 3;                       // partial projections in flight
+constexpr long long kSeqBuildSteps = 48;          // steps for which a block layout is built (p > 2^16)
 constexpr int kVsStride = 24;                     // halves per staged row (no bank conflicts for ldmatrix)
 constexpr unsigned kDefaultSpins = 1u << 22;      // x <= 64 ns sleeps: well under a second
 
@@ -544,7 +545,8 @@ struct SeqState {
     u32 *partial = nullptr;
     unsigned *bar = nullptr;
     int nblocks = 0;
-    // per-launch path buffers
+    // per-launch path buffers, and the steps it was asked for
+    long long steps = 0;
     void *gwork = nullptr;
     size_t gwork_bytes = 0;
     // graph cache: the kernel arguments and the two input blocks that the
@@ -678,11 +680,14 @@ ffspmv_status sequence_per_launch(ffspmv_handle *h, SeqState &q, const u32 *X, c
     const Mod M = make_mod(h->m, 1, 0);
     // m > 2^16 and a format of the library's choice: one launch per step on the
     // block layout (4 001 rows, s = 8, p = 2^31 - 1: 6.4 us per step against
-    // 14.1 with a projection, its finish and the plan's product); the layout
-    // has to be there or worth building
+    // 14.1 with a projection, its finish and the plan's product).  The layout
+    // has to be there or worth building: that takes 0.4 ms at 4 000 rows, 12 ms at
+    // a million, what 20 to 60 steps gain (s = 1 to 16).  Steps of earlier calls
+    // count (a sequence resumed piece by piece)
     const BlockPlan *B = nullptr;
+    q.steps = std::min<long long>(q.steps + nsteps, 1LL << 40);
     if (h->m > 65536u && n > 0 && h->opt.sequence_mode == 0 && h->opt.priority_format == FFSPMV_FMT_AUTO &&
-        nsteps > 0 && !(h->opt.test_hooks & 12) && (h->block[0] || nsteps >= 16))
+        nsteps > 0 && !(h->opt.test_hooks & 12) && (h->block[0] || q.steps >= kSeqBuildSteps))
         B = ensure_block(h, false, nullptr, 0, 0, st);
     const int ldv = B ? (s + 3) / 4 * 4 : s;
     size_t vb = ((size_t)n * ldv * 4 + 255) / 256 * 256 + 256;
