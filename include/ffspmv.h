@@ -103,7 +103,8 @@ typedef struct {
                                   the 2- and 4-vector passes, without the timing that decides it;
                                   bit 3 = x-panel blocks never take them (one-vector passes);
                                   bit 4 = the first attempt at a block layout of A, and of A^T,
-                                  finds no device memory */
+                                  finds no device memory; bit 5 = a block sequence finds none
+                                  for its steps on the block layout */
     int32_t panel_cluster;     /* x-panel layout: CTAs per cluster (column groups); 0 = chosen by
                                   the builder, 1, 2 or 4 to force one */
 } ffspmv_options;

@@ -689,15 +689,25 @@ ffspmv_status sequence_per_launch(ffspmv_handle *h, SeqState &q, const u32 *X, c
     if (h->m > 65536u && n > 0 && h->opt.sequence_mode == 0 && h->opt.priority_format == FFSPMV_FMT_AUTO &&
         nsteps > 0 && !(h->opt.test_hooks & 12) && (h->block[0] || q.steps >= kSeqBuildSteps))
         B = ensure_block(h, false, nullptr, 0, 0, st);
-    const int ldv = B ? (s + 3) / 4 * 4 : s;
-    size_t vb = ((size_t)n * ldv * 4 + 255) / 256 * 256 + 256;
-    size_t need = 2 * vb + std::max((size_t)s * s * 8, B ? block_steps_bytes(n, s) : 0) + 256;
-    if (need > q.gwork_bytes) {
+    int ldv = s;
+    size_t vb = 0;
+    for (;;) {
+        ldv = B ? (s + 3) / 4 * 4 : s;
+        vb = ((size_t)n * ldv * 4 + 255) / 256 * 256 + 256;
+        const size_t need = 2 * vb + std::max((size_t)s * s * 8, B ? block_steps_bytes(n, s) : 0) + 256;
+        if (need <= q.gwork_bytes) break;
         if (q.gwork) cudaFree(q.gwork);
         q.gwork = nullptr;
         q.gwork_bytes = 0;
-        if (cudaMalloc(&q.gwork, need) != cudaSuccess) return FFSPMV_ERR_OOM;
-        q.gwork_bytes = need;
+        const bool deny = B && (h->opt.test_hooks & 32);   // testing
+        if (!deny && cudaMalloc(&q.gwork, need) == cudaSuccess) {
+            q.gwork_bytes = need;
+            break;
+        }
+        cudaGetLastError();
+        q.gwork = nullptr;
+        if (!B) return FFSPMV_ERR_OOM;
+        B = nullptr;   // the layout's steps take up to four times the rows of V at s < 4: without it, then
     }
     u32 *V[2] = {(u32 *)q.gwork, (u32 *)((char *)q.gwork + vb)};
     u64 *Sacc = (u64 *)((char *)q.gwork + 2 * vb);

@@ -43,3 +43,15 @@ def test_short_sequences_build_together(lib):
         assert ("blocks:" in M.describe()) == (k > 2)      # 16, 32, then 48 steps
         got.append(to_host(M.resume_sequence(to_dev(X), V, 16 * k, 16)))
     assert np.array_equal(np.concatenate(got), want) and np.array_equal(to_host(V), Vw)
+
+
+@pytest.mark.parametrize("s", [1, 7, 16])
+def test_no_memory_for_the_steps(lib, s):
+    # test hook 32: the scratch of the layout's steps cannot be had
+    m = 2**31 - 1
+    A, X, Y = _case(700, s, m)
+    M = lib.Matrix.from_csr(A, transpose_mode=lib.TRANSPOSE.NONE, test_hooks=32)
+    want, Vw = oracle.csr_block_sequence(A, X, Y, 50, want_next=True)
+    for _ in range(2):
+        S, V = M.block_sequence(to_dev(X), to_dev(Y), 50, want_next=True)
+        assert np.array_equal(to_host(S), want) and np.array_equal(to_host(V), Vw)
