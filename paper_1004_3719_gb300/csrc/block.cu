@@ -986,6 +986,7 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
         B.n = b[j].n;
         B.ncols = J.transpose ? J.h->A.nrows : J.h->A.ncols;
         B.small = b[j].small != 0;
+        B.nsm = std::max(nsm, 1);
         B.nlong = (long long)(cur[kBlockClasses] >> 32);
         B.nchunk = (long long)cur[kBlockClasses + 1];
         u64 quads = cur[kBlockClasses] & 0xffffffffull, rows = 0;
@@ -1295,7 +1296,7 @@ static long long block_warps(const BlockPlan &B, BlockArgs &a)
             const int rpw = 32 >> (a.m.lgt + lg);
             warps += (B.cls_row[c + 1] - B.cls_row[c] + rpw - 1) / rpw;
         }
-        if (warps >= 16 * 152) break;
+        if (warps >= 16LL * B.nsm) break;
     }
     a.row0[kBlockClasses] = (u32)B.cls_row[kBlockClasses];
     a.warp0[kBlockClasses] = (u32)warps;

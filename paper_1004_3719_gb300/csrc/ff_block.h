@@ -48,6 +48,7 @@ struct BlockPlan {
     void *arena = nullptr;
     long long n = 0, ncols = 0;
     bool small = true;                 // m <= 2^16: u16 values and staged x
+    int nsm = 1;                       // the device's SMs
     long long nlong = 0, nchunk = 0;   // rows split over warps, and their chunks
     long long cls_row[kBlockClasses + 1] = {};  // rows of class c: [cls_row[c], cls_row[c + 1]) of row / ptr
     const u32 *ptr = nullptr;          // [n - nlong + 1] offsets in quads, rows in class order
