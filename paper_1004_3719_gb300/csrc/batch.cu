@@ -77,7 +77,10 @@ static ffspmv_status batch_apply(int32_t count, const ffspmv_t *hs, const uint32
     }
     for (int j = 0; j < count; ++j) {
         if (round[j] >= 0 || hs[j]->A.nrows == 0) continue;
-        const ffspmv_status s = run_plan(hs[j]->A, d_x[j], nvec[j], d_y[j], nvec[j], nvec[j], hs[j]->m, 1, 0, st);
+        PanelCtl ctl;   // an x-panel plan's waits report to the handle, as in spmv_apply
+        ctl.status = hs[j]->d_status + 2;
+        ctl.skip_stage = (hs[j]->opt.test_hooks & 2) ? 1 : -1;
+        const ffspmv_status s = run_plan(hs[j]->A, d_x[j], nvec[j], d_y[j], nvec[j], nvec[j], hs[j]->m, 1, 0, st, &ctl);
         if (s != FFSPMV_OK) return s;
     }
     std::vector<const BlockPlan *> B;

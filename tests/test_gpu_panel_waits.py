@@ -59,3 +59,17 @@ def test_ctas_of_a_cluster_with_uneven_work(lib, m, q, n):
         want = oracle.csr_spmv(A, x)
         for y in ys:
             assert np.array_equal(to_host(y).reshape(want.shape), want)
+
+
+def test_batch_without_a_layout_reports_a_wait_that_ran_out(lib):
+    # no memory for the block layout (hook 16), so the x-panel plan runs, without its copies (hook 2)
+    A = gen.powerlaw_matrix(seed=8, n=150_001, lmax=10_000, m=65521)
+    M = lib.Matrix.from_csr(A, priority_format=lib.FMT.PANEL, transpose_mode=lib.TRANSPOSE.NONE, test_hooks=2 | 16)
+    x, y = to_dev(rand_block(5, A.ncols, 1, 65521)), to_dev(np.zeros(A.nrows, dtype=np.uint32))
+    lib.spmv_batch_apply([M.handle], [x], [y], [1])
+    with pytest.raises(lib.FFSPMVError) as e:
+        M.check_status()
+    assert e.value.status == 6
+    lib.spmv_batch_apply([M.handle], [x], [y], [1])     # on its layout now
+    M.check_status()
+    assert np.array_equal(to_host(y), oracle.csr_spmv(A, to_host(x)))
