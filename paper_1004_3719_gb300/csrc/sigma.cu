@@ -75,7 +75,7 @@ constexpr int kSbThreads = 32 * kSbWarps;
 constexpr int kSbSend = 32 * (kSbWarps - kSbElim);
 constexpr int kSbApply = 6;                 // CTAs that apply the operations to P and to R's later coefficients
 constexpr int kSbCtas = 1 + kSbApply;
-constexpr int kSbPolls = 256;               // tries of a wait before it looks at the clock
+constexpr u32 kSbPolls = 64;                // tries of a wait between two looks at the clock
 constexpr u64 kSbWaitNs = 700ull * 1000 * 1000, kSbDrainNs = 50ull * 1000 * 1000;   // its limit; that of messages in flight
 constexpr size_t kSbSmemMax = 227 * 1024;
 constexpr size_t kSbAlign = 256;
@@ -217,37 +217,25 @@ __device__ __forceinline__ void sb_bar_init(u32 bar, u32 bytes)
     asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// The rare rest of sb_bar_wait: `ns` nanoseconds of tries that return at once.
-__device__ __noinline__ bool sb_bar_wait_on(u32 bar, u64 ns)
-{
-    u32 ok;
-    const u64 t0 = global_ns();
-    do {
-        asm volatile("{\n.reg .pred q;\nmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n"
-                     "selp.u32 %0, 1, 0, q;\n}"
-                     : "=r"(ok)
-                     : "r"(bar)
-                     : "memory");
-        if (ok) return true;
-        __nanosleep(64);
-    } while (global_ns() - t0 < ns);
-    return false;
-}
-
-// Every mbarrier is used once.  False when the wait ran out: after kSbPolls
-// tries, which the hardware may draw out, and `ns` nanoseconds.
+// Every mbarrier is used once.  False when the wait ran out: `ns` nanoseconds
+// after the first kSbPolls tries (the clock is read every kSbPolls tries; the
+// hardware may draw each of them out).
 __device__ __forceinline__ bool sb_bar_wait(u32 bar, u64 ns = kSbWaitNs)
 {
-    u32 ok;
-    for (int i = 0; i < kSbPolls; ++i) {
+    u64 t0 = 0;
+    for (u32 i = 1;; ++i) {
+        u32 ok;
         asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n"
                      "selp.u32 %0, 1, 0, q;\n}"
                      : "=r"(ok)
                      : "r"(bar)
                      : "memory");
         if (ok) return true;
+        if (i % kSbPolls) continue;
+        const u64 t = global_ns();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > ns) return false;
     }
-    return sb_bar_wait_on(bar, ns);
 }
 
 __device__ __forceinline__ void sb_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
