@@ -26,6 +26,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <thread>
 #include <type_traits>
 
 #include "ff_internal.cuh"
@@ -794,42 +795,97 @@ ffspmv_status block_limits(const BlockJob &J)
     return FFSPMV_OK;
 }
 
-// Uploads of a handle's arrays go through page-locked memory: the copy engine
-// reads pageable memory page by page, and where the host's pages are small (a
-// machine that has been up for a while) that is 3 GB/s: 126 MB of a 15.8M-entry
-// matrix took 1.6 ms to 45 ms.  Through two slots of kUpSlot bytes, filled by
-// the host while the other one is sent: 9 ms.  One buffer for the process,
-// taken in turn, given back with the last handle.
-constexpr size_t kUpSlot = 2 << 20, kUpDirect = 64 * 1024;   // smaller copies leave the host's memory at once
+// Uploads of a handle's arrays go through page-locked memory.  The copy engine
+// reads pageable memory at 130 GB/s on a good day, but it makes the pages it
+// touches candidates for migration, and once that has begun the 126 MB of a
+// 15.8M-entry matrix take 20 to 45 ms.  Here kUpLanes host threads fill a slot
+// each and send it (one thread copies 12 to 16 GB/s, four 55): 5.3 ms for the
+// whole first block.  Builds of less than kUpLeast bytes do without: locking the
+// buffer and starting the threads takes 0.5 ms (2.7M entries: 0.8 ms without on a
+// good day, 1.3 with).
+constexpr int kUpLanes = 4;
+constexpr size_t kUpSlot = 1 << 20, kUpDirect = 64 * 1024;   // smaller copies leave the host's memory at once
+constexpr size_t kUpLeast = 32 << 20;
 
-struct BlockRing {
-    std::mutex use;
+// What the library keeps while it has handles: that buffer, used by one build at
+// a time, and per device a pool for the builds' temporary memory (up to
+// kKeepPool bytes of it: a default pool gives all of it back at once, 0.2 ms).
+constexpr int kKeepDevices = 16;
+constexpr unsigned long long kKeepPool = 32ull << 20;
+struct BlockKeep {
+    std::mutex use;      // of buf
+    std::mutex state;    // of the rest
     long long handles = 0;
     char *buf = nullptr;
+    cudaMemPool_t pool[kKeepDevices] = {};
 };
-BlockRing &block_ring()
+BlockKeep &block_keep()
 {
-    static BlockRing *r = new BlockRing();   // (outlives the handles of a process that ends without freeing them)
-    return *r;
+    static BlockKeep *k = new BlockKeep();   // (outlives the handles of a process that ends without freeing them)
+    return *k;
+}
+
+// The current device's pool; null: the default one.
+cudaMemPool_t block_pool()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kKeepDevices) return nullptr;
+    BlockKeep &K = block_keep();
+    std::lock_guard<std::mutex> lock(K.state);
+    if (!K.pool[dev]) {
+        cudaMemPoolProps p = {};
+        p.allocType = cudaMemAllocationTypePinned;
+        p.location.type = cudaMemLocationTypeDevice;
+        p.location.id = dev;
+        unsigned long long keep = kKeepPool;
+        if (cudaMemPoolCreate(&K.pool[dev], &p) != cudaSuccess) {
+            cudaGetLastError();
+            K.pool[dev] = nullptr;
+        } else {
+            cudaMemPoolSetAttribute(K.pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+        }
+    }
+    return K.pool[dev];
 }
 
 class BlockUpload {
+    struct Piece {
+        char *dst;
+        const char *src;
+        size_t bytes;
+    };
     std::unique_lock<std::mutex> lock;
+    std::vector<Piece> pieces;   // at most kUpSlot bytes each
     cudaStream_t st;
-    cudaEvent_t sent[2] = {nullptr, nullptr};
+    cudaEvent_t sent[kUpLanes] = {};
     char *buf = nullptr;
-    int slot = 0;
+
+    // pieces k, k + kUpLanes, ... through slot k
+    cudaError_t lane(int k) const
+    {
+        char *h = buf + (size_t)k * kUpSlot;
+        for (size_t i = (size_t)k; i < pieces.size(); i += kUpLanes) {
+            const Piece &p = pieces[i];
+            cudaError_t e = cudaEventSynchronize(sent[k]);   // (never recorded: done)
+            if (e != cudaSuccess) return e;
+            memcpy(h, p.src, p.bytes);
+            if ((e = cudaMemcpyAsync(p.dst, h, p.bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
+            if ((e = cudaEventRecord(sent[k], st)) != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
 
 public:
     BlockUpload(cudaStream_t s, size_t bytes) : st(s)
     {
-        if (bytes < kUpDirect) return;
-        BlockRing &R = block_ring();
-        lock = std::unique_lock<std::mutex>(R.use);
-        if (!R.buf && cudaHostAlloc((void **)&R.buf, 2 * kUpSlot, cudaHostAllocPortable) != cudaSuccess) R.buf = nullptr;
-        if (R.buf && cudaEventCreateWithFlags(&sent[0], cudaEventDisableTiming) == cudaSuccess &&
-            cudaEventCreateWithFlags(&sent[1], cudaEventDisableTiming) == cudaSuccess)
-            buf = R.buf;
+        if (bytes < kUpLeast) return;
+        pieces.reserve(bytes / kUpSlot + 64);
+        BlockKeep &K = block_keep();
+        lock = std::unique_lock<std::mutex>(K.use);
+        if (!K.buf && cudaHostAlloc((void **)&K.buf, kUpLanes * kUpSlot, cudaHostAllocPortable) != cudaSuccess) K.buf = nullptr;
+        bool ok = K.buf != nullptr;
+        for (cudaEvent_t &e : sent) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+        if (ok) buf = K.buf;
         cudaGetLastError();   // (without it: ordinary copies)
     }
     ~BlockUpload()
@@ -839,6 +895,8 @@ public:
             if (e) cudaEventDestroy(e);
     }
     BlockUpload(const BlockUpload &) = delete;
+
+    // The copy is made by send() unless it is small.
     ffspmv_status copy(void *dst, const void *src, size_t bytes)
     {
         if (!bytes) return FFSPMV_OK;
@@ -846,14 +904,32 @@ public:
             FF_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st));
             return FFSPMV_OK;
         }
-        for (size_t at = 0; at < bytes; at += kUpSlot, slot ^= 1) {
-            const size_t n = std::min(kUpSlot, bytes - at);
-            char *h = buf + slot * kUpSlot;
-            FF_CUDA(cudaEventSynchronize(sent[slot]));   // (never recorded: done)
-            memcpy(h, (const char *)src + at, n);
-            FF_CUDA(cudaMemcpyAsync((char *)dst + at, h, n, cudaMemcpyHostToDevice, st));
-            FF_CUDA(cudaEventRecord(sent[slot], st));
+        for (size_t at = 0; at < bytes; at += kUpSlot)
+            pieces.push_back({(char *)dst + at, (const char *)src + at, std::min(kUpSlot, bytes - at)});
+        return FFSPMV_OK;
+    }
+    ffspmv_status send()
+    {
+        cudaError_t err[kUpLanes] = {};
+        std::thread helper[kUpLanes];
+        int dev = 0;
+        cudaGetDevice(&dev);
+        // a thread is worth starting for a few pieces
+        const int helpers = pieces.size() >= 4 * kUpLanes ? kUpLanes - 1 : 0;
+        for (int k = 0; k < helpers; ++k)
+            try {
+                helper[k] = std::thread([this, k, dev, &err] {
+                    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+                    cudaThreadExchangeStreamCaptureMode(&mode);
+                    if ((err[k] = cudaSetDevice(dev)) == cudaSuccess) err[k] = lane(k);
+                });
+            } catch (const std::exception &) {   // no thread: this one does it
+            }
+        for (int k = kUpLanes - 1; k >= 0; --k) {
+            if (helper[k].joinable()) helper[k].join();
+            else err[k] = lane(k);
         }
+        for (cudaError_t e : err) FF_CUDA(e);
         return FFSPMV_OK;
     }
 };
@@ -936,7 +1012,8 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
             most = std::max(most, std::max(n, jobs[j].h->A.nrows));
         }
     const size_t o_start = starts[0];
-    if (cudaMallocAsync(&S.tmp, o, st) != cudaSuccess) {
+    const cudaMemPool_t pool = block_pool();
+    if ((pool ? cudaMallocFromPoolAsync(&S.tmp, o, pool, st) : cudaMallocAsync(&S.tmp, o, st)) != cudaSuccess) {
         cudaGetLastError();
         S.tmp = nullptr;
         return FFSPMV_ERR_OOM;
@@ -964,6 +1041,7 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
     ffspmv_status r = to_device.copy(t, up.data(), packed);
     for (const Array &a : arr)
         if (r == FFSPMV_OK && a.bytes >= kPack) r = to_device.copy(t + a.at, a.src, a.bytes);
+    if (r == FFSPMV_OK) r = to_device.send();
     if (r != FFSPMV_OK) return r;
     FF_CUDA(cudaMemsetAsync(t + o_len, 0, o_start - o_len, st));
     int dev = 0, nsm = 0;
@@ -1113,12 +1191,16 @@ ffspmv_status make_block(const ffspmv_handle *h, bool transpose, bool odd, int l
 
 void block_handles(int more)
 {
-    BlockRing &R = block_ring();
-    std::lock_guard<std::mutex> use(R.use);
-    R.handles += more;
-    if (R.handles == 0 && R.buf) {
-        cudaFreeHost(R.buf);
-        R.buf = nullptr;
+    BlockKeep &K = block_keep();
+    std::lock_guard<std::mutex> state(K.state);
+    K.handles += more;
+    if (K.handles) return;
+    // no handle, so no build
+    if (K.buf) cudaFreeHost(K.buf);
+    K.buf = nullptr;
+    for (cudaMemPool_t &p : K.pool) {
+        if (p) cudaMemPoolDestroy(p);
+        p = nullptr;
     }
 }
 
