@@ -890,7 +890,7 @@ public:
     }
     ~BlockUpload()
     {
-        if (buf) cudaStreamSynchronize(st);   // the next build may fill the slots
+        cudaStreamSynchronize(st);   // the next build may fill the slots, the sources may go
         for (cudaEvent_t e : sent)
             if (e) cudaEventDestroy(e);
     }
@@ -1033,7 +1033,10 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
         b[j].odd = J.odd ? 1 : 0;
         b[j].transpose = J.transpose ? 1 : 0;
     }
+    // host ends of copies, here so that none is freed while one goes on
+    // (to_device waits for the stream when it goes)
     std::vector<char> up(packed, 0);
+    std::vector<u64> curs((size_t)kBlockCursors * count);
     memcpy(up.data(), b.data(), sizeof(BlockBuild) * b.size());
     for (const Array &a : arr)
         if (a.bytes && a.bytes < kPack) memcpy(up.data() + a.at, a.src, a.bytes);
@@ -1052,7 +1055,6 @@ ffspmv_status build_blocks(BlockJob *jobs, int count, BlockScope &S)
     k_block_lengths<<<grid, kBlockThreads, 0, st>>>(dj);
     k_block_place<<<grid, kBlockThreads, 0, st>>>(dj, 0);
     FF_CUDA(cudaGetLastError());
-    std::vector<u64> curs((size_t)kBlockCursors * count);
     FF_CUDA(cudaMemcpyAsync(curs.data(), t + o_cur, sizeof(u64) * curs.size(), cudaMemcpyDeviceToHost, st));
     FF_CUDA(cudaStreamSynchronize(st));
     for (int j = 0; j < count; ++j) {
