@@ -18,17 +18,17 @@ extern "C" {
 #endif
 
 /*
- * Device workspace that polymat_mul needs for these sizes (bytes, written
- * to *bytes).  1 <= s <= 32, da, db >= 0; FFSPMV_ERR_UNSUPPORTED when
- * da + db + 1 > 2^15 (the transform length is limited by shared memory).
+ * Device workspace that polymat_mul needs for these sizes at any p (bytes,
+ * written to *bytes).  1 <= s <= 32, da, db >= 0; FFSPMV_ERR_UNSUPPORTED when
+ * da + db + 1 > 2^15 (the longest transform: two axes of at most 256 points).
  */
 ffspmv_status polymat_mul_workspace(int32_t s, int64_t da, int64_t db, int64_t *bytes);
 
 /*
  * d_C = d_A * d_B mod p (device arrays as above; d_C must not overlap the
  * inputs).  2 <= p <= 2^31; inputs must be below p.  The exact integer
- * coefficients are computed modulo three primes by number-theoretic
- * transforms and recombined by the Chinese remainder theorem, which needs
+ * coefficients are computed modulo as many of three primes as they need, by
+ * number-theoretic transforms and the Chinese remainder theorem, which takes
  * s * (min(da, db) + 1) * (p - 1)^2 < 998244353 * 167772161 * 469762049
  * (about 2^86), else FFSPMV_ERR_UNSUPPORTED.  d_work: device memory of at
  * least polymat_mul_workspace bytes, 16-byte aligned, owned by the caller

@@ -6,13 +6,13 @@
 // looks its matrix up in the launch parameters), so another set of handles that
 // have their layouts costs nothing but the call.  Layouts that are missing are
 // built together first: a first batch over 48 new handles of 200 to 5 000 rows
-// takes 2.1 ms (4.6 with the work list described below, 5.0 with a build for
-// each), of 1 000 to 200 000 rows 25 ms (60).
+// takes 1.9 ms (4.6 with the work list described below, 5.0 with a build for
+// each), of 1 000 to 200 000 rows 13 ms (60).
 //
 // Measured, 48 problems of 1 000 to 200 000 rows, 1 to 32 vectors, primes near
-// 2^31, another set of handles on every call: 22.9 ms with a work list that
-// was rebuilt, uploaded and timed in six tile shapes for each new set, 0.47 ms
-// here; the same set again: 512 us before, 427 us now.
+// 2^31, handles with their layouts, another set on every call: 23.4 ms with a work
+// list that was rebuilt, uploaded and timed in six tile shapes for each new set,
+// 0.41 ms here; the same set again 0.51 ms and 0.41.
 #include <algorithm>
 #include <exception>
 #include <vector>

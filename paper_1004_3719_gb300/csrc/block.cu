@@ -1240,7 +1240,7 @@ void ensure_blocks(int count, ffspmv_handle *const *hs, const u32 *const *x, con
 {
     // builds share a stream and two waits, as many as fit this much temporary
     // memory: the first batch over 48 handles of 200 to 5 000 rows takes 11.6 ms
-    // with a build each, 2.1 so
+    // with a build each, 1.9 so
     constexpr size_t kTogether = (size_t)64 << 20;
     if (capturing(st)) return;
     std::vector<BlockJob> jobs;

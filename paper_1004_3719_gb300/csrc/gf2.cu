@@ -17,7 +17,7 @@
 // The gathers bound it: one random L2 sector per entry, 63 us for 15.8M at 250 G
 // sectors/s.  1M power-law pattern, 64 / 256 vectors: 91 / 211 us with a lane
 // group per short row, a second launch for the long rows and 8-byte offsets;
-// 66 / 87 us here (16 words: 1359 -> 302).
+// 66 / 82 us here (16 words: 1359 -> 302).
 #include <algorithm>
 
 #include "ff_block.h"

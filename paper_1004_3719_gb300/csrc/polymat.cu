@@ -850,6 +850,7 @@ extern "C" ffspmv_status polymat_mul_workspace(int32_t s, int64_t da, int64_t db
     if (!bytes || s < 1 || s > 32 || da < 0 || db < 0) return FFSPMV_ERR_ARG;
     if (da + db + 1 > (1LL << kPmMaxLog)) return FFSPMV_ERR_UNSUPPORTED;
     const long long L = 1LL << pm_log2(da + db + 1);
+    // the planes for any p (three primes); the rest is no longer used, but callers know the size
     *bytes = 3LL * kPmPrimes * s * s * L * 4 + (long long)kPmPrimes * L * 8 + 256;
     return FFSPMV_OK;
 }

@@ -679,8 +679,8 @@ ffspmv_status sequence_per_launch(ffspmv_handle *h, SeqState &q, const u32 *X, c
     const long long n = h->A.nrows;
     const Mod M = make_mod(h->m, 1, 0);
     // m > 2^16 and a format of the library's choice: one launch per step on the
-    // block layout (4 001 rows, s = 8, p = 2^31 - 1: 6.4 us per step against
-    // 14.1 with a projection, its finish and the plan's product).  The layout
+    // block layout (4 001 rows, s = 8, p = 2^31 - 1: 5.2 us per step against
+    // 17 with a projection, its finish and the plan's product).  The layout
     // has to be there or worth building: that takes 0.4 ms at 4 000 rows, 12 ms at
     // a million, what 20 to 60 steps gain (s = 1 to 16).  Steps of earlier calls
     // count (a sequence resumed piece by piece)
