@@ -419,9 +419,10 @@ static ffspmv_status next_pass(ffspmv_t h, bool transpose, const Plan *P, int le
 //     (20 000 x 20 000, 10 per row, m = 65521: 4 vectors in 10 us against 12,
 //     16 in 15.8 against 12; 90 001 x 120 011 power-law, 23 per row: 2
 //     vectors in 62 us against 17, 16 in 515 against 20).  The first such
-//     block still takes the plan: building the layout costs 0.1 to 2 ms,
-//     which a single product would not earn back (a panel plan's first block
-//     would build panel layouts instead, which takes longer).
+//     block still takes the plan: building the layout costs 0.4 ms (20 000
+//     rows) to 5 ms (15.8M entries), which a single product would not earn back
+//     (a panel plan's first block would build panel layouts instead, which takes
+//     longer).
 static BlockPlan *block_path(ffspmv_t h, bool transpose, const u32 *x, long long ldx, int nvec, cudaStream_t st,
                              bool counting = false)
 {
